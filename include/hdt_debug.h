@@ -51,8 +51,7 @@ extern "C" {
  *                    stage-1 kernel does the completion (off by default).
  *   "no_overlap"     1: the stages above 0 run after stage 0 on the caller's stream instead of
  *                    beside it on an internal stream.
- *   "no_graph"       1: hdt_build_index launches its kernels one by one instead of replaying a
- *                    cached CUDA graph.
+ *   "no_graph"       accepted and without effect (the index build is two launches; there is no graph to leave out).
  *   "no_pdl"         1: the kernels of hdt_build_index are ordinary stream successors instead of
  *                    programmatic dependents.
  *   "phase_stamps"   (only in a library built with HDT_WORKBENCH defined; otherwise ignored)

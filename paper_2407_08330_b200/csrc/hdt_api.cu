@@ -66,7 +66,6 @@ int *device_status_ptr() {
 // on first use.
 static thread_local Side g_side[64];
 int g_no_overlap = 0;
-int g_no_graph = 0;
 int g_phase_stamps = 0;
 int g_no_fwd_mc = 0;
 int g_no_pdl = 0;
@@ -90,7 +89,6 @@ int get_side(Side **out) {
         HDT_CUDA_CHECK(cudaEventCreateWithFlags(&sd.join2, cudaEventDisableTiming));
         HDT_CUDA_CHECK(cudaEventCreateWithFlags(&sd.fork0, cudaEventDisableTiming));
         HDT_CUDA_CHECK(cudaEventCreateWithFlags(&sd.join0, cudaEventDisableTiming));
-        for (int i = 0; i < 2 * HDT_MAX_STAGES; ++i) HDT_CUDA_CHECK(cudaEventCreateWithFlags(&sd.stage_ev[i], cudaEventDisableTiming));
         sd.ready = true;
     }
     *out = &sd;
@@ -176,7 +174,7 @@ extern "C" int hdt_set_option(const char *name, int32_t value) {
     if (name && std::strcmp(name, "no_persistent") == 0) { g_no_persistent = value; return HDT_OK; }
     if (name && std::strcmp(name, "simt_upper") == 0) { g_simt_upper = value; return HDT_OK; }
     if (name && std::strcmp(name, "no_overlap") == 0) { g_no_overlap = value; return HDT_OK; }
-    if (name && std::strcmp(name, "no_graph") == 0) { g_no_graph = value; return HDT_OK; }
+    if (name && std::strcmp(name, "no_graph") == 0) return HDT_OK;
     if (name && std::strcmp(name, "phase_stamps") == 0) { g_phase_stamps = value; return HDT_OK; }
     if (name && std::strcmp(name, "no_fused_delta") == 0) { g_no_fused_delta = value; return HDT_OK; }
     if (name && std::strcmp(name, "no_fold") == 0) { g_no_fold = value; return HDT_OK; }

@@ -1,15 +1,22 @@
 // Device-side index builder: (level, parent, cu_seqlens) -> staged family ranges, row blocks,
 // work queues.  Integer work only; every array must equal the sequential definition bit for bit.
 //
+// Two launches, whatever the number of stages:
+//   k_seq     one CTA per sequence, its arrays in shared memory: validation, child counts, family
+//             ranges, compaction to the next stage, greedy packing of row blocks, block records - for
+//             all stages of the sequence, in sequence-relative numbers, beside the counts of the stage
+//   k_finish  adds the sequences' offsets (sums over the sequences before it), ranks the blocks of a
+//             stage by cost (longest first), and sends the header to the host
 // Per stage (array of n elements in document order):
-//   count     cnt[p] = children of p; nlc[p] = children of p that have children
+//   counts    cnt[p] = children of p, and whether one of them has children
 //   ranges    a node whose children are all childless heads a family; head and children get
 //             their key range; children of heads (and PAD) are removed for the next stage
-//   scan      exclusive prefix sum of the keep flags -> position in the next stage's array
-//   compact   tok / par / sequence offsets of the next stage
-//   walk      greedy packing of row blocks per sequence (one CTA per sequence, list in smem)
-//   blocks    per block key span, flags, cost
-//   queue     rank sort by cost (longest first)
+//   compact   tok / par of the kept elements in the next stage's array
+//   walk      greedy packing of row blocks
+// What bounds it: latency (about 40 bytes a token move; a chain of barriers and shared-memory round
+// trips per stage).  The stages of a sequence only meet the other sequences' in their offsets, so the
+// grid-wide steps (formerly nine launches for three stages and a hundred for twenty, each a launch
+// latency behind the one before) are one kernel boundary.
 #include <cstdio>
 #include <cstring>
 #include <atomic>
@@ -20,39 +27,39 @@
 
 namespace hdt {
 
-static constexpr int CHUNK = 1024;  // elements per CTA in the element-wise kernels
+// What k_seq leaves about one sequence for k_finish.
+struct SeqInfo {
+    int stages;                // stages this sequence's own hierarchy needs (at least 1)
+    int res;                   // elements it still has in any later stage of the batch: its root, or nothing
+    int err, err_pos;          // structure error, 0 = none
+    int more, pad;             // elements were left after the last allowed stage
+    long long nnz, visited;
+};
 
 struct Layout {
-    size_t header, cnt, nlc, pre, keep, fpos, blocksum, bstart, seqcount, cost, stage0, stage_stride;
-    size_t fpos2, bstart2, seqcount2, cost2;   // second set for the upper stages, built beside stage 0's blocks
-    size_t rank;                               // per token: its number among its siblings (written where its family is found)
+    size_t header, info, counts, rank, recs, el, upl, glob, keys, stage0, stage_stride;
     size_t s_tok, s_par, s_rng, s_up, s_scu, s_blocks, s_queue, s_queue2;  // offsets inside a stage
     size_t total;
-    int capnb, nchunk;
+    int capnb;
 };
 
 static size_t al(size_t x) { return (x + 255) & ~size_t(255); }
 
+static constexpr int NGLOB = 9;      // element arrays of the sequences that do not fit in shared memory
+
 static Layout make_layout(int B, int T, int bm, int max_stages) {   // bm: the smaller of the two block sizes
     Layout L;
     L.capnb = 2 * (T / bm + 1) + 4 * B + 2;
-    L.nchunk = (T + CHUNK - 1) / CHUNK + 1;
     size_t o = 0;
     L.header = o; o += al(sizeof(DevHeader));
-    L.cnt = o; o += al(sizeof(int) * (size_t)T);
-    L.nlc = o; o += al(sizeof(int) * (size_t)T);
-    L.pre = o; o += al(sizeof(int) * (size_t)T);
-    L.keep = o; o += al((size_t)T);
-    L.fpos = o; o += al((size_t)T);
-    L.blocksum = o; o += al(sizeof(int) * (size_t)L.nchunk);
-    L.bstart = o; o += al(sizeof(int) * (size_t)L.capnb);
-    L.seqcount = o; o += al(sizeof(int) * (size_t)(B + 1));
-    L.cost = o; o += al(sizeof(long long) * (size_t)L.capnb);
-    L.fpos2 = o; o += al((size_t)T);
-    L.bstart2 = o; o += al(sizeof(int) * (size_t)L.capnb);
-    L.seqcount2 = o; o += al(sizeof(int) * (size_t)(B + 1));
-    L.cost2 = o; o += al(sizeof(long long) * (size_t)L.capnb);
+    L.info = o; o += al(sizeof(SeqInfo) * (size_t)B);
+    L.counts = o; o += al(sizeof(int) * 4 * (size_t)max_stages * B);
     L.rank = o; o += al(sizeof(int) * (size_t)T);
+    L.recs = o; o += al(sizeof(int4) * (size_t)max_stages * L.capnb);
+    L.keys = o; o += al(sizeof(long long) * (size_t)max_stages * L.capnb);
+    L.el = o; o += al(sizeof(int4) * (size_t)(max_stages - 1) * T);
+    L.upl = o; o += al(sizeof(int) * (size_t)(max_stages - 1) * T);
+    L.glob = o; o += NGLOB * al(sizeof(int) * (size_t)T);
     L.stage0 = o;
     size_t s = 0;
     L.s_tok = s; s += al(sizeof(int) * (size_t)T);
@@ -68,66 +75,10 @@ static Layout make_layout(int B, int T, int bm, int max_stages) {   // bm: the s
     return L;
 }
 
-__device__ __forceinline__ void dev_fail(DevHeader *h, int code, int pos) {
-    if (atomicCAS(&h->status, 0, code) == 0) h->err_pos = pos;
-}
+// First block slot of a sequence that starts at token c: a walk packs two consecutive blocks into
+// more than bm elements, so a sequence of n elements has at most 2 ceil(n / bm) + 1 blocks.
+__device__ __forceinline__ int block_slot(int c, int b, int bm) { return 2 * (c / bm) + 4 * b; }
 
-// ---------------------------------------------------------------------------------------------
-// stage 0 set-up: validation of the caller's arrays, global parent indices
-// ---------------------------------------------------------------------------------------------
-__global__ void k_init(const int8_t *__restrict__ level, const int32_t *__restrict__ parent,
-                       const int32_t *__restrict__ cu, int B, int T, int max_level, DevHeader *hdr,
-                       int *tok, int *par, int *scu, int *cnt, int *nlc) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i <= B) {
-        const int c = cu[i];
-        scu[i] = c;
-        if (i == 0 && c != 0) dev_fail(hdr, HDT_ERR_BAD_HIERARCHY, 0);
-        if (i == B && c != T) dev_fail(hdr, HDT_ERR_BAD_HIERARCHY, B);
-        if (i < B && cu[i + 1] < c) dev_fail(hdr, HDT_ERR_BAD_HIERARCHY, i);
-        if (c < 0 || c > T) dev_fail(hdr, HDT_ERR_BAD_HIERARCHY, i);
-    }
-    if (i == 0) hdr->st[0].n = T;
-    if (i >= T) return;
-    // sequence of token i: last b with cu[b] <= i  (cu clamped so a bad cu cannot fault)
-    int lo = 0, hi = B;  // invariant: cu[lo] <= i
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (cu[mid] <= i) lo = mid; else hi = mid;
-    }
-    const int s0 = min(max(cu[lo], 0), T);
-    const int r = i - s0;
-    const int l = level[i], p = parent[i];
-    int gp = -1;
-    bool ok = true;
-    if (l < 0) {
-        ok = (l == -1 && p == -1);
-    } else {
-        if (l > max_level) ok = false;
-        if (r <= 0) {
-            ok = ok && (r == 0 && l == 0 && p == -1);
-        } else {
-            if (p < 0 || p >= r) ok = false;
-            else {
-                gp = s0 + p;
-                if ((int)level[gp] != l - 1) ok = false;
-            }
-            if ((int)level[i - 1] < 0) ok = false;  // PAD only as a suffix
-        }
-    }
-    if (!ok) { dev_fail(hdr, HDT_ERR_BAD_HIERARCHY, i); gp = -1; }
-    tok[i] = i;
-    par[i] = gp;
-    // cnt and nlc were zeroed with the header.  nlc[x] = children of x that have children: the first
-    // child to register with its parent reports that parent to the grandparent, once per parent
-    // (no second pass over the elements after the counts are complete).
-    if (gp >= 0 && atomicAdd(&cnt[gp], 1) == 0) {
-        const int pg = parent[gp];
-        if (pg >= 0 && pg < gp - s0) atomicAdd(&nlc[s0 + pg], 1);   // (gp's own thread reports a bad entry)
-    }
-}
-
-// One CTA per CHUNK elements (needed for the per-chunk keep counts).
 // Keys of row e with range [lo, hi) that the direction bits keep.  A row whose range starts at or
 // after itself is the head of its family (the keys after it are its children); otherwise lo is
 // the row's parent and the remaining keys are its siblings.  dirs: 1 = child -> parent,
@@ -138,582 +89,668 @@ __device__ __forceinline__ int row_pairs(int e, int lo, int hi, int dirs) {
     return 1 + ((dirs & 1) ? 1 : 0) + ((dirs & 2) ? hi - lo - 2 : 0);
 }
 
-__global__ void __launch_bounds__(CHUNK)
-k_ranges(DevHeader *hdr, int s, const int8_t *__restrict__ level /* stage 0 only */,
-         const int *__restrict__ par, const int *__restrict__ cnt, const int *__restrict__ nlc,
-         int *rng, uint8_t *keep, uint8_t *fpos, int *blocksum, int dirs, const int *__restrict__ tok /* nullptr: identity */,
-         int *rank) {
-    pdl_launch_dependents();      // the kernel queued behind this one may be scheduled now; it waits likewise
-    pdl_wait();                   // the kernel before this one has completed
-    const int n = hdr->st[s].n;
-    const int e = blockIdx.x * CHUNK + threadIdx.x;
-    int kp = 0;
-    long long deg = 0;
-    if (e < n) {
-        const bool real = level ? (level[e] >= 0) : true;
-        const int p = par[e], c = cnt[e];
-        const bool head = real && ((c > 0 && nlc[e] == 0) || (s == 0 && p < 0 && c == 0));
-        int lo = 0, hi = 0, fp = 0;
-        kp = real ? 1 : 0;
-        if (head) {
-            lo = (p < 0) ? e : e + 1;
-            hi = e + 1 + c;
-        } else if (p >= 0) {
-            const int cp = cnt[p];
-            if (cp > 0 && nlc[p] == 0) {  // child of a head
-                if (!(p < e && e <= p + cp)) dev_fail(hdr, HDT_ERR_BAD_HIERARCHY, e);
-                lo = p;
-                hi = p + 1 + cp;
-                fp = min(e - p, 255);
-                kp = 0;
-                rank[tok ? tok[e] : e] = e - p;     // the token's number among its siblings (hierarchical positions)
+// Element numbers and child counts of a stage: 16 bits in shared memory, 32 bits in the workspace
+// for sequences too long for it.  The top bit of a count says that a child has children itself.
+template <class I> struct Elem;
+template <> struct Elem<uint16_t> {
+    static constexpr unsigned NONE = 0xffffu, FLAG = 0x8000u, MASK = 0x7fffu;
+    static __device__ __forceinline__ void add(uint16_t *c, unsigned i) {
+        atomicAdd(reinterpret_cast<unsigned *>(c) + (i >> 1), 1u << ((i & 1) * 16));
+    }
+    static __device__ __forceinline__ void flag(uint16_t *c, unsigned i) {
+        atomicOr(reinterpret_cast<unsigned *>(c) + (i >> 1), FLAG << ((i & 1) * 16));
+    }
+};
+template <> struct Elem<uint32_t> {
+    static constexpr unsigned NONE = 0xffffffffu, FLAG = 0x80000000u, MASK = 0x7fffffffu;
+    static __device__ __forceinline__ void add(uint32_t *c, unsigned i) { atomicAdd(c + i, 1u); }
+    static __device__ __forceinline__ void flag(uint32_t *c, unsigned i) { atomicOr(c + i, FLAG); }
+};
+
+static constexpr int SEQ_CAP_MAX = 32768;   // tokens of a sequence held in shared memory (15-bit counts)
+static constexpr int SB0 = 1024, SBU = 256; // block starts of stage 0 / an upper stage held in shared memory
+
+struct SeqArgs {
+    const int8_t *level;
+    const int32_t *parent, *cu;
+    int B, T, ms, bm, bmu, bmin, dirs;
+    int cap, uc;               // tokens of stage 0 / elements of an upper stage that fit in shared memory
+    int overlay;               // the upper stages' arrays lie over stage 0's prefix sums
+    int *tok, *par, *rng, *up, *scu;     // stage 0 (final, but for `up`: relative to the sequence)
+    int *rank;
+    SeqInfo *info;
+    int *counts;               // [4][ms][B]: elements, blocks, SELF non-EMPTY blocks, EMPTY blocks
+    int4 *recs;                // [ms][capnb]: r0, a, b, rows | flags << 8, relative to the sequence
+    int capnb;
+    int4 *el;                  // [ms - 1][T]: tok, par, lo, hi of the upper stages, relative to the sequence
+    int *upl;                  // [ms - 1][T]: index in the next stage, -1 = removed
+    uint32_t *glob;            // NGLOB arrays of glob_stride elements
+    size_t glob_stride;
+};
+
+struct SeqShared {
+    int bst0[SB0], bst[SBU];
+    int wtot[32], wtotu[32];
+    int err, err_pos, flag0, flag, nb0, nb, nf0, ne0, nf, ne;
+    unsigned long long nnz, vis;
+};
+
+__device__ __forceinline__ void seq_fail(SeqShared &sh, int pos) {
+    if (atomicCAS(&sh.err, 0, HDT_ERR_BAD_HIERARCHY) == 0) sh.err_pos = pos;
+}
+
+// Barrier of the warps that build the upper stages (the last warp meanwhile walks stage 0's blocks).
+__device__ __forceinline__ void bar_upper(int n) { asm volatile("bar.sync 1, %0;" ::"r"(n) : "memory"); }
+
+// Range and fate of one element.  root_real (stage 0 only): the sequence's first token is a root, not
+// PAD; a root without children is a family of its own there.  Returns whether a family holds it as a child.
+template <class I>
+__device__ __forceinline__ bool elem_range(const I *par, const I *cnt, int e, bool stage0, bool root_real, unsigned &p, unsigned &lo,
+                                           unsigned &hi) {
+    using E = Elem<I>;
+    p = par[e];
+    const unsigned y = cnt[e], c = y & E::MASK;
+    lo = hi = 0;
+    if ((c > 0 && !(y & E::FLAG)) || (stage0 && e == 0 && c == 0 && root_real)) {
+        lo = (p == E::NONE) ? e : e + 1;
+        hi = e + 1 + c;
+    } else if (p != E::NONE) {
+        const unsigned yp = cnt[p], cp = yp & E::MASK;
+        if (cp > 0 && !(yp & E::FLAG)) {
+            lo = p;
+            hi = p + 1 + cp;
+            return true;
+        }
+    }
+    return false;
+}
+
+// Greedy packing of row blocks (one thread): a cut that would split a family which starts inside the
+// block moves to the family's head.
+template <class I>
+__device__ __forceinline__ int walk_blocks(const I *par, const I *cnt, int n, int bm, int *bst, int nbst, int4 *rec) {
+    using E = Elem<I>;
+    int pos = 0, nb = 0;
+    while (pos < n) {
+        int end = min(pos + bm, n);
+        if (end < n) {
+            const unsigned p = par[end];
+            if (p != E::NONE && (int)p > pos) {
+                const unsigned yp = cnt[p];
+                const unsigned y = cnt[end];
+                const bool head = (y & E::MASK) > 0 && !(y & E::FLAG);
+                if (!head && (yp & E::MASK) > 0 && !(yp & E::FLAG)) end = (int)p;
             }
         }
-        rng[2 * e] = lo;
-        rng[2 * e + 1] = hi;
-        keep[e] = (uint8_t)kp;
-        fpos[e] = (uint8_t)fp;
-        deg = row_pairs(e, lo, hi, dirs);
-        if (kp && p >= 0) hdr->st[s].has_next = 1;  // same value from every writer
-    }
-    // CTA reductions: keep count and nnz
-    __shared__ int s_k[32];
-    __shared__ long long s_d[32];
-    int k = kp;
-    long long d = deg;
-    for (int o = 16; o; o >>= 1) {
-        k += __shfl_xor_sync(0xffffffffu, k, o);
-        d += __shfl_xor_sync(0xffffffffu, d, o);
-    }
-    if ((threadIdx.x & 31) == 0) { s_k[threadIdx.x >> 5] = k; s_d[threadIdx.x >> 5] = d; }
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        k = s_k[threadIdx.x];
-        d = s_d[threadIdx.x];
-        for (int o = 16; o; o >>= 1) {
-            k += __shfl_xor_sync(0xffffffffu, k, o);
-            d += __shfl_xor_sync(0xffffffffu, d, o);
-        }
-        if (threadIdx.x == 0) {
-            blocksum[blockIdx.x] = k;
-            if (d) atomicAdd((unsigned long long *)&hdr->nnz, (unsigned long long)d);
-        }
-    }
-}
-
-// Exclusive scan of keep[] (per-CTA offset = sum of the chunk counts before it), next-stage tok.
-__global__ void __launch_bounds__(CHUNK)
-k_scan(DevHeader *hdr, int s, int nchunk_cap, const uint8_t *__restrict__ keep,
-       const int *__restrict__ blocksum, const int *__restrict__ tok, int *pre, int *up, int *tok2, int *cnt_clear,
-       int *nlc_clear) {
-    pdl_launch_dependents();      // the kernel queued behind this one may be scheduled now; it waits likewise
-    pdl_wait();                   // the kernel before this one has completed
-    const int n = hdr->st[s].n;
-    const int nchunk = (n + CHUNK - 1) / CHUNK;
-    if ((int)blockIdx.x >= nchunk && blockIdx.x != 0) return;
-    __shared__ int s_w[32];
-    __shared__ int s_off, s_tot;
-    // offset of this chunk and grand total
-    int part = 0, tot = 0;
-    for (int c = threadIdx.x; c < nchunk; c += CHUNK) {
-        const int v = blocksum[c];
-        tot += v;
-        if (c < (int)blockIdx.x) part += v;
-    }
-    for (int o = 16; o; o >>= 1) {
-        part += __shfl_xor_sync(0xffffffffu, part, o);
-        tot += __shfl_xor_sync(0xffffffffu, tot, o);
-    }
-    __shared__ int s_p[32], s_t[32];
-    if ((threadIdx.x & 31) == 0) { s_p[threadIdx.x >> 5] = part; s_t[threadIdx.x >> 5] = tot; }
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        part = s_p[threadIdx.x];
-        tot = s_t[threadIdx.x];
-        for (int o = 16; o; o >>= 1) {
-            part += __shfl_xor_sync(0xffffffffu, part, o);
-            tot += __shfl_xor_sync(0xffffffffu, tot, o);
-        }
-        if (threadIdx.x == 0) { s_off = part; s_tot = tot; }
-    }
-    __syncthreads();
-    const int has_next = hdr->st[s].has_next;
-    if (blockIdx.x == 0 && threadIdx.x == 0) hdr->st[s + 1].n = has_next ? s_tot : 0;
-    const int e = blockIdx.x * CHUNK + threadIdx.x;
-    const int kp = (e < n) ? keep[e] : 0;
-    // block exclusive scan
-    int v = kp;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += t;
-    }
-    if (lane == 31) s_w[w] = v;
-    __syncthreads();
-    if (w == 0) {
-        int x = s_w[lane];
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += t;
-        }
-        s_w[lane] = x;
-    }
-    __syncthreads();
-    const int excl = s_off + (w ? s_w[w - 1] : 0) + v - kp;
-    if (e < n) {
-        pre[e] = excl;
-        const int u = (kp && has_next) ? excl : -1;
-        up[e] = u;
-        if (u >= 0) tok2[u] = tok[e];
-        // (this stage's counts are dead: cleared here where k_compact goes on to count the next stage's children)
-        if (cnt_clear != nullptr) { cnt_clear[e] = 0; nlc_clear[e] = 0; }
-    }
-}
-
-// count_next: cnt and nlc were cleared by k_scan; the next stage's child counts (and nlc, as in k_init) are taken
-// here, where its parent indices are formed, instead of in a kernel of their own.
-__global__ void k_compact(const DevHeader *hdr, int s, int B, const int *__restrict__ par,
-                          const int *__restrict__ up, const int *__restrict__ pre,
-                          const int *__restrict__ scu, int *par2, int *scu2, int *cnt, int *nlc, int count_next) {
-    pdl_launch_dependents();      // the kernel queued behind this one may be scheduled now; it waits likewise
-    pdl_wait();                   // the kernel before this one has completed
-    const int n = hdr->st[s].n, n2 = hdr->st[s + 1].n;
-    const int gtid = blockIdx.x * blockDim.x + threadIdx.x, gsz = gridDim.x * blockDim.x;
-    for (int e = gtid; e < n; e += gsz) {
-        const int u = up[e];
-        if (u >= 0) {
-            const int p = par[e];
-            const int q = (p >= 0) ? pre[p] : -1;
-            par2[u] = q;
-            if (count_next && n2 > 0 && q >= 0 && atomicAdd(&cnt[q], 1) == 0) {      // (a kept element's ancestors are kept)
-                const int pp = par[p];
-                if (pp >= 0) atomicAdd(&nlc[pre[pp]], 1);
-            }
-        }
-    }
-    if (!count_next)
-        for (int e = gtid; e < n2; e += gsz) { cnt[e] = 0; nlc[e] = 0; }
-    for (int b = gtid; b <= B; b += gsz) {
-        const int x = scu[b];
-        scu2[b] = (n2 > 0) ? ((x < n) ? pre[x] : n2) : 0;
-    }
-}
-
-// Greedy block packing of one sequence.  fpos[e] = distance of e from the head of its family
-// (0 for heads and for elements in no family, capped at 255 >= block_m).
-__global__ void k_walk(const DevHeader *hdr, int s, int bm, const int *__restrict__ scu,
-                       const uint8_t *__restrict__ fpos, int *bstart, int *seqcount, int smem_cap) {
-    pdl_launch_dependents();      // the kernel queued behind this one may be scheduled now; it waits likewise
-    pdl_wait();                   // the kernel before this one has completed
-    extern __shared__ __align__(16) uint8_t s_fp[];
-    const int n = hdr->st[s].n;
-    const int b = blockIdx.x;
-    if (s > 0 && n == 0) { if (threadIdx.x == 0) seqcount[b] = 0; return; }
-    const int s0 = scu[b], s1 = scu[b + 1], len = s1 - s0;
-    // capacity offset of this sequence in bstart: sum over earlier sequences of 2*ceil(len/bm)+2
-    __shared__ int s_red[32];
-    int off = 0;
-    for (int c = threadIdx.x; c < b; c += blockDim.x) off += 2 * ((scu[c + 1] - scu[c] + bm - 1) / bm) + 2;
-    for (int o = 16; o; o >>= 1) off += __shfl_xor_sync(0xffffffffu, off, o);
-    if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = off;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        off = (threadIdx.x < (blockDim.x >> 5)) ? s_red[threadIdx.x] : 0;
-        for (int o = 16; o; o >>= 1) off += __shfl_xor_sync(0xffffffffu, off, o);
-        if (threadIdx.x == 0) s_red[0] = off;
-    }
-    __syncthreads();
-    off = s_red[0];
-    // stage fpos[a0 .. s1) from the 16-byte boundary a0 <= s0 with vector loads
-    const int a0 = s0 & ~15, skew = s0 - a0;
-    const bool in_smem = len + 32 <= smem_cap;
-    if (in_smem) {
-        const uint4 *src = reinterpret_cast<const uint4 *>(fpos + a0);
-        uint4 *dst = reinterpret_cast<uint4 *>(s_fp);
-        const int nv = (skew + len + 15) >> 4;   // the workspace array is padded to 256 bytes: no overrun
-        for (int i = threadIdx.x; i < nv; i += blockDim.x) dst[i] = src[i];
-    }
-    __syncthreads();
-    if (threadIdx.x != 0) return;
-    const uint8_t *fp = in_smem ? (s_fp + skew) : (fpos + s0);
-    int pos = 0, cntb = 0;
-    while (pos < len) {
-        int end = min(pos + bm, len);
-        if (end < len) {
-            const int f = fp[end];
-            if (f >= 1 && f < end - pos) end -= f;  // cut would split a family that starts after pos
-        }
-        bstart[off + cntb] = s0 + pos;
-        ++cntb;
+        if (nb < nbst) bst[nb] = pos; else rec[nb].x = pos;
+        ++nb;
         pos = end;
     }
-    seqcount[b] = cntb;
+    return nb;
 }
 
-// Block records of one sequence: one warp per block.
-__global__ void k_blocks(DevHeader *hdr, int s, int bm, int B, const int *__restrict__ scu,
-                         const int *__restrict__ bstart, const int *__restrict__ seqcount,
-                         const int *__restrict__ rng, const int *__restrict__ up, int *blocks,
-                         long long *cost) {
-    pdl_launch_dependents();      // the kernel queued behind this one may be scheduled now; it waits likewise
-    pdl_wait();                   // the kernel before this one has completed
-    const int n = hdr->st[s].n;
-    const int b = blockIdx.x;
-    if (s > 0 && n == 0) return;
-    __shared__ int s_red[2][32];
-    int off = 0, base = 0;
-    for (int c = threadIdx.x; c < b; c += blockDim.x) {
-        off += 2 * ((scu[c + 1] - scu[c] + bm - 1) / bm) + 2;
-        base += seqcount[c];
-    }
-    for (int o = 16; o; o >>= 1) {
-        off += __shfl_xor_sync(0xffffffffu, off, o);
-        base += __shfl_xor_sync(0xffffffffu, base, o);
-    }
-    if ((threadIdx.x & 31) == 0) { s_red[0][threadIdx.x >> 5] = off; s_red[1][threadIdx.x >> 5] = base; }
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        const bool in = threadIdx.x < (blockDim.x >> 5);
-        off = in ? s_red[0][threadIdx.x] : 0;
-        base = in ? s_red[1][threadIdx.x] : 0;
-        for (int o = 16; o; o >>= 1) {
-            off += __shfl_xor_sync(0xffffffffu, off, o);
-            base += __shfl_xor_sync(0xffffffffu, base, o);
-        }
-        if (threadIdx.x == 0) { s_red[0][0] = off; s_red[1][0] = base; }
-    }
-    __syncthreads();
-    off = s_red[0][0];
-    base = s_red[1][0];
-    const int nb_seq = seqcount[b], s1 = scu[b + 1];
-    if (b == B - 1 && threadIdx.x == 0 && blockIdx.y == 0) hdr->st[s].nb = base + nb_seq;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+// Block records of one stage, one warp per block.
+template <class I>
+__device__ __forceinline__ void make_records(const I *par, const I *cnt, int n, bool stage0, bool root_real, int nb, const int *bst, int nbst,
+                                             int4 *rec, int w, int nw, int lane, int *nf, int *ne, unsigned long long *vis_out) {
+    using E = Elem<I>;
     long long vis = 0;
-    for (int i = blockIdx.y * nw + w; i < nb_seq; i += nw * gridDim.y) {   // grid.y CTAs share a sequence
-        const int r0 = bstart[off + i];
-        const int r1 = (i + 1 < nb_seq) ? bstart[off + i + 1] : s1;
+    int mf = 0, me = 0;
+    for (int i = w; i < nb; i += nw) {
+        const int r0 = i < nbst ? bst[i] : rec[i].x;
+        const int r1 = (i + 1 < nb) ? (i + 1 < nbst ? bst[i + 1] : rec[i + 1].x) : n;
         int a = INT_MAX, bb = INT_MIN, carry = 0;
-        for (int e = r0 + lane; e < r1; e += 32) {
-            const int lo = rng[2 * e], hi = rng[2 * e + 1];
-            if (hi > lo) { a = min(a, lo); bb = max(bb, hi); }
-            if (up[e] >= 0) carry = 1;
+        unsigned lo[4], hi[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int e = r0 + lane + 32 * k;
+            lo[k] = hi[k] = 0;
+            if (e < r1) {
+                unsigned p;
+                const bool child = elem_range<I>(par, cnt, e, stage0, root_real, p, lo[k], hi[k]);
+                if (hi[k] > lo[k]) { a = min(a, (int)lo[k]); bb = max(bb, (int)hi[k]); }
+                const bool real = !stage0 || p != E::NONE || (e == 0 && root_real);
+                if (real && !child) carry = 1;
+            }
         }
-        for (int o = 16; o; o >>= 1) {
-            a = min(a, __shfl_xor_sync(0xffffffffu, a, o));
-            bb = max(bb, __shfl_xor_sync(0xffffffffu, bb, o));
-            carry |= __shfl_xor_sync(0xffffffffu, carry, o);
-        }
+        a = __reduce_min_sync(0xffffffffu, a);
+        bb = __reduce_max_sync(0xffffffffu, bb);
+        carry = __any_sync(0xffffffffu, carry);
         const bool any = bb > a;
         if (!any) { a = r0; bb = r0; }
         int dense = 1;
-        for (int e = r0 + lane; e < r1; e += 32)
-            if (rng[2 * e] != a || rng[2 * e + 1] != bb) dense = 0;
-        for (int o = 16; o; o >>= 1) dense &= __shfl_xor_sync(0xffffffffu, dense, o);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (r0 + lane + 32 * k < r1 && ((int)lo[k] != a || (int)hi[k] != bb)) dense = 0;
+        dense = __all_sync(0xffffffffu, dense);
         if (lane == 0) {
             int fl = 0;
             if (a >= r0 && bb <= r1) fl |= HDT_BLK_SELF;
             if (dense && any) fl |= HDT_BLK_DENSE;
             if (carry) fl |= HDT_BLK_CARRY;
             if (!any) fl |= HDT_BLK_EMPTY;
-            int *rec = blocks + 5 * (size_t)(base + i);
-            rec[0] = r0; rec[1] = r1; rec[2] = a; rec[3] = bb; rec[4] = fl;
-            const long long c = (long long)(r1 - r0) * (long long)(bb - a);
-            cost[base + i] = c;
-            vis += c;
+            rec[i] = make_int4(r0, a, bb, (r1 - r0) | (fl << 8));
+            vis += (long long)(r1 - r0) * (bb - a);
+            mf += (fl & HDT_BLK_SELF) && any;
+            me += !any;
         }
     }
-    if (lane == 0 && vis) atomicAdd((unsigned long long *)&hdr->visited, (unsigned long long)vis);
-}
-
-// Rank sort: queue[rank] = block id, cost descending, id ascending.  queue_split: the same order
-// inside two groups, blocks that are SELF and not EMPTY first (n_fused of them), then the others.
-// One warp per block: its lanes share the scan over all blocks and add up their counts.
-__global__ void __launch_bounds__(256)
-k_queue(DevHeader *hdr, int s, const long long *__restrict__ cost, const int *__restrict__ blocks, int *queue,
-        int *queue_split) {
-    pdl_launch_dependents();      // the kernel queued behind this one may be scheduled now; it waits likewise
-    pdl_wait();                   // the kernel before this one has completed
-    const int nb = hdr->st[s].nb;
-    const int lane = threadIdx.x & 31;
-    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
-    int mine = 0, mine_empty = 0;
-    for (int i = gw; i < nb; i += nw) {
-        const long long ci = cost[i];
-        const int fi = blocks[5 * i + 4];
-        const int ei = ((fi & HDT_BLK_SELF) && !(fi & HDT_BLK_EMPTY)) ? 1 : 0;
-        int rank = 0, rank2 = 0;
-        for (int j = lane; j < nb; j += 32) {
-            const long long cj = cost[j];
-            const int fj = blocks[5 * j + 4];
-            const int ej = ((fj & HDT_BLK_SELF) && !(fj & HDT_BLK_EMPTY)) ? 1 : 0;
-            const int before = (cj > ci) || (cj == ci && j < i);
-            rank += before;
-            rank2 += (ej > ei) || (ej == ei && before);
-        }
-        for (int o = 16; o; o >>= 1) {
-            rank += __shfl_xor_sync(0xffffffffu, rank, o);
-            rank2 += __shfl_xor_sync(0xffffffffu, rank2, o);
-        }
-        if (lane == 0) {
-            queue[rank] = i;
-            queue_split[rank2] = i;
-            mine += ei;
-            mine_empty += (fi & HDT_BLK_EMPTY) ? 1 : 0;
-        }
+    if (lane == 0) {
+        if (mf) atomicAdd(nf, mf);
+        if (me) atomicAdd(ne, me);
+        if (vis) atomicAdd(vis_out, (unsigned long long)vis);
     }
-    if (lane == 0 && mine) atomicAdd(&hdr->st[s].n_fused, mine);
-    if (lane == 0 && mine_empty) atomicAdd(&hdr->st[s].n_empty, mine_empty);
 }
 
-// ---------------------------------------------------------------------------------------------
-// All stages above 0 in one CTA.  Their arrays are a few percent of the tokens, so a single CTA
-// with block-wide barriers between the steps replaces eight launches per stage.
-// ---------------------------------------------------------------------------------------------
-struct UpperArgs {
-    StagePtrs st[HDT_MAX_STAGES];
-    int max_stages, B, bm, dirs;
-    int *cnt, *nlc, *pre, *bstart, *seqcount, *rank;
-    uint8_t *keep, *fpos;
-    long long *cost;
-};
+// log2 of the contiguous elements each of nw warps takes of n (at least one 32-element step).
+__device__ __forceinline__ int seg_shift(int n, int nw) {
+    int k = 5;
+    while (((long long)nw << k) < n) ++k;
+    return k;
+}
+// Exclusive offsets of the warps (lane w holds that of warp w) and the total.
+__device__ __forceinline__ int warp_offsets(const int *wtot, int nw, int lane, int &total) {
+    const int v0 = lane < nw ? wtot[lane] : 0;
+    int v = v0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += x;
+    }
+    total = __shfl_sync(0xffffffffu, v, 31);
+    return v - v0;
+}
 
-static constexpr int UT = 1024;      // threads of the fused kernel
-static constexpr int UMAXB = 1024;   // sequences it handles (per-sequence offsets live in shared memory)
-static constexpr int UCAP = 4096;    // elements of a stage whose scratch fits in shared memory
-static constexpr int USB = 2048;     // block slots of a stage whose block starts, costs and flags stay in shared memory
-static constexpr int USMEM = UCAP * (8 * 4 + 2) + USB * (4 + 8 + 1);   // bytes of that scratch
-
-__global__ void __launch_bounds__(UT) k_upper_stages(DevHeader *hdr, const UpperArgs u) {
-    // Stages of at most UCAP elements keep their per-element scratch (tokens, parents, child counts,
-    // keep flags, prefix sums, ranges, next-stage indices) in shared memory, and with at most USB
-    // block slots the block starts, costs and flags too: a dozen barrier-separated steps per stage
-    // would otherwise each pay a round trip to global memory (after the loads at a stage's start
-    // such a stage only writes to it).
-    extern __shared__ __align__(16) int s_dyn[];
-    int *s_par = s_dyn, *s_cnt = s_par + UCAP, *s_nlc = s_cnt + UCAP, *s_pre = s_nlc + UCAP, *s_up = s_pre + UCAP;
-    int *s_rng = s_up + UCAP;                                   // 2 * UCAP
-    int *s_tok = s_rng + 2 * UCAP;
-    long long *s_cst = reinterpret_cast<long long *>(s_tok + UCAP);   // (8-byte aligned: the arrays before it are multiples of 16 KB)
-    int *s_bst = reinterpret_cast<int *>(s_cst + USB);
-    uint8_t *s_keep = reinterpret_cast<uint8_t *>(s_bst + USB), *s_fpos = s_keep + UCAP, *s_bfl = s_fpos + UCAP;
-    __shared__ int s_off[UMAXB], s_base[UMAXB + 1], s_nbs[UMAXB], s_scu[UMAXB + 1];   // per sequence: block slots, first block, block count, offsets
-    __shared__ int s_w[32];
-    __shared__ int s_carry, s_flag, s_cap;
-    __shared__ long long s_ll[32];
-    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    const int B = u.B, bm = u.bm;
-    int n = hdr->st[1].n;                // (stage 0's kernels wrote it; the later ones are computed here)
-    for (int s = 1; s < u.max_stages; ++s) {
-        if (n == 0) break;
-        const StagePtrs P = u.st[s];
-        const bool last = (s + 1 == u.max_stages);
-        const StagePtrs N = u.st[last ? s : s + 1];
-        const bool small = n <= UCAP;
-        int *cnt = small ? s_cnt : u.cnt, *nlc = small ? s_nlc : u.nlc, *pre = small ? s_pre : u.pre;
-        uint8_t *keep = small ? s_keep : u.keep, *fpos = small ? s_fpos : u.fpos;
-        const int *par = small ? s_par : P.par, *tokr = small ? s_tok : P.tok;
-        const int *rngr = small ? s_rng : P.rng, *upr = small ? s_up : P.up;    // read-back of this stage's results
-        for (int b = t; b <= B; b += UT) s_scu[b] = P.scu[b];
-        if (small)
-            for (int e = t; e < n; e += UT) { s_par[e] = P.par[e]; s_tok[e] = P.tok[e]; s_cnt[e] = 0; s_nlc[e] = 0; }
-        __syncthreads();
-        // children counts (cnt, nlc are zero for [0, n))
-        for (int e = t; e < n; e += UT) { const int p = par[e]; if (p >= 0) atomicAdd(&cnt[p], 1); }
-        if (t == 0) { s_flag = 0; s_carry = 0; }
-        __syncthreads();
-        for (int e = t; e < n; e += UT) { const int p = par[e]; if (p >= 0 && cnt[e] > 0) atomicAdd(&nlc[p], 1); }
-        __syncthreads();
-        // ranges, keep flags
-        long long deg = 0;
-        for (int e = t; e < n; e += UT) {
-            const int p = par[e], c = cnt[e];
-            const bool head = (c > 0 && nlc[e] == 0);
-            int lo = 0, hi = 0, fp = 0, kp = 1;
-            if (head) {
-                lo = (p < 0) ? e : e + 1;
-                hi = e + 1 + c;
-            } else if (p >= 0) {
-                const int cp = cnt[p];
-                if (cp > 0 && nlc[p] == 0) {
-                    if (!(p < e && e <= p + cp)) dev_fail(hdr, HDT_ERR_BAD_HIERARCHY, e);
-                    lo = p; hi = p + 1 + cp; fp = min(e - p, 255); kp = 0;
-                    u.rank[tokr[e]] = e - p;
-                }
+// Stage 0 of one sequence up to the compaction, by all threads of the CTA.  X: parents, Y: counts,
+// Z: levels, then prefix sums of the keep flags.  Returns the number of kept elements.
+template <class I>
+__device__ __forceinline__ void seq_stage0(const SeqArgs &a, SeqShared &sh, I *X, I *Y, I *Z, int s0, int L, bool root_real) {
+    using E = Elem<I>;
+    const int t = threadIdx.x, nt = blockDim.x, lane = t & 31, w = t >> 5, nw = nt >> 5;
+    for (int e = t; e < L; e += nt) {
+        const int p = a.parent[s0 + e], l = a.level[s0 + e];
+        bool ok = true;
+        unsigned q = E::NONE;
+        if (l < 0) ok = (l == -1 && p == -1);
+        else if (e == 0) ok = (l == 0 && p == -1);
+        else if (l > HDT_MAX_STAGES * 8 || p < 0 || p >= e) ok = false;
+        else q = (unsigned)p;
+        X[e] = (I)q;
+        Z[e] = (I)(uint8_t)l;
+        Y[e] = 0;
+        if (!ok) seq_fail(sh, s0 + e);
+    }
+    __syncthreads();
+    for (int e = t; e < L; e += nt) {
+        const unsigned p = X[e];
+        const int l = (int8_t)(uint8_t)Z[e];
+        if (l >= 0 && e > 0) {
+            if (p != E::NONE && (int)(int8_t)(uint8_t)Z[p] != l - 1) seq_fail(sh, s0 + e);
+            if ((int8_t)(uint8_t)Z[e - 1] < 0) seq_fail(sh, s0 + e);     // PAD only as a suffix
+        }
+        if (p != E::NONE) E::add(Y, p);
+    }
+    __syncthreads();
+    for (int e = t; e < L; e += nt) {
+        const unsigned p = X[e];
+        if (p != E::NONE && (Y[e] & E::MASK) > 0) E::flag(Y, p);
+    }
+    __syncthreads();
+    const int k = seg_shift(L, nw);
+    int run = 0, next = 0;
+    long long deg = 0;
+    for (int i = 0; i < (1 << (k - 5)); ++i) {
+        const int base = (w << k) + 32 * i, e = base + lane;
+        if (base >= L) break;
+        bool kp = false;
+        if (e < L) {
+            const bool real = (int8_t)(uint8_t)Z[e] >= 0;
+            unsigned p, lo, hi;
+            const bool child = elem_range<I>(X, Y, e, true, root_real, p, lo, hi);
+            if (child) {
+                if (!((int)p < e && e < (int)hi)) seq_fail(sh, s0 + e);
+                a.rank[s0 + e] = e - (int)p;        // the token's number among its siblings (hierarchical positions)
             }
-            P.rng[2 * e] = lo;
-            P.rng[2 * e + 1] = hi;
-            if (small) { s_rng[2 * e] = lo; s_rng[2 * e + 1] = hi; }
-            keep[e] = (uint8_t)kp;
-            fpos[e] = (uint8_t)fp;
-            deg += row_pairs(e, lo, hi, u.dirs);
-            if (kp && p >= 0) s_flag = 1;
+            kp = real && !child;
+            const bool has = hi > lo;
+            reinterpret_cast<int2 *>(a.rng)[s0 + e] = make_int2(has ? s0 + (int)lo : 0, has ? s0 + (int)hi : 0);
+            a.tok[s0 + e] = s0 + e;
+            a.par[s0 + e] = (p == E::NONE) ? -1 : s0 + (int)p;
+            deg += row_pairs(e, (int)lo, (int)hi, a.dirs);
+            if (kp && p != E::NONE) next = 1;
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, kp);
+        if (e < L) Z[e] = (I)(kp ? (unsigned)(run + __popc(m & ((1u << lane) - 1u))) : E::NONE);
+        run += __popc(m);
+    }
+    for (int o = 16; o; o >>= 1) deg += __shfl_xor_sync(0xffffffffu, deg, o);
+    next = __any_sync(0xffffffffu, next);
+    if (lane == 0) {
+        sh.wtot[w] = run;
+        if (deg) atomicAdd(&sh.nnz, (unsigned long long)deg);
+        if (next) sh.flag0 = 1;
+    }
+}
+
+// Stage 0 -> stage 1: the kept elements' parents and tokens (only when the sequence has a stage 1), `up`.
+template <class I, class J>
+__device__ __forceinline__ void seq_compact0(const SeqArgs &a, const SeqShared &sh, const I *X, const I *Z, J *par2, J *tok2, int s0, int L, bool next) {
+    using E = Elem<I>;
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5, nw = blockDim.x >> 5;
+    const int k = seg_shift(L, nw);
+    int total;
+    const int wo = warp_offsets(sh.wtot, nw, lane, total);
+    const int mine = __shfl_sync(0xffffffffu, wo, w);
+    for (int i = 0; i < (1 << (k - 5)); ++i) {
+        const int base = (w << k) + 32 * i, e = base + lane;
+        if (base >= L) break;
+        const unsigned z = e < L ? Z[e] : E::NONE;
+        unsigned p = E::NONE, q = E::NONE;
+        if (z != E::NONE) { p = X[e]; if (p != E::NONE) q = Z[p]; }
+        const int wp = __shfl_sync(0xffffffffu, wo, q != E::NONE ? (int)(p >> k) : 0);
+        const int u = z != E::NONE ? (int)z + mine : -1;
+        if (e < L) a.up[s0 + e] = u;
+        if (u >= 0 && next) {
+            par2[u] = (J)(q != E::NONE ? q + (unsigned)wp : Elem<J>::NONE);
+            tok2[u] = (J)e;
+        }
+    }
+}
+
+// All stages above 0 of one sequence, by the first nw warps of the CTA (tu threads).
+template <class J>
+__device__ __forceinline__ void seq_upper(const SeqArgs &a, SeqShared &sh, J *par, J *tok, J *par2, J *tok2, J *cnt, J *pre, int b, int s0,
+                                          int slot, int n, int &stages, int &res, int &more) {
+    using E = Elem<J>;
+    const int t = threadIdx.x, tu = blockDim.x - 32, lane = t & 31, w = t >> 5, nw = tu >> 5;
+    int s = 1;
+    while (true) {
+        if (s == a.ms) { more = 1; break; }          // elements left that no stage may take
+        int4 *rec = a.recs + (size_t)s * a.capnb + slot;
+        int4 *el = a.el + (size_t)(s - 1) * a.T + s0;
+        int *upl = a.upl + (size_t)(s - 1) * a.T + s0;
+        for (int e = t; e < n; e += tu) cnt[e] = 0;
+        if (t == 0) { sh.flag = 0; sh.nf = 0; sh.ne = 0; }
+        bar_upper(tu);
+        for (int e = t; e < n; e += tu) { const unsigned p = par[e]; if (p != E::NONE) E::add(cnt, p); }
+        bar_upper(tu);
+        for (int e = t; e < n; e += tu) {
+            const unsigned p = par[e];
+            if (p != E::NONE && (cnt[e] & E::MASK) > 0) E::flag(cnt, p);
+        }
+        bar_upper(tu);
+        if (t == 0) sh.nb = walk_blocks<J>(par, cnt, n, a.bmu, sh.bst, SBU, rec);
+        __syncwarp();
+        const int k = seg_shift(n, nw);
+        int run = 0, next = 0;
+        long long deg = 0;
+        for (int i = 0; i < (1 << (k - 5)); ++i) {
+            const int base = (w << k) + 32 * i, e = base + lane;
+            if (base >= n) break;
+            bool kp = false;
+            if (e < n) {
+                unsigned p, lo, hi;
+                const bool child = elem_range<J>(par, cnt, e, false, false, p, lo, hi);
+                const int tk = tok[e];
+                if (child) {
+                    if (!((int)p < e && e < (int)hi)) seq_fail(sh, s0 + tk);
+                    a.rank[s0 + tk] = e - (int)p;
+                }
+                kp = !child;
+                el[e] = make_int4(tk, (p == E::NONE) ? -1 : (int)p, (int)lo, (int)hi);
+                deg += row_pairs(e, (int)lo, (int)hi, a.dirs);
+                if (kp && p != E::NONE) next = 1;
+            }
+            const unsigned m = __ballot_sync(0xffffffffu, kp);
+            if (e < n) pre[e] = (J)(kp ? (unsigned)(run + __popc(m & ((1u << lane) - 1u))) : E::NONE);
+            run += __popc(m);
         }
         for (int o = 16; o; o >>= 1) deg += __shfl_xor_sync(0xffffffffu, deg, o);
-        if (lane == 0) s_ll[w] = deg;
-        __syncthreads();
+        next = __any_sync(0xffffffffu, next);
+        if (lane == 0) {
+            sh.wtotu[w] = run;
+            if (deg) atomicAdd(&sh.nnz, (unsigned long long)deg);
+            if (next) sh.flag = 1;
+        }
+        bar_upper(tu);
+        const bool go_on = sh.flag != 0;
+        int total;
+        const int wo = warp_offsets(sh.wtotu, nw, lane, total);
+        const int mine = __shfl_sync(0xffffffffu, wo, w);
+        for (int i = 0; i < (1 << (k - 5)); ++i) {
+            const int base = (w << k) + 32 * i, e = base + lane;
+            if (base >= n) break;
+            const unsigned z = e < n ? pre[e] : E::NONE;
+            unsigned p = E::NONE, q = E::NONE;
+            if (z != E::NONE) { p = par[e]; if (p != E::NONE) q = pre[p]; }
+            const int wp = __shfl_sync(0xffffffffu, wo, q != E::NONE ? (int)(p >> k) : 0);
+            const int u = z != E::NONE ? (int)z + mine : -1;
+            if (e < n) upl[e] = u;
+            if (u >= 0 && go_on) {
+                par2[u] = (J)(q != E::NONE ? q + (unsigned)wp : E::NONE);
+                tok2[u] = tok[e];
+            }
+        }
+        make_records<J>(par, cnt, n, false, false, sh.nb, sh.bst, SBU, rec, w, nw, lane, &sh.nf, &sh.ne, &sh.vis);
+        bar_upper(tu);
         if (t == 0) {
-            long long d = 0;
-            for (int i = 0; i < UT / 32; ++i) d += s_ll[i];
-            if (d) atomicAdd((unsigned long long *)&hdr->nnz, (unsigned long long)d);
-            hdr->st[s].has_next = s_flag;
+            int *c = a.counts + (size_t)s * a.B + b;
+            const size_t q = (size_t)a.ms * a.B;
+            c[0] = n; c[q] = sh.nb; c[2 * q] = sh.nf; c[3 * q] = sh.ne;
         }
-        const int has_next = s_flag;
-        // exclusive scan of keep[] in chunks of UT
-        for (int base = 0; base < n; base += UT) {
-            const int e = base + t;
-            const int kp = (e < n) ? keep[e] : 0;
-            int v = kp;
-            for (int o = 1; o < 32; o <<= 1) { const int x = __shfl_up_sync(0xffffffffu, v, o); if (lane >= o) v += x; }
-            if (lane == 31) s_w[w] = v;
-            __syncthreads();
-            if (w == 0) {
-                int x = s_w[lane];
-                for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(0xffffffffu, x, o); if (lane >= o) x += y; }
-                s_w[lane] = x;
-            }
-            __syncthreads();
-            const int excl = s_carry + (w ? s_w[w - 1] : 0) + v - kp;
-            if (e < n) {
-                pre[e] = excl;
-                const int up = (kp && has_next) ? excl : -1;
-                P.up[e] = up;
-                if (small) s_up[e] = up;
-                if (up >= 0 && !last) N.tok[up] = tokr[e];
-            }
-            __syncthreads();
-            if (t == 0) s_carry += s_w[31];
-            __syncthreads();
+        ++s;
+        res = total;
+        if (!go_on) break;
+        n = total;
+        J *x = par; par = par2; par2 = x;
+        x = tok; tok = tok2; tok2 = x;
+    }
+    stages = s;
+}
+
+// A sequence's stages.  Shared memory per token of `cap`: 6 bytes (parents, counts, prefix sums) and,
+// per upper element of `uc`, 12 (two sets of parents and tokens, counts, prefix sums), of which 8 may
+// lie over stage 0's prefix sums, which are dead after its compaction.
+__global__ void __launch_bounds__(1024) k_seq(const SeqArgs a) {
+    pdl_launch_dependents();
+    extern __shared__ __align__(16) uint16_t s_dyn[];
+    __shared__ SeqShared sh;
+    const int b = blockIdx.x, t = threadIdx.x, lane = t & 31, w = t >> 5, nw = blockDim.x >> 5;
+    const int c0 = a.cu[b], c1 = a.cu[b + 1];
+    const int s0 = min(max(c0, 0), a.T), L = min(max(c1, s0), a.T) - s0;
+    if (t == 0) {
+        sh.err = 0; sh.err_pos = 0; sh.flag0 = 0; sh.nf0 = 0; sh.ne0 = 0; sh.nnz = 0; sh.vis = 0;
+        if (c1 < c0 || c0 < 0 || c1 > a.T || (b == 0 && c0 != 0) || (b == a.B - 1 && c1 != a.T)) seq_fail(sh, b);
+        a.scu[b] = c0;
+        if (b == a.B - 1) a.scu[a.B] = c1;
+    }
+    const bool root_real = L > 0 && a.level[s0] >= 0;
+    const int slot = block_slot(s0, b, a.bmin);
+    __syncthreads();
+    const bool in_smem = L <= a.cap;
+    uint16_t *X = s_dyn, *Y = X + a.cap, *Z = Y + a.cap, *U = Z + a.cap;
+    uint32_t *G[NGLOB];
+    for (int i = 0; i < NGLOB; ++i) G[i] = a.glob + a.glob_stride * i + s0;
+    if (in_smem) seq_stage0<uint16_t>(a, sh, X, Y, Z, s0, L, root_real);
+    else seq_stage0<uint32_t>(a, sh, G[0], G[1], G[2], s0, L, root_real);
+    __syncthreads();
+    int n1;
+    (void)warp_offsets(sh.wtot, nw, lane, n1);
+    const bool next = sh.flag0 != 0;
+    const bool up_smem = n1 <= a.uc;
+    // (the first parent / token set of the upper stages never lies over the prefix sums)
+    uint16_t *P0 = U, *T0 = U + a.uc, *V = a.overlay ? Z : U + 2 * a.uc;
+    if (in_smem && up_smem) seq_compact0<uint16_t, uint16_t>(a, sh, X, Z, P0, T0, s0, L, next);
+    else if (in_smem) seq_compact0<uint16_t, uint32_t>(a, sh, X, Z, G[3], G[4], s0, L, next);
+    else if (up_smem && L < 65535) seq_compact0<uint32_t, uint16_t>(a, sh, G[0], G[2], P0, T0, s0, L, next);
+    else seq_compact0<uint32_t, uint32_t>(a, sh, G[0], G[2], G[3], G[4], s0, L, next);
+    __syncthreads();
+    int stages = 1, res = n1, more = 0;
+    if (w == nw - 1) {
+        if (lane == 0)
+            sh.nb0 = in_smem ? walk_blocks<uint16_t>(X, Y, L, a.bm, sh.bst0, SB0, a.recs + slot)
+                             : walk_blocks<uint32_t>(G[0], G[1], L, a.bm, sh.bst0, SB0, a.recs + slot);
+    } else if (next) {
+        if (up_smem && (in_smem || L < 65535)) seq_upper<uint16_t>(a, sh, P0, T0, V, V + a.uc, V + 2 * a.uc, V + 3 * a.uc, b, s0, slot, n1, stages, res, more);
+        else seq_upper<uint32_t>(a, sh, G[3], G[4], G[5], G[6], G[7], G[8], b, s0, slot, n1, stages, res, more);
+    }
+    __syncthreads();
+    if (in_smem) make_records<uint16_t>(X, Y, L, true, root_real, sh.nb0, sh.bst0, SB0, a.recs + slot, w, nw, lane, &sh.nf0, &sh.ne0, &sh.vis);
+    else make_records<uint32_t>(G[0], G[1], L, true, root_real, sh.nb0, sh.bst0, SB0, a.recs + slot, w, nw, lane, &sh.nf0, &sh.ne0, &sh.vis);
+    __syncthreads();
+    if (t == 0) {
+        const size_t q = (size_t)a.ms * a.B;
+        int *c = a.counts + b;
+        c[0] = L; c[q] = sh.nb0; c[2 * q] = sh.nf0; c[3 * q] = sh.ne0;
+        for (int s = stages; s < a.ms; ++s) {          // beyond its own stages: its root in a block of its own
+            c = a.counts + (size_t)s * a.B + b;
+            c[0] = res; c[q] = res; c[2 * q] = 0; c[3 * q] = res;
         }
-        const int n2 = has_next ? s_carry : 0;
-        if (t == 0) hdr->st[s + 1].n = n2;
-        // next stage's parents and sequence offsets; clear cnt / nlc for it
-        if (!last) {
-            for (int e = t; e < n; e += UT) {
-                const int up = upr[e];
-                if (up >= 0) { const int p = par[e]; N.par[up] = (p >= 0) ? pre[p] : -1; }
-            }
-            for (int b = t; b <= B; b += UT) {
-                const int x = s_scu[b];
-                N.scu[b] = (n2 > 0) ? ((x < n) ? pre[x] : n2) : 0;
-            }
+        SeqInfo f;
+        f.stages = stages; f.res = res; f.err = sh.err; f.err_pos = sh.err_pos; f.more = more; f.pad = 0;
+        f.nnz = (long long)sh.nnz; f.visited = (long long)sh.vis;
+        a.info[b] = f;
+    }
+}
+
+struct FinishArgs {
+    StagePtrs st[HDT_MAX_STAGES];
+    const int32_t *cu;
+    int B, T, ms, bm, bmu, bmin, capnb, gy, r0;   // gy: CTAs of a sequence; r0: CTAs that rank stage 0's blocks
+    const SeqInfo *info;
+    const int *counts;
+    const int4 *recs, *el;
+    const int *upl;
+    long long *keys;
+    DevHeader *hdr, *host;         // host: pinned landing buffer (its words are not 0 at `tail` before)
+};
+
+static constexpr int FT = 256;     // threads of k_finish
+static constexpr int FKEYS = 4096; // blocks of a stage whose sort keys fit in shared memory
+
+__device__ __forceinline__ long long warp_sum(long long v) {
+#pragma unroll
+    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Header: totals over the sequences.  The words go to the workspace (kernels read them there) and
+// straight to the host's pinned buffer, the tail word last and behind a system-wide fence: the host
+// watches for it, so no copy has to be queued behind the build.
+__device__ void finish_header(const FinishArgs &f, int S) {
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    __shared__ int s_err, s_more;
+    __shared__ long long s_sum[2];
+    if (t == 0) { s_err = 0x7fffffff; s_more = 0; s_sum[0] = s_sum[1] = 0; }
+    __syncthreads();
+    const size_t q = (size_t)f.ms * f.B;
+    for (int i = w; i < 4 * S; i += FT / 32) {
+        const int s = i >> 2, c = i & 3;
+        int v = 0;
+        for (int b = lane; b < f.B; b += 32) v += f.counts[c * q + (size_t)s * f.B + b];
+        v = __reduce_add_sync(0xffffffffu, v);
+        if (lane == 0) {
+            StageDesc &d = f.hdr->st[s], &h = f.host->st[s];
+            int *pd = c == 0 ? &d.n : c == 1 ? &d.nb : c == 2 ? &d.n_fused : &d.n_empty;
+            int *ph = c == 0 ? &h.n : c == 1 ? &h.nb : c == 2 ? &h.n_fused : &h.n_empty;
+            *pd = v;
+            *reinterpret_cast<volatile int *>(ph) = v;
         }
-        __syncthreads();   // every cnt / nlc / pre read of this stage is done
-        if (!small)
-            for (int e = t; e < max(n2, 0); e += UT) { u.cnt[e] = 0; u.nlc[e] = 0; }
-        // per-sequence capacity offsets, greedy walk (one lane per sequence)
-        for (int b = t; b < B; b += UT) {
-            int off = 0;
-            for (int c = 0; c < b; ++c) off += 2 * ((s_scu[c + 1] - s_scu[c] + bm - 1) / bm) + 2;
-            s_off[b] = off;
-            if (b == B - 1) s_cap = off + 2 * ((s_scu[b + 1] - s_scu[b] + bm - 1) / bm) + 2;
+    }
+    long long nnz = 0, vis = 0;
+    for (int b = t; b < f.B; b += FT) {
+        const SeqInfo &x = f.info[b];
+        nnz += x.nnz; vis += x.visited;
+        if (x.err) atomicMin(&s_err, b);
+        if (x.more) s_more = 1;
+    }
+    nnz = warp_sum(nnz); vis = warp_sum(vis);
+    if (lane == 0) { atomicAdd((unsigned long long *)&s_sum[0], (unsigned long long)nnz); atomicAdd((unsigned long long *)&s_sum[1], (unsigned long long)vis); }
+    __syncthreads();
+    if (t <= HDT_MAX_STAGES) {
+        const int more = (t + 1 < S) || (t + 1 == S && s_more);
+        f.hdr->st[t].has_next = more;
+        *reinterpret_cast<volatile int *>(&f.host->st[t].has_next) = more;
+        if (t >= S) {
+            StageDesc &d = f.hdr->st[t];
+            d.n = d.nb = d.n_fused = d.n_empty = 0;
+            volatile StageDesc *h = &f.host->st[t];
+            h->n = 0; h->nb = 0; h->n_fused = 0; h->n_empty = 0;
         }
+    }
+    if (t == 0) {
+        int err = 0, pos = 0;
+        if (f.B == 0) { f.st[0].scu[0] = f.cu[0]; if (f.cu[0] != 0 || f.T != 0) err = HDT_ERR_BAD_HIERARCHY; }
+        else if (s_err != 0x7fffffff) { err = f.info[s_err].err; pos = f.info[s_err].err_pos; }
+        volatile DevHeader *h = f.host;
+        f.hdr->status = err; f.hdr->err_pos = pos; f.hdr->nnz = s_sum[0]; f.hdr->visited = s_sum[1]; f.hdr->tail = 0;
+        h->status = err; h->err_pos = pos; h->nnz = s_sum[0]; h->visited = s_sum[1];
+    }
+    __threadfence_system();
+    __syncthreads();
+    if (t == 0) *reinterpret_cast<volatile int *>(&f.host->tail) = 0;
+}
+
+// Rank sort of a stage's blocks: queue[rank] = block id, cost descending, id ascending.  queue_split:
+// the same order inside two groups, blocks that are SELF and not EMPTY first, then the others.
+// Every CTA gathers all keys (cost << 1 | SELF non-EMPTY), a warp ranks a block at a time.
+__device__ void finish_rank(const FinishArgs &f, int s, int part, int parts, long long *s_keys) {
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5, nw = FT / 32;
+    __shared__ int s_base[FT], s_cnt[FT], s_w[FT / 32];
+    const int *cb = f.counts + (size_t)f.ms * f.B + (size_t)s * f.B;
+    int nb = 0;
+    for (int b = t; b < f.B; b += FT) nb += cb[b];
+    nb = __reduce_add_sync(0xffffffffu, nb);
+    if (lane == 0) s_w[w] = nb;
+    __syncthreads();
+    nb = 0;
+    for (int i = 0; i < nw; ++i) nb += s_w[i];
+    __syncthreads();
+    long long *keys = nb <= FKEYS ? s_keys : f.keys + (size_t)s * f.capnb;    // (every CTA of the stage writes the same values)
+    int run = 0;
+    for (int b0 = 0; b0 < f.B; b0 += FT) {
+        const int b = b0 + t, c = b < f.B ? cb[b] : 0;
+        int v = c;
+        for (int o = 1; o < 32; o <<= 1) { const int x = __shfl_up_sync(0xffffffffu, v, o); if (lane >= o) v += x; }
+        if (lane == 31) s_w[w] = v;
         __syncthreads();
-        const bool few = B > 0 && s_cap <= USB;        // block slots of this stage fit in shared memory
-        int *bst = few ? s_bst : u.bstart;
-        long long *cst = few ? s_cst : u.cost;
-        for (int b = w; b < B; b += UT / 32) {
-            if (lane == 0) {
-                const int s0 = s_scu[b], len = s_scu[b + 1] - s0, off = s_off[b];
-                int pos = 0, cntb = 0;
-                while (pos < len) {
-                    int end = min(pos + bm, len);
-                    if (end < len) {
-                        const int f = fpos[s0 + end];
-                        if (f >= 1 && f < end - pos) end -= f;
-                    }
-                    bst[off + cntb] = s0 + pos;
-                    ++cntb;
-                    pos = end;
-                }
-                u.seqcount[b] = cntb;
-                s_nbs[b] = cntb;
-            }
-        }
+        int off = run, all = 0;
+        for (int i = 0; i < nw; ++i) { if (i < w) off += s_w[i]; all += s_w[i]; }
+        s_base[t] = off + v - c;
+        s_cnt[t] = c;
         __syncthreads();
-        for (int b = t; b < B; b += UT) {
-            int base = 0;
-            for (int c = 0; c < b; ++c) base += s_nbs[c];
-            s_base[b] = base;
-            if (b == B - 1) { hdr->st[s].nb = base + s_nbs[b]; s_base[B] = base + s_nbs[b]; }
+        const int nseq = min(FT, f.B - b0);
+        for (int i = w; i < nseq; i += nw) {
+            const int bb = b0 + i;
+            const bool own = s < f.info[bb].stages;     // else its root alone, in a block without keys: cost 0
+            const int4 *rec = f.recs + (size_t)s * f.capnb + block_slot(min(max(f.cu[bb], 0), f.T), bb, f.bmin);
+            for (int j = lane; j < s_cnt[i]; j += 32) {
+                long long k = 0;
+                if (own) {
+                    const int4 r = rec[j];
+                    const int fl = r.w >> 8;
+                    k = ((long long)(r.w & 255) * (r.z - r.y)) * 2 + ((fl & HDT_BLK_SELF) && !(fl & HDT_BLK_EMPTY) ? 1 : 0);
+                }
+                keys[s_base[i] + j] = k;
+            }
         }
+        run += all;
         __syncthreads();
-        // block records, one warp per block over all sequences (the block's sequence by bisection of s_base)
-        long long vis = 0;
-        {
-            const int nb_all = (B > 0) ? s_base[B] : 0;
-            for (int gb = w; gb < nb_all; gb += UT / 32) {
-                int lo_b = 0, hi_b = B;
-                while (hi_b - lo_b > 1) { const int mid = (lo_b + hi_b) >> 1; if (s_base[mid] <= gb) lo_b = mid; else hi_b = mid; }
-                // (the largest b with s_base[b] <= gb always owns blocks: an empty sequence has the base of its successor)
-                const int b = lo_b, i = gb - s_base[b];
-                const int nb_seq = s_nbs[b], off = s_off[b], base = s_base[b], s1 = s_scu[b + 1];
-                const int r0 = bst[off + i];
-                const int r1 = (i + 1 < nb_seq) ? bst[off + i + 1] : s1;
-                int a = 0x7fffffff, bb = (int)0x80000000, carry = 0;
-                for (int e = r0 + lane; e < r1; e += 32) {
-                    const int lo = rngr[2 * e], hi = rngr[2 * e + 1];
-                    if (hi > lo) { a = min(a, lo); bb = max(bb, hi); }
-                    if (upr[e] >= 0) carry = 1;
-                }
-                for (int o = 16; o; o >>= 1) {
-                    a = min(a, __shfl_xor_sync(0xffffffffu, a, o));
-                    bb = max(bb, __shfl_xor_sync(0xffffffffu, bb, o));
-                    carry |= __shfl_xor_sync(0xffffffffu, carry, o);
-                }
-                const bool any = bb > a;
-                if (!any) { a = r0; bb = r0; }
-                int dense = 1;
-                for (int e = r0 + lane; e < r1; e += 32)
-                    if (rngr[2 * e] != a || rngr[2 * e + 1] != bb) dense = 0;
-                for (int o = 16; o; o >>= 1) dense &= __shfl_xor_sync(0xffffffffu, dense, o);
-                if (lane == 0) {
-                    int fl = 0;
-                    if (a >= r0 && bb <= r1) fl |= HDT_BLK_SELF;
-                    if (dense && any) fl |= HDT_BLK_DENSE;
-                    if (carry) fl |= HDT_BLK_CARRY;
-                    if (!any) fl |= HDT_BLK_EMPTY;
-                    int *rec = P.blocks + 5 * (size_t)(base + i);
-                    rec[0] = r0; rec[1] = r1; rec[2] = a; rec[3] = bb; rec[4] = fl;
-                    const long long c = (long long)(r1 - r0) * (long long)(bb - a);
-                    cst[base + i] = c;
-                    if (few) s_bfl[base + i] = (uint8_t)fl;
-                    vis += c;
-                }
-            }
+    }
+    for (int i = part * nw + w; i < nb; i += nw * parts) {
+        const long long ki = keys[i];
+        int rank = 0, rank2 = 0;
+        for (int j = lane; j < nb; j += 32) {
+            const long long kj = keys[j];
+            const int before = ((kj >> 1) > (ki >> 1)) || ((kj >> 1) == (ki >> 1) && j < i);
+            rank += before;
+            rank2 += ((kj & 1) > (ki & 1)) || ((kj & 1) == (ki & 1) && before);
         }
-        if (lane == 0 && vis) atomicAdd((unsigned long long *)&hdr->visited, (unsigned long long)vis);
-        __syncthreads();
-        // queues
-        const int nb = (B > 0) ? s_base[B] : 0;
-        int mine = 0, mine_empty = 0;
-        for (int i = w; i < nb; i += UT / 32) {      // one warp per block, lanes share the scan
-            const long long ci = cst[i];
-            const int fi = few ? (int)s_bfl[i] : P.blocks[5 * i + 4];
-            const int ei = ((fi & HDT_BLK_SELF) && !(fi & HDT_BLK_EMPTY)) ? 1 : 0;
-            int rank = 0, rank2 = 0;
-            for (int j = lane; j < nb; j += 32) {
-                const long long cj = cst[j];
-                const int fj = few ? (int)s_bfl[j] : P.blocks[5 * j + 4];
-                const int ej = ((fj & HDT_BLK_SELF) && !(fj & HDT_BLK_EMPTY)) ? 1 : 0;
-                const int before = (cj > ci) || (cj == ci && j < i);
-                rank += before;
-                rank2 += (ej > ei) || (ej == ei && before);
-            }
-            for (int o = 16; o; o >>= 1) {
-                rank += __shfl_xor_sync(0xffffffffu, rank, o);
-                rank2 += __shfl_xor_sync(0xffffffffu, rank2, o);
-            }
-            if (lane == 0) {
-                P.queue[rank] = i;
-                P.queue_split[rank2] = i;
-                mine += ei;
-                mine_empty += (fi & HDT_BLK_EMPTY) ? 1 : 0;
-            }
+        rank = __reduce_add_sync(0xffffffffu, rank);
+        rank2 = __reduce_add_sync(0xffffffffu, rank2);
+        if (lane == 0) {
+            f.st[s].queue[rank] = i;
+            f.st[s].queue_split[rank2] = i;
         }
-        if (mine) atomicAdd(&hdr->st[s].n_fused, mine);
-        if (mine_empty) atomicAdd(&hdr->st[s].n_empty, mine_empty);
-        __syncthreads();   // every read of this stage's scratch is done before the next stage overwrites it
-        n = n2;
+    }
+}
+
+// CTA 0: header; then r0 CTAs rank stage 0's blocks and one each those of the other stages; then gy
+// CTAs per sequence move its elements and block records to their place in the batch's arrays.
+__global__ void __launch_bounds__(FT) k_finish(const FinishArgs f) {
+    pdl_launch_dependents();
+    pdl_wait();
+    __shared__ long long s_keys[FKEYS];
+    __shared__ int s_stages, s_bad;
+    __shared__ int s_n[HDT_MAX_STAGES + 1], s_b[HDT_MAX_STAGES + 1], s_tot[HDT_MAX_STAGES + 1];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5, nw = FT / 32;
+    if (t == 0) { s_stages = 1; s_bad = 0; }
+    __syncthreads();
+    {
+        int m = 1, bad = 0;
+        for (int b = t; b < f.B; b += FT) { m = max(m, f.info[b].stages); bad |= f.info[b].err; }
+        m = __reduce_max_sync(0xffffffffu, m);
+        bad = __any_sync(0xffffffffu, bad);
+        if (lane == 0) { atomicMax(&s_stages, m); if (bad) s_bad = 1; }
+    }
+    __syncthreads();
+    const int S = s_stages;
+    int id = blockIdx.x;
+    if (id == 0) { finish_header(f, S); return; }
+    if (s_bad) return;               // (offsets of a broken hierarchy mean nothing)
+    id -= 1;
+    if (id < f.r0) { finish_rank(f, 0, id, f.r0, s_keys); return; }
+    id -= f.r0;
+    if (id < f.ms - 1) { if (id + 1 < S) finish_rank(f, id + 1, 0, 1, s_keys); return; }
+    id -= f.ms - 1;
+    const int b = id / f.gy, y = id % f.gy;
+    // sums over the sequences before this one: elements and blocks of every stage
+    const size_t q = (size_t)f.ms * f.B;
+    for (int i = w; i < 2 * S; i += nw) {
+        const int s = i >> 1;
+        const int *c = f.counts + ((i & 1) ? q : 0) + (size_t)s * f.B;
+        int v = 0;
+        for (int j = lane; j < b; j += 32) v += c[j];
+        v = __reduce_add_sync(0xffffffffu, v);
+        if (lane == 0) {
+            if (i & 1) s_b[s] = v;
+            else { s_n[s] = v; s_tot[s] = v + c[b]; }      // (s_tot: the batch's elements where b is the last sequence)
+        }
+    }
+    __syncthreads();
+    const SeqInfo info = f.info[b];
+    const int s0 = f.cu[b], L = f.cu[b + 1] - s0;
+    const int step = FT * f.gy, me = y * FT + t;
+    {
+        int *up = f.st[0].up;
+        const int off = S > 1 ? s_n[1] : 0;
+        for (int e = me; e < L; e += step) {
+            const int v = up[s0 + e];
+            if (v >= 0) up[s0 + e] = S > 1 ? v + off : -1;
+        }
+    }
+    const int slot = block_slot(s0, b, f.bmin);
+    for (int s = 0; s < S; ++s) {
+        const StagePtrs &P = f.st[s];
+        const int off = s ? s_n[s] : s0, boff = s_b[s];
+        const bool last = s + 1 == S;
+        const int n = f.counts[(size_t)s * f.B + b], nb = f.counts[q + (size_t)s * f.B + b];
+        if (s > 0 && me == 0) {
+            P.scu[b] = off;
+            if (b == f.B - 1) P.scu[f.B] = s_tot[s];
+        }
+        if (s < info.stages) {
+            if (s > 0) {
+                const int4 *el = f.el + (size_t)(s - 1) * f.T + s0;
+                const int *upl = f.upl + (size_t)(s - 1) * f.T + s0;
+                const int noff = last ? 0 : s_n[s + 1];
+                for (int e = me; e < n; e += step) {
+                    const int4 x = el[e];
+                    const int u = upl[e];
+                    const bool has = x.w > x.z;
+                    P.tok[off + e] = s0 + x.x;
+                    P.par[off + e] = x.y < 0 ? -1 : off + x.y;
+                    reinterpret_cast<int2 *>(P.rng)[off + e] = make_int2(has ? off + x.z : 0, has ? off + x.w : 0);
+                    P.up[off + e] = (u < 0 || last) ? -1 : u + noff;
+                }
+            }
+            const int4 *rec = f.recs + (size_t)s * f.capnb + slot;
+            for (int i = me; i < nb; i += step) {
+                const int4 r = rec[i];
+                int fl = r.w >> 8;
+                if (last) fl &= ~HDT_BLK_CARRY;
+                int *o = P.blocks + 5 * (size_t)(boff + i);
+                o[0] = off + r.x; o[1] = off + r.x + (r.w & 255); o[2] = off + r.y; o[3] = off + r.z; o[4] = fl;
+            }
+        } else if (info.res && me == 0) {       // (res is 0 or 1 here)
+            P.tok[off] = s0;
+            P.par[off] = -1;
+            reinterpret_cast<int2 *>(P.rng)[off] = make_int2(0, 0);
+            P.up[off] = last ? -1 : s_n[s + 1];
+            int *o = P.blocks + 5 * (size_t)boff;
+            o[0] = off; o[1] = off + 1; o[2] = off; o[3] = off;
+            o[4] = HDT_BLK_SELF | HDT_BLK_EMPTY | (last ? 0 : HDT_BLK_CARRY);
+        }
     }
 }
 
@@ -738,54 +775,31 @@ extern "C" size_t hdt_index_workspace_bytes(int32_t batch, int32_t total_tokens,
     return make_layout(batch, total_tokens, min(bm, bmu), ms).total;
 }
 
-// Launch as a programmatic dependent of the kernel before it on the stream (its CTAs are scheduled
-// while that kernel ends and wait for it with pdl_wait): the dozen tiny kernels of a build are a
-// chain, and most of each link is launch latency.
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_chain(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = g_no_pdl ? 0 : 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
-}
-
-// Pinned landing buffers for index headers: a small pool shared by all host threads (a deferred
-// index keeps its buffer until the header has been read).
+// Pinned landing buffers for index headers: a small pool shared by all host threads (an index keeps
+// its buffer until the header has been read).
 static const int kUnset = 0x7fffffff;
 static std::mutex g_pinned_mu;
-// A landing buffer for the header with the event that marks the end of its copy.
-struct PinnedSlot { DevHeader *p; cudaEvent_t ev; };
-static std::vector<PinnedSlot> g_pinned_free;
-static bool pinned_acquire(PinnedSlot *out) {
+static std::vector<DevHeader *> g_pinned_free;
+static DevHeader *pinned_acquire() {
     {
         std::lock_guard<std::mutex> lk(g_pinned_mu);
         if (!g_pinned_free.empty()) {
-            *out = g_pinned_free.back();
+            DevHeader *p = g_pinned_free.back();
             g_pinned_free.pop_back();
-            return true;
+            return p;
         }
     }
-    PinnedSlot s{nullptr, nullptr};
-    if (cudaMallocHost((void **)&s.p, sizeof(DevHeader)) != cudaSuccess) { (void)cudaGetLastError(); return false; }
-    if (cudaEventCreateWithFlags(&s.ev, cudaEventDisableTiming) != cudaSuccess) {
+    DevHeader *p = nullptr;
+    if (cudaHostAlloc((void **)&p, sizeof(DevHeader), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
         (void)cudaGetLastError();
-        cudaFreeHost(s.p);
-        return false;
+        return nullptr;
     }
-    *out = s;
-    return true;
+    return p;
 }
-static void pinned_release(DevHeader *p, cudaEvent_t ev) {
+static void pinned_release(DevHeader *p) {
     if (!p) return;
     std::lock_guard<std::mutex> lk(g_pinned_mu);
-    g_pinned_free.push_back(PinnedSlot{p, ev});
+    g_pinned_free.push_back(p);
 }
 
 extern "C" int hdt_build_index(const int8_t *level, const int32_t *parent, const int32_t *cu_seqlens,
@@ -806,18 +820,37 @@ extern "C" int hdt_build_index(const int8_t *level, const int32_t *parent, const
     if (((uintptr_t)workspace & 255) != 0)
         return set_error(HDT_ERR_INVALID_ARG, "hdt_build_index: workspace must be 256-byte aligned");
     const int B = batch, T = total_tokens;
-    const Layout L = make_layout(B, T, min(bm, bmu), ms);
+    const int bmin = min(bm, bmu);
+    const Layout L = make_layout(B, T, bmin, ms);
     if (workspace_bytes < L.total)
         return set_error(HDT_ERR_WORKSPACE, "hdt_build_index: workspace %zu < required %zu", workspace_bytes,
                          L.total);
     cudaStream_t st = (cudaStream_t)stream;
     char *ws = (char *)workspace;
-    DevHeader *hdr = (DevHeader *)(ws + L.header);
-    int *cnt = (int *)(ws + L.cnt), *nlc = (int *)(ws + L.nlc), *pre = (int *)(ws + L.pre);
-    uint8_t *keep = (uint8_t *)(ws + L.keep), *fpos = (uint8_t *)(ws + L.fpos);
-    int *blocksum = (int *)(ws + L.blocksum), *bstart = (int *)(ws + L.bstart);
-    int *seqcount = (int *)(ws + L.seqcount);
-    long long *cost = (long long *)(ws + L.cost);
+
+    // Shared memory of k_seq.  The host knows the mean length, not the longest: room for four times the
+    // mean (documents of one batch differ that much; a longer one works in the workspace), in powers of
+    // two up to SEQ_CAP_MAX.  Up to 8192 tokens the upper stages' arrays have room of their own for as
+    // many elements as tokens (deep trees keep most of them above stage 0); beyond, for 4096 elements
+    // (documents keep a few percent), over stage 0's prefix sums.
+    const long long mean = B > 0 ? ((long long)T + B - 1) / B : 0;
+    const long long want = B == 1 ? T : 4 * mean;
+    int cap = 1024;
+    while (cap < want && cap < SEQ_CAP_MAX) cap *= 2;
+    SeqArgs a{};
+    a.cap = cap;
+    a.uc = min(cap, 4096);
+    a.overlay = cap > 8192 ? 1 : 0;
+    const size_t smem = sizeof(uint16_t) * (3 * (size_t)cap + (a.overlay ? 2 : 6) * (size_t)a.uc);
+    static constexpr size_t kSmemMax = sizeof(uint16_t) * (3 * (size_t)SEQ_CAP_MAX + 2 * 4096);
+    static DevOnce attr_done;
+    if (!attr_done.done()) {
+        HDT_CUDA_CHECK(cudaFuncSetAttribute(k_seq, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+        attr_done.set();
+    }
+    DevHeader *hp = pinned_acquire();
+    if (!hp) return set_error(HDT_ERR_CUDA, "hdt_build_index: no pinned host memory for the index header");
+    hp->tail = kUnset;
 
     hdt_index *ix = new hdt_index();
     ix->batch = B; ix->total_tokens = T; ix->block_m = bm; ix->block_m_upper = bmu; ix->n_stages = 0;
@@ -830,212 +863,62 @@ extern "C" int hdt_build_index(const int8_t *level, const int32_t *parent, const
                               (int *)(base + L.s_up), (int *)(base + L.s_scu), (int *)(base + L.s_blocks),
                               (int *)(base + L.s_queue), (int *)(base + L.s_queue2)};
     }
-#define HDT_BUILD_CHECK(expr)                                                          \
-    do {                                                                               \
-        cudaError_t e_ = (expr);                                                       \
-        if (e_ != cudaSuccess) {                                                       \
-            delete ix;                                                                 \
-            return set_error(HDT_ERR_CUDA, "%s failed: %s", #expr, cudaGetErrorString(e_)); \
-        }                                                                              \
-    } while (0)
-
-    const int nel = max(T, B + 1);
-    const int g_el = (nel + 255) / 256;
-    const int g_chunk = max(1, (T + CHUNK - 1) / CHUNK);
-    const int g_stride = max(1, min((T + 255) / 256, 148 * 8));
-    static const int kSmemCap = 200 * 1024;
-    static DevOnce attr_done;
-    if (!attr_done.done()) {
-        HDT_BUILD_CHECK(cudaFuncSetAttribute(k_walk, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap));
-        HDT_BUILD_CHECK(cudaFuncSetAttribute(k_upper_stages, cudaFuncAttributeMaxDynamicSharedMemorySize, USMEM));
-        attr_done.set();
-    }
-    // One CTA builds all stages above 0 when they are small (documents: a few percent of the
-    // tokens, up to 3-4 stages).  A caller that allows many stages expects deep trees, whose upper
-    // stages hold most of the elements: those go through the per-stage kernels.
-    const bool fused_upper = (B <= UMAXB) && ms <= 8;
-    // The upper stages only need stage 0's compaction; with their own scratch they are built on the
-    // side stream while stage 0's blocks and queues are built on the caller's stream.
-    Side *sd = nullptr;
-    if (ms > 1 && !g_no_overlap && get_side(&sd) != HDT_OK) sd = nullptr;
-    // The per-stage kernels (deep trees, many sequences) as two chains: what the next stage waits for (counts,
-    // ranges, scan, compaction) on the caller's stream, the stage's blocks and queues (walk, block records,
-    // ranking), which nothing but the attention kernels reads, on the side stream behind the stage's compaction.
-    // The two share the family positions and the block scratch, so those alternate between two sets by stage
-    // parity, and stage s + 2 takes a set only when the walk of stage s has read it.
-    const bool piped = !fused_upper && sd != nullptr && ms > 1;
-
-    // Everything the build enqueues; returns the first CUDA error.  Called directly or under
-    // stream capture (see below).
-    int n_launched = 0;
-    auto enqueue_all = [&]() -> cudaError_t {
-        cudaError_t e;
-#define HDT_ENQ(expr) do { e = (expr); if (e != cudaSuccess) return e; } while (0)
-        // header, cnt and nlc are adjacent in the workspace: one memset clears all three
-        HDT_ENQ(cudaMemsetAsync(ws + L.header, 0, L.pre - L.header, st));
-        k_init<<<g_el, 256, 0, st>>>(level, parent, cu_seqlens, B, T, HDT_MAX_STAGES * 8, hdr, ix->st[0].tok,
-                                     ix->st[0].par, ix->st[0].scu, cnt, nlc);
-        ++n_launched;
-        auto launch_upper = [&](cudaStream_t s_) {
-            UpperArgs u;
-            for (int i = 0; i < HDT_MAX_STAGES; ++i) u.st[i] = ix->st[i < ms ? i : ms - 1];
-            u.max_stages = ms; u.B = B; u.bm = bmu; u.dirs = dirs;
-            u.cnt = cnt; u.nlc = nlc; u.pre = pre; u.keep = keep;
-            u.bstart = (int *)(ws + L.bstart2); u.seqcount = (int *)(ws + L.seqcount2);
-            u.fpos = (uint8_t *)(ws + L.fpos2); u.cost = (long long *)(ws + L.cost2);
-            u.rank = (int *)(ws + L.rank);
-            k_upper_stages<<<1, UT, USMEM, s_>>>(hdr, u);
-            ++n_launched;
-        };
-        for (int s = 0; s < ms; ++s) {
-            if (s >= 1 && fused_upper) {
-                if (sd) HDT_ENQ(cudaStreamWaitEvent(st, sd->join, 0));
-                else launch_upper(st);
-                break;
-            }
-            // (piped: the scratch set of this stage's parity)
-            const bool set2 = piped && (s & 1);
-            uint8_t *fpos_s = set2 ? (uint8_t *)(ws + L.fpos2) : fpos;
-            int *bstart_s = set2 ? (int *)(ws + L.bstart2) : bstart, *seqcount_s = set2 ? (int *)(ws + L.seqcount2) : seqcount;
-            long long *cost_s = set2 ? (long long *)(ws + L.cost2) : cost;
-            if (piped && s >= 2) HDT_ENQ(cudaStreamWaitEvent(st, sd->stage_ev[2 * (s - 2) + 1], 0));   // the walk of stage s - 2 has read fpos
-            const StagePtrs &P = ix->st[s];
-            // the last possible stage writes its (unused) next-stage arrays into its own up/pre scratch
-            const StagePtrs &N = ix->st[(s + 1 < ms) ? s + 1 : s];
-            const bool last = (s + 1 == ms);
-            // (a kernel chain per stage: the stage before counted this stage's children in its compaction)
-            HDT_ENQ(launch_chain(k_ranges, dim3(g_chunk), dim3(CHUNK), 0, st, hdr, s, s == 0 ? level : (const int8_t *)nullptr, P.par, cnt, nlc,
-                                 P.rng, keep, fpos_s, blocksum, dirs, s == 0 ? (const int *)nullptr : (const int *)P.tok, (int *)(ws + L.rank)));
-            // tok2 of the last possible stage is never read: point it at scratch (pre is rewritten first)
-            const bool chain = !fused_upper;     // (else the one-CTA builder counts for itself and expects cleared arrays)
-            HDT_ENQ(launch_chain(k_scan, dim3(g_chunk), dim3(CHUNK), 0, st, hdr, s, L.nchunk, keep, blocksum, P.tok, pre, P.up,
-                                 last ? cnt : N.tok, chain ? cnt : (int *)nullptr, chain ? nlc : (int *)nullptr));
-            n_launched += 2;
-            if (!last) {
-                HDT_ENQ(launch_chain(k_compact, dim3(g_stride), dim3(256), 0, st, hdr, s, B, P.par, P.up, pre, P.scu, N.par, N.scu, cnt, nlc,
-                                     chain ? 1 : 0));
-                ++n_launched;
-                if (s == 0 && sd && fused_upper) {   // fork: the upper stages start now
-                    HDT_ENQ(cudaEventRecord(sd->fork, st));
-                    HDT_ENQ(cudaStreamWaitEvent(sd->s, sd->fork, 0));
-                    launch_upper(sd->s);
-                    HDT_ENQ(cudaEventRecord(sd->join, sd->s));
-                }
-            }
-            cudaStream_t sb = st;        // the stream of the stage's blocks and queues
-            if (piped) {
-                sb = sd->s;
-                HDT_ENQ(cudaEventRecord(sd->stage_ev[2 * s], st));
-                HDT_ENQ(cudaStreamWaitEvent(sb, sd->stage_ev[2 * s], 0));
-            }
-            if (B > 0) {
-                int maxlen_smem = kSmemCap;  // sequences longer than this walk through global memory
-                const int bms = (s == 0) ? bm : bmu;
-                HDT_ENQ(launch_chain(k_walk, dim3(B), dim3(256), (size_t)kSmemCap, sb, hdr, s, bms, P.scu, fpos_s, bstart_s, seqcount_s, maxlen_smem));
-                if (piped) HDT_ENQ(cudaEventRecord(sd->stage_ev[2 * s + 1], sb));
-                const int gy = max(1, min(64, 2048 / max(B, 1)));   // enough CTAs to spread a few long sequences
-                HDT_ENQ(launch_chain(k_blocks, dim3(B, gy), dim3(256), 0, sb, hdr, s, bms, B, P.scu, bstart_s, seqcount_s, P.rng, P.up, P.blocks, cost_s));
-                HDT_ENQ(launch_chain(k_queue, dim3(max(1, min(L.capnb / 8 + 1, 148 * 4))), dim3(256), 0, sb, hdr, s, cost_s, P.blocks, P.queue, P.queue_split));
-                n_launched += 3;
-            } else if (piped) {
-                HDT_ENQ(cudaEventRecord(sd->stage_ev[2 * s + 1], sb));
-            }
-        }
-        if (piped) {      // the side chain joins the caller's stream
-            HDT_ENQ(cudaEventRecord(sd->join, sd->s));
-            HDT_ENQ(cudaStreamWaitEvent(st, sd->join, 0));
-        }
-        return cudaGetLastError();
-#undef HDT_ENQ
-    };
-
-    {
-        ProfScope ps(PROF_INDEX, st);
-        // The build is a dozen tiny kernels: launching them one by one is slower than running them.
-        // They are captured once into a CUDA graph, which is replayed while the same buffers, sizes
-        // and parameters come back (a few cached graphs per host thread).
-        struct GraphKey { const void *a, *b, *c, *w; int B, T, bm, ms, bmu, ov, dirs, pad; };   // no padding bytes: compared with memcmp
-        struct GraphCache { GraphKey key; cudaGraphExec_t exec; int launches; bool valid; unsigned long long used; };
-        // (a few entries, least recently used replaced: a loop that alternates between buffer sets replays instead of capturing again)
-        constexpr int kGraphs = 4;
-        static thread_local GraphCache cache[kGraphs]{};
-        static thread_local unsigned long long tick = 0;
-        const GraphKey key{level, parent, cu_seqlens, workspace, B, T, bm, ms, bmu, sd ? 1 : 0, dirs, 0};
-        static_assert(sizeof(GraphKey) == 4 * sizeof(void *) + 8 * sizeof(int), "GraphKey must not contain padding");
-        bool done = false;
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        // (the legacy and per-thread default streams cannot be captured)
-        const bool capturable = st != nullptr && st != cudaStreamLegacy && st != cudaStreamPerThread;
-        if (!g_no_graph && capturable && cudaStreamIsCapturing(st, &cap) == cudaSuccess &&
-            cap == cudaStreamCaptureStatusNone) {
-            GraphCache *hit = nullptr, *victim = &cache[0];
-            for (int i = 0; i < kGraphs; ++i) {
-                if (cache[i].valid && std::memcmp(&cache[i].key, &key, sizeof(key)) == 0) hit = &cache[i];
-                if (!cache[i].valid || (victim->valid && cache[i].used < victim->used)) victim = &cache[i];
-            }
-            if (hit) {
-                hit->used = ++tick;
-                if (cudaGraphLaunch(hit->exec, st) == cudaSuccess) { done = true; count_launch(hit->launches); }
-            } else if (cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
-                const cudaError_t e = enqueue_all();
-                cudaGraph_t g = nullptr;
-                const cudaError_t e2 = cudaStreamEndCapture(st, &g);
-                cudaGraphExec_t exec = nullptr;
-                if (e == cudaSuccess && e2 == cudaSuccess && g && cudaGraphInstantiate(&exec, g, 0) == cudaSuccess) {
-                    if (victim->valid) cudaGraphExecDestroy(victim->exec);
-                    *victim = GraphCache{key, exec, n_launched, true, ++tick};
-                    if (cudaGraphLaunch(exec, st) == cudaSuccess) { done = true; count_launch(n_launched); }
-                }
-                if (g) cudaGraphDestroy(g);
-                if (!done) (void)cudaGetLastError();   // fall back to direct launches below
-            }
-        }
-        if (!done) {
-            n_launched = 0;
-            HDT_BUILD_CHECK(enqueue_all());
-            count_launch(n_launched);
-        }
-    }
-    // The header comes back through a pinned host buffer (a copy to pageable memory would be staged
-    // by the driver).  First and last word of the buffer are set to a value the device never writes
-    // (status is 0 or negative, tail is 0) so that the host can watch the copy land: it is the last
-    // operation of the build on the stream, and its words arrive in order.
-    PinnedSlot slot_{nullptr, nullptr};
-    DevHeader *h_pinned = pinned_acquire(&slot_) ? slot_.p : nullptr;
-    if (!h_pinned) {
-        delete ix;
-        return set_error(HDT_ERR_CUDA, "hdt_build_index: no pinned host memory for the index header");
-    }
-    // every word of the (reused) landing buffer is poisoned, not only the two the host watches
-    for (size_t w = 0; w < sizeof(DevHeader) / sizeof(int); ++w) reinterpret_cast<int *>(h_pinned)[w] = kUnset;
-    ix->h_pinned = h_pinned;
-    ix->hdr_ev = slot_.ev;
-    ix->hdr_dev = hdr;
+    ix->h_pinned = hp;
+    ix->hdr_dev = (const DevHeader *)(ws + L.header);
     ix->stream = st;
     ix->max_stages = ms;
     ix->pending = 1;
+
+    a.level = level; a.parent = parent; a.cu = cu_seqlens;
+    a.B = B; a.T = T; a.ms = ms; a.bm = bm; a.bmu = bmu; a.bmin = bmin; a.dirs = dirs;
+    a.tok = ix->st[0].tok; a.par = ix->st[0].par; a.rng = ix->st[0].rng; a.up = ix->st[0].up; a.scu = ix->st[0].scu;
+    a.rank = (int *)(ws + L.rank);
+    a.info = (SeqInfo *)(ws + L.info);
+    a.counts = (int *)(ws + L.counts);
+    a.recs = (int4 *)(ws + L.recs);
+    a.capnb = L.capnb;
+    a.el = (int4 *)(ws + L.el);
+    a.upl = (int *)(ws + L.upl);
+    a.glob = (uint32_t *)(ws + L.glob);
+    a.glob_stride = al(sizeof(int) * (size_t)T) / sizeof(int);
+    FinishArgs f{};
+    for (int s = 0; s < ms; ++s) f.st[s] = ix->st[s];
+    f.cu = cu_seqlens; f.B = B; f.T = T; f.ms = ms; f.bm = bm; f.bmu = bmu; f.bmin = bmin; f.capnb = L.capnb;
+    f.gy = (int)min(16LL, max(1LL, mean / 2048));
+    f.r0 = max(1, min(32, L.capnb / 64));
+    f.info = a.info; f.counts = a.counts; f.recs = a.recs; f.el = a.el; f.upl = a.upl;
+    f.keys = (long long *)(ws + L.keys);
+    f.hdr = (DevHeader *)(ws + L.header);
+    f.host = hp;
+    cudaError_t e = cudaSuccess;
     {
-        // A deferred build leaves the caller's stream free for the attention kernel that follows: the
-        // copy goes to the side stream, behind an event (the fallback wait of index_ready is then on
-        // that stream).  Compute -> copy -> compute on one stream costs the kernel behind the copy a
-        // few microseconds.
-        cudaStream_t cs = st;
-        Side *sdc = nullptr;
-        if (params && params->deferred && !g_no_overlap && get_side(&sdc) == HDT_OK && sdc != nullptr &&
-            cudaEventRecord(sdc->fork, st) == cudaSuccess && cudaStreamWaitEvent(sdc->s, sdc->fork, 0) == cudaSuccess) {
-            cs = sdc->s;
-            ix->stream = cs;
+        ProfScope ps(PROF_INDEX, st);
+        if (B > 0) {
+            // a thread per element of short sequences: 8 warps (7 build the upper stages), else 32
+            k_seq<<<B, mean <= 1024 ? 256 : 1024, smem, st>>>(a);
+            count_launch();
+            e = cudaGetLastError();
         }
-        cudaError_t e_ = cudaMemcpyAsync(h_pinned, hdr, sizeof(DevHeader), cudaMemcpyDeviceToHost, cs);
-        if (e_ == cudaSuccess) e_ = cudaEventRecord(slot_.ev, cs);      // the end of the copy, as the runtime sees it
-        if (e_ != cudaSuccess) {
-            (void)cudaStreamSynchronize(cs);                              // the copy may be queued: let it land first
-            pinned_release(h_pinned, slot_.ev);
-            delete ix;
-            return set_error(HDT_ERR_CUDA, "queueing the copy of the index header failed: %s", cudaGetErrorString(e_));
+        if (e == cudaSuccess) {
+            // a programmatic dependent: its CTAs are scheduled while k_seq runs and wait for its end
+            cudaLaunchConfig_t cfg{};
+            cfg.gridDim = dim3((unsigned)(1 + f.r0 + (ms - 1) + (size_t)B * f.gy));
+            cfg.blockDim = dim3(FT);
+            cfg.stream = st;
+            cudaLaunchAttribute at[1];
+            at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            at[0].val.programmaticStreamSerializationAllowed = g_no_pdl ? 0 : 1;
+            cfg.attrs = at;
+            cfg.numAttrs = 1;
+            e = cudaLaunchKernelEx(&cfg, k_finish, f);
+            count_launch();
         }
     }
-#undef HDT_BUILD_CHECK
+    if (e != cudaSuccess) {
+        pinned_release(hp);
+        delete ix;
+        return set_error(HDT_ERR_CUDA, "hdt_build_index: launch failed: %s", cudaGetErrorString(e));
+    }
     if (!(params && params->deferred)) {
         const int rc = index_ready(ix);
         if (rc) {
@@ -1051,38 +934,32 @@ namespace hdt {
 int index_ready(const hdt_index *cix) {
     hdt_index *ix = const_cast<hdt_index *>(cix);
     if (ix->pending) {
-        // The host watches the copy land instead of sleeping in the driver: the first and the last
-        // word of the buffer change when (parts of) the copy have arrived.  That is only a hint — the
-        // bytes of one copy need not reach host memory in address order — so the event recorded
-        // behind the copy decides: it is polled (about a microsecond per query) and, after a bounded
-        // number of polls, waited for.
+        // The host watches the tail word of the pinned header, which the device writes last, behind a
+        // system-wide fence.  After a bounded number of looks it waits for the stream instead.
         DevHeader *hp = ix->h_pinned;
-        volatile int *p_status = &hp->status, *p_tail = &hp->tail;
-        bool landed = false;
-        for (long long spin = 0; spin < 20000000LL && !landed; ++spin) landed = (*p_tail != kUnset && *p_status != kUnset);
-        cudaError_t e_ = cudaErrorNotReady;
-        for (int poll = 0; poll < 200000 && e_ == cudaErrorNotReady; ++poll) e_ = cudaEventQuery(ix->hdr_ev);
-        if (e_ == cudaErrorNotReady) e_ = cudaEventSynchronize(ix->hdr_ev);
+        volatile int *p_tail = &hp->tail;
+        for (long long spin = 0; spin < 20000000LL && *p_tail == kUnset; ++spin) {}
+        cudaError_t e_ = cudaSuccess;
+        if (*p_tail == kUnset) {
+            e_ = cudaStreamSynchronize(ix->stream);
+            if (e_ == cudaSuccess && *p_tail == kUnset) e_ = cudaErrorUnknown;
+        }
+        ix->pending = 0;
+        ix->h_pinned = nullptr;
         if (e_ != cudaSuccess) {
             (void)cudaGetLastError();
-            (void)cudaStreamSynchronize(ix->stream);
-            ix->pending = 0;
             ix->failed = HDT_ERR_CUDA;
-            pinned_release(hp, ix->hdr_ev);
-            ix->h_pinned = nullptr;
+            pinned_release(hp);
             return set_error(HDT_ERR_CUDA, "waiting for the index build failed: %s", cudaGetErrorString(e_));
         }
         std::atomic_thread_fence(std::memory_order_acquire);
         const DevHeader h = *hp;
-        pinned_release(hp, ix->hdr_ev);
-        ix->h_pinned = nullptr;
-        ix->pending = 0;
+        pinned_release(hp);
         ix->failed = h.status;
         ix->err_pos = h.err_pos;
         if (h.status == 0) {
             int ns = 1;
             while (ns < ix->max_stages && h.st[ns].n > 0) ++ns;
-            // (a last stage that found "has_next" without one being built cannot happen below max_stages)
             if (h.st[ns - 1].has_next && ns == ix->max_stages) {
                 ix->failed = HDT_ERR_BAD_HIERARCHY;
                 ix->err_pos = -1;
@@ -1127,7 +1004,7 @@ extern "C" int hdt_index_export(const hdt_index_t *ix, int32_t stage, hdt_stage_
 }
 
 extern "C" int hdt_index_destroy(hdt_index_t *ix) {
-    if (ix && ix->pending) (void)index_ready(ix);     // the header copy must not land in a recycled buffer
+    if (ix && ix->pending) (void)index_ready(ix);     // the header must not land in a recycled buffer
     delete ix;
     return HDT_OK;
 }

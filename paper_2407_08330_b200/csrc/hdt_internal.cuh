@@ -49,7 +49,6 @@ struct hdt_index {
     int failed;                       // hdt_status_t found in the header (or by its check), 0 = fine
     int err_pos, max_stages;
     hdt::DevHeader *h_pinned;         // pinned landing buffer (from a pool), nullptr once released
-    cudaEvent_t hdr_ev;               // recorded behind the copy of the header into h_pinned
     const hdt::DevHeader *hdr_dev;    // the header in the index workspace
     cudaStream_t stream;              // stream of the build
 };
@@ -103,13 +102,11 @@ int sm_count(int *n_sm);
 struct Side {
     cudaStream_t s, s2, s3;
     cudaEvent_t fork, join, join2, join3, fork0, join0;      // fork0 / join0: a hand-over of their own for work that starts before `fork`
-    cudaEvent_t stage_ev[2 * HDT_MAX_STAGES];                // index build with a kernel chain per stage: [2 s] the stage's compaction is queued, [2 s + 1] its walk
     bool ready;
 };
 int get_side(Side **out);
 extern int g_no_overlap;   // option "no_overlap"
 extern int g_force_simt;   // option "force_simt"
-extern int g_no_graph;     // option "no_graph"
 extern int g_phase_stamps; // option "phase_stamps": the transposed backward runs its instrumented instantiation
 extern int g_no_fwd_mc;    // option "no_fwd_mc": blocks that are not self-contained stay on the 128-thread general forward kernel
 
