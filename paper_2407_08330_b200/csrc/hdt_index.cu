@@ -16,11 +16,15 @@
 // What bounds it: latency (about 40 bytes a token move; a chain of barriers and shared-memory round
 // trips per stage).  The stages of a sequence only meet the other sequences' in their offsets, so the
 // grid-wide steps (formerly nine launches for three stages and a hundred for twenty, each a launch
-// latency behind the one before) are one kernel boundary.
+// latency behind the one before) are one kernel boundary.  Device time: 57 tokens 15 us, 4 x 8192 tokens 24,
+// 2 x 32768 51, 200 trees of 20 stages 48; whole passes with the nine launches and with these: 81 -> 57 us
+// (57 tokens, fp32, build and forward), 76 -> 56 (8 x 2048, build and forward), 1100 -> 807 (200 trees, build,
+// forward and backward).
 #include <cstdio>
 #include <cstring>
 #include <atomic>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "hdt_internal.cuh"
@@ -45,7 +49,7 @@ struct Layout {
 
 static size_t al(size_t x) { return (x + 255) & ~size_t(255); }
 
-static constexpr int NGLOB = 9;      // element arrays of the sequences that do not fit in shared memory
+static constexpr int NGLOB = 11;      // element arrays of the sequences that do not fit in shared memory
 
 static Layout make_layout(int B, int T, int bm, int max_stages) {   // bm: the smaller of the two block sizes
     Layout L;
@@ -94,28 +98,74 @@ __device__ __forceinline__ int row_pairs(int e, int lo, int hi, int dirs) {
 template <class I> struct Elem;
 template <> struct Elem<uint16_t> {
     static constexpr unsigned NONE = 0xffffu, FLAG = 0x8000u, MASK = 0x7fffu;
-    static __device__ __forceinline__ void add(uint16_t *c, unsigned i) {
-        atomicAdd(reinterpret_cast<unsigned *>(c) + (i >> 1), 1u << ((i & 1) * 16));
+    static __device__ __forceinline__ unsigned *word(uint16_t *c, int &sh) {
+        sh = ((uintptr_t)c & 2) * 8;
+        return reinterpret_cast<unsigned *>((uintptr_t)c & ~(uintptr_t)3);
     }
-    static __device__ __forceinline__ void flag(uint16_t *c, unsigned i) {
-        atomicOr(reinterpret_cast<unsigned *>(c) + (i >> 1), FLAG << ((i & 1) * 16));
-    }
+    static __device__ __forceinline__ void add(uint16_t *c, unsigned v) { int sh; unsigned *q = word(c, sh); atomicAdd(q, v << sh); }
+    static __device__ __forceinline__ void flag(uint16_t *c) { int sh; unsigned *q = word(c, sh); atomicOr(q, FLAG << sh); }
 };
 template <> struct Elem<uint32_t> {
     static constexpr unsigned NONE = 0xffffffffu, FLAG = 0x80000000u, MASK = 0x7fffffffu;
-    static __device__ __forceinline__ void add(uint32_t *c, unsigned i) { atomicAdd(c + i, 1u); }
-    static __device__ __forceinline__ void flag(uint32_t *c, unsigned i) { atomicOr(c + i, FLAG); }
+    static __device__ __forceinline__ void add(uint32_t *c, unsigned v) { atomicAdd(c, v); }
+    static __device__ __forceinline__ void flag(uint32_t *c) { atomicOr(c, FLAG); }
 };
 
+// Arrays of a sequence.  Flat: in one piece.  Sliced: 2^sl elements in the shared memory of each CTA of the
+// sequence's cluster; another CTA's slice is read and added to over distributed shared memory (parents
+// of anchors, rows of a block that straddles two slices: a few percent of the accesses).
+template <class T> struct Flat {
+    using I = T;
+    I *base;
+    __device__ __forceinline__ I *ptr(unsigned e) const { return base + e; }
+    __device__ __forceinline__ unsigned get(unsigned e) const { return base[e]; }
+};
+template <class T>
+__device__ __forceinline__ T *map_rank(T *p, unsigned rank) {
+    uint64_t r;
+    asm("mapa.u64 %0, %1, %2;" : "=l"(r) : "l"(p), "r"(rank));
+    return reinterpret_cast<T *>(r);
+}
+struct Sliced {
+    using I = uint16_t;
+    I *loc;
+    unsigned sl, rank;
+    __device__ __forceinline__ I *ptr(unsigned e) const {
+        I *p = loc + (e & ((1u << sl) - 1u));
+        const unsigned r = e >> sl;
+        return r == rank ? p : map_rank(p, r);
+    }
+    __device__ __forceinline__ unsigned get(unsigned e) const {
+        const unsigned r = e >> sl;
+        return r == rank ? loc[e & ((1u << sl) - 1u)] : *ptr(e);
+    }
+};
+
+// Child counts of 32 consecutive elements (one per lane, NONE beyond the end): siblings follow one another,
+// so a run of equal parents is one addition (thirty additions to one word are thirty turns of the
+// shared-memory atomic unit).
+template <class A>
+__device__ __forceinline__ void count_children(const A &cnt, unsigned p, int lane) {
+    using E = Elem<typename A::I>;
+    const unsigned before = __shfl_up_sync(0xffffffffu, p, 1);
+    const bool first = lane == 0 || p != before;
+    const unsigned m = __ballot_sync(0xffffffffu, first);
+    if (first && p != E::NONE) {
+        const unsigned rest = lane == 31 ? 0u : m >> (lane + 1);
+        E::add(cnt.ptr(p), rest ? (unsigned)__ffs(rest) : 32u - (unsigned)lane);
+    }
+}
+
 static constexpr int SEQ_CAP_MAX = 32768;   // tokens of a sequence held in shared memory (15-bit counts)
-static constexpr int SB0 = 1024, SBU = 256; // block starts of stage 0 / an upper stage held in shared memory
+static constexpr int UC_MAX = 4096;         // elements of an upper stage held there
+static constexpr int SB0 = 1024, SBU = 256, SBW = 64; // block starts of stage 0 / an upper stage (by the CTA, by a warp) held there
+static constexpr int SEQ_CLUSTER = 8;       // CTAs of a long sequence
 
 struct SeqArgs {
     const int8_t *level;
     const int32_t *parent, *cu;
     int B, T, ms, bm, bmu, bmin, dirs;
-    int cap, uc;               // tokens of stage 0 / elements of an upper stage that fit in shared memory
-    int overlay;               // the upper stages' arrays lie over stage 0's prefix sums
+    int cap, uc, pool;         // tokens of stage 0 / elements of an upper stage that fit in shared memory; bytes for the upper stages
     int *tok, *par, *rng, *up, *scu;     // stage 0 (final, but for `up`: relative to the sequence)
     int *rank;
     SeqInfo *info;
@@ -130,57 +180,51 @@ struct SeqArgs {
 
 struct SeqShared {
     int bst0[SB0], bst[SBU];
-    int wtot[32], wtotu[32];
+    int wtot[32], wtotu[32], ctot[SEQ_CLUSTER];
     int err, err_pos, flag0, flag, nb0, nb, nf0, ne0, nf, ne;
+    int ns[HDT_MAX_STAGES], bsw[16][SBW], nfs[16], nes[16];     // (seq_upper_all)
     unsigned long long nnz, vis;
 };
 
-__device__ __forceinline__ void seq_fail(SeqShared &sh, int pos) {
-    if (atomicCAS(&sh.err, 0, HDT_ERR_BAD_HIERARCHY) == 0) sh.err_pos = pos;
+__device__ __forceinline__ void seq_fail(SeqShared *sh, int pos) {
+    if (atomicCAS(&sh->err, 0, HDT_ERR_BAD_HIERARCHY) == 0) sh->err_pos = pos;
 }
 
-// Barrier of the warps that build the upper stages (the last warp meanwhile walks stage 0's blocks).
+// Barrier of the warps that build the upper stages (with one CTA per sequence its last warp meanwhile walks stage 0's blocks).
 __device__ __forceinline__ void bar_upper(int n) { asm volatile("bar.sync 1, %0;" ::"r"(n) : "memory"); }
+__device__ __forceinline__ void seq_sync(unsigned cs) {
+    __syncwarp();
+    if (cs > 1) asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    else __syncthreads();
+}
 
-// Range and fate of one element.  root_real (stage 0 only): the sequence's first token is a root, not
-// PAD; a root without children is a family of its own there.  Returns whether a family holds it as a child.
-template <class I>
-__device__ __forceinline__ bool elem_range(const I *par, const I *cnt, int e, bool stage0, bool root_real, unsigned &p, unsigned &lo,
-                                           unsigned &hi) {
-    using E = Elem<I>;
-    p = par[e];
-    const unsigned y = cnt[e], c = y & E::MASK;
+// Range and fate of element e with parent p; y, yp: count words of the two.  lone_root: stage 0's root without children,
+// a family of its own there.  Returns whether a family holds the element as a child.
+template <class E>
+__device__ __forceinline__ bool elem_range(unsigned e, unsigned p, unsigned y, unsigned yp, bool lone_root, unsigned &lo, unsigned &hi) {
+    const unsigned c = y & E::MASK, cp = yp & E::MASK;
     lo = hi = 0;
-    if ((c > 0 && !(y & E::FLAG)) || (stage0 && e == 0 && c == 0 && root_real)) {
+    if ((c > 0 && !(y & E::FLAG)) || (lone_root && c == 0)) {
         lo = (p == E::NONE) ? e : e + 1;
         hi = e + 1 + c;
-    } else if (p != E::NONE) {
-        const unsigned yp = cnt[p], cp = yp & E::MASK;
-        if (cp > 0 && !(yp & E::FLAG)) {
-            lo = p;
-            hi = p + 1 + cp;
-            return true;
-        }
+    } else if (p != E::NONE && cp > 0 && !(yp & E::FLAG)) {
+        lo = p;
+        hi = p + 1 + cp;
+        return true;
     }
     return false;
 }
 
 // Greedy packing of row blocks (one thread): a cut that would split a family which starts inside the
-// block moves to the family's head.
-template <class I>
-__device__ __forceinline__ int walk_blocks(const I *par, const I *cnt, int n, int bm, int *bst, int nbst, int4 *rec) {
-    using E = Elem<I>;
+// block moves to the family's head.  fpos[e]: distance of e from the head of the family that holds it as
+// a child (0 = none, capped at 255 >= bm): one dependent load per block.
+__device__ __forceinline__ int walk_blocks(const uint8_t *fpos, int n, int bm, int *bst, int nbst, int4 *rec) {
     int pos = 0, nb = 0;
     while (pos < n) {
         int end = min(pos + bm, n);
         if (end < n) {
-            const unsigned p = par[end];
-            if (p != E::NONE && (int)p > pos) {
-                const unsigned yp = cnt[p];
-                const unsigned y = cnt[end];
-                const bool head = (y & E::MASK) > 0 && !(y & E::FLAG);
-                if (!head && (yp & E::MASK) > 0 && !(yp & E::FLAG)) end = (int)p;
-            }
+            const int f = fpos[end];
+            if (f < end - pos) end -= f;
         }
         if (nb < nbst) bst[nb] = pos; else rec[nb].x = pos;
         ++nb;
@@ -189,44 +233,42 @@ __device__ __forceinline__ int walk_blocks(const I *par, const I *cnt, int n, in
     return nb;
 }
 
-// Block records of one stage, one warp per block.
-template <class I>
-__device__ __forceinline__ void make_records(const I *par, const I *cnt, int n, bool stage0, bool root_real, int nb, const int *bst, int nbst,
-                                             int4 *rec, int w, int nw, int lane, int *nf, int *ne, unsigned long long *vis_out) {
-    using E = Elem<I>;
+// Records of the blocks i = i0, i0 + di, ... < i1 of a stage with nb blocks and n elements, one warp per block.
+// get(e, lo, hi) gives the range of an element and returns whether it lives on.  (The loops stay rolled: nearly
+// every instruction of this kernel is executed once or twice by a warp, and fetching it costs more than that.)
+template <class Get>
+__device__ __forceinline__ void make_records(Get get, int n, int nb, const int *bst, int nbst, int4 *rec, int i0, int i1, int di, int lane, int *nf,
+                                             int *ne, unsigned long long *vis_out) {
     long long vis = 0;
     int mf = 0, me = 0;
-    for (int i = w; i < nb; i += nw) {
+#pragma unroll 1
+    for (int i = i0; i < i1; i += di) {
         const int r0 = i < nbst ? bst[i] : rec[i].x;
         const int r1 = (i + 1 < nb) ? (i + 1 < nbst ? bst[i + 1] : rec[i + 1].x) : n;
-        int a = INT_MAX, bb = INT_MIN, carry = 0;
-        unsigned lo[4], hi[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int e = r0 + lane + 32 * k;
-            lo[k] = hi[k] = 0;
-            if (e < r1) {
-                unsigned p;
-                const bool child = elem_range<I>(par, cnt, e, stage0, root_real, p, lo[k], hi[k]);
-                if (hi[k] > lo[k]) { a = min(a, (int)lo[k]); bb = max(bb, (int)hi[k]); }
-                const bool real = !stage0 || p != E::NONE || (e == 0 && root_real);
-                if (real && !child) carry = 1;
-            }
+        // a block is dense where all its rows have one range
+        int a = INT_MAX, bb = INT_MIN, a2 = INT_MIN, bb2 = INT_MAX;
+        bool carry = false, none = false;
+#pragma unroll 1
+        for (int e = r0 + lane; e < r1; e += 32) {
+            int lo, hi;
+            carry |= get(e, lo, hi);
+            if (hi > lo) { a = min(a, lo); bb = max(bb, hi); a2 = max(a2, lo); bb2 = min(bb2, hi); }
+            else none = true;
         }
+        __syncwarp();
         a = __reduce_min_sync(0xffffffffu, a);
         bb = __reduce_max_sync(0xffffffffu, bb);
+        a2 = __reduce_max_sync(0xffffffffu, a2);
+        bb2 = __reduce_min_sync(0xffffffffu, bb2);
         carry = __any_sync(0xffffffffu, carry);
+        none = __any_sync(0xffffffffu, none);
         const bool any = bb > a;
+        const bool dense = any && !none && a == a2 && bb == bb2;
         if (!any) { a = r0; bb = r0; }
-        int dense = 1;
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-            if (r0 + lane + 32 * k < r1 && ((int)lo[k] != a || (int)hi[k] != bb)) dense = 0;
-        dense = __all_sync(0xffffffffu, dense);
         if (lane == 0) {
             int fl = 0;
             if (a >= r0 && bb <= r1) fl |= HDT_BLK_SELF;
-            if (dense && any) fl |= HDT_BLK_DENSE;
+            if (dense) fl |= HDT_BLK_DENSE;
             if (carry) fl |= HDT_BLK_CARRY;
             if (!any) fl |= HDT_BLK_EMPTY;
             rec[i] = make_int4(r0, a, bb, (r1 - r0) | (fl << 8));
@@ -261,108 +303,131 @@ __device__ __forceinline__ int warp_offsets(const int *wtot, int nw, int lane, i
     return v - v0;
 }
 
-// Stage 0 of one sequence up to the compaction, by all threads of the CTA.  X: parents, Y: counts,
-// Z: levels, then prefix sums of the keep flags.  Returns the number of kept elements.
-template <class I>
-__device__ __forceinline__ void seq_stage0(const SeqArgs &a, SeqShared &sh, I *X, I *Y, I *Z, int s0, int L, bool root_real) {
+// The part of a sequence one CTA holds in stage 0.
+struct Slice {
+    unsigned rank, cs, sl;     // CTA in the cluster, its size, log2 of the slice length
+    int s0, L, e0, ne;         // sequence start and length; first element of the slice and their number
+};
+
+// Stage 0 of one slice up to the keep flags: X parents, Y counts, Z levels and then the number of kept
+// elements before each kept one, relative to the slice.  sh: this CTA's, sh0: the first CTA's shared state.
+template <class A>
+__device__ __forceinline__ void seq_stage0(const SeqArgs &a, SeqShared &sh, SeqShared *sh0, const A &X, const A &Y, const A &Z, const Slice &c,
+                                           uint8_t *fpos, bool &root_real) {
+    using I = typename A::I;
     using E = Elem<I>;
     const int t = threadIdx.x, nt = blockDim.x, lane = t & 31, w = t >> 5, nw = nt >> 5;
-    for (int e = t; e < L; e += nt) {
-        const int p = a.parent[s0 + e], l = a.level[s0 + e];
-        bool ok = true;
-        unsigned q = E::NONE;
-        if (l < 0) ok = (l == -1 && p == -1);
-        else if (e == 0) ok = (l == 0 && p == -1);
-        else if (l > HDT_MAX_STAGES * 8 || p < 0 || p >= e) ok = false;
-        else q = (unsigned)p;
-        X[e] = (I)q;
-        Z[e] = (I)(uint8_t)l;
-        Y[e] = 0;
-        if (!ok) seq_fail(sh, s0 + e);
-    }
-    __syncthreads();
-    for (int e = t; e < L; e += nt) {
-        const unsigned p = X[e];
-        const int l = (int8_t)(uint8_t)Z[e];
-        if (l >= 0 && e > 0) {
-            if (p != E::NONE && (int)(int8_t)(uint8_t)Z[p] != l - 1) seq_fail(sh, s0 + e);
-            if ((int8_t)(uint8_t)Z[e - 1] < 0) seq_fail(sh, s0 + e);     // PAD only as a suffix
+    I *x = X.ptr(c.e0), *y = Y.ptr(c.e0), *z = Z.ptr(c.e0);
+    int bad = -1;
+    for (int i0 = 0; i0 < c.ne; i0 += 8 * nt) {          // (eight loads in flight per thread)
+        int p8[8], l8[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int i = i0 + k * nt + t;
+            if (i < c.ne) { p8[k] = a.parent[c.s0 + c.e0 + i]; l8[k] = a.level[c.s0 + c.e0 + i]; }
         }
-        if (p != E::NONE) E::add(Y, p);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int i = i0 + k * nt + t, e = c.e0 + i;
+            if (i >= c.ne) break;
+            const int p = p8[k], l = l8[k];
+            bool ok = true;
+            unsigned q = E::NONE;
+            if (l < 0) ok = (l == -1 && p == -1);
+            else if (e == 0) ok = (l == 0 && p == -1);
+            else if (l > HDT_MAX_STAGES * 8 || p < 0 || p >= e) ok = false;
+            else q = (unsigned)p;
+            x[i] = (I)q;
+            z[i] = (I)(uint8_t)l;
+            y[i] = 0;
+            if (!ok) bad = e;
+        }
     }
-    __syncthreads();
-    for (int e = t; e < L; e += nt) {
-        const unsigned p = X[e];
-        if (p != E::NONE && (Y[e] & E::MASK) > 0) E::flag(Y, p);
+    seq_sync(c.cs);
+    if (bad >= 0) seq_fail(sh0, c.s0 + bad);
+    root_real = c.L > 0 && (int8_t)(uint8_t)Z.get(0) >= 0;
+    for (int i0 = 32 * w; i0 < c.ne; i0 += nt) {
+        const int i = i0 + lane, e = c.e0 + i;
+        unsigned p = E::NONE;
+        if (i < c.ne) {
+            p = x[i];
+            const int l = (int8_t)(uint8_t)z[i];
+            if (l >= 0 && e > 0) {
+                if (p != E::NONE && (int)(int8_t)(uint8_t)Z.get(p) != l - 1) seq_fail(sh0, c.s0 + e);
+                if ((int8_t)(uint8_t)Z.get(e - 1) < 0) seq_fail(sh0, c.s0 + e);     // PAD only as a suffix
+            }
+        }
+        count_children(Y, p, lane);
     }
-    __syncthreads();
-    const int k = seg_shift(L, nw);
+    seq_sync(c.cs);
+    for (int i = t; i < c.ne; i += nt) {
+        const unsigned p = x[i];
+        if ((y[i] & E::MASK) > 0 && p != E::NONE) E::flag(Y.ptr(p));
+    }
+    seq_sync(c.cs);
+    const int k = seg_shift(c.ne, nw);
     int run = 0, next = 0;
     long long deg = 0;
-    for (int i = 0; i < (1 << (k - 5)); ++i) {
-        const int base = (w << k) + 32 * i, e = base + lane;
-        if (base >= L) break;
+    for (int i0 = w << k; i0 < min((w + 1) << k, c.ne); i0 += 32) {
+        const int i = i0 + lane, e = c.e0 + i, g = c.s0 + e;
         bool kp = false;
-        if (e < L) {
-            const bool real = (int8_t)(uint8_t)Z[e] >= 0;
-            unsigned p, lo, hi;
-            const bool child = elem_range<I>(X, Y, e, true, root_real, p, lo, hi);
-            if (child) {
-                if (!((int)p < e && e < (int)hi)) seq_fail(sh, s0 + e);
-                a.rank[s0 + e] = e - (int)p;        // the token's number among its siblings (hierarchical positions)
-            }
+        if (i < c.ne) {
+            const bool real = (int8_t)(uint8_t)z[i] >= 0;
+            const unsigned p = x[i];
+            unsigned lo, hi;
+            const bool child = elem_range<E>(e, p, y[i], p != E::NONE ? Y.get(p) : 0u, e == 0 && root_real, lo, hi);
+            if (child && !((int)p < e && e < (int)hi)) seq_fail(sh0, g);
             kp = real && !child;
-            const bool has = hi > lo;
-            reinterpret_cast<int2 *>(a.rng)[s0 + e] = make_int2(has ? s0 + (int)lo : 0, has ? s0 + (int)hi : 0);
-            a.tok[s0 + e] = s0 + e;
-            a.par[s0 + e] = (p == E::NONE) ? -1 : s0 + (int)p;
+            fpos[e] = child ? (uint8_t)min(e - (int)p, 255) : 0;
             deg += row_pairs(e, (int)lo, (int)hi, a.dirs);
             if (kp && p != E::NONE) next = 1;
         }
         const unsigned m = __ballot_sync(0xffffffffu, kp);
-        if (e < L) Z[e] = (I)(kp ? (unsigned)(run + __popc(m & ((1u << lane) - 1u))) : E::NONE);
+        if (i < c.ne) z[i] = (I)(kp ? (unsigned)(run + __popc(m & ((1u << lane) - 1u))) : E::NONE);
         run += __popc(m);
     }
     for (int o = 16; o; o >>= 1) deg += __shfl_xor_sync(0xffffffffu, deg, o);
     next = __any_sync(0xffffffffu, next);
     if (lane == 0) {
         sh.wtot[w] = run;
-        if (deg) atomicAdd(&sh.nnz, (unsigned long long)deg);
-        if (next) sh.flag0 = 1;
+        if (deg) atomicAdd(&sh0->nnz, (unsigned long long)deg);
+        if (next) sh0->flag0 = 1;
     }
+    __syncthreads();
+    int total;
+    const int mine = __shfl_sync(0xffffffffu, warp_offsets(sh.wtot, nw, lane, total), w);
+    if (mine)
+        for (int i = (w << k) + lane; i < min((w + 1) << k, c.ne); i += 32)
+            if (z[i] != E::NONE) z[i] = (I)(z[i] + mine);
+    if (t < (int)c.cs) (c.cs > 1 ? map_rank(&sh, t) : &sh)->ctot[c.rank] = total;      // to every CTA of the cluster
 }
 
-// Stage 0 -> stage 1: the kept elements' parents and tokens (only when the sequence has a stage 1), `up`.
-template <class I, class J>
-__device__ __forceinline__ void seq_compact0(const SeqArgs &a, const SeqShared &sh, const I *X, const I *Z, J *par2, J *tok2, int s0, int L, bool next) {
+// Stage 0 -> stage 1: the kept elements' parents and tokens.
+template <class A, class J>
+__device__ __forceinline__ void seq_compact0(const SeqArgs &a, const A &X, const A &Z, const int *coff, J *par2, J *tok2, const Slice &c) {
+    using I = typename A::I;
     using E = Elem<I>;
-    const int t = threadIdx.x, lane = t & 31, w = t >> 5, nw = blockDim.x >> 5;
-    const int k = seg_shift(L, nw);
-    int total;
-    const int wo = warp_offsets(sh.wtot, nw, lane, total);
-    const int mine = __shfl_sync(0xffffffffu, wo, w);
-    for (int i = 0; i < (1 << (k - 5)); ++i) {
-        const int base = (w << k) + 32 * i, e = base + lane;
-        if (base >= L) break;
-        const unsigned z = e < L ? Z[e] : E::NONE;
-        unsigned p = E::NONE, q = E::NONE;
-        if (z != E::NONE) { p = X[e]; if (p != E::NONE) q = Z[p]; }
-        const int wp = __shfl_sync(0xffffffffu, wo, q != E::NONE ? (int)(p >> k) : 0);
-        const int u = z != E::NONE ? (int)z + mine : -1;
-        if (e < L) a.up[s0 + e] = u;
-        if (u >= 0 && next) {
-            par2[u] = (J)(q != E::NONE ? q + (unsigned)wp : Elem<J>::NONE);
-            tok2[u] = (J)e;
+    const I *x = X.ptr(c.e0), *z = Z.ptr(c.e0);
+    for (int i = threadIdx.x; i < c.ne; i += blockDim.x) {
+        const unsigned v = z[i];
+        if (v != E::NONE) {
+            const int u = (int)v + coff[c.rank];
+            const unsigned p = x[i];
+            unsigned q = E::NONE;
+            if (p != E::NONE) q = Z.get(p);
+            par2[u] = (J)(q != E::NONE ? q + (unsigned)coff[p >> c.sl] : Elem<J>::NONE);
+            tok2[u] = (J)(c.e0 + i);
         }
     }
 }
 
-// All stages above 0 of one sequence, by the first nw warps of the CTA (tu threads).
+// All stages above 0 of one sequence, by the first nw warps of its first CTA.
 template <class J>
-__device__ __forceinline__ void seq_upper(const SeqArgs &a, SeqShared &sh, J *par, J *tok, J *par2, J *tok2, J *cnt, J *pre, int b, int s0,
-                                          int slot, int n, int &stages, int &res, int &more) {
+__device__ __forceinline__ void seq_upper(const SeqArgs &a, SeqShared &sh, J *par, J *tok, J *par2, J *tok2, J *cnt, J *pre, uint8_t *fpos, int b,
+                                          int s0, int slot, int n, int nw, int &stages, int &res, int &more) {
     using E = Elem<J>;
-    const int t = threadIdx.x, tu = blockDim.x - 32, lane = t & 31, w = t >> 5, nw = tu >> 5;
+    const int t = threadIdx.x, tu = nw * 32, lane = t & 31, w = t >> 5;
+    const Flat<J> C{cnt};
     int s = 1;
     while (true) {
         if (s == a.ms) { more = 1; break; }          // elements left that no stage may take
@@ -372,32 +437,31 @@ __device__ __forceinline__ void seq_upper(const SeqArgs &a, SeqShared &sh, J *pa
         for (int e = t; e < n; e += tu) cnt[e] = 0;
         if (t == 0) { sh.flag = 0; sh.nf = 0; sh.ne = 0; }
         bar_upper(tu);
-        for (int e = t; e < n; e += tu) { const unsigned p = par[e]; if (p != E::NONE) E::add(cnt, p); }
+        for (int e0 = 32 * w; e0 < n; e0 += tu) count_children(C, e0 + lane < n ? (unsigned)par[e0 + lane] : E::NONE, lane);
         bar_upper(tu);
         for (int e = t; e < n; e += tu) {
             const unsigned p = par[e];
-            if (p != E::NONE && (cnt[e] & E::MASK) > 0) E::flag(cnt, p);
+            if (p != E::NONE && (cnt[e] & E::MASK) > 0) E::flag(cnt + p);
         }
         bar_upper(tu);
-        if (t == 0) sh.nb = walk_blocks<J>(par, cnt, n, a.bmu, sh.bst, SBU, rec);
-        __syncwarp();
         const int k = seg_shift(n, nw);
         int run = 0, next = 0;
         long long deg = 0;
-        for (int i = 0; i < (1 << (k - 5)); ++i) {
-            const int base = (w << k) + 32 * i, e = base + lane;
-            if (base >= n) break;
+        for (int i0 = w << k; i0 < min((w + 1) << k, n); i0 += 32) {
+            const int e = i0 + lane;
             bool kp = false;
             if (e < n) {
-                unsigned p, lo, hi;
-                const bool child = elem_range<J>(par, cnt, e, false, false, p, lo, hi);
+                const unsigned p = par[e];
+                unsigned lo, hi;
+                const bool child = elem_range<E>(e, p, cnt[e], p != E::NONE ? cnt[p] : 0u, false, lo, hi);
                 const int tk = tok[e];
                 if (child) {
-                    if (!((int)p < e && e < (int)hi)) seq_fail(sh, s0 + tk);
+                    if (!((int)p < e && e < (int)hi)) seq_fail(&sh, s0 + tk);
                     a.rank[s0 + tk] = e - (int)p;
                 }
                 kp = !child;
                 el[e] = make_int4(tk, (p == E::NONE) ? -1 : (int)p, (int)lo, (int)hi);
+                fpos[e] = child ? (uint8_t)min(e - (int)p, 255) : 0;
                 deg += row_pairs(e, (int)lo, (int)hi, a.dirs);
                 if (kp && p != E::NONE) next = 1;
             }
@@ -414,16 +478,17 @@ __device__ __forceinline__ void seq_upper(const SeqArgs &a, SeqShared &sh, J *pa
         }
         bar_upper(tu);
         const bool go_on = sh.flag != 0;
+        if (t == tu - 1) sh.nb = walk_blocks(fpos, n, a.bmu, sh.bst, SBU, rec);
+        __syncwarp();
         int total;
         const int wo = warp_offsets(sh.wtotu, nw, lane, total);
-        const int mine = __shfl_sync(0xffffffffu, wo, w);
-        for (int i = 0; i < (1 << (k - 5)); ++i) {
-            const int base = (w << k) + 32 * i, e = base + lane;
-            if (base >= n) break;
+        for (int i0 = w << k; i0 < min((w + 1) << k, n); i0 += 32) {
+            const int e = i0 + lane;
             const unsigned z = e < n ? pre[e] : E::NONE;
             unsigned p = E::NONE, q = E::NONE;
             if (z != E::NONE) { p = par[e]; if (p != E::NONE) q = pre[p]; }
             const int wp = __shfl_sync(0xffffffffu, wo, q != E::NONE ? (int)(p >> k) : 0);
+            const int mine = __shfl_sync(0xffffffffu, wo, w);
             const int u = z != E::NONE ? (int)z + mine : -1;
             if (e < n) upl[e] = u;
             if (u >= 0 && go_on) {
@@ -431,7 +496,15 @@ __device__ __forceinline__ void seq_upper(const SeqArgs &a, SeqShared &sh, J *pa
                 tok2[u] = tok[e];
             }
         }
-        make_records<J>(par, cnt, n, false, false, sh.nb, sh.bst, SBU, rec, w, nw, lane, &sh.nf, &sh.ne, &sh.vis);
+        bar_upper(tu);
+        make_records([&](int e, int &lo, int &hi) {
+                         const unsigned p = par[e];
+                         unsigned l, h;
+                         const bool child = elem_range<E>(e, p, cnt[e], p != E::NONE ? cnt[p] : 0u, false, l, h);
+                         lo = (int)l; hi = (int)h;
+                         return !child;
+                     },
+                     n, sh.nb, sh.bst, SBU, rec, w, sh.nb, nw, lane, &sh.nf, &sh.ne, &sh.vis);
         bar_upper(tu);
         if (t == 0) {
             int *c = a.counts + (size_t)s * a.B + b;
@@ -448,63 +521,246 @@ __device__ __forceinline__ void seq_upper(const SeqArgs &a, SeqShared &sh, J *pa
     stages = s;
 }
 
-// A sequence's stages.  Shared memory per token of `cap`: 6 bytes (parents, counts, prefix sums) and,
-// per upper element of `uc`, 12 (two sets of parents and tokens, counts, prefix sums), of which 8 may
-// lie over stage 0's prefix sums, which are dead after its compaction.
-__global__ void __launch_bounds__(1024) k_seq(const SeqArgs a) {
+// The same for all stages at once, where the maps fit in the pool.  With g(e) the height of e in stage 1's
+// tree, e lives in the stages 1 .. g(parent of e) and heads its family in stage g(e): every stage's elements and
+// ranges follow from the heights, and the stages need not follow one another (twenty stages of a
+// 500-token tree: 50 us one by one, each a chain of six barriers).  Returns whether they fitted.
+__device__ __forceinline__ bool seq_upper_all(const SeqArgs &a, SeqShared &sh, const uint16_t *par, const uint16_t *tok, uint32_t *pool, size_t pool_bytes,
+                                              int b, int s0, int slot, int n, int nw, int &stages, int &res, int &more) {
+    using E = Elem<uint16_t>;
+    const int t = threadIdx.x, tu = nw * 32, lane = t & 31, w = t >> 5;
+    uint32_t *g = pool;
+    uint16_t *cn = reinterpret_cast<uint16_t *>(g + n);
+    const int n2 = (n + 1) & ~1;
+    for (int e = t; e < n2; e += tu) { if (e < n) g[e] = 0; cn[e] = 0; }
+    bar_upper(tu);
+    for (int e0 = 32 * w; e0 < n; e0 += tu) count_children(Flat<uint16_t>{cn}, e0 + lane < n ? (unsigned)par[e0 + lane] : E::NONE, lane);
+    bar_upper(tu);
+    for (int e = t; e < n; e += tu) {
+        if (cn[e] != 0) continue;
+        unsigned p = par[e];
+        for (unsigned k = 1; p != E::NONE; ++k) {          // climb while this leaf is the deepest seen
+            if (atomicMax(&g[p], k) >= k) break;
+            p = par[p];
+        }
+    }
+    bar_upper(tu);
+    const int S = min(1 + (int)g[0], a.ms);
+    uint16_t *map = cn + n2 - 2 * (size_t)n2;              // (used from stage 2 on)
+    uint8_t *fp = reinterpret_cast<uint8_t *>(cn + n2 + (size_t)max(S - 2, 0) * n2) - n2;      // (from stage 1 on)
+    const int nch = (n + 31) / 32;
+    uint16_t *coff = reinterpret_cast<uint16_t *>(fp + (size_t)max(S, 1) * n2) - 2 * nch;    // (from stage 2 on)
+    if (reinterpret_cast<uint8_t *>(pool) + pool_bytes < reinterpret_cast<uint8_t *>(coff + S * nch)) return false;
+    more = 1 + (int)g[0] > a.ms;
+    stages = S;
+    res = 1;
+    // tasks of 32 elements of one stage, dealt to the warps
+    for (int i = w; i < nch * (S - 2); i += nw) {
+        const int s = 2 + i / nch, ch = i % nch, e = 32 * ch + lane;
+        bool in = false;
+        if (e < n) { const unsigned p = par[e]; in = p == E::NONE || (int)g[p] >= s; }
+        const unsigned m = __ballot_sync(0xffffffffu, in);
+        if (e < n) map[s * (size_t)n2 + e] = in ? (uint16_t)__popc(m & ((1u << lane) - 1u)) : (uint16_t)E::NONE;
+        if (lane == 0) coff[s * nch + ch] = (uint16_t)__popc(m);
+    }
+    bar_upper(tu);
+    for (int s = 2 + w; s < S; s += nw) {
+        int run = 0;
+        for (int c0 = 0; c0 < nch; c0 += 32) {
+            const int c = c0 + lane, v0 = c < nch ? coff[s * nch + c] : 0;
+            int v = v0;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int x = __shfl_up_sync(0xffffffffu, v, o);
+                if (lane >= o) v += x;
+            }
+            if (c < nch) coff[s * nch + c] = (uint16_t)(run + v - v0);
+            run += __shfl_sync(0xffffffffu, v, 31);
+        }
+        if (lane == 0) sh.ns[s] = run;
+    }
+    if (t == 0) sh.ns[1] = n;
+    bar_upper(tu);
+    long long deg = 0;
+    for (int i = w; i < nch * (S - 1); i += nw) {
+        const int s = 1 + i / nch, ch = i % nch, e = 32 * ch + lane;
+        if (e >= n) continue;
+        const uint16_t *ms = map + s * (size_t)n2, *mn = ms + n2;
+        const unsigned p = par[e];
+        const int tk = tok[e], ge = (int)g[e], ce = cn[e];
+        int pos = e, pp = -1, gp = INT_MAX, cp = 0;
+        if (p != E::NONE) { gp = (int)g[p]; cp = cn[p]; }
+        if (gp < s) continue;                               // not in this stage
+        if (s > 1) pos = ms[e] + coff[s * nch + ch];
+        if (p != E::NONE) pp = s > 1 ? (int)ms[p] + coff[s * nch + (p >> 5)] : (int)p;
+        const bool child = gp == s;
+        int lo = 0, hi = 0;
+        if (ge == s) {
+            lo = p == E::NONE ? pos : pos + 1;
+            hi = pos + 1 + ce;
+        } else if (child) {
+            lo = pp;
+            hi = pp + 1 + cp;
+            if (!(pp < pos && pos < hi)) seq_fail(&sh, s0 + tk);
+            a.rank[s0 + tk] = pos - pp;
+        }
+        const size_t o = (size_t)(s - 1) * a.T + s0 + pos;
+        a.el[o] = make_int4(tk, pp, lo, hi);
+        a.upl[o] = child ? -1 : (s + 1 < S ? (int)mn[e] + coff[(s + 1) * nch + ch] : 0);
+        fp[s * (size_t)n2 + pos] = child ? (uint8_t)min(pos - pp, 255) : 0;
+        deg += row_pairs(pos, lo, hi, a.dirs);
+    }
+    for (int o = 16; o; o >>= 1) deg += __shfl_xor_sync(0xffffffffu, deg, o);
+    if (lane == 0 && deg) atomicAdd(&sh.nnz, (unsigned long long)deg);
+    bar_upper(tu);
+    for (int s = 1 + w; s < S; s += nw) {          // a warp per stage: its blocks
+        int4 *rec = a.recs + (size_t)s * a.capnb + slot;
+        const int4 *el = a.el + (size_t)(s - 1) * a.T + s0;
+        const int *upl = a.upl + (size_t)(s - 1) * a.T + s0;
+        const int ns = sh.ns[s];
+        int *bst = sh.bsw[w];
+        int nb = 0;
+        if (lane == 0) nb = walk_blocks(fp + s * (size_t)n2, ns, a.bmu, bst, SBW, rec);
+        nb = __shfl_sync(0xffffffffu, nb, 0);
+        if (lane == 0) { sh.nfs[w] = 0; sh.nes[w] = 0; }
+        __syncwarp();
+        make_records([&](int e, int &lo, int &hi) {
+            const int4 x = el[e];
+            lo = x.z; hi = x.w;
+            return upl[e] >= 0;
+        }, ns, nb, bst, SBW, rec, 0, nb, 1, lane, &sh.nfs[w], &sh.nes[w], &sh.vis);
+        if (lane == 0) {
+            int *c = a.counts + (size_t)s * a.B + b;
+            const size_t q = (size_t)a.ms * a.B;
+            c[0] = ns; c[q] = nb; c[2 * q] = sh.nfs[w]; c[3 * q] = sh.nes[w];
+        }
+        __syncwarp();
+    }
+    return true;
+}
+
+// A sequence's stages, by one CTA or, for long sequences, a cluster of SEQ_CLUSTER CTAs: stage 0 a slice per CTA
+// (one SM issues about 1500 instructions per 32 tokens of it: 25 us of an 8192-token sequence on one CTA), then
+// the stages above it on the first CTA while a thread of the second one walks stage 0's blocks, then the
+// records of stage 0's blocks, each by the CTA that holds its first row.
+// Shared memory: 6 bytes per token of the slice (parents, counts, prefix sums), `pool` for the upper stages, one
+// per token of `cap` for the walk.
+__global__ void __launch_bounds__(512) k_seq(const SeqArgs a) {
     pdl_launch_dependents();
     extern __shared__ __align__(16) uint16_t s_dyn[];
     __shared__ SeqShared sh;
-    const int b = blockIdx.x, t = threadIdx.x, lane = t & 31, w = t >> 5, nw = blockDim.x >> 5;
+    Slice c;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(c.rank));
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(c.cs));
+    const int b = blockIdx.x / c.cs, t = threadIdx.x, lane = t & 31, w = t >> 5, nw = blockDim.x >> 5;
     const int c0 = a.cu[b], c1 = a.cu[b + 1];
-    const int s0 = min(max(c0, 0), a.T), L = min(max(c1, s0), a.T) - s0;
+    c.s0 = min(max(c0, 0), a.T);
+    c.L = min(max(c1, c.s0), a.T) - c.s0;
+    c.sl = 5;
+    while (((long long)c.cs << c.sl) < c.L) ++c.sl;
+    c.e0 = min((int)(c.rank << c.sl), c.L);
+    c.ne = min(1 << c.sl, c.L - c.e0);
+    const bool first = c.rank == 0;
     if (t == 0) {
         sh.err = 0; sh.err_pos = 0; sh.flag0 = 0; sh.nf0 = 0; sh.ne0 = 0; sh.nnz = 0; sh.vis = 0;
-        if (c1 < c0 || c0 < 0 || c1 > a.T || (b == 0 && c0 != 0) || (b == a.B - 1 && c1 != a.T)) seq_fail(sh, b);
-        a.scu[b] = c0;
-        if (b == a.B - 1) a.scu[a.B] = c1;
+        if (first) {
+            if (c1 < c0 || c0 < 0 || c1 > a.T || (b == 0 && c0 != 0) || (b == a.B - 1 && c1 != a.T)) seq_fail(&sh, b);
+            a.scu[b] = c0;
+            if (b == a.B - 1) a.scu[a.B] = c1;
+        }
     }
-    const bool root_real = L > 0 && a.level[s0] >= 0;
-    const int slot = block_slot(s0, b, a.bmin);
-    __syncthreads();
-    const bool in_smem = L <= a.cap;
-    uint16_t *X = s_dyn, *Y = X + a.cap, *Z = Y + a.cap, *U = Z + a.cap;
+    SeqShared *sh0 = c.cs > 1 ? map_rank(&sh, 0) : &sh;
+    const int slot = block_slot(c.s0, b, a.bmin);
+    const int piece = a.cap / c.cs;
+    uint16_t *U = s_dyn + 3 * piece;
+    uint8_t *fu = reinterpret_cast<uint8_t *>(U + 6 * a.uc), *f0 = reinterpret_cast<uint8_t *>(U) + a.pool;
+    const unsigned wr = c.cs > 1 ? 1 : 0;          // CTA of the walk
+    const bool in_smem = c.L <= a.cap;
+    const Sliced X{s_dyn, c.sl, c.rank}, Y{s_dyn + piece, c.sl, c.rank}, Z{s_dyn + 2 * piece, c.sl, c.rank};
     uint32_t *G[NGLOB];
-    for (int i = 0; i < NGLOB; ++i) G[i] = a.glob + a.glob_stride * i + s0;
-    if (in_smem) seq_stage0<uint16_t>(a, sh, X, Y, Z, s0, L, root_real);
-    else seq_stage0<uint32_t>(a, sh, G[0], G[1], G[2], s0, L, root_real);
-    __syncthreads();
+    for (int i = 0; i < NGLOB; ++i) G[i] = a.glob + a.glob_stride * i + c.s0;
+    if (!in_smem) f0 = reinterpret_cast<uint8_t *>(a.glob + a.glob_stride * 9) + c.s0;
+    uint8_t *fw = (in_smem && c.cs > 1) ? map_rank(f0, wr) : f0;
+    const Flat<uint32_t> GX{G[0]}, GY{G[1]}, GZ{G[2]};
+    bool root_real = false;
+    if (in_smem) seq_stage0(a, sh, sh0, X, Y, Z, c, fw, root_real);
+    else seq_stage0(a, sh, sh0, GX, GY, GZ, c, fw, root_real);
+    seq_sync(c.cs);
     int n1;
-    (void)warp_offsets(sh.wtot, nw, lane, n1);
-    const bool next = sh.flag0 != 0;
-    const bool up_smem = n1 <= a.uc;
-    // (the first parent / token set of the upper stages never lies over the prefix sums)
-    uint16_t *P0 = U, *T0 = U + a.uc, *V = a.overlay ? Z : U + 2 * a.uc;
-    if (in_smem && up_smem) seq_compact0<uint16_t, uint16_t>(a, sh, X, Z, P0, T0, s0, L, next);
-    else if (in_smem) seq_compact0<uint16_t, uint32_t>(a, sh, X, Z, G[3], G[4], s0, L, next);
-    else if (up_smem && L < 65535) seq_compact0<uint32_t, uint16_t>(a, sh, G[0], G[2], P0, T0, s0, L, next);
-    else seq_compact0<uint32_t, uint32_t>(a, sh, G[0], G[2], G[3], G[4], s0, L, next);
+    const int coff_ = warp_offsets(sh.ctot, c.cs, lane, n1);
     __syncthreads();
+    if (w == 0 && lane < (int)c.cs) sh.ctot[lane] = coff_;          // (now the slices' offsets)
+    __syncthreads();
+    const bool next = sh0->flag0 != 0;
+    const bool up_smem = n1 <= a.uc && c.L < 65535;
+    uint16_t *P0 = c.cs > 1 ? map_rank(U, 0) : U, *T0 = P0 + a.uc;
+    if (!next) {}
+    else if (in_smem && up_smem) seq_compact0(a, X, Z, sh.ctot, P0, T0, c);
+    else if (in_smem) seq_compact0(a, X, Z, sh.ctot, G[3], G[4], c);
+    else if (up_smem) seq_compact0(a, GX, GZ, sh.ctot, P0, T0, c);
+    else seq_compact0(a, GX, GZ, sh.ctot, G[3], G[4], c);
+    seq_sync(c.cs);
     int stages = 1, res = n1, more = 0;
-    if (w == nw - 1) {
-        if (lane == 0)
-            sh.nb0 = in_smem ? walk_blocks<uint16_t>(X, Y, L, a.bm, sh.bst0, SB0, a.recs + slot)
-                             : walk_blocks<uint32_t>(G[0], G[1], L, a.bm, sh.bst0, SB0, a.recs + slot);
-    } else if (next) {
-        if (up_smem && (in_smem || L < 65535)) seq_upper<uint16_t>(a, sh, P0, T0, V, V + a.uc, V + 2 * a.uc, V + 3 * a.uc, b, s0, slot, n1, stages, res, more);
-        else seq_upper<uint32_t>(a, sh, G[3], G[4], G[5], G[6], G[7], G[8], b, s0, slot, n1, stages, res, more);
+    const int nwu = c.cs > 1 ? nw : nw - 1;
+    if (c.rank == wr && w == nw - 1) {
+        if (lane == 0) sh.nb0 = walk_blocks(f0, c.L, a.bm, sh.bst0, SB0, a.recs + slot);
+    } else if (first && next) {
+        const bool done = up_smem && seq_upper_all(a, sh, U, U + a.uc, reinterpret_cast<uint32_t *>(U + 2 * a.uc), a.pool - 4 * (size_t)a.uc, b, c.s0, slot, n1,
+                                                   nwu, stages, res, more);
+        if (done) {}
+        else if (up_smem) seq_upper<uint16_t>(a, sh, U, U + a.uc, U + 2 * a.uc, U + 3 * a.uc, U + 4 * a.uc, U + 5 * a.uc, fu, b, c.s0, slot, n1, nwu, stages, res, more);
+        else seq_upper<uint32_t>(a, sh, G[3], G[4], G[5], G[6], G[7], G[8], reinterpret_cast<uint8_t *>(a.glob + a.glob_stride * 10) + c.s0, b, c.s0, slot, n1, nwu, stages, res, more);
     }
+    seq_sync(c.cs);
+    const SeqShared *shw = c.cs > 1 ? map_rank(&sh, wr) : &sh;
+    const int nb0 = shw->nb0;
+    if (c.rank != wr)
+        for (int i = t; i < min(nb0, SB0); i += blockDim.x) sh.bst0[i] = shw->bst0[i];
     __syncthreads();
-    if (in_smem) make_records<uint16_t>(X, Y, L, true, root_real, sh.nb0, sh.bst0, SB0, a.recs + slot, w, nw, lane, &sh.nf0, &sh.ne0, &sh.vis);
-    else make_records<uint32_t>(G[0], G[1], L, true, root_real, sh.nb0, sh.bst0, SB0, a.recs + slot, w, nw, lane, &sh.nf0, &sh.ne0, &sh.vis);
-    __syncthreads();
-    if (t == 0) {
+    int i0 = 0, i1 = nb0, di = nw;      // the blocks that start in this slice
+    if (c.cs > 1 && nb0 <= SB0) {
+        auto before = [&](int e) {      // blocks that start before element e
+            int lo = 0, hi = nb0;
+            while (lo < hi) { const int mid = (lo + hi) >> 1; if (sh.bst0[mid] < e) lo = mid + 1; else hi = mid; }
+            return lo;
+        };
+        i0 = before(c.e0);
+        i1 = c.rank + 1 == c.cs ? nb0 : before(c.e0 + c.ne);
+    } else if (c.cs > 1) {
+        i0 = c.rank * nw;
+        di = c.cs * nw;
+    }
+    // (the elements' arrays are written here, not where they are first known: a cluster barrier waits for the
+    // CTA's outstanding stores, and the blocks cover every token)
+    auto records = [&](const auto &par, const auto &cnt, const auto &pre) {
+        using E = Elem<typename std::remove_reference_t<decltype(par)>::I>;
+        make_records([&](int e, int &lo, int &hi) {
+            const unsigned p = par.get(e);
+            const bool root = e == 0 && root_real;
+            unsigned l, h;
+            const bool child = elem_range<E>(e, p, cnt.get(e), p != E::NONE ? cnt.get(p) : 0u, root, l, h);
+            const bool kept = !child && (p != E::NONE || root);
+            lo = (int)l; hi = (int)h;
+            const bool has = h > l;
+            const int g = c.s0 + e;
+            reinterpret_cast<int2 *>(a.rng)[g] = make_int2(has ? c.s0 + lo : 0, has ? c.s0 + hi : 0);
+            a.tok[g] = g;
+            a.par[g] = p == E::NONE ? -1 : c.s0 + (int)p;
+            a.up[g] = kept ? (int)pre.get(e) + sh.ctot[e >> c.sl] : -1;
+            if (child) a.rank[g] = e - (int)p;       // the token's number among its siblings (hierarchical positions)
+            return kept;
+        }, c.L, nb0, sh.bst0, SB0, a.recs + slot, i0 + w, i1, di, lane, &sh0->nf0, &sh0->ne0, &sh0->vis);
+    };
+    if (in_smem) records(X, Y, Z);
+    else records(GX, GY, GZ);
+    seq_sync(c.cs);
+    if (first && t == 0) {
         const size_t q = (size_t)a.ms * a.B;
-        int *c = a.counts + b;
-        c[0] = L; c[q] = sh.nb0; c[2 * q] = sh.nf0; c[3 * q] = sh.ne0;
+        int *p = a.counts + b;
+        p[0] = c.L; p[q] = nb0; p[2 * q] = sh.nf0; p[3 * q] = sh.ne0;
         for (int s = stages; s < a.ms; ++s) {          // beyond its own stages: its root in a block of its own
-            c = a.counts + (size_t)s * a.B + b;
-            c[0] = res; c[q] = res; c[2 * q] = 0; c[3 * q] = res;
+            p = a.counts + (size_t)s * a.B + b;
+            p[0] = res; p[q] = res; p[2 * q] = 0; p[3 * q] = res;
         }
         SeqInfo f;
         f.stages = stages; f.res = res; f.err = sh.err; f.err_pos = sh.err_pos; f.more = more; f.pad = 0;
@@ -516,7 +772,7 @@ __global__ void __launch_bounds__(1024) k_seq(const SeqArgs a) {
 struct FinishArgs {
     StagePtrs st[HDT_MAX_STAGES];
     const int32_t *cu;
-    int B, T, ms, bm, bmu, bmin, capnb, gy, r0;   // gy: CTAs of a sequence; r0: CTAs that rank stage 0's blocks
+    int B, T, ms, bm, bmu, bmin, capnb, gy, r0, r1;   // gy: CTAs of a sequence; r0 / r1: CTAs that rank the blocks of stage 0 / of another stage
     const SeqInfo *info;
     const int *counts;
     const int4 *recs, *el;
@@ -534,6 +790,24 @@ __device__ __forceinline__ long long warp_sum(long long v) {
     return v;
 }
 
+// Sums over sequences [0, m) of rows row(i), i = w, w + nw, ...: four rows of a warp at a time, so that the
+// loads of one pass are in flight together.  put(i, sum) runs on lane 0.
+template <class Row, class Put>
+__device__ __forceinline__ void row_sums(int rows, int m, int w, int nw, int lane, Row row, Put put) {
+    for (int i0 = w; i0 < rows; i0 += 4 * nw) {
+        int v[4] = {0, 0, 0, 0};
+        for (int b = lane; b < m; b += 32)
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (i0 + k * nw < rows) v[k] += row(i0 + k * nw)[b];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int x = __reduce_add_sync(0xffffffffu, v[k]);
+            if (lane == 0 && i0 + k * nw < rows) put(i0 + k * nw, x);
+        }
+    }
+}
+
 // Header: totals over the sequences.  The words go to the workspace (kernels read them there) and
 // straight to the host's pinned buffer, the tail word last and behind a system-wide fence: the host
 // watches for it, so no copy has to be queued behind the build.
@@ -544,19 +818,15 @@ __device__ void finish_header(const FinishArgs &f, int S) {
     if (t == 0) { s_err = 0x7fffffff; s_more = 0; s_sum[0] = s_sum[1] = 0; }
     __syncthreads();
     const size_t q = (size_t)f.ms * f.B;
-    for (int i = w; i < 4 * S; i += FT / 32) {
-        const int s = i >> 2, c = i & 3;
-        int v = 0;
-        for (int b = lane; b < f.B; b += 32) v += f.counts[c * q + (size_t)s * f.B + b];
-        v = __reduce_add_sync(0xffffffffu, v);
-        if (lane == 0) {
-            StageDesc &d = f.hdr->st[s], &h = f.host->st[s];
-            int *pd = c == 0 ? &d.n : c == 1 ? &d.nb : c == 2 ? &d.n_fused : &d.n_empty;
-            int *ph = c == 0 ? &h.n : c == 1 ? &h.nb : c == 2 ? &h.n_fused : &h.n_empty;
-            *pd = v;
-            *reinterpret_cast<volatile int *>(ph) = v;
-        }
-    }
+    row_sums(4 * S, f.B, w, FT / 32, lane, [&](int i) { return f.counts + (i & 3) * q + (size_t)(i >> 2) * f.B; },
+             [&](int i, int v) {
+                 StageDesc &d = f.hdr->st[i >> 2], &h = f.host->st[i >> 2];
+                 const int c = i & 3;
+                 int *pd = c == 0 ? &d.n : c == 1 ? &d.nb : c == 2 ? &d.n_fused : &d.n_empty;
+                 int *ph = c == 0 ? &h.n : c == 1 ? &h.nb : c == 2 ? &h.n_fused : &h.n_empty;
+                 *pd = v;
+                 *reinterpret_cast<volatile int *>(ph) = v;
+             });
     long long nnz = 0, vis = 0;
     for (int b = t; b < f.B; b += FT) {
         const SeqInfo &x = f.info[b];
@@ -596,7 +866,7 @@ __device__ void finish_header(const FinishArgs &f, int S) {
 // Every CTA gathers all keys (cost << 1 | SELF non-EMPTY), a warp ranks a block at a time.
 __device__ void finish_rank(const FinishArgs &f, int s, int part, int parts, long long *s_keys) {
     const int t = threadIdx.x, lane = t & 31, w = t >> 5, nw = FT / 32;
-    __shared__ int s_base[FT], s_cnt[FT], s_w[FT / 32];
+    __shared__ int s_base[FT], s_slot[FT], s_w[FT / 32];
     const int *cb = f.counts + (size_t)f.ms * f.B + (size_t)s * f.B;
     int nb = 0;
     for (int b = t; b < f.B; b += FT) nb += cb[b];
@@ -613,26 +883,24 @@ __device__ void finish_rank(const FinishArgs &f, int s, int part, int parts, lon
         int v = c;
         for (int o = 1; o < 32; o <<= 1) { const int x = __shfl_up_sync(0xffffffffu, v, o); if (lane >= o) v += x; }
         if (lane == 31) s_w[w] = v;
+        // (beyond its own stages a sequence has its root alone, in a block without keys: cost 0)
+        s_slot[t] = (b < f.B && s < f.info[b].stages) ? block_slot(min(max(f.cu[b], 0), f.T), b, f.bmin) : -1;
         __syncthreads();
         int off = run, all = 0;
         for (int i = 0; i < nw; ++i) { if (i < w) off += s_w[i]; all += s_w[i]; }
         s_base[t] = off + v - c;
-        s_cnt[t] = c;
         __syncthreads();
-        const int nseq = min(FT, f.B - b0);
-        for (int i = w; i < nseq; i += nw) {
-            const int bb = b0 + i;
-            const bool own = s < f.info[bb].stages;     // else its root alone, in a block without keys: cost 0
-            const int4 *rec = f.recs + (size_t)s * f.capnb + block_slot(min(max(f.cu[bb], 0), f.T), bb, f.bmin);
-            for (int j = lane; j < s_cnt[i]; j += 32) {
-                long long k = 0;
-                if (own) {
-                    const int4 r = rec[j];
-                    const int fl = r.w >> 8;
-                    k = ((long long)(r.w & 255) * (r.z - r.y)) * 2 + ((fl & HDT_BLK_SELF) && !(fl & HDT_BLK_EMPTY) ? 1 : 0);
-                }
-                keys[s_base[i] + j] = k;
+        // a thread per block; its sequence is the last one that starts at or before it (an empty one has the base of its successor)
+        for (int j = run + t; j < run + all; j += FT) {
+            int lo = 0, hi = FT;
+            while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (s_base[mid] <= j) lo = mid; else hi = mid; }
+            long long k = 0;
+            if (s_slot[lo] >= 0) {
+                const int4 r = f.recs[(size_t)s * f.capnb + s_slot[lo] + (j - s_base[lo])];
+                const int fl = r.w >> 8;
+                k = ((long long)(r.w & 255) * (r.z - r.y)) * 2 + ((fl & HDT_BLK_SELF) && !(fl & HDT_BLK_EMPTY) ? 1 : 0);
             }
+            keys[j] = k;
         }
         run += all;
         __syncthreads();
@@ -655,24 +923,44 @@ __device__ void finish_rank(const FinishArgs &f, int s, int part, int parts, lon
     }
 }
 
-// CTA 0: header; then r0 CTAs rank stage 0's blocks and one each those of the other stages; then gy
+// CTA 0: header; then r0 CTAs rank stage 0's blocks and r1 each those of the other stages; then gy
 // CTAs per sequence move its elements and block records to their place in the batch's arrays.
 __global__ void __launch_bounds__(FT) k_finish(const FinishArgs f) {
     pdl_launch_dependents();
-    pdl_wait();
     __shared__ long long s_keys[FKEYS];
     __shared__ int s_stages, s_bad;
-    __shared__ int s_n[HDT_MAX_STAGES + 1], s_b[HDT_MAX_STAGES + 1], s_tot[HDT_MAX_STAGES + 1];
+    __shared__ int s_n[HDT_MAX_STAGES], s_b[HDT_MAX_STAGES], s_cn[HDT_MAX_STAGES], s_cb[HDT_MAX_STAGES];
     const int t = threadIdx.x, lane = t & 31, w = t >> 5, nw = FT / 32;
+    const int first_seq = 1 + f.r0 + f.r1 * (f.ms - 1);
+    const bool seq = (int)blockIdx.x >= first_seq;
+    const int b = seq ? ((int)blockIdx.x - first_seq) / f.gy : 0, y = seq ? ((int)blockIdx.x - first_seq) % f.gy : 0;
+    const size_t q = (size_t)f.ms * f.B;
     if (t == 0) { s_stages = 1; s_bad = 0; }
     __syncthreads();
-    {
-        int m = 1, bad = 0;
-        for (int b = t; b < f.B; b += FT) { m = max(m, f.info[b].stages); bad |= f.info[b].err; }
-        m = __reduce_max_sync(0xffffffffu, m);
-        bad = __any_sync(0xffffffffu, bad);
-        if (lane == 0) { atomicMax(&s_stages, m); if (bad) s_bad = 1; }
+    pdl_wait();
+    // One round of loads: the stages of the batch and its errors; in a sequence's CTA also the sums over the
+    // sequences before it (elements and blocks of every stage) and its own numbers.
+    int m = 1, bad = 0, s0 = 0, L = 0;
+    SeqInfo info{};
+    if (seq) {
+        info = f.info[b];
+        s0 = f.cu[b];
+        L = f.cu[b + 1] - s0;
+        if (t < f.ms) {
+            s_cn[t] = f.counts[(size_t)t * f.B + b];
+            s_cb[t] = f.counts[q + (size_t)t * f.B + b];
+        }
     }
+    for (int i = t; i < f.B; i += FT) { m = max(m, f.info[i].stages); bad |= f.info[i].err; }
+    if (seq)
+        row_sums(2 * f.ms, b, w, nw, lane, [&](int i) { return f.counts + ((i & 1) ? q : 0) + (size_t)(i >> 1) * f.B; },
+                 [&](int i, int v) {
+                     if (i & 1) s_b[i >> 1] = v;
+                     else s_n[i >> 1] = v;
+                 });
+    m = __reduce_max_sync(0xffffffffu, m);
+    bad = __any_sync(0xffffffffu, bad);
+    if (lane == 0) { atomicMax(&s_stages, m); if (bad) s_bad = 1; }
     __syncthreads();
     const int S = s_stages;
     int id = blockIdx.x;
@@ -681,73 +969,65 @@ __global__ void __launch_bounds__(FT) k_finish(const FinishArgs f) {
     id -= 1;
     if (id < f.r0) { finish_rank(f, 0, id, f.r0, s_keys); return; }
     id -= f.r0;
-    if (id < f.ms - 1) { if (id + 1 < S) finish_rank(f, id + 1, 0, 1, s_keys); return; }
-    id -= f.ms - 1;
-    const int b = id / f.gy, y = id % f.gy;
-    // sums over the sequences before this one: elements and blocks of every stage
-    const size_t q = (size_t)f.ms * f.B;
-    for (int i = w; i < 2 * S; i += nw) {
-        const int s = i >> 1;
-        const int *c = f.counts + ((i & 1) ? q : 0) + (size_t)s * f.B;
-        int v = 0;
-        for (int j = lane; j < b; j += 32) v += c[j];
-        v = __reduce_add_sync(0xffffffffu, v);
-        if (lane == 0) {
-            if (i & 1) s_b[s] = v;
-            else { s_n[s] = v; s_tot[s] = v + c[b]; }      // (s_tot: the batch's elements where b is the last sequence)
-        }
-    }
-    __syncthreads();
-    const SeqInfo info = f.info[b];
-    const int s0 = f.cu[b], L = f.cu[b + 1] - s0;
+    if (!seq) { if (id / f.r1 + 1 < S) finish_rank(f, id / f.r1 + 1, id % f.r1, f.r1, s_keys); return; }
     const int step = FT * f.gy, me = y * FT + t;
+    const int slot = block_slot(s0, b, f.bmin);
     {
         int *up = f.st[0].up;
         const int off = S > 1 ? s_n[1] : 0;
-        for (int e = me; e < L; e += step) {
-            const int v = up[s0 + e];
-            if (v >= 0) up[s0 + e] = S > 1 ? v + off : -1;
+        for (int e = me; e < L; e += 4 * step) {
+            int v[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) v[k] = e + k * step < L ? up[s0 + e + k * step] : -1;
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (v[k] >= 0) up[s0 + e + k * step] = S > 1 ? v[k] + off : -1;
         }
     }
-    const int slot = block_slot(s0, b, f.bmin);
-    for (int s = 0; s < S; ++s) {
+    // stage 0's records by all threads, then a stage per warp (deep trees have twenty small ones)
+    auto put_records = [&](int s, int i0, int di) {
         const StagePtrs &P = f.st[s];
         const int off = s ? s_n[s] : s0, boff = s_b[s];
+        const int4 *rec = f.recs + (size_t)s * f.capnb + slot;
+        for (int i = i0; i < s_cb[s]; i += di) {
+            const int4 r = rec[i];
+            int fl = r.w >> 8;
+            if (s + 1 == S) fl &= ~HDT_BLK_CARRY;
+            int *o = P.blocks + 5 * (size_t)(boff + i);
+            o[0] = off + r.x; o[1] = off + r.x + (r.w & 255); o[2] = off + r.y; o[3] = off + r.z; o[4] = fl;
+        }
+    };
+    put_records(0, me, step);
+    const int split = S > 4 ? 1 : nw / max(S - 1, 1);      // warps that share a stage of a hierarchy of few
+    for (int s = 1 + w / split; s < S; s += nw / split) {
+        const StagePtrs &P = f.st[s];
+        const int off = s_n[s], n = s_cn[s];
         const bool last = s + 1 == S;
-        const int n = f.counts[(size_t)s * f.B + b], nb = f.counts[q + (size_t)s * f.B + b];
-        if (s > 0 && me == 0) {
+        const int noff = last ? 0 : s_n[s + 1];
+        const int i0 = (y * split + w % split) * 32 + lane, di = f.gy * split * 32;
+        if (i0 == 0) {
             P.scu[b] = off;
-            if (b == f.B - 1) P.scu[f.B] = s_tot[s];
+            if (b == f.B - 1) P.scu[f.B] = off + n;
         }
         if (s < info.stages) {
-            if (s > 0) {
-                const int4 *el = f.el + (size_t)(s - 1) * f.T + s0;
-                const int *upl = f.upl + (size_t)(s - 1) * f.T + s0;
-                const int noff = last ? 0 : s_n[s + 1];
-                for (int e = me; e < n; e += step) {
-                    const int4 x = el[e];
-                    const int u = upl[e];
-                    const bool has = x.w > x.z;
-                    P.tok[off + e] = s0 + x.x;
-                    P.par[off + e] = x.y < 0 ? -1 : off + x.y;
-                    reinterpret_cast<int2 *>(P.rng)[off + e] = make_int2(has ? off + x.z : 0, has ? off + x.w : 0);
-                    P.up[off + e] = (u < 0 || last) ? -1 : u + noff;
-                }
+            const int4 *el = f.el + (size_t)(s - 1) * f.T + s0;
+            const int *upl = f.upl + (size_t)(s - 1) * f.T + s0;
+            for (int e = i0; e < n; e += di) {
+                const int4 x = el[e];
+                const int u = upl[e];
+                const bool has = x.w > x.z;
+                P.tok[off + e] = s0 + x.x;
+                P.par[off + e] = x.y < 0 ? -1 : off + x.y;
+                reinterpret_cast<int2 *>(P.rng)[off + e] = make_int2(has ? off + x.z : 0, has ? off + x.w : 0);
+                P.up[off + e] = (u < 0 || last) ? -1 : u + noff;
             }
-            const int4 *rec = f.recs + (size_t)s * f.capnb + slot;
-            for (int i = me; i < nb; i += step) {
-                const int4 r = rec[i];
-                int fl = r.w >> 8;
-                if (last) fl &= ~HDT_BLK_CARRY;
-                int *o = P.blocks + 5 * (size_t)(boff + i);
-                o[0] = off + r.x; o[1] = off + r.x + (r.w & 255); o[2] = off + r.y; o[3] = off + r.z; o[4] = fl;
-            }
-        } else if (info.res && me == 0) {       // (res is 0 or 1 here)
+            put_records(s, i0, di);
+        } else if (info.res && i0 == 0) {       // (res is 0 or 1 here)
             P.tok[off] = s0;
             P.par[off] = -1;
             reinterpret_cast<int2 *>(P.rng)[off] = make_int2(0, 0);
-            P.up[off] = last ? -1 : s_n[s + 1];
-            int *o = P.blocks + 5 * (size_t)boff;
+            P.up[off] = last ? -1 : noff;
+            int *o = P.blocks + 5 * (size_t)s_b[s];
             o[0] = off; o[1] = off + 1; o[2] = off; o[3] = off;
             o[4] = HDT_BLK_SELF | HDT_BLK_EMPTY | (last ? 0 : HDT_BLK_CARRY);
         }
@@ -830,19 +1110,20 @@ extern "C" int hdt_build_index(const int8_t *level, const int32_t *parent, const
 
     // Shared memory of k_seq.  The host knows the mean length, not the longest: room for four times the
     // mean (documents of one batch differ that much; a longer one works in the workspace), in powers of
-    // two up to SEQ_CAP_MAX.  Up to 8192 tokens the upper stages' arrays have room of their own for as
-    // many elements as tokens (deep trees keep most of them above stage 0); beyond, for 4096 elements
-    // (documents keep a few percent), over stage 0's prefix sums.
+    // two up to SEQ_CAP_MAX.  Upper stages: as many elements as tokens up to UC_MAX (deep trees keep most of
+    // their tokens above stage 0, documents a few percent).  One CTA where a mean sequence is an element
+    // or two per thread of it, else a cluster.
     const long long mean = B > 0 ? ((long long)T + B - 1) / B : 0;
     const long long want = B == 1 ? T : 4 * mean;
     int cap = 1024;
     while (cap < want && cap < SEQ_CAP_MAX) cap *= 2;
+    const int cs = mean > 768 ? SEQ_CLUSTER : 1, threads = 512;
     SeqArgs a{};
     a.cap = cap;
-    a.uc = min(cap, 4096);
-    a.overlay = cap > 8192 ? 1 : 0;
-    const size_t smem = sizeof(uint16_t) * (3 * (size_t)cap + (a.overlay ? 2 : 6) * (size_t)a.uc);
-    static constexpr size_t kSmemMax = sizeof(uint16_t) * (3 * (size_t)SEQ_CAP_MAX + 2 * 4096);
+    a.uc = min(cap, UC_MAX);
+    a.pool = (cap <= 2048 ? 32 : 16) * a.uc;       // (13 at least, for the stages one by one)
+    const size_t smem = 6 * (size_t)(cap / cs) + a.pool + cap;
+    static constexpr size_t kSmemMax = 6 * 8192 + 16 * UC_MAX + SEQ_CAP_MAX;
     static DevOnce attr_done;
     if (!attr_done.done()) {
         HDT_CUDA_CHECK(cudaFuncSetAttribute(k_seq, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
@@ -885,7 +1166,8 @@ extern "C" int hdt_build_index(const int8_t *level, const int32_t *parent, const
     for (int s = 0; s < ms; ++s) f.st[s] = ix->st[s];
     f.cu = cu_seqlens; f.B = B; f.T = T; f.ms = ms; f.bm = bm; f.bmu = bmu; f.bmin = bmin; f.capnb = L.capnb;
     f.gy = (int)min(16LL, max(1LL, mean / 2048));
-    f.r0 = max(1, min(32, L.capnb / 64));
+    f.r0 = max(1, min(64, L.capnb / 16));
+    f.r1 = ms > 4 ? max(1, min(8, L.capnb / 128)) : max(1, min(16, L.capnb / 64));
     f.info = a.info; f.counts = a.counts; f.recs = a.recs; f.el = a.el; f.upl = a.upl;
     f.keys = (long long *)(ws + L.keys);
     f.hdr = (DevHeader *)(ws + L.header);
@@ -894,15 +1176,23 @@ extern "C" int hdt_build_index(const int8_t *level, const int32_t *parent, const
     {
         ProfScope ps(PROF_INDEX, st);
         if (B > 0) {
-            // a thread per element of short sequences: 8 warps (7 build the upper stages), else 32
-            k_seq<<<B, mean <= 1024 ? 256 : 1024, smem, st>>>(a);
+            cudaLaunchConfig_t cfg{};
+            cfg.gridDim = dim3((unsigned)(B * cs));
+            cfg.blockDim = dim3(threads);
+            cfg.dynamicSmemBytes = smem;
+            cfg.stream = st;
+            cudaLaunchAttribute at[1];
+            at[0].id = cudaLaunchAttributeClusterDimension;
+            at[0].val.clusterDim.x = cs; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+            cfg.attrs = at;
+            cfg.numAttrs = 1;
+            e = cudaLaunchKernelEx(&cfg, k_seq, a);
             count_launch();
-            e = cudaGetLastError();
         }
         if (e == cudaSuccess) {
             // a programmatic dependent: its CTAs are scheduled while k_seq runs and wait for its end
             cudaLaunchConfig_t cfg{};
-            cfg.gridDim = dim3((unsigned)(1 + f.r0 + (ms - 1) + (size_t)B * f.gy));
+            cfg.gridDim = dim3((unsigned)(1 + f.r0 + f.r1 * (ms - 1) + (size_t)B * f.gy));
             cfg.blockDim = dim3(FT);
             cfg.stream = st;
             cudaLaunchAttribute at[1];
