@@ -73,6 +73,8 @@ static int g_no_multi_upper = 0;
 static int g_no_self_beside = 0;
 static int g_no_fused_delta = 0;
 static int g_no_fold = 0;
+static int g_no_rows = 0;
+static long long g_rows_lim[4] = {2000000000, 30000000, 10, 64};
 
 int get_side(Side **out) {
     int dev = -1;
@@ -183,6 +185,8 @@ extern "C" int hdt_set_option(const char *name, int32_t value) {
     if (name && std::strcmp(name, "bwd_walk") == 0) { g_bwd_walk = value; return HDT_OK; }
     if (name && std::strcmp(name, "no_multi_upper") == 0) { g_no_multi_upper = value; return HDT_OK; }
     if (name && std::strcmp(name, "no_self_beside") == 0) { g_no_self_beside = value; return HDT_OK; }
+    if (name && std::strcmp(name, "no_rows") == 0) { g_no_rows = value; return HDT_OK; }
+    if (name && std::strncmp(name, "rows_lim", 8) == 0) { g_rows_lim[name[8] - '0'] = value; return HDT_OK; }
     return set_error(HDT_ERR_INVALID_ARG, "hdt_set_option: unknown option");
 }
 
@@ -233,6 +237,22 @@ extern "C" int hdt_profile_read(int32_t id, int64_t *launches, double *total_ms,
     return HDT_OK;
 }
 
+// Whether a call may use the row-wise kernels at all: not where an option asks for one of the others.
+static bool rows_allowed() {
+    return !g_no_rows && !g_force_simt && !g_simt_upper && !g_no_overlap && !g_no_fold && !g_no_multi_upper && g_no_persistent == 0;
+}
+// All stages row by row.
+static bool rows_all(const hdt_index *ix, int dtype) {
+    return rows_allowed() && ix->nnz <= g_rows_lim[dtype == HDT_F32 ? 3 : 2] * ix->total_tokens;
+}
+// The stages above 0 row by row.
+static bool rows_upper(const hdt_index *ix, int heads, int head_dim, int bwd) {
+    return rows_allowed() && ix->n_stages > 1 && ix->nnz_upper * heads * (head_dim / 64) <= g_rows_lim[bwd];
+}
+static void row_stages(const hdt_index *ix, RowStage *st) {
+    for (int s = 0; s < ix->n_stages; ++s) st[s] = RowStage{ix->st[s].tok, ix->st[s].rng, ix->st[s].up};
+}
+
 extern "C" size_t hdt_attn_workspace_bytes(const hdt_index_t *ix, int32_t heads, int32_t head_dim,
                                            int32_t dtype, int32_t bwd) {
     (void)dtype;
@@ -264,7 +284,7 @@ extern "C" int hdt_attn_fwd(const hdt_index_t *ix, const void *q, const void *k,
     bool early = false;
     std::unique_ptr<ProfScope> ps_early;      // stage 0's time when a kernel goes ahead: from its start to the end of the stage's other kernel
     if (ix->pending && ix->total_tokens > 0 && dtype == HDT_BF16 && !g_force_simt && g_no_persistent == 0 &&
-        !g_no_overlap && (workspace == nullptr || ((uintptr_t)workspace & 255) == 0)) {
+        !g_no_overlap && ix->max_stages <= 8 && (workspace == nullptr || ((uintptr_t)workspace & 255) == 0)) {
         Side *sd = nullptr;
         rc = get_side(&sd);
         if (rc) return rc;
@@ -294,6 +314,19 @@ extern "C" int hdt_attn_fwd(const hdt_index_t *ix, const void *q, const void *k,
     rc = check_common(ix, heads, head_dim, dtype, workspace, workspace_bytes, L.total, "hdt_attn_fwd");
     if (rc) return rc;
     if (ix->total_tokens == 0) return HDT_OK;
+    const bool all_rows = !early && rows_all(ix, dtype);
+    const bool up_rows = all_rows || rows_upper(ix, heads, head_dim, 0);
+    auto upper_rows = [&](int first) {      // the elements of stage `first` with everything above it
+        RowFwdArgs a{};
+        a.n = ix->desc[first].n; a.H = heads; a.T = ix->total_tokens; a.first = first; a.dirs = ix->directions;
+        a.q = q; a.k = k; a.v = v; a.o = o; a.lse = lse;
+        a.scale_log2 = scale * 1.4426950408889634f;
+        if (first) { a.base_o = (const float *)(ws + L.part[1][0]); a.base_lse = (const float *)(ws + L.part[1][1]); }
+        row_stages(ix, a.st);
+        ProfScope ps(first ? PROF_FWD_UPPER : PROF_FWD_STAGE0, st);
+        return launch_fwd_rows(a, head_dim, dtype, st);
+    };
+    if (all_rows) return upper_rows(0);
     auto stage_args = [&](int s) {
         const StagePtrs &P = ix->st[s];
         FwdStageArgs a{};
@@ -328,14 +361,14 @@ extern "C" int hdt_attn_fwd(const hdt_index_t *ix, const void *q, const void *k,
         rc = get_side(&sd);
         if (rc) return rc;
         if (!early) HDT_CUDA_CHECK(cudaEventRecord(sd->fork, st));
-        HDT_CUDA_CHECK(cudaStreamWaitEvent(sd->s, sd->fork, 0));
+        if (!up_rows) HDT_CUDA_CHECK(cudaStreamWaitEvent(sd->s, sd->fork, 0));
         const bool tc0 = dtype == HDT_BF16 && !g_force_simt;
         // Stage 0's blocks that are not self-contained (split families, EMPTY blocks) have a kernel of
         // their own.  Where the split families are the smaller part it runs on the second side stream beside the
         // looping kernel (measured: a batch of padded documents gains 7 %); where split families
         // dominate, one kernel after the other is faster (the skewed batch loses 3 % side by side).
         const bool rest_beside = early || (tc0 && 2 * (ix->desc[0].nb - ix->desc[0].n_fused - ix->desc[0].n_empty) <= ix->desc[0].nb);
-        const bool two = ix->n_stages > 2;
+        const bool two = ix->n_stages > 2 && !up_rows;
         if (two) HDT_CUDA_CHECK(cudaStreamWaitEvent(sd->s2, sd->fork, 0));
         // Stages above 0 of bf16 calls run on the gathering tensor-core kernels, whatever the depth of the
         // hierarchy (option "simt_upper" = 1: on the fp32 SIMT kernels, which take trees of more than three
@@ -363,7 +396,7 @@ extern "C" int hdt_attn_fwd(const hdt_index_t *ix, const void *q, const void *k,
         // takes every SM ahead of stage 0 and was slower, 1.253 against 1.234 ms on the expression trees.)
         const bool multi = !tc_upper && ix->n_stages > 3 && !g_no_multi_upper;
         MultiFwdArgs mf{};
-        for (int s = 1; s < ix->n_stages; ++s) {
+        for (int s = 1; s < ix->n_stages && !up_rows; ++s) {
             FwdStageArgs a = stage_args(s);
             a.own_o = (float *)(ws + L.own[s][0]);
             a.own_lse = (float *)(ws + L.own[s][1]);
@@ -383,7 +416,7 @@ extern "C" int hdt_attn_fwd(const hdt_index_t *ix, const void *q, const void *k,
             else rc = launch_fwd_simt(a, head_dim, dtype, ss);
             if (rc) return rc;
         }
-        if (multi) {
+        if (multi && !up_rows) {
             rc = launch_fwd_simt_multi(mf, head_dim, dtype, sd->s);
             if (rc) return rc;
         }
@@ -396,7 +429,7 @@ extern "C" int hdt_attn_fwd(const hdt_index_t *ix, const void *q, const void *k,
             rc = launch_fwd_tc(a, head_dim, sd->s3);
             if (rc) return rc;
         }
-        HDT_CUDA_CHECK(cudaEventRecord(sd->join, sd->s));
+        if (!up_rows) HDT_CUDA_CHECK(cudaEventRecord(sd->join, sd->s));
         if (two) HDT_CUDA_CHECK(cudaEventRecord(sd->join2, sd->s2));
         if (rest_beside) HDT_CUDA_CHECK(cudaEventRecord(sd->join3, sd->s3));
         {   // stage 0 after the small side kernels are queued: they take their SM share first (the
@@ -418,6 +451,7 @@ extern "C" int hdt_attn_fwd(const hdt_index_t *ix, const void *q, const void *k,
         }
         if (rest_beside) HDT_CUDA_CHECK(cudaStreamWaitEvent(st, sd->join3, 0));
         ps_early.reset();                    // (stage 0 ends here: both of its kernels are done)
+        if (up_rows) return upper_rows(1);
         HDT_CUDA_CHECK(cudaStreamWaitEvent(st, sd->join, 0));
         if (two) HDT_CUDA_CHECK(cudaStreamWaitEvent(st, sd->join2, 0));
         ProfScope ps(PROF_FWD_UPPER, st);
@@ -466,6 +500,18 @@ extern "C" int hdt_attn_bwd(const hdt_index_t *ix, const void *q, const void *k,
     int *status = device_status_ptr();
     if (!status) return HDT_ERR_CUDA;
     const bool overlap = ix->n_stages > 1 && !g_no_overlap;
+    const bool all_rows = rows_all(ix, dtype), up_rows = all_rows || rows_upper(ix, heads, head_dim, 1);
+    auto upper_rows = [&](int first, const float *delta_) {      // (see hdt_attn_fwd)
+        RowBwdArgs a{};
+        a.n = ix->desc[first].n; a.H = heads; a.T = ix->total_tokens; a.first = first; a.dirs = ix->directions;
+        a.q = q; a.k = k; a.v = v; a.o = o; a.d_o = d_o; a.lse = lse; a.delta = delta_;
+        a.scale = scale; a.scale_log2 = scale * 1.4426950408889634f;
+        a.dq = dq; a.dk = dk; a.dv = dv;
+        if (first) for (int i = 0; i < 3; ++i) a.base[i] = (const float *)(ws + L.part[1][i]);
+        row_stages(ix, a.st);
+        ProfScope ps(first ? PROF_BWD_UPPER : PROF_BWD_STAGE0, st);
+        return launch_bwd_rows(a, head_dim, dtype, st);
+    };
     // Stages above 0 of bf16 calls: the gathering tensor-core kernels (see hdt_attn_fwd).
     const bool tc_upper = dtype == HDT_BF16 && !g_force_simt && !g_simt_upper;
     // No delta pass when every kernel of this call computes dO . O of its rows itself: stage 0
@@ -477,7 +523,7 @@ extern "C" int hdt_attn_bwd(const hdt_index_t *ix, const void *q, const void *k,
     // Families longer than a row block (head_dim 64): one walk over their tile pairs, dQ tiles summed
     // in an fp32 buffer that starts at zero (option "bwd_walk" = 1: two walks, no buffer).
     float *dq_acc = nullptr;
-    if (L.has_dq_acc && !g_force_simt && g_bwd_walk != 1 &&
+    if (!all_rows && L.has_dq_acc && !g_force_simt && g_bwd_walk != 1 &&
         (g_no_persistent == 0 || g_no_persistent == 4 || g_no_persistent == 6)) {
         dq_acc = (float *)(ws + L.dq_acc);
     }
@@ -496,6 +542,13 @@ extern "C" int hdt_attn_bwd(const hdt_index_t *ix, const void *q, const void *k,
             ProfScope ps(PROF_BWD_STAGE0, st);
             HDT_CUDA_CHECK(cudaMemsetAsync(dq_acc, 0, bytes, st));
         }
+    }
+    if (all_rows) {
+        {
+            ProfScope ps(PROF_DELTA, st);
+            rc = launch_delta(o, d_o, delta, ix->total_tokens, heads, head_dim, dtype, st);
+        }
+        return rc ? rc : upper_rows(0, delta);
     }
     if (!fused_delta) {
         ProfScope ps(PROF_DELTA, st);
@@ -538,11 +591,11 @@ extern "C" int hdt_attn_bwd(const hdt_index_t *ix, const void *q, const void *k,
         rc = get_side(&sd);
         if (rc) return rc;
         HDT_CUDA_CHECK(cudaEventRecord(sd->fork, st));
-        HDT_CUDA_CHECK(cudaStreamWaitEvent(sd->s, sd->fork, 0));
+        if (!up_rows) HDT_CUDA_CHECK(cudaStreamWaitEvent(sd->s, sd->fork, 0));
         // (with the one-walk kernel the self-contained blocks' kernel goes to the second side stream: its CTAs take
         // the SMs that the one-walk kernel's CTAs leave first, and it shares HBM with the pass that converts dQ)
         const bool self_beside = dq_acc != nullptr && ix->desc[0].n_fused > 0 && !g_no_self_beside;
-        const bool two = ix->n_stages > 2 || self_beside;
+        const bool two = (ix->n_stages > 2 && !up_rows) || self_beside;
         if (two) HDT_CUDA_CHECK(cudaStreamWaitEvent(sd->s2, sd->fork, 0));
         ChainArgs c{};
         c.n1 = ix->desc[1].n; c.H = heads; c.T = ix->total_tokens; c.n_stages = ix->n_stages; c.nt = 3;
@@ -552,7 +605,7 @@ extern "C" int hdt_attn_bwd(const hdt_index_t *ix, const void *q, const void *k,
         BwdStageArgs a1{};
         const bool multi = !tc_upper && ix->n_stages > 3 && !g_no_multi_upper;      // (see hdt_attn_fwd)
         MultiBwdArgs mb{};
-        for (int s = 1; s < ix->n_stages; ++s) {
+        for (int s = 1; s < ix->n_stages && !up_rows; ++s) {
             BwdStageArgs a = stage_args(s);
             a.own_dq = (float *)(ws + L.own[s][0]);
             a.own_dk = (float *)(ws + L.own[s][1]);
@@ -578,11 +631,11 @@ extern "C" int hdt_attn_bwd(const hdt_index_t *ix, const void *q, const void *k,
             else rc = launch_bwd_simt(a, head_dim, dtype, ss);
             if (rc) return rc;
         }
-        if (multi) {
+        if (multi && !up_rows) {
             rc = launch_bwd_simt_multi(mb, head_dim, dtype, sd->s);
             if (rc) return rc;
         }
-        HDT_CUDA_CHECK(cudaEventRecord(sd->join, sd->s));
+        if (!up_rows) HDT_CUDA_CHECK(cudaEventRecord(sd->join, sd->s));
         if (two && !self_beside) HDT_CUDA_CHECK(cudaEventRecord(sd->join2, sd->s2));
         {
             BwdStageArgs a = stage_args(0);
@@ -596,8 +649,9 @@ extern "C" int hdt_attn_bwd(const hdt_index_t *ix, const void *q, const void *k,
                 HDT_CUDA_CHECK(cudaStreamWaitEvent(st, sd->join2, 0));
             }
         }
-        HDT_CUDA_CHECK(cudaStreamWaitEvent(st, sd->join, 0));
+        if (!up_rows) HDT_CUDA_CHECK(cudaStreamWaitEvent(st, sd->join, 0));
         if (two && !self_beside) HDT_CUDA_CHECK(cudaStreamWaitEvent(st, sd->join2, 0));
+        if (up_rows) return upper_rows(1, fused_delta ? nullptr : delta);
         ProfScope ps(PROF_BWD_UPPER, st);
         if (fold) {
             a1.final_merge = 1;

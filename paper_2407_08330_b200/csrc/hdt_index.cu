@@ -37,7 +37,7 @@ struct SeqInfo {
     int res;                   // elements it still has in any later stage of the batch: its root, or nothing
     int err, err_pos;          // structure error, 0 = none
     int more, pad;             // elements were left after the last allowed stage
-    long long nnz, visited;
+    long long nnz, nnz_upper, visited;
 };
 
 struct Layout {
@@ -183,7 +183,7 @@ struct SeqShared {
     int wtot[32], wtotu[32], ctot[SEQ_CLUSTER];
     int err, err_pos, flag0, flag, nb0, nb, nf0, ne0, nf, ne;
     int ns[HDT_MAX_STAGES], bsw[16][SBW], nfs[16], nes[16];     // (seq_upper_all)
-    unsigned long long nnz, vis;
+    unsigned long long nnz, nnz_upper, vis;
 };
 
 __device__ __forceinline__ void seq_fail(SeqShared *sh, int pos) {
@@ -473,7 +473,7 @@ __device__ __forceinline__ void seq_upper(const SeqArgs &a, SeqShared &sh, J *pa
         next = __any_sync(0xffffffffu, next);
         if (lane == 0) {
             sh.wtotu[w] = run;
-            if (deg) atomicAdd(&sh.nnz, (unsigned long long)deg);
+            if (deg) atomicAdd(&sh.nnz_upper, (unsigned long long)deg);
             if (next) sh.flag = 1;
         }
         bar_upper(tu);
@@ -611,7 +611,7 @@ __device__ __forceinline__ bool seq_upper_all(const SeqArgs &a, SeqShared &sh, c
         deg += row_pairs(pos, lo, hi, a.dirs);
     }
     for (int o = 16; o; o >>= 1) deg += __shfl_xor_sync(0xffffffffu, deg, o);
-    if (lane == 0 && deg) atomicAdd(&sh.nnz, (unsigned long long)deg);
+    if (lane == 0 && deg) atomicAdd(&sh.nnz_upper, (unsigned long long)deg);
     bar_upper(tu);
     for (int s = 1 + w; s < S; s += nw) {          // a warp per stage: its blocks
         int4 *rec = a.recs + (size_t)s * a.capnb + slot;
@@ -662,7 +662,7 @@ __global__ void __launch_bounds__(512) k_seq(const SeqArgs a) {
     c.ne = min(1 << c.sl, c.L - c.e0);
     const bool first = c.rank == 0;
     if (t == 0) {
-        sh.err = 0; sh.err_pos = 0; sh.flag0 = 0; sh.nf0 = 0; sh.ne0 = 0; sh.nnz = 0; sh.vis = 0;
+        sh.err = 0; sh.err_pos = 0; sh.flag0 = 0; sh.nf0 = 0; sh.ne0 = 0; sh.nnz = 0; sh.nnz_upper = 0; sh.vis = 0;
         if (first) {
             if (c1 < c0 || c0 < 0 || c1 > a.T || (b == 0 && c0 != 0) || (b == a.B - 1 && c1 != a.T)) seq_fail(&sh, b);
             a.scu[b] = c0;
@@ -764,7 +764,7 @@ __global__ void __launch_bounds__(512) k_seq(const SeqArgs a) {
         }
         SeqInfo f;
         f.stages = stages; f.res = res; f.err = sh.err; f.err_pos = sh.err_pos; f.more = more; f.pad = 0;
-        f.nnz = (long long)sh.nnz; f.visited = (long long)sh.vis;
+        f.nnz = (long long)(sh.nnz + sh.nnz_upper); f.nnz_upper = (long long)sh.nnz_upper; f.visited = (long long)sh.vis;
         a.info[b] = f;
     }
 }
@@ -814,8 +814,8 @@ __device__ __forceinline__ void row_sums(int rows, int m, int w, int nw, int lan
 __device__ void finish_header(const FinishArgs &f, int S) {
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     __shared__ int s_err, s_more;
-    __shared__ long long s_sum[2];
-    if (t == 0) { s_err = 0x7fffffff; s_more = 0; s_sum[0] = s_sum[1] = 0; }
+    __shared__ long long s_sum[3];
+    if (t == 0) { s_err = 0x7fffffff; s_more = 0; s_sum[0] = s_sum[1] = s_sum[2] = 0; }
     __syncthreads();
     const size_t q = (size_t)f.ms * f.B;
     row_sums(4 * S, f.B, w, FT / 32, lane, [&](int i) { return f.counts + (i & 3) * q + (size_t)(i >> 2) * f.B; },
@@ -827,15 +827,15 @@ __device__ void finish_header(const FinishArgs &f, int S) {
                  *pd = v;
                  *reinterpret_cast<volatile int *>(ph) = v;
              });
-    long long nnz = 0, vis = 0;
+    long long nnz = 0, vis = 0, nup = 0;
     for (int b = t; b < f.B; b += FT) {
         const SeqInfo &x = f.info[b];
-        nnz += x.nnz; vis += x.visited;
+        nnz += x.nnz; vis += x.visited; nup += x.nnz_upper;
         if (x.err) atomicMin(&s_err, b);
         if (x.more) s_more = 1;
     }
-    nnz = warp_sum(nnz); vis = warp_sum(vis);
-    if (lane == 0) { atomicAdd((unsigned long long *)&s_sum[0], (unsigned long long)nnz); atomicAdd((unsigned long long *)&s_sum[1], (unsigned long long)vis); }
+    nnz = warp_sum(nnz); vis = warp_sum(vis); nup = warp_sum(nup);
+    if (lane == 0) { atomicAdd((unsigned long long *)&s_sum[0], (unsigned long long)nnz); atomicAdd((unsigned long long *)&s_sum[1], (unsigned long long)vis); atomicAdd((unsigned long long *)&s_sum[2], (unsigned long long)nup); }
     __syncthreads();
     if (t <= HDT_MAX_STAGES) {
         const int more = (t + 1 < S) || (t + 1 == S && s_more);
@@ -853,8 +853,8 @@ __device__ void finish_header(const FinishArgs &f, int S) {
         if (f.B == 0) { f.st[0].scu[0] = f.cu[0]; if (f.cu[0] != 0 || f.T != 0) err = HDT_ERR_BAD_HIERARCHY; }
         else if (s_err != 0x7fffffff) { err = f.info[s_err].err; pos = f.info[s_err].err_pos; }
         volatile DevHeader *h = f.host;
-        f.hdr->status = err; f.hdr->err_pos = pos; f.hdr->nnz = s_sum[0]; f.hdr->visited = s_sum[1]; f.hdr->tail = 0;
-        h->status = err; h->err_pos = pos; h->nnz = s_sum[0]; h->visited = s_sum[1];
+        f.hdr->status = err; f.hdr->err_pos = pos; f.hdr->nnz = s_sum[0]; f.hdr->visited = s_sum[1]; f.hdr->nnz_upper = s_sum[2]; f.hdr->tail = 0;
+        h->status = err; h->err_pos = pos; h->nnz = s_sum[0]; h->visited = s_sum[1]; h->nnz_upper = s_sum[2];
     }
     __threadfence_system();
     __syncthreads();
@@ -1257,6 +1257,7 @@ int index_ready(const hdt_index *cix) {
                 ix->n_stages = ns;
                 ix->nnz = h.nnz;
                 ix->visited = h.visited;
+                ix->nnz_upper = h.nnz_upper;
                 for (int s = 0; s <= HDT_MAX_STAGES; ++s) ix->desc[s] = h.st[s];
             }
         }

@@ -22,6 +22,7 @@ struct DevHeader {
     int status;              // hdt_status_t, first error wins
     int err_pos;             // element / sequence where it was detected
     long long nnz;           // unmasked pairs
+    long long nnz_upper;     // those of the stages above 0
     long long visited;       // sum over blocks of rows x span
     StageDesc st[HDT_MAX_STAGES + 1];
     int tail;                // always 0 on the device: the last word of the header to arrive on the host
@@ -37,7 +38,7 @@ struct StagePtrs {
 struct hdt_index {
     int batch, total_tokens, block_m, block_m_upper, n_stages;
     int directions;   // bits 1 | 2 | 4: child->parent, sibling<->sibling, parent->child entries kept (7 = full rule)
-    long long nnz, visited;
+    long long nnz, nnz_upper, visited;
     hdt::StageDesc desc[HDT_MAX_STAGES + 1];
     hdt::StagePtrs st[HDT_MAX_STAGES];
     void *workspace;
@@ -269,6 +270,27 @@ int read_fwd_timeline(long long *out4096);       // per CTA of the last instrume
 int launch_bwd_simt(const BwdStageArgs &a, int head_dim, int dtype, cudaStream_t st);
 int launch_delta(const void *o, const void *d_o, float *delta, int T, int H, int head_dim, int dtype,
                  cudaStream_t st);
+// Row-wise kernels (hdt_attn_rows.cu): the elements of stage `first` with all stages they live in from there on.
+struct RowStage { const int *tok, *rng, *up; };
+struct RowFwdArgs {
+    int n, H, T, first, dirs;            // n: elements of stage `first`
+    const void *q, *k, *v;
+    void *o;
+    float *lse, scale_log2;
+    const float *base_o, *base_lse;      // first = 1: stage 0's partial results of its elements, [n, H, D] and [n, H]
+    RowStage st[HDT_MAX_STAGES];
+};
+struct RowBwdArgs {
+    int n, H, T, first, dirs;
+    const void *q, *k, *v, *o, *d_o;
+    const float *lse, *delta;            // delta nullptr: computed from o
+    float scale, scale_log2;
+    void *dq, *dk, *dv;
+    const float *base[3];                // first = 1: stage 0's partial gradients, [n, H, D]
+    RowStage st[HDT_MAX_STAGES];
+};
+int launch_fwd_rows(const RowFwdArgs &a, int head_dim, int dtype, cudaStream_t st);
+int launch_bwd_rows(const RowBwdArgs &a, int head_dim, int dtype, cudaStream_t st);
 // One launch that completes every token of stage 1 (= every token that lives in a stage above 0):
 // stage 0's partial merged with the own partials of all upper stages the token belongs to, found
 // by following the `up` maps.  nt = 1 tensor (forward: O with LSE) or 3 (backward: dQ, dK, dV).
