@@ -25,15 +25,15 @@ __device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) { f2 r; asm("fma.rn.f32x2 %
 __device__ __forceinline__ f2 mul2(f2 a, f2 b) { f2 r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
 __device__ __forceinline__ f2 add2(f2 a, f2 b) { f2 r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
 
-// Eight consecutive values of a row as loaded, and as four packed pairs.
+// Eight consecutive values of a row as loaded, and as four packed pairs.  Offsets count groups of eight values.
 template <bool BF16> struct Raw;
 template <> struct Raw<true> {
     uint4 u;
-    __device__ __forceinline__ void load(const void *p, size_t i) { u = __ldg(reinterpret_cast<const uint4 *>(reinterpret_cast<const __nv_bfloat16 *>(p) + i)); }
+    __device__ __forceinline__ void load(const void *p, unsigned i) { u = __ldg(reinterpret_cast<const uint4 *>(p) + i); }
     __device__ __forceinline__ void zero() { u = make_uint4(0, 0, 0, 0); }
     static __device__ __forceinline__ f2 two(uint32_t x) { return pack2(__uint_as_float(x << 16), __uint_as_float(x & 0xffff0000u)); }
     __device__ __forceinline__ void get(f2 (&v)[4]) const { v[0] = two(u.x); v[1] = two(u.y); v[2] = two(u.z); v[3] = two(u.w); }
-    static __device__ __forceinline__ void store(void *p, size_t i, const f2 (&v)[4]) {
+    static __device__ __forceinline__ void store(void *p, unsigned i, const f2 (&v)[4]) {
         uint32_t w[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -42,21 +42,21 @@ template <> struct Raw<true> {
             const __nv_bfloat162 x = __floats2bfloat162_rn(a, b);
             w[k] = *reinterpret_cast<const uint32_t *>(&x);
         }
-        *reinterpret_cast<uint4 *>(reinterpret_cast<__nv_bfloat16 *>(p) + i) = make_uint4(w[0], w[1], w[2], w[3]);
+        reinterpret_cast<uint4 *>(p)[i] = make_uint4(w[0], w[1], w[2], w[3]);
     }
 };
 template <> struct Raw<false> {
     float4 a, b;
-    __device__ __forceinline__ void load(const void *p, size_t i) {
-        const float4 *q = reinterpret_cast<const float4 *>(reinterpret_cast<const float *>(p) + i);
+    __device__ __forceinline__ void load(const void *p, unsigned i) {
+        const float4 *q = reinterpret_cast<const float4 *>(p) + 2 * (size_t)i;
         a = __ldg(q); b = __ldg(q + 1);
     }
     __device__ __forceinline__ void zero() { a = b = make_float4(0.f, 0.f, 0.f, 0.f); }
     __device__ __forceinline__ void get(f2 (&v)[4]) const { v[0] = pack2(a.x, a.y); v[1] = pack2(a.z, a.w); v[2] = pack2(b.x, b.y); v[3] = pack2(b.z, b.w); }
-    static __device__ __forceinline__ void store(void *p, size_t i, const f2 (&v)[4]) {
+    static __device__ __forceinline__ void store(void *p, unsigned i, const f2 (&v)[4]) {
         float4 x, y;
         unpack2(v[0], x.x, x.y); unpack2(v[1], x.z, x.w); unpack2(v[2], y.x, y.y); unpack2(v[3], y.z, y.w);
-        float4 *q = reinterpret_cast<float4 *>(reinterpret_cast<float *>(p) + i);
+        float4 *q = reinterpret_cast<float4 *>(p) + 2 * (size_t)i;
         q[0] = x; q[1] = y;
     }
 };
@@ -68,6 +68,37 @@ __device__ __forceinline__ float dot8(const f2 (&a)[4], const f2 (&b)[4]) {
     float x, y;
     unpack2(s, x, y);
     return x + y;
+}
+
+template <bool BF16>
+__device__ __forceinline__ float dot(const Raw<BF16> &a, const Raw<BF16> &b) {
+    f2 x[4], y[4];
+    a.get(x); b.get(y);
+    return dot8(x, y);
+}
+template <int C, bool BF16>
+__device__ __forceinline__ void dots(const Raw<BF16> &a, const Raw<BF16> (&b)[C], float (&out)[C]) {
+    f2 x[4];
+    a.get(x);
+#pragma unroll
+    for (int i = 0; i < C; ++i) {
+        f2 y[4];
+        b[i].get(y);
+        out[i] = dot8(x, y);
+    }
+}
+// acc += sum over the chunk of w (one per lane) times its row
+template <int C, bool BF16>
+__device__ __forceinline__ void axpys(f2 (&acc)[4], float w, const Raw<BF16> (&x)[C], unsigned mask, int src) {
+#pragma unroll
+    for (int i = 0; i < C; ++i) {
+        const float wi = __shfl_sync(mask, w, src + i, 32);
+        const f2 w2 = pack2(wi, wi);
+        f2 y[4];
+        x[i].get(y);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[u] = fma2(w2, y[u], acc[u]);
+    }
 }
 
 // Sums of C values over the LPK lanes of a group; lane g keeps the total of value g % C.
@@ -90,12 +121,51 @@ __device__ __forceinline__ float reduce_scatter(float (&v)[C], int g, unsigned m
 
 static constexpr int ROW_THREADS = 128;
 
+// The keys of a row over the stages it lives in, a chunk at a time.  What the next stage needs first (range,
+// next index) is loaded on entering a stage, and the tokens of a chunk while the one before it is worked
+// on: the walk is a chain of dependent loads, and the kernels are bound by its length.
+template <int C, int STEP>
+struct RowCursor {
+    const RowStage *st;
+    int s, e, up, upn, j0;
+    int2 r, rn;
+    __device__ __forceinline__ void peek() {
+        if (up >= 0) {
+            rn = __ldg(reinterpret_cast<const int2 *>(st[s + 1].rng) + up);
+            upn = __ldg(st[s + 1].up + up);
+        }
+    }
+    __device__ __forceinline__ bool settle(int first) {      // to the next stage while this one is exhausted; false: no keys left
+        while (j0 >= r.y) {
+            if (up < 0) return false;
+            e = up; r = rn; up = upn; ++s;
+            j0 = r.x + first;
+            peek();
+        }
+        return true;
+    }
+    __device__ __forceinline__ bool start(const RowStage *st_, int s_, int e_, int first) {
+        st = st_; s = s_; e = e_;
+        r = __ldg(reinterpret_cast<const int2 *>(st[s].rng) + e);
+        up = __ldg(st[s].up + e);
+        j0 = r.x + first;
+        peek();
+        return settle(first);
+    }
+    __device__ __forceinline__ bool next(int first) { j0 += STEP; return settle(first); }
+    // token of this lane's key (keys past the end read the last one: in bounds, weight 0)
+    __device__ __forceinline__ int token(int c) const {
+        const int j = min(j0 + c, r.y - 1);
+        return s ? __ldg(st[s].tok + j) : j;
+    }
+};
+
 // ---------------------------------------------------------------------------------------------
 // forward
 // ---------------------------------------------------------------------------------------------
-template <int D, bool BF16, int KP>
+template <int D, bool BF16, int KP, int C>
 __global__ void __launch_bounds__(ROW_THREADS) k_fwd_rows(const RowFwdArgs a) {
-    constexpr int LPK = D / 8, G = LPK * KP, C = 8;
+    constexpr int LPK = D / 8, G = LPK * KP;
     const float NEG = -INFINITY;
     const int lane = threadIdx.x & 31, sub = lane % G, g = sub % LPK, kp = sub / LPK;
     const unsigned all = G == 32 ? 0xffffffffu : ((1u << G) - 1u) << (lane - sub);     // the lanes of the row
@@ -103,10 +173,9 @@ __global__ void __launch_bounds__(ROW_THREADS) k_fwd_rows(const RowFwdArgs a) {
     const unsigned mask = ((1u << LPK) - 1u) << src;
     const unsigned long long id = ((unsigned long long)blockIdx.x * ROW_THREADS + threadIdx.x) / G;
     if (id >= (unsigned long long)a.n * a.H) return;
-    int e = (int)(id / a.H);
-    const int h = (int)(id % a.H), e_first = e;
+    const int e = (int)(id / a.H), h = (int)(id % a.H);
     const int t = a.first ? a.st[a.first].tok[e] : e;
-    const size_t row = ((size_t)t * a.H + h) * D + 8 * g;
+    const unsigned row = ((unsigned)t * a.H + h) * LPK + g;
     f2 q[4], acc[4];
     {
         Raw<BF16> r;
@@ -117,24 +186,22 @@ __global__ void __launch_bounds__(ROW_THREADS) k_fwd_rows(const RowFwdArgs a) {
         for (int i = 0; i < 4; ++i) { q[i] = mul2(q[i], c); acc[i] = 0ull; }
     }
     float m = NEG, l = 0.f;          // l: this lane's keys only
-    for (int s = a.first; ; ++s) {
-        const RowStage &S = a.st[s];
-        const int2 r = __ldg(reinterpret_cast<const int2 *>(S.rng) + e);
-        const int up = __ldg(S.up + e);
-        for (int j0 = r.x + kp * C; j0 < r.y; j0 += KP * C) {
-            const int jm = j0 + (g & (C - 1));
-            const bool ok = jm < r.y && (a.dirs == 7 || dir_ok(e, jm, r.x, a.dirs));
-            int tm = jm < r.y ? jm : r.y - 1;         // (keys past the end read the last one: in bounds, weight 0)
-            if (s) tm = __ldg(S.tok + tm);
+    RowCursor<C, KP * C> cur;
+    bool more = cur.start(a.st, a.first, e, kp * C);
+    int tm = more ? cur.token(g & (C - 1)) : 0;
+    {
+        while (more) {
+            const int jm = cur.j0 + (g & (C - 1)), tc = tm;
+            const bool ok = jm < cur.r.y && (a.dirs == 7 || dir_ok(cur.e, jm, cur.r.x, a.dirs));
             Raw<BF16> kr[C], vr[C];
-            size_t at[C];
 #pragma unroll
             for (int i = 0; i < C; ++i) {
-                at[i] = ((size_t)__shfl_sync(mask, tm, src + i, 32) * a.H + h) * D + 8 * g;
-                kr[i].load(a.k, at[i]);
+                const unsigned at = ((unsigned)__shfl_sync(mask, tc, src + i, 32) * a.H + h) * LPK + g;
+                kr[i].load(a.k, at);
+                vr[i].load(a.v, at);
             }
-#pragma unroll
-            for (int i = 0; i < C; ++i) vr[i].load(a.v, at[i]);
+            more = cur.next(kp * C);
+            if (more) tm = cur.token(g & (C - 1));
             float sc[C];
 #pragma unroll
             for (int i = 0; i < C; ++i) {
@@ -165,8 +232,6 @@ __global__ void __launch_bounds__(ROW_THREADS) k_fwd_rows(const RowFwdArgs a) {
                 for (int u = 0; u < 4; ++u) acc[u] = fma2(w2, v[u], acc[u]);
             }
         }
-        if (up < 0) break;
-        e = up;
     }
     // l over the C lanes that hold different keys (lanes g and g + C of a 16-lane group hold the same ones)
 #pragma unroll
@@ -183,7 +248,7 @@ __global__ void __launch_bounds__(ROW_THREADS) k_fwd_rows(const RowFwdArgs a) {
         for (int i = 0; i < 4; ++i) acc[i] = fma2(p2, __shfl_xor_sync(all, acc[i], o), mul2(acc[i], p1));
     }
     if (a.base_o != nullptr) {              // stage 0's partial result, normalised, as one more key
-        const size_t r1 = (size_t)e_first * a.H + h;
+        const size_t r1 = (size_t)e * a.H + h;
         const float s0 = a.base_lse[r1] * 1.4426950408889634f;
         const float4 *bo = reinterpret_cast<const float4 *>(a.base_o + r1 * D + 8 * g);
         const float4 x = bo[0], y = bo[1];
@@ -214,107 +279,87 @@ __global__ void __launch_bounds__(ROW_THREADS) k_fwd_rows(const RowFwdArgs a) {
 // one walk gives the row's dQ (as a query), dK and dV (as a key), each complete: no atomics.
 // DELTA: rowsum(dO . O) is given; else it is computed from O here (one more row per key to read).
 template <int D, bool BF16, int KP, bool DELTA>
-__global__ void __launch_bounds__(ROW_THREADS) k_bwd_rows(const RowBwdArgs a) {
-    constexpr int LPK = D / 8, G = LPK * KP, C = 4;
+__global__ void __launch_bounds__(ROW_THREADS, BF16 ? 4 : 3) k_bwd_rows(const RowBwdArgs a) {
+    constexpr int LPK = D / 8, G = LPK * KP, C = BF16 ? 4 : 2;
     const int lane = threadIdx.x & 31, sub = lane % G, g = sub % LPK, kp = sub / LPK;
     const unsigned all = G == 32 ? 0xffffffffu : ((1u << G) - 1u) << (lane - sub);     // the lanes of the row
     const int src = lane - g;                                                             // and of the group that shares a key
     const unsigned mask = ((1u << LPK) - 1u) << src;
     const unsigned long long id = ((unsigned long long)blockIdx.x * ROW_THREADS + threadIdx.x) / G;
     if (id >= (unsigned long long)a.n * a.H) return;
-    int e = (int)(id / a.H);
-    const int h = (int)(id % a.H), e_first = e;
+    const int e = (int)(id / a.H), h = (int)(id % a.H);
     const int t = a.first ? a.st[a.first].tok[e] : e;
-    const size_t row = ((size_t)t * a.H + h) * D + 8 * g;
+    const unsigned row = ((unsigned)t * a.H + h) * LPK + g;
     const float L2E = 1.4426950408889634f;
-    f2 q[4], k[4], v[4], go[4], dq[4], dk[4], dv[4];
-    float lse_i, dl_i;
-    {
-        Raw<BF16> rq, rk, rv, rg;
-        rq.load(a.q, row); rk.load(a.k, row); rv.load(a.v, row); rg.load(a.d_o, row);
-        lse_i = __ldg(a.lse + (size_t)h * a.T + t) * L2E;
-        const f2 c = pack2(a.scale_log2, a.scale_log2);
-        rq.get(q); rk.get(k); rv.get(v); rg.get(go);
-        if constexpr (DELTA) dl_i = __ldg(a.delta + (size_t)h * a.T + t);
-        else {
-            Raw<BF16> ro;
-            f2 o[4];
-            ro.load(a.o, row);
-            ro.get(o);
-            dl_i = dot8(go, o);
+    // (the row's own values stay as loaded and are unpacked once per chunk: registers decide how many warps hide
+    // the loads' latency here)
+    Raw<BF16> q, k, v, go;
+    f2 dq[4], dk[4], dv[4];
+    q.load(a.q, row); k.load(a.k, row); v.load(a.v, row); go.load(a.d_o, row);
+    const float lse_i = __ldg(a.lse + (size_t)h * a.T + t) * L2E;
+    float dl_i;
+    if constexpr (DELTA) dl_i = __ldg(a.delta + (size_t)h * a.T + t);
+    else {
+        Raw<BF16> ro;
+        ro.load(a.o, row);
+        dl_i = dot(go, ro);
 #pragma unroll
-            for (int x = 1; x < LPK; x *= 2) dl_i += __shfl_xor_sync(mask, dl_i, x);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) { q[i] = mul2(q[i], c); k[i] = mul2(k[i], c); dq[i] = dk[i] = dv[i] = 0ull; }
+        for (int x = 1; x < LPK; x *= 2) dl_i += __shfl_xor_sync(mask, dl_i, x);
     }
-    for (int s = a.first; ; ++s) {
-        const RowStage &S = a.st[s];
-        const int2 r = __ldg(reinterpret_cast<const int2 *>(S.rng) + e);
-        const int up = __ldg(S.up + e);
-        for (int j0 = r.x + kp * C; j0 < r.y; j0 += KP * C) {
-            const int jm = j0 + (g & (C - 1));
-            const bool in = jm < r.y;
-            const bool ok_q = in && (a.dirs == 7 || dir_ok(e, jm, r.x, a.dirs));          // the row attends to it
-            const bool ok_k = in && (a.dirs == 7 || dir_ok_key(e, jm, r.x, a.dirs));      // it attends to the row
-            int tm = in ? jm : r.y - 1;
-            if (s) tm = __ldg(S.tok + tm);
-            const float lse_j = __ldg(a.lse + (size_t)h * a.T + tm) * L2E;
-            float dl_j = 0.f;
-            if constexpr (DELTA) dl_j = __ldg(a.delta + (size_t)h * a.T + tm);
-            Raw<BF16> kr[C], qr[C], gr[C], xr[C];
-            size_t at[C];
 #pragma unroll
-            for (int i = 0; i < C; ++i) {
-                at[i] = ((size_t)__shfl_sync(mask, tm, src + i, 32) * a.H + h) * D + 8 * g;
-                kr[i].load(a.k, at[i]);
-                xr[i].load(a.v, at[i]);
-            }
+    for (int i = 0; i < 4; ++i) dq[i] = dk[i] = dv[i] = 0ull;
+    RowCursor<C, KP * C> cur;
+    bool more = cur.start(a.st, a.first, e, kp * C);
+    int tm = more ? cur.token(g & (C - 1)) : 0;
+    while (more) {
+        const int jm = cur.j0 + (g & (C - 1)), tc = tm;
+        const bool in = jm < cur.r.y;
+        const bool ok_q = in && (a.dirs == 7 || dir_ok(cur.e, jm, cur.r.x, a.dirs));          // the row attends to it
+        const bool ok_k = in && (a.dirs == 7 || dir_ok_key(cur.e, jm, cur.r.x, a.dirs));      // it attends to the row
+        const float lse_j = __ldg(a.lse + (size_t)h * a.T + tc) * L2E;
+        float dl_j = 0.f;
+        if constexpr (DELTA) dl_j = __ldg(a.delta + (size_t)h * a.T + tc);
+        Raw<BF16> x[C], y[C];
+        unsigned at[C];
+        float v1[C], v2[C];
+        // the row as a query: K and V of its keys
 #pragma unroll
-            for (int i = 0; i < C; ++i) { qr[i].load(a.q, at[i]); gr[i].load(a.d_o, at[i]); }
-            float sc[C], x1[C], x2[C], x3[C];
-#pragma unroll
-            for (int i = 0; i < C; ++i) {
-                f2 y[4];
-                kr[i].get(y); sc[i] = dot8(q, y);
-                xr[i].get(y); x1[i] = dot8(go, y);
-                qr[i].get(y); x2[i] = dot8(k, y);
-                gr[i].get(y); x3[i] = dot8(v, y);
-            }
-            if constexpr (!DELTA) {
-                float x4[C];
-#pragma unroll
-                for (int i = 0; i < C; ++i) {
-                    f2 y[4], z[4];
-                    xr[i].load(a.o, at[i]);
-                    xr[i].get(y); gr[i].get(z);
-                    x4[i] = dot8(z, y);
-                }
-                dl_j = reduce_scatter<C, LPK>(x4, g, mask);
-            }
-            const float s_ij = reduce_scatter<C, LPK>(sc, g, mask), dp_ij = reduce_scatter<C, LPK>(x1, g, mask);
-            const float s_ji = reduce_scatter<C, LPK>(x2, g, mask), dp_ji = reduce_scatter<C, LPK>(x3, g, mask);
-            const float p_ij = ok_q ? exp2f(s_ij - lse_i) : 0.f, p_ji = ok_k ? exp2f(s_ji - lse_j) : 0.f;
-            const float ds_ij = p_ij * (dp_ij - dl_i), ds_ji = p_ji * (dp_ji - dl_j);
-#pragma unroll
-            for (int i = 0; i < C; ++i) {
-                const float w1 = __shfl_sync(mask, ds_ij, src + i, 32), w2 = __shfl_sync(mask, ds_ji, src + i, 32),
-                            w3 = __shfl_sync(mask, p_ji, src + i, 32);
-                const f2 c1 = pack2(w1, w1), c2 = pack2(w2, w2), c3 = pack2(w3, w3);
-                f2 y[4];
-                kr[i].get(y);
-#pragma unroll
-                for (int u = 0; u < 4; ++u) dq[u] = fma2(c1, y[u], dq[u]);
-                qr[i].get(y);
-#pragma unroll
-                for (int u = 0; u < 4; ++u) dk[u] = fma2(c2, y[u], dk[u]);
-                gr[i].get(y);
-#pragma unroll
-                for (int u = 0; u < 4; ++u) dv[u] = fma2(c3, y[u], dv[u]);
-            }
+        for (int i = 0; i < C; ++i) {
+            at[i] = ((unsigned)__shfl_sync(mask, tc, src + i, 32) * a.H + h) * LPK + g;
+            x[i].load(a.k, at[i]);
+            y[i].load(a.v, at[i]);
         }
-        if (up < 0) break;
-        e = up;
+        more = cur.next(kp * C);
+        if (more) tm = cur.token(g & (C - 1));
+        dots<C>(q, x, v1);
+        dots<C>(go, y, v2);
+        {
+            const float s_ij = reduce_scatter<C, LPK>(v1, g, mask) * a.scale_log2, dp_ij = reduce_scatter<C, LPK>(v2, g, mask);
+            const float p_ij = ok_q ? exp2f(s_ij - lse_i) : 0.f;
+            axpys<C>(dq, p_ij * (dp_ij - dl_i), x, mask, src);
+        }
+        // the row as a key: Q and dO of the queries that attend to it
+#pragma unroll
+        for (int i = 0; i < C; ++i) {
+            x[i].load(a.q, at[i]);
+            y[i].load(a.d_o, at[i]);
+        }
+        if constexpr (!DELTA) {
+            float v3[C];
+#pragma unroll
+            for (int i = 0; i < C; ++i) {
+                Raw<BF16> o;
+                o.load(a.o, at[i]);
+                v3[i] = dot(o, y[i]);
+            }
+            dl_j = reduce_scatter<C, LPK>(v3, g, mask);
+        }
+        dots<C>(k, x, v1);
+        dots<C>(v, y, v2);
+        const float s_ji = reduce_scatter<C, LPK>(v1, g, mask) * a.scale_log2, dp_ji = reduce_scatter<C, LPK>(v2, g, mask);
+        const float p_ji = ok_k ? exp2f(s_ji - lse_j) : 0.f;
+        axpys<C>(dk, p_ji * (dp_ji - dl_j), x, mask, src);
+        axpys<C>(dv, p_ji, y, mask, src);
     }
 #pragma unroll
     for (int o = LPK; o < G; o *= 2) {
@@ -330,7 +375,7 @@ __global__ void __launch_bounds__(ROW_THREADS) k_bwd_rows(const RowBwdArgs a) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) { dq[i] = mul2(dq[i], c); dk[i] = mul2(dk[i], c); }
         if (a.base[0] != nullptr) {         // stage 0's partial gradients
-            const size_t r1 = ((size_t)e_first * a.H + h) * D + 8 * g;
+            const size_t r1 = ((size_t)e * a.H + h) * D + 8 * g;
             auto plus = [&](f2 (&x)[4], const float *b) {
                 const float4 y = *reinterpret_cast<const float4 *>(b + r1), z = *reinterpret_cast<const float4 *>(b + r1 + 4);
                 x[0] = add2(x[0], pack2(y.x, y.y)); x[1] = add2(x[1], pack2(y.z, y.w));
@@ -344,35 +389,36 @@ __global__ void __launch_bounds__(ROW_THREADS) k_bwd_rows(const RowBwdArgs a) {
     }
 }
 
-// Lanes per row: with few rows several groups of lanes share one, for latency; with many, one group each
-// (no final merge, fewer idle lanes in short families).
+// Lanes per row: while all rows fit on the SMs at once several groups of lanes share one, for latency; beyond, one
+// group each (no final merge, fewer idle lanes in short families).
+static int row_groups(long long rows, int D) {
+    for (int kp = 256 / D; kp > 1; kp /= 2)
+        if (rows * kp * (D / 8) <= 148LL * 20 * 32) return kp;
+    return 1;
+}
 template <int D, bool BF16>
 static int launch_fwd_rows_t(const RowFwdArgs &a, cudaStream_t st) {
     const long long rows = (long long)a.n * a.H;
     if (rows == 0) return HDT_OK;
-    const bool share = rows * (D / 8) < 148LL * 1024;
-    const int g = share ? 32 : D / 8;
-    const unsigned grid = (unsigned)((rows * g + ROW_THREADS - 1) / ROW_THREADS);
-    if (share) k_fwd_rows<D, BF16, 256 / D><<<grid, ROW_THREADS, 0, st>>>(a);
-    else k_fwd_rows<D, BF16, 1><<<grid, ROW_THREADS, 0, st>>>(a);
+    const int kp = row_groups(rows, D);
+    const unsigned grid = (unsigned)((rows * kp * (D / 8) + ROW_THREADS - 1) / ROW_THREADS);
+    if (kp == 4) k_fwd_rows<D, BF16, D == 64 ? 4 : 1, 8><<<grid, ROW_THREADS, 0, st>>>(a);
+    else if (kp == 2) k_fwd_rows<D, BF16, 2, 8><<<grid, ROW_THREADS, 0, st>>>(a);
+    else if (a.first) k_fwd_rows<D, BF16, 1, 8><<<grid, ROW_THREADS, 0, st>>>(a);
+    else k_fwd_rows<D, BF16, 1, 4><<<grid, ROW_THREADS, 0, st>>>(a);
     count_launch();
     HDT_CUDA_CHECK(cudaGetLastError());
     return HDT_OK;
 }
-template <int D, bool BF16>
+template <int D, bool BF16, bool DELTA>
 static int launch_bwd_rows_t(const RowBwdArgs &a, cudaStream_t st) {
     const long long rows = (long long)a.n * a.H;
     if (rows == 0) return HDT_OK;
-    const bool share = rows * (D / 8) < 148LL * 1024;
-    const int g = share ? 32 : D / 8;
-    const unsigned grid = (unsigned)((rows * g + ROW_THREADS - 1) / ROW_THREADS);
-    if (a.delta) {
-        if (share) k_bwd_rows<D, BF16, 256 / D, true><<<grid, ROW_THREADS, 0, st>>>(a);
-        else k_bwd_rows<D, BF16, 1, true><<<grid, ROW_THREADS, 0, st>>>(a);
-    } else {
-        if (share) k_bwd_rows<D, BF16, 256 / D, false><<<grid, ROW_THREADS, 0, st>>>(a);
-        else k_bwd_rows<D, BF16, 1, false><<<grid, ROW_THREADS, 0, st>>>(a);
-    }
+    const int kp = row_groups(2 * rows, D);
+    const unsigned grid = (unsigned)((rows * kp * (D / 8) + ROW_THREADS - 1) / ROW_THREADS);
+    if (kp == 4) k_bwd_rows<D, BF16, D == 64 ? 4 : 1, DELTA><<<grid, ROW_THREADS, 0, st>>>(a);
+    else if (kp == 2) k_bwd_rows<D, BF16, 2, DELTA><<<grid, ROW_THREADS, 0, st>>>(a);
+    else k_bwd_rows<D, BF16, 1, DELTA><<<grid, ROW_THREADS, 0, st>>>(a);
     count_launch();
     HDT_CUDA_CHECK(cudaGetLastError());
     return HDT_OK;
@@ -382,9 +428,13 @@ int launch_fwd_rows(const RowFwdArgs &a, int D, int dtype, cudaStream_t st) {
     if (D == 128) return dtype == HDT_BF16 ? launch_fwd_rows_t<128, true>(a, st) : launch_fwd_rows_t<128, false>(a, st);
     return set_error(HDT_ERR_UNSUPPORTED, "head_dim %d not supported (64 or 128)", D);
 }
+template <int D, bool BF16>
+static int launch_bwd_rows_d(const RowBwdArgs &a, cudaStream_t st) {
+    return a.delta ? launch_bwd_rows_t<D, BF16, true>(a, st) : launch_bwd_rows_t<D, BF16, false>(a, st);
+}
 int launch_bwd_rows(const RowBwdArgs &a, int D, int dtype, cudaStream_t st) {
-    if (D == 64) return dtype == HDT_BF16 ? launch_bwd_rows_t<64, true>(a, st) : launch_bwd_rows_t<64, false>(a, st);
-    if (D == 128) return dtype == HDT_BF16 ? launch_bwd_rows_t<128, true>(a, st) : launch_bwd_rows_t<128, false>(a, st);
+    if (D == 64) return dtype == HDT_BF16 ? launch_bwd_rows_d<64, true>(a, st) : launch_bwd_rows_d<64, false>(a, st);
+    if (D == 128) return dtype == HDT_BF16 ? launch_bwd_rows_d<128, true>(a, st) : launch_bwd_rows_d<128, false>(a, st);
     return set_error(HDT_ERR_UNSUPPORTED, "head_dim %d not supported (64 or 128)", D);
 }
 
