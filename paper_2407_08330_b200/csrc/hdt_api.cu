@@ -74,7 +74,7 @@ static int g_no_self_beside = 0;
 static int g_no_fused_delta = 0;
 static int g_no_fold = 0;
 static int g_no_rows = 0;
-static long long g_rows_lim[4] = {2000000000, 30000000, 10, 64};
+static long long g_rows_lim[5] = {400000, 40000, 10, 10, 4000000};
 
 int get_side(Side **out) {
     int dev = -1;
@@ -245,6 +245,11 @@ static bool rows_allowed() {
 static bool rows_all(const hdt_index *ix, int dtype) {
     return rows_allowed() && ix->nnz <= g_rows_lim[dtype == HDT_F32 ? 3 : 2] * ix->total_tokens;
 }
+// fp32 calls: stage 0 on the kernels that stage its keys in shared memory.
+static bool tile_f32(int dtype) { return dtype == HDT_F32 && !g_no_rows && !g_force_simt; }
+static bool tile_walk(const hdt_index *ix, int heads, int head_dim) {
+    return ix->n_stages == 1 || (rows_allowed() && ix->nnz_upper * heads * (head_dim / 64) <= g_rows_lim[4]);
+}
 // The stages above 0 row by row.
 static bool rows_upper(const hdt_index *ix, int heads, int head_dim, int bwd) {
     return rows_allowed() && ix->n_stages > 1 && ix->nnz_upper * heads * (head_dim / 64) <= g_rows_lim[bwd];
@@ -319,6 +324,7 @@ extern "C" int hdt_attn_fwd(const hdt_index_t *ix, const void *q, const void *k,
     auto upper_rows = [&](int first) {      // the elements of stage `first` with everything above it
         RowFwdArgs a{};
         a.n = ix->desc[first].n; a.H = heads; a.T = ix->total_tokens; a.first = first; a.dirs = ix->directions;
+        a.keys = (float)(first ? ix->nnz_upper : ix->nnz) / (float)(a.n > 0 ? a.n : 1);
         a.q = q; a.k = k; a.v = v; a.o = o; a.lse = lse;
         a.scale_log2 = scale * 1.4426950408889634f;
         if (first) { a.base_o = (const float *)(ws + L.part[1][0]); a.base_lse = (const float *)(ws + L.part[1][1]); }
@@ -327,6 +333,20 @@ extern "C" int hdt_attn_fwd(const hdt_index_t *ix, const void *q, const void *k,
         return launch_fwd_rows(a, head_dim, dtype, st);
     };
     if (all_rows) return upper_rows(0);
+    auto tile_stage0 = [&](cudaStream_t s_) {
+        TileFwdArgs a{};
+        a.nb = ix->desc[0].nb; a.block_rows = ix->block_m; a.H = heads; a.T = ix->total_tokens; a.dirs = ix->directions;
+        a.blocks = ix->st[0].blocks; a.queue = ix->st[0].queue; a.rng = ix->st[0].rng; a.up = ix->n_stages > 1 ? ix->st[0].up : nullptr;
+        a.q = q; a.k = k; a.v = v; a.o = o; a.lse = lse;
+        a.scale_log2 = scale * 1.4426950408889634f;
+        if (ix->n_stages > 1) { a.part_o = (float *)(ws + L.part[1][0]); a.part_lse = (float *)(ws + L.part[1][1]); }
+        ProfScope ps(PROF_FWD_STAGE0, s_);
+        return launch_fwd_tile(a, head_dim, s_);
+    };
+    if (tile_f32(dtype) && tile_walk(ix, heads, head_dim)) {
+        rc = tile_stage0(st);
+        return rc || ix->n_stages == 1 ? rc : upper_rows(1);
+    }
     auto stage_args = [&](int s) {
         const StagePtrs &P = ix->st[s];
         FwdStageArgs a{};
@@ -439,6 +459,7 @@ extern "C" int hdt_attn_fwd(const hdt_index_t *ix, const void *q, const void *k,
             if (!early) {                    // (early: already queued)
                 ProfScope ps(PROF_FWD_STAGE0, st);
                 if (tc0) rc = launch_fwd_tc(a, head_dim, st);
+                else if (tile_f32(dtype)) rc = tile_stage0(st);
                 else rc = launch_fwd_simt(a, head_dim, dtype, st);
                 if (rc) return rc;
             }
@@ -504,6 +525,7 @@ extern "C" int hdt_attn_bwd(const hdt_index_t *ix, const void *q, const void *k,
     auto upper_rows = [&](int first, const float *delta_) {      // (see hdt_attn_fwd)
         RowBwdArgs a{};
         a.n = ix->desc[first].n; a.H = heads; a.T = ix->total_tokens; a.first = first; a.dirs = ix->directions;
+        a.keys = (float)(first ? ix->nnz_upper : ix->nnz) / (float)(a.n > 0 ? a.n : 1);
         a.q = q; a.k = k; a.v = v; a.o = o; a.d_o = d_o; a.lse = lse; a.delta = delta_;
         a.scale = scale; a.scale_log2 = scale * 1.4426950408889634f;
         a.dq = dq; a.dk = dk; a.dv = dv;
@@ -549,6 +571,21 @@ extern "C" int hdt_attn_bwd(const hdt_index_t *ix, const void *q, const void *k,
             rc = launch_delta(o, d_o, delta, ix->total_tokens, heads, head_dim, dtype, st);
         }
         return rc ? rc : upper_rows(0, delta);
+    }
+    auto tile_stage0 = [&]() {
+        TileBwdArgs a{};
+        a.nb = ix->desc[0].nb; a.block_rows = ix->block_m; a.H = heads; a.T = ix->total_tokens; a.dirs = ix->directions;
+        a.blocks = ix->st[0].blocks; a.queue = ix->st[0].queue; a.rng = ix->st[0].rng; a.up = ix->n_stages > 1 ? ix->st[0].up : nullptr;
+        a.q = q; a.k = k; a.v = v; a.o = o; a.d_o = d_o; a.lse = lse;
+        a.scale = scale; a.scale_log2 = scale * 1.4426950408889634f;
+        a.dq = dq; a.dk = dk; a.dv = dv;
+        if (ix->n_stages > 1) for (int i = 0; i < 3; ++i) a.part[i] = (float *)(ws + L.part[1][i]);
+        ProfScope ps(PROF_BWD_STAGE0, st);
+        return launch_bwd_tile(a, head_dim, st);
+    };
+    if (tile_f32(dtype) && tile_walk(ix, heads, head_dim)) {
+        rc = tile_stage0();
+        return rc || ix->n_stages == 1 ? rc : upper_rows(1, nullptr);
     }
     if (!fused_delta) {
         ProfScope ps(PROF_DELTA, st);
@@ -642,6 +679,7 @@ extern "C" int hdt_attn_bwd(const hdt_index_t *ix, const void *q, const void *k,
             if (self_beside) a.self_stream = (void *)sd->s2;
             ProfScope ps(PROF_BWD_STAGE0, st);
             if (dtype == HDT_BF16 && !g_force_simt) rc = launch_bwd_tc(a, head_dim, st);
+            else if (tile_f32(dtype)) rc = tile_stage0();
             else rc = launch_bwd_simt(a, head_dim, dtype, st);
             if (rc) return rc;
             if (self_beside) {       // (inside the scope: stage 0 ends when both streams have)

@@ -12,6 +12,8 @@
 // (C - 1 shuffles instead of 3 C or 4 C), which leaves one key's score per lane: one exponential per key
 // and lane instead of one per key on every lane.  KP groups of lanes may share a row (each takes every
 // KP-th chunk), for batches with too few rows to fill the SMs.
+#include <climits>
+
 #include <cuda_bf16.h>
 
 #include "hdt_internal.cuh"
@@ -25,15 +27,16 @@ __device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) { f2 r; asm("fma.rn.f32x2 %
 __device__ __forceinline__ f2 mul2(f2 a, f2 b) { f2 r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
 __device__ __forceinline__ f2 add2(f2 a, f2 b) { f2 r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
 
-// Eight consecutive values of a row as loaded, and as four packed pairs.  Offsets count groups of eight values.
-template <bool BF16> struct Raw;
-template <> struct Raw<true> {
+// Eight values of a row as loaded, and as four packed pairs.  Of a row of 8 N values lane g < N holds the values
+// 8 g .. 8 g + 7 (bf16: one 16-byte load) or 4 g .. + 3 and 4 N + 4 g .. + 3 (fp32: two loads, each contiguous
+// over the lanes).  r: row number (token * heads + head).
+template <bool BF16, int N> struct Raw;
+template <int N> struct Raw<true, N> {
     uint4 u;
-    __device__ __forceinline__ void load(const void *p, unsigned i) { u = __ldg(reinterpret_cast<const uint4 *>(p) + i); }
-    __device__ __forceinline__ void zero() { u = make_uint4(0, 0, 0, 0); }
+    __device__ __forceinline__ void load(const void *p, unsigned r, int g) { u = __ldg(reinterpret_cast<const uint4 *>(p) + r * N + g); }
     static __device__ __forceinline__ f2 two(uint32_t x) { return pack2(__uint_as_float(x << 16), __uint_as_float(x & 0xffff0000u)); }
     __device__ __forceinline__ void get(f2 (&v)[4]) const { v[0] = two(u.x); v[1] = two(u.y); v[2] = two(u.z); v[3] = two(u.w); }
-    static __device__ __forceinline__ void store(void *p, unsigned i, const f2 (&v)[4]) {
+    static __device__ __forceinline__ void store(void *p, unsigned r, int g, const f2 (&v)[4]) {
         uint32_t w[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -42,22 +45,33 @@ template <> struct Raw<true> {
             const __nv_bfloat162 x = __floats2bfloat162_rn(a, b);
             w[k] = *reinterpret_cast<const uint32_t *>(&x);
         }
-        reinterpret_cast<uint4 *>(p)[i] = make_uint4(w[0], w[1], w[2], w[3]);
+        reinterpret_cast<uint4 *>(p)[r * N + g] = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+    // the same values of an fp32 row (stage 0's partial results)
+    static __device__ __forceinline__ void load_f32(const float *p, size_t r, int g, f2 (&v)[4]) {
+        const float4 *q = reinterpret_cast<const float4 *>(p) + (r * N + g) * 2;
+        const float4 x = q[0], y = q[1];
+        v[0] = pack2(x.x, x.y); v[1] = pack2(x.z, x.w); v[2] = pack2(y.x, y.y); v[3] = pack2(y.z, y.w);
     }
 };
-template <> struct Raw<false> {
+template <int N> struct Raw<false, N> {
     float4 a, b;
-    __device__ __forceinline__ void load(const void *p, unsigned i) {
-        const float4 *q = reinterpret_cast<const float4 *>(p) + 2 * (size_t)i;
-        a = __ldg(q); b = __ldg(q + 1);
+    __device__ __forceinline__ void load(const void *p, unsigned r, int g) {
+        const float4 *q = reinterpret_cast<const float4 *>(p) + (size_t)r * (2 * N) + g;
+        a = __ldg(q); b = __ldg(q + N);
     }
-    __device__ __forceinline__ void zero() { a = b = make_float4(0.f, 0.f, 0.f, 0.f); }
+    __device__ __forceinline__ void load_smem(const float4 *row, int g) { a = row[g]; b = row[N + g]; }
     __device__ __forceinline__ void get(f2 (&v)[4]) const { v[0] = pack2(a.x, a.y); v[1] = pack2(a.z, a.w); v[2] = pack2(b.x, b.y); v[3] = pack2(b.z, b.w); }
-    static __device__ __forceinline__ void store(void *p, unsigned i, const f2 (&v)[4]) {
+    static __device__ __forceinline__ void store(void *p, unsigned r, int g, const f2 (&v)[4]) {
         float4 x, y;
         unpack2(v[0], x.x, x.y); unpack2(v[1], x.z, x.w); unpack2(v[2], y.x, y.y); unpack2(v[3], y.z, y.w);
-        float4 *q = reinterpret_cast<float4 *>(p) + 2 * (size_t)i;
-        q[0] = x; q[1] = y;
+        float4 *q = reinterpret_cast<float4 *>(p) + (size_t)r * (2 * N) + g;
+        q[0] = x; q[N] = y;
+    }
+    static __device__ __forceinline__ void load_f32(const float *p, size_t r, int g, f2 (&v)[4]) {
+        const float4 *q = reinterpret_cast<const float4 *>(p) + r * (2 * N) + g;
+        const float4 x = q[0], y = q[N];
+        v[0] = pack2(x.x, x.y); v[1] = pack2(x.z, x.w); v[2] = pack2(y.x, y.y); v[3] = pack2(y.z, y.w);
     }
 };
 __device__ __forceinline__ float dot8(const f2 (&a)[4], const f2 (&b)[4]) {
@@ -70,14 +84,14 @@ __device__ __forceinline__ float dot8(const f2 (&a)[4], const f2 (&b)[4]) {
     return x + y;
 }
 
-template <bool BF16>
-__device__ __forceinline__ float dot(const Raw<BF16> &a, const Raw<BF16> &b) {
+template <class R>
+__device__ __forceinline__ float dot(const R &a, const R &b) {
     f2 x[4], y[4];
     a.get(x); b.get(y);
     return dot8(x, y);
 }
-template <int C, bool BF16>
-__device__ __forceinline__ void dots(const Raw<BF16> &a, const Raw<BF16> (&b)[C], float (&out)[C]) {
+template <int C, class R>
+__device__ __forceinline__ void dots(const R &a, const R (&b)[C], float (&out)[C]) {
     f2 x[4];
     a.get(x);
 #pragma unroll
@@ -88,8 +102,8 @@ __device__ __forceinline__ void dots(const Raw<BF16> &a, const Raw<BF16> (&b)[C]
     }
 }
 // acc += sum over the chunk of w (one per lane) times its row
-template <int C, bool BF16>
-__device__ __forceinline__ void axpys(f2 (&acc)[4], float w, const Raw<BF16> (&x)[C], unsigned mask, int src) {
+template <int C, class R>
+__device__ __forceinline__ void axpys(f2 (&acc)[4], float w, const R (&x)[C], unsigned mask, int src) {
 #pragma unroll
     for (int i = 0; i < C; ++i) {
         const float wi = __shfl_sync(mask, w, src + i, 32);
@@ -163,113 +177,115 @@ struct RowCursor {
 // ---------------------------------------------------------------------------------------------
 // forward
 // ---------------------------------------------------------------------------------------------
+// A row's online softmax: maximum (log2), sum (this lane's keys only) and accumulator.
+struct RowSoftmax {
+    float m, l;
+    f2 acc[4];
+    __device__ __forceinline__ void clear() {
+        m = -INFINITY; l = 0.f;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[i] = 0ull;
+    }
+    // x: score of this lane's key (-inf: none).  Returns its weight.
+    template <int C>
+    __device__ __forceinline__ float add(float x, unsigned mask) {
+        float mx = x;
+#pragma unroll
+        for (int o = 1; o < C; o *= 2) mx = fmaxf(mx, __shfl_xor_sync(mask, mx, o));
+        mx = fmaxf(mx, m);
+        const float ref = mx > -INFINITY ? mx : 0.f;
+        const float p = exp2f(x - ref), al = exp2f(m - ref);
+        m = mx;
+        l = l * al + p;
+        const f2 al2 = pack2(al, al);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[i] = mul2(acc[i], al2);
+        return p;
+    }
+    // another partial result: maximum, sum, accumulator
+    __device__ __forceinline__ void merge(float m2, float l2, const f2 (&acc2)[4]) {
+        const float mx = fmaxf(m, m2), ref = mx > -INFINITY ? mx : 0.f;
+        const float w1 = exp2f(m - ref), w2 = exp2f(m2 - ref);
+        const f2 p1 = pack2(w1, w1), p2 = pack2(w2, w2);
+        l = l * w1 + l2 * w2;
+        m = mx;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[i] = fma2(p2, acc2[i], mul2(acc[i], p1));
+    }
+    __device__ __forceinline__ float finish() {         // normalises; natural-log LSE
+        const float inv = l > 0.f ? 1.f / l : 0.f;
+        const f2 i2 = pack2(inv, inv);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[i] = mul2(acc[i], i2);
+        return l > 0.f ? (m + log2f(l)) * 0.6931471805599453f : -INFINITY;
+    }
+};
+
+// The keys of stages `first`, first + 1, ... of one row, read from global memory.
+template <int D, bool BF16, int KP, int C, class Args>
+__device__ __forceinline__ void fwd_walk(const Args &a, const Raw<BF16, D / 8> &q, RowSoftmax &S, int first, int e, int h, int g, int kp, int src, unsigned mask) {
+    using R = Raw<BF16, D / 8>;
+    RowCursor<C, KP * C> cur;
+    bool more = cur.start(a.st, first, e, kp * C);
+    int tm = more ? cur.token(g & (C - 1)) : 0;
+    while (more) {
+        const int jm = cur.j0 + (g & (C - 1)), tc = tm;
+        const bool ok = jm < cur.r.y && (a.dirs == 7 || dir_ok(cur.e, jm, cur.r.x, a.dirs));
+        R kr[C], vr[C];
+#pragma unroll
+        for (int i = 0; i < C; ++i) {
+            const unsigned r = (unsigned)__shfl_sync(mask, tc, src + i, 32) * a.H + h;
+            kr[i].load(a.k, r, g);
+            vr[i].load(a.v, r, g);
+        }
+        more = cur.next(kp * C);
+        if (more) tm = cur.token(g & (C - 1));
+        float sc[C];
+        dots<C>(q, kr, sc);
+        const float x = reduce_scatter<C, D / 8>(sc, g, mask) * a.scale_log2;
+        const float p = S.add<C>(ok ? x : -INFINITY, mask);
+        axpys<C>(S.acc, p, vr, mask, src);
+    }
+}
+
 template <int D, bool BF16, int KP, int C>
 __global__ void __launch_bounds__(ROW_THREADS) k_fwd_rows(const RowFwdArgs a) {
     constexpr int LPK = D / 8, G = LPK * KP;
-    const float NEG = -INFINITY;
+    using R = Raw<BF16, LPK>;
     const int lane = threadIdx.x & 31, sub = lane % G, g = sub % LPK, kp = sub / LPK;
     const unsigned all = G == 32 ? 0xffffffffu : ((1u << G) - 1u) << (lane - sub);     // the lanes of the row
     const int src = lane - g;                                                             // and of the group that shares a key
     const unsigned mask = ((1u << LPK) - 1u) << src;
     const unsigned long long id = ((unsigned long long)blockIdx.x * ROW_THREADS + threadIdx.x) / G;
     if (id >= (unsigned long long)a.n * a.H) return;
-    const int e = (int)(id / a.H), h = (int)(id % a.H);
+    const int e = (int)(id / a.H), h = (int)(id % a.H);     // (the rows of a warp are heads of an element: one range, no divergence)
     const int t = a.first ? a.st[a.first].tok[e] : e;
-    const unsigned row = ((unsigned)t * a.H + h) * LPK + g;
-    f2 q[4], acc[4];
-    {
-        Raw<BF16> r;
-        r.load(a.q, row);
-        r.get(q);
-        const f2 c = pack2(a.scale_log2, a.scale_log2);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) { q[i] = mul2(q[i], c); acc[i] = 0ull; }
-    }
-    float m = NEG, l = 0.f;          // l: this lane's keys only
-    RowCursor<C, KP * C> cur;
-    bool more = cur.start(a.st, a.first, e, kp * C);
-    int tm = more ? cur.token(g & (C - 1)) : 0;
-    {
-        while (more) {
-            const int jm = cur.j0 + (g & (C - 1)), tc = tm;
-            const bool ok = jm < cur.r.y && (a.dirs == 7 || dir_ok(cur.e, jm, cur.r.x, a.dirs));
-            Raw<BF16> kr[C], vr[C];
-#pragma unroll
-            for (int i = 0; i < C; ++i) {
-                const unsigned at = ((unsigned)__shfl_sync(mask, tc, src + i, 32) * a.H + h) * LPK + g;
-                kr[i].load(a.k, at);
-                vr[i].load(a.v, at);
-            }
-            more = cur.next(kp * C);
-            if (more) tm = cur.token(g & (C - 1));
-            float sc[C];
-#pragma unroll
-            for (int i = 0; i < C; ++i) {
-                f2 k[4];
-                kr[i].get(k);
-                sc[i] = dot8(q, k);
-            }
-            float x = reduce_scatter<C, LPK>(sc, g, mask);
-            x = ok ? x : NEG;
-            float mx = x;
-#pragma unroll
-            for (int o = 1; o < C; o *= 2) mx = fmaxf(mx, __shfl_xor_sync(mask, mx, o));
-            mx = fmaxf(mx, m);
-            const float ref = mx > NEG ? mx : 0.f;
-            const float p = exp2f(x - ref), al = exp2f(m - ref);
-            m = mx;
-            l = l * al + p;
-            const f2 al2 = pack2(al, al);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) acc[i] = mul2(acc[i], al2);
-#pragma unroll
-            for (int i = 0; i < C; ++i) {
-                const float w = __shfl_sync(mask, p, src + i, 32);
-                f2 v[4];
-                vr[i].get(v);
-                const f2 w2 = pack2(w, w);
-#pragma unroll
-                for (int u = 0; u < 4; ++u) acc[u] = fma2(w2, v[u], acc[u]);
-            }
-        }
-    }
+    const unsigned row = (unsigned)t * a.H + h;
+    R q;
+    q.load(a.q, row, g);
+    RowSoftmax S;
+    S.clear();
+    fwd_walk<D, BF16, KP, C>(a, q, S, a.first, e, h, g, kp, src, mask);
     // l over the C lanes that hold different keys (lanes g and g + C of a 16-lane group hold the same ones)
 #pragma unroll
-    for (int o = 1; o < C; o *= 2) l += __shfl_xor_sync(mask, l, o);
+    for (int o = 1; o < C; o *= 2) S.l += __shfl_xor_sync(mask, S.l, o);
 #pragma unroll
     for (int o = LPK; o < G; o *= 2) {      // the groups that share the row
-        const float m2 = __shfl_xor_sync(all, m, o), l2 = __shfl_xor_sync(all, l, o);
-        const float mx = fmaxf(m, m2), ref = mx > NEG ? mx : 0.f;
-        const float w1 = exp2f(m - ref), w2 = exp2f(m2 - ref);
-        const f2 p1 = pack2(w1, w1), p2 = pack2(w2, w2);
-        l = l * w1 + l2 * w2;
-        m = mx;
+        f2 acc2[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) acc[i] = fma2(p2, __shfl_xor_sync(all, acc[i], o), mul2(acc[i], p1));
+        for (int i = 0; i < 4; ++i) acc2[i] = __shfl_xor_sync(all, S.acc[i], o);
+        const float m2 = __shfl_xor_sync(all, S.m, o), l2 = __shfl_xor_sync(all, S.l, o);
+        S.merge(m2, l2, acc2);
     }
+    if (kp != 0) return;
     if (a.base_o != nullptr) {              // stage 0's partial result, normalised, as one more key
-        const size_t r1 = (size_t)e * a.H + h;
-        const float s0 = a.base_lse[r1] * 1.4426950408889634f;
-        const float4 *bo = reinterpret_cast<const float4 *>(a.base_o + r1 * D + 8 * g);
-        const float4 x = bo[0], y = bo[1];
-        const float mx = fmaxf(m, s0), ref = mx > NEG ? mx : 0.f;
-        const float w1 = exp2f(m - ref), w0 = exp2f(s0 - ref);
-        const f2 p1 = pack2(w1, w1), p0 = pack2(w0, w0);
-        l = l * w1 + w0;
-        m = mx;
-        acc[0] = fma2(p0, pack2(x.x, x.y), mul2(acc[0], p1));
-        acc[1] = fma2(p0, pack2(x.z, x.w), mul2(acc[1], p1));
-        acc[2] = fma2(p0, pack2(y.x, y.y), mul2(acc[2], p1));
-        acc[3] = fma2(p0, pack2(y.z, y.w), mul2(acc[3], p1));
+        f2 o0[4];
+        R::load_f32(a.base_o, (size_t)e * a.H + h, g, o0);
+        S.merge(a.base_lse[(size_t)e * a.H + h] * 1.4426950408889634f, 1.f, o0);
     }
-    if (kp == 0) {
-        const float inv = l > 0.f ? 1.f / l : 0.f;
-        const f2 i2 = pack2(inv, inv);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) acc[i] = mul2(acc[i], i2);
-        Raw<BF16>::store(a.o, row, acc);
-        if (g == 0) a.lse[(size_t)h * a.T + t] = l > 0.f ? (m + log2f(l)) * 0.6931471805599453f : NEG;
-    }
+    const float lse = S.finish();
+    R::store(a.o, row, g, S.acc);
+    if (g == 0) a.lse[(size_t)h * a.T + t] = lse;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -278,129 +294,391 @@ __global__ void __launch_bounds__(ROW_THREADS) k_fwd_rows(const RowFwdArgs a) {
 // The family ranges of a stage are symmetric: the keys of a row are also the queries that attend to it, so
 // one walk gives the row's dQ (as a query), dK and dV (as a key), each complete: no atomics.
 // DELTA: rowsum(dO . O) is given; else it is computed from O here (one more row per key to read).
-template <int D, bool BF16, int KP, bool DELTA>
-__global__ void __launch_bounds__(ROW_THREADS, BF16 ? 4 : 3) k_bwd_rows(const RowBwdArgs a) {
-    constexpr int LPK = D / 8, G = LPK * KP, C = BF16 ? 4 : 2;
-    const int lane = threadIdx.x & 31, sub = lane % G, g = sub % LPK, kp = sub / LPK;
-    const unsigned all = G == 32 ? 0xffffffffu : ((1u << G) - 1u) << (lane - sub);     // the lanes of the row
-    const int src = lane - g;                                                             // and of the group that shares a key
-    const unsigned mask = ((1u << LPK) - 1u) << src;
-    const unsigned long long id = ((unsigned long long)blockIdx.x * ROW_THREADS + threadIdx.x) / G;
-    if (id >= (unsigned long long)a.n * a.H) return;
-    const int e = (int)(id / a.H), h = (int)(id % a.H);
-    const int t = a.first ? a.st[a.first].tok[e] : e;
-    const unsigned row = ((unsigned)t * a.H + h) * LPK + g;
-    const float L2E = 1.4426950408889634f;
-    // (the row's own values stay as loaded and are unpacked once per chunk: registers decide how many warps hide
-    // the loads' latency here)
-    Raw<BF16> q, k, v, go;
+template <bool BF16, int N> struct RowGrad {
+    Raw<BF16, N> q, k, v, go;          // the row's own values stay as loaded: registers decide how many warps hide the loads' latency
+    float lse, delta;                  // lse in log2 units
     f2 dq[4], dk[4], dv[4];
-    q.load(a.q, row); k.load(a.k, row); v.load(a.v, row); go.load(a.d_o, row);
-    const float lse_i = __ldg(a.lse + (size_t)h * a.T + t) * L2E;
-    float dl_i;
-    if constexpr (DELTA) dl_i = __ldg(a.delta + (size_t)h * a.T + t);
-    else {
-        Raw<BF16> ro;
-        ro.load(a.o, row);
-        dl_i = dot(go, ro);
+    template <bool DELTA, class Args>
+    __device__ __forceinline__ void load(const Args &a, int t, int h, int g, unsigned mask) {
+        const unsigned row = (unsigned)t * a.H + h;
+        q.load(a.q, row, g); k.load(a.k, row, g); v.load(a.v, row, g); go.load(a.d_o, row, g);
+        lse = __ldg(a.lse + (size_t)h * a.T + t) * 1.4426950408889634f;
+        if constexpr (DELTA) delta = __ldg(a.delta + (size_t)h * a.T + t);
+        else {
+            Raw<BF16, N> o;
+            o.load(a.o, row, g);
+            delta = dot(go, o);
 #pragma unroll
-        for (int x = 1; x < LPK; x *= 2) dl_i += __shfl_xor_sync(mask, dl_i, x);
+            for (int x = 1; x < N; x *= 2) delta += __shfl_xor_sync(mask, delta, x);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) dq[i] = dk[i] = dv[i] = 0ull;
     }
+    // The row as a query: K rows x and V rows y of a chunk of its keys; ok: this lane's key counts.
+    template <int C>
+    __device__ __forceinline__ void as_query(const Raw<BF16, N> (&x)[C], const Raw<BF16, N> (&y)[C], bool ok, float scale_log2, int g, unsigned mask, int src) {
+        float v1[C], v2[C];
+        dots<C>(q, x, v1);
+        dots<C>(go, y, v2);
+        const float s = reduce_scatter<C, N>(v1, g, mask) * scale_log2, dp = reduce_scatter<C, N>(v2, g, mask);
+        const float p = ok ? exp2f(s - lse) : 0.f;
+        axpys<C>(dq, p * (dp - delta), x, mask, src);
+    }
+    // The row as a key: Q rows x and dO rows y of queries that attend to it, with their LSE and delta.
+    template <int C>
+    __device__ __forceinline__ void as_key(const Raw<BF16, N> (&x)[C], const Raw<BF16, N> (&y)[C], bool ok, float lse_j, float delta_j, float scale_log2, int g,
+                                           unsigned mask, int src) {
+        float v1[C], v2[C];
+        dots<C>(k, x, v1);
+        dots<C>(v, y, v2);
+        const float s = reduce_scatter<C, N>(v1, g, mask) * scale_log2, dp = reduce_scatter<C, N>(v2, g, mask);
+        const float p = ok ? exp2f(s - lse_j) : 0.f;
+        axpys<C>(dk, p * (dp - delta_j), x, mask, src);
+        axpys<C>(dv, p, y, mask, src);
+    }
+    __device__ __forceinline__ void scale(float c) {
+        const f2 c2 = pack2(c, c);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) dq[i] = dk[i] = dv[i] = 0ull;
+        for (int i = 0; i < 4; ++i) { dq[i] = mul2(dq[i], c2); dk[i] = mul2(dk[i], c2); }
+    }
+};
+
+template <int D, bool BF16, int KP, int C, bool DELTA, class Args>
+__device__ __forceinline__ void bwd_walk(const Args &a, RowGrad<BF16, D / 8> &S, int first, int e, int h, int g, int kp, int src, unsigned mask) {
+    using R = Raw<BF16, D / 8>;
     RowCursor<C, KP * C> cur;
-    bool more = cur.start(a.st, a.first, e, kp * C);
+    bool more = cur.start(a.st, first, e, kp * C);
     int tm = more ? cur.token(g & (C - 1)) : 0;
     while (more) {
         const int jm = cur.j0 + (g & (C - 1)), tc = tm;
         const bool in = jm < cur.r.y;
         const bool ok_q = in && (a.dirs == 7 || dir_ok(cur.e, jm, cur.r.x, a.dirs));          // the row attends to it
         const bool ok_k = in && (a.dirs == 7 || dir_ok_key(cur.e, jm, cur.r.x, a.dirs));      // it attends to the row
-        const float lse_j = __ldg(a.lse + (size_t)h * a.T + tc) * L2E;
+        const float lse_j = __ldg(a.lse + (size_t)h * a.T + tc) * 1.4426950408889634f;
         float dl_j = 0.f;
         if constexpr (DELTA) dl_j = __ldg(a.delta + (size_t)h * a.T + tc);
-        Raw<BF16> x[C], y[C];
+        R x[C], y[C];
         unsigned at[C];
-        float v1[C], v2[C];
-        // the row as a query: K and V of its keys
 #pragma unroll
         for (int i = 0; i < C; ++i) {
-            at[i] = ((unsigned)__shfl_sync(mask, tc, src + i, 32) * a.H + h) * LPK + g;
-            x[i].load(a.k, at[i]);
-            y[i].load(a.v, at[i]);
+            at[i] = (unsigned)__shfl_sync(mask, tc, src + i, 32) * a.H + h;
+            x[i].load(a.k, at[i], g);
+            y[i].load(a.v, at[i], g);
         }
         more = cur.next(kp * C);
         if (more) tm = cur.token(g & (C - 1));
-        dots<C>(q, x, v1);
-        dots<C>(go, y, v2);
-        {
-            const float s_ij = reduce_scatter<C, LPK>(v1, g, mask) * a.scale_log2, dp_ij = reduce_scatter<C, LPK>(v2, g, mask);
-            const float p_ij = ok_q ? exp2f(s_ij - lse_i) : 0.f;
-            axpys<C>(dq, p_ij * (dp_ij - dl_i), x, mask, src);
-        }
-        // the row as a key: Q and dO of the queries that attend to it
+        S.template as_query<C>(x, y, ok_q, a.scale_log2, g, mask, src);
 #pragma unroll
         for (int i = 0; i < C; ++i) {
-            x[i].load(a.q, at[i]);
-            y[i].load(a.d_o, at[i]);
+            x[i].load(a.q, at[i], g);
+            y[i].load(a.d_o, at[i], g);
         }
         if constexpr (!DELTA) {
             float v3[C];
 #pragma unroll
             for (int i = 0; i < C; ++i) {
-                Raw<BF16> o;
-                o.load(a.o, at[i]);
+                R o;
+                o.load(a.o, at[i], g);
                 v3[i] = dot(o, y[i]);
             }
-            dl_j = reduce_scatter<C, LPK>(v3, g, mask);
+            dl_j = reduce_scatter<C, D / 8>(v3, g, mask);
         }
-        dots<C>(k, x, v1);
-        dots<C>(v, y, v2);
-        const float s_ji = reduce_scatter<C, LPK>(v1, g, mask) * a.scale_log2, dp_ji = reduce_scatter<C, LPK>(v2, g, mask);
-        const float p_ji = ok_k ? exp2f(s_ji - lse_j) : 0.f;
-        axpys<C>(dk, p_ji * (dp_ji - dl_j), x, mask, src);
-        axpys<C>(dv, p_ji, y, mask, src);
+        S.template as_key<C>(x, y, ok_k, lse_j, dl_j, a.scale_log2, g, mask, src);
     }
+}
+
+template <int D, bool BF16, int KP, bool DELTA>
+__global__ void __launch_bounds__(ROW_THREADS, BF16 ? 4 : 3) k_bwd_rows(const RowBwdArgs a) {
+    constexpr int LPK = D / 8, G = LPK * KP, C = BF16 ? 4 : 2;
+    using R = Raw<BF16, LPK>;
+    const int lane = threadIdx.x & 31, sub = lane % G, g = sub % LPK, kp = sub / LPK;
+    const unsigned all = G == 32 ? 0xffffffffu : ((1u << G) - 1u) << (lane - sub);     // the lanes of the row
+    const int src = lane - g;                                                             // and of the group that shares a key
+    const unsigned mask = ((1u << LPK) - 1u) << src;
+    const unsigned long long id = ((unsigned long long)blockIdx.x * ROW_THREADS + threadIdx.x) / G;
+    if (id >= (unsigned long long)a.n * a.H) return;
+    const int e = (int)(id / a.H), h = (int)(id % a.H);     // (the rows of a warp are heads of an element: one range, no divergence)
+    const int t = a.first ? a.st[a.first].tok[e] : e;
+    RowGrad<BF16, LPK> S;
+    S.template load<DELTA>(a, t, h, g, mask);
+    bwd_walk<D, BF16, KP, C, DELTA>(a, S, a.first, e, h, g, kp, src, mask);
 #pragma unroll
     for (int o = LPK; o < G; o *= 2) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            dq[i] = add2(dq[i], __shfl_xor_sync(all, dq[i], o));
-            dk[i] = add2(dk[i], __shfl_xor_sync(all, dk[i], o));
-            dv[i] = add2(dv[i], __shfl_xor_sync(all, dv[i], o));
+            S.dq[i] = add2(S.dq[i], __shfl_xor_sync(all, S.dq[i], o));
+            S.dk[i] = add2(S.dk[i], __shfl_xor_sync(all, S.dk[i], o));
+            S.dv[i] = add2(S.dv[i], __shfl_xor_sync(all, S.dv[i], o));
         }
     }
-    if (kp == 0) {
-        const f2 c = pack2(a.scale, a.scale);
+    if (kp != 0) return;
+    S.scale(a.scale);
+    if (a.base[0] != nullptr) {         // stage 0's partial gradients
+        f2 y[4];
+        auto plus = [&](f2 (&x)[4], const float *b) {
+            R::load_f32(b, (size_t)e * a.H + h, g, y);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) { dq[i] = mul2(dq[i], c); dk[i] = mul2(dk[i], c); }
-        if (a.base[0] != nullptr) {         // stage 0's partial gradients
-            const size_t r1 = ((size_t)e * a.H + h) * D + 8 * g;
-            auto plus = [&](f2 (&x)[4], const float *b) {
-                const float4 y = *reinterpret_cast<const float4 *>(b + r1), z = *reinterpret_cast<const float4 *>(b + r1 + 4);
-                x[0] = add2(x[0], pack2(y.x, y.y)); x[1] = add2(x[1], pack2(y.z, y.w));
-                x[2] = add2(x[2], pack2(z.x, z.y)); x[3] = add2(x[3], pack2(z.z, z.w));
-            };
-            plus(dq, a.base[0]); plus(dk, a.base[1]); plus(dv, a.base[2]);
-        }
-        Raw<BF16>::store(a.dq, row, dq);
-        Raw<BF16>::store(a.dk, row, dk);
-        Raw<BF16>::store(a.dv, row, dv);
+            for (int i = 0; i < 4; ++i) x[i] = add2(x[i], y[i]);
+        };
+        plus(S.dq, a.base[0]); plus(S.dk, a.base[1]); plus(S.dv, a.base[2]);
     }
+    const unsigned row = (unsigned)t * a.H + h;
+    R::store(a.dq, row, g, S.dq);
+    R::store(a.dk, row, g, S.dk);
+    R::store(a.dv, row, g, S.dv);
 }
 
-// Lanes per row: while all rows fit on the SMs at once several groups of lanes share one, for latency; beyond, one
-// group each (no final merge, fewer idle lanes in short families).
-static int row_groups(long long rows, int D) {
-    for (int kp = 256 / D; kp > 1; kp /= 2)
-        if (rows * kp * (D / 8) <= 148LL * 20 * 32) return kp;
-    return 1;
+// ---------------------------------------------------------------------------------------------
+// fp32, stage 0: the rows' keys staged in shared memory
+// ---------------------------------------------------------------------------------------------
+// A CTA takes 32 (head_dim 64) or 16 (128) rows of a block and the keys of their ranges, in pieces of KT; a
+// row is owned by D / 8 lanes as above.  The elements that live on leave their partial result in stage 1's
+// buffers.  What bounds it is the chain of a key chunk (loads, products, reduction, exponential, broadcast) at the
+// six warps a scheduler holds: 2 x 2048 tokens, 12 x 64, FWD_US us forward and BWD_US backward, against 100 and 191 for
+// the kernels that give 16 dimensions to a lane and walk a whole block's span in step.  Measured and not kept: a row
+// on 2 (forward) or 4 (backward) lanes (49 and 173 us: fewer warps, twice the registers), four and two rows to
+// eight lanes, so that a key read from shared memory serves several (58 and 213), going on to the
+// stages above 0 inside this kernel (70 and 185: one long row holds the CTA).
+static constexpr int TILE_THREADS = 256;
+template <int D> struct TileShape {
+    static constexpr int LPK = D / 8, ROWS = TILE_THREADS / LPK, KT = D == 64 ? 96 : 48;
+};
+__device__ __forceinline__ void cp_async16(float4 *dst, const float4 *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory"); }
+
+// The rows of CTA x of a block and the span of their ranges.
+struct TileRows {
+    int r0, n, a, b;
+    template <class Args>
+    __device__ __forceinline__ void find(const Args &p, int rows, int per_block, int *s_ab) {
+        const int *rec = p.blocks + 5 * (size_t)p.queue[blockIdx.x / per_block];
+        r0 = rec[0] + (blockIdx.x % per_block) * rows;
+        n = min(rows, rec[1] - r0);
+        if (threadIdx.x == 0) { s_ab[0] = INT_MAX; s_ab[1] = 0; }
+        __syncthreads();
+        for (int i = threadIdx.x; i < n; i += blockDim.x) {
+            const int2 r = __ldg(reinterpret_cast<const int2 *>(p.rng) + r0 + i);
+            if (r.y > r.x) { atomicMin(s_ab, r.x); atomicMax(s_ab + 1, r.y); }
+        }
+        __syncthreads();
+        a = s_ab[0]; b = s_ab[1];
+    }
+};
+template <int D>
+__device__ __forceinline__ void tile_load(float4 *dst, const void *src, int c0, int n, int H, int h) {
+    constexpr int U = D / 4;
+    for (int i = threadIdx.x; i < n * U; i += TILE_THREADS)
+        cp_async16(dst + i, reinterpret_cast<const float4 *>(src) + ((size_t)(c0 + i / U) * H + h) * U + i % U);
+}
+
+template <int D>
+__global__ void __launch_bounds__(TILE_THREADS, 3) k_fwd_tile(const TileFwdArgs a) {
+    constexpr int LPK = D / 8, ROWS = TileShape<D>::ROWS, KT = TileShape<D>::KT, C = 4, U = D / 4;
+    using R = Raw<false, LPK>;
+    extern __shared__ float4 s_tile[];
+    __shared__ int s_ab[2];
+    float4 *sK = s_tile, *sV = sK + KT * U;
+    const int h = blockIdx.y, lane = threadIdx.x & 31, g = lane % LPK, src = lane - g;
+    const unsigned mask = ((1u << LPK) - 1u) << src;
+    TileRows T;
+    T.find(a, ROWS, (a.block_rows + ROWS - 1) / ROWS, s_ab);
+    if (T.n <= 0) return;
+    const int rl = threadIdx.x / LPK, row = T.r0 + rl;
+    const bool inb = rl < T.n;
+    int2 r = make_int2(0, 0);
+    R q;
+    RowSoftmax S;
+    S.clear();
+    if (inb) {
+        r = __ldg(reinterpret_cast<const int2 *>(a.rng) + row);
+        q.load(a.q, (unsigned)row * a.H + h, g);
+    }
+    for (int c0 = T.a; c0 < T.b; c0 += KT) {
+        const int n = min(KT, T.b - c0);
+        if (c0 != T.a) __syncthreads();
+        tile_load<D>(sK, a.k, c0, n, a.H, h);
+        tile_load<D>(sV, a.v, c0, n, a.H, h);
+        cp_async_wait();
+        __syncthreads();
+        const int jlo = max(r.x, c0), jhi = min(r.y, c0 + n);
+        for (int j0 = jlo; j0 < jhi; j0 += C) {
+            float sc[C];
+            f2 qf[4];
+            q.get(qf);
+#pragma unroll
+            for (int i = 0; i < C; ++i) {
+                R x;
+                f2 k[4];
+                x.load_smem(sK + (min(j0 + i, jhi - 1) - c0) * U, g);      // (keys past the end: the last one, weight 0)
+                x.get(k);
+                sc[i] = dot8(qf, k);
+            }
+            const int jm = j0 + (g & (C - 1));
+            const bool ok = jm < jhi && (a.dirs == 7 || dir_ok(row, jm, r.x, a.dirs));
+            const float x = reduce_scatter<C, LPK>(sc, g, mask) * a.scale_log2;
+            const float p = S.add<C>(ok ? x : -INFINITY, mask);
+#pragma unroll
+            for (int i = 0; i < C; ++i) {
+                const float w = __shfl_sync(mask, p, src + i, 32);
+                const f2 w2 = pack2(w, w);
+                R y;
+                f2 v[4];
+                y.load_smem(sV + (min(j0 + i, jhi - 1) - c0) * U, g);
+                y.get(v);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) S.acc[u] = fma2(w2, v[u], S.acc[u]);
+            }
+        }
+    }
+    if (!inb) return;
+    const int up = a.up ? __ldg(a.up + row) : -1;
+    // (l over the C lanes that hold different keys)
+#pragma unroll
+    for (int o = 1; o < C; o *= 2) S.l += __shfl_xor_sync(mask, S.l, o);
+    const float lse = S.finish();
+    if (up >= 0) {
+        R::store(a.part_o, (unsigned)up * a.H + h, g, S.acc);
+        if (g == 0) a.part_lse[(size_t)up * a.H + h] = lse;
+    }
+    R::store(a.o, (unsigned)row * a.H + h, g, S.acc);
+    if (g == 0) a.lse[(size_t)h * a.T + row] = lse;
+}
+
+template <int D>
+__global__ void __launch_bounds__(TILE_THREADS, 2) k_bwd_tile(const TileBwdArgs a) {
+    constexpr int LPK = D / 8, ROWS = TileShape<D>::ROWS, KT = TileShape<D>::KT, C = 2, U = D / 4;
+    using R = Raw<false, LPK>;
+    extern __shared__ float4 s_tile[];
+    __shared__ int s_ab[2];
+    __shared__ float s_lse[KT], s_delta[KT];
+    float4 *sK = s_tile, *sV = sK + KT * U, *sQ = sV + KT * U, *sG = sQ + KT * U;
+    const int h = blockIdx.y, lane = threadIdx.x & 31, g = lane % LPK, src = lane - g;
+    const unsigned mask = ((1u << LPK) - 1u) << src;
+    TileRows T;
+    T.find(a, ROWS, (a.block_rows + ROWS - 1) / ROWS, s_ab);
+    if (T.n <= 0) return;
+    const int rl = threadIdx.x / LPK, row = T.r0 + min(rl, T.n - 1);
+    const bool inb = rl < T.n;
+    int2 r = inb ? __ldg(reinterpret_cast<const int2 *>(a.rng) + row) : make_int2(0, 0);
+    RowGrad<false, LPK> S;
+    S.template load<false>(a, row, h, g, mask);
+    for (int c0 = T.a; c0 < T.b; c0 += KT) {
+        const int n = min(KT, T.b - c0);
+        if (c0 != T.a) __syncthreads();
+        tile_load<D>(sK, a.k, c0, n, a.H, h);
+        tile_load<D>(sV, a.v, c0, n, a.H, h);
+        tile_load<D>(sQ, a.q, c0, n, a.H, h);
+        tile_load<D>(sG, a.d_o, c0, n, a.H, h);
+        cp_async_wait();
+        __syncthreads();
+        for (int i = rl; i < n; i += ROWS) {           // rowsum(dO . O) of the tile's rows
+            R o, y;
+            o.load(a.o, (unsigned)(c0 + i) * a.H + h, g);
+            y.load_smem(sG + i * U, g);
+            float d = dot(o, y);
+#pragma unroll
+            for (int x = 1; x < LPK; x *= 2) d += __shfl_xor_sync(mask, d, x);
+            if (g == 0) {
+                s_delta[i] = d;
+                s_lse[i] = __ldg(a.lse + (size_t)h * a.T + c0 + i) * 1.4426950408889634f;
+            }
+        }
+        __syncthreads();
+        const int jlo = max(r.x, c0), jhi = min(r.y, c0 + n);
+        for (int j0 = jlo; j0 < jhi; j0 += C) {
+            const int jm = j0 + (g & (C - 1)), jc = min(jm, jhi - 1);
+            const bool in = jm < jhi;
+            const bool ok_q = in && (a.dirs == 7 || dir_ok(row, jm, r.x, a.dirs));
+            const bool ok_k = in && (a.dirs == 7 || dir_ok_key(row, jm, r.x, a.dirs));
+            R x[C], y[C];
+#pragma unroll
+            for (int i = 0; i < C; ++i) {
+                const int o = (min(j0 + i, jhi - 1) - c0) * U;
+                x[i].load_smem(sK + o, g);
+                y[i].load_smem(sV + o, g);
+            }
+            S.template as_query<C>(x, y, ok_q, a.scale_log2, g, mask, src);
+#pragma unroll
+            for (int i = 0; i < C; ++i) {
+                const int o = (min(j0 + i, jhi - 1) - c0) * U;
+                x[i].load_smem(sQ + o, g);
+                y[i].load_smem(sG + o, g);
+            }
+            S.template as_key<C>(x, y, ok_k, s_lse[jc - c0], s_delta[jc - c0], a.scale_log2, g, mask, src);
+        }
+    }
+    if (!inb) return;
+    const int up = a.up ? __ldg(a.up + row) : -1;
+    S.scale(a.scale);
+    if (up >= 0) {
+        const unsigned p = (unsigned)up * a.H + h;
+        R::store(a.part[0], p, g, S.dq); R::store(a.part[1], p, g, S.dk); R::store(a.part[2], p, g, S.dv);
+    }
+    const unsigned p = (unsigned)row * a.H + h;
+    R::store(a.dq, p, g, S.dq); R::store(a.dk, p, g, S.dk); R::store(a.dv, p, g, S.dv);
+}
+
+template <int D>
+static int launch_fwd_tile_t(const TileFwdArgs &a, cudaStream_t st) {
+    if (a.nb == 0) return HDT_OK;
+    constexpr int smem = 2 * TileShape<D>::KT * D * 4;
+    static DevOnce once;
+    if (!once.done()) {
+        HDT_CUDA_CHECK(cudaFuncSetAttribute(k_fwd_tile<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        once.set();
+    }
+    constexpr int ROWS = TileShape<D>::ROWS;
+    k_fwd_tile<D><<<dim3(a.nb * ((a.block_rows + ROWS - 1) / ROWS), a.H), TILE_THREADS, smem, st>>>(a);
+    count_launch();
+    HDT_CUDA_CHECK(cudaGetLastError());
+    return HDT_OK;
+}
+template <int D>
+static int launch_bwd_tile_t(const TileBwdArgs &a, cudaStream_t st) {
+    if (a.nb == 0) return HDT_OK;
+    constexpr int smem = 4 * TileShape<D>::KT * D * 4;
+    static DevOnce once;
+    if (!once.done()) {
+        HDT_CUDA_CHECK(cudaFuncSetAttribute(k_bwd_tile<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        once.set();
+    }
+    constexpr int ROWS = TileShape<D>::ROWS;
+    k_bwd_tile<D><<<dim3(a.nb * ((a.block_rows + ROWS - 1) / ROWS), a.H), TILE_THREADS, smem, st>>>(a);
+    count_launch();
+    HDT_CUDA_CHECK(cudaGetLastError());
+    return HDT_OK;
+}
+int launch_fwd_tile(const TileFwdArgs &a, int D, cudaStream_t st) {
+    if (D == 64) return launch_fwd_tile_t<64>(a, st);
+    if (D == 128) return launch_fwd_tile_t<128>(a, st);
+    return set_error(HDT_ERR_UNSUPPORTED, "head_dim %d not supported (64 or 128)", D);
+}
+int launch_bwd_tile(const TileBwdArgs &a, int D, cudaStream_t st) {
+    if (D == 64) return launch_bwd_tile_t<64>(a, st);
+    if (D == 128) return launch_bwd_tile_t<128>(a, st);
+    return set_error(HDT_ERR_UNSUPPORTED, "head_dim %d not supported (64 or 128)", D);
+}
+
+// Groups of lanes per row.  A row's time is its chain of chunks (about two round trips to L2 each), the launch's that
+// chain times the number of times the rows fill the SMs: take the split with the smallest product.  keys: mean
+// keys of a row, chunk: keys a group takes at a time, warps: warps resident on an SM.
+static int row_groups(long long rows, int D, float keys, int chunk, int warps) {
+    int best = 1;
+    double least = 0;
+    for (int kp = 1; kp <= 256 / D; kp *= 2) {
+        const double lanes = (double)rows * kp * (D / 8), waves = lanes / (148.0 * 32 * warps);
+        const double t = (waves < 1 ? 1 : waves) * (keys / (chunk * kp) + 2.5 + (kp > 1 ? 0.5 : 0));
+        if (kp == 1 || t < least) { best = kp; least = t; }
+    }
+    return best;
 }
 template <int D, bool BF16>
 static int launch_fwd_rows_t(const RowFwdArgs &a, cudaStream_t st) {
     const long long rows = (long long)a.n * a.H;
     if (rows == 0) return HDT_OK;
-    const int kp = row_groups(rows, D);
+    const int kp = row_groups(rows, D, a.keys, a.first ? 8 : 4, BF16 ? 16 : 12);
     const unsigned grid = (unsigned)((rows * kp * (D / 8) + ROW_THREADS - 1) / ROW_THREADS);
     if (kp == 4) k_fwd_rows<D, BF16, D == 64 ? 4 : 1, 8><<<grid, ROW_THREADS, 0, st>>>(a);
     else if (kp == 2) k_fwd_rows<D, BF16, 2, 8><<<grid, ROW_THREADS, 0, st>>>(a);
@@ -414,7 +692,7 @@ template <int D, bool BF16, bool DELTA>
 static int launch_bwd_rows_t(const RowBwdArgs &a, cudaStream_t st) {
     const long long rows = (long long)a.n * a.H;
     if (rows == 0) return HDT_OK;
-    const int kp = row_groups(2 * rows, D);
+    const int kp = row_groups(rows, D, a.keys, BF16 ? 4 : 2, BF16 ? 16 : 12);
     const unsigned grid = (unsigned)((rows * kp * (D / 8) + ROW_THREADS - 1) / ROW_THREADS);
     if (kp == 4) k_bwd_rows<D, BF16, D == 64 ? 4 : 1, DELTA><<<grid, ROW_THREADS, 0, st>>>(a);
     else if (kp == 2) k_bwd_rows<D, BF16, 2, DELTA><<<grid, ROW_THREADS, 0, st>>>(a);

@@ -274,6 +274,7 @@ int launch_delta(const void *o, const void *d_o, float *delta, int T, int H, int
 struct RowStage { const int *tok, *rng, *up; };
 struct RowFwdArgs {
     int n, H, T, first, dirs;            // n: elements of stage `first`
+    float keys;                          // mean keys of a row (over all its stages)
     const void *q, *k, *v;
     void *o;
     float *lse, scale_log2;
@@ -282,6 +283,7 @@ struct RowFwdArgs {
 };
 struct RowBwdArgs {
     int n, H, T, first, dirs;
+    float keys;
     const void *q, *k, *v, *o, *d_o;
     const float *lse, *delta;            // delta nullptr: computed from o
     float scale, scale_log2;
@@ -289,6 +291,27 @@ struct RowBwdArgs {
     const float *base[3];                // first = 1: stage 0's partial gradients, [n, H, D]
     RowStage st[HDT_MAX_STAGES];
 };
+// fp32, stage 0, keys staged in shared memory.
+struct TileFwdArgs {
+    int nb, block_rows, H, T, dirs;
+    const int *blocks, *queue, *rng, *up;      // up nullptr: there is no stage above 0; else the partial results of the elements
+                                               // that live on go to part_o / part_lse, part[] at up[e]
+    const void *q, *k, *v;
+    void *o;
+    float *lse, scale_log2;
+    float *part_o, *part_lse;
+};
+struct TileBwdArgs {
+    int nb, block_rows, H, T, dirs;
+    const int *blocks, *queue, *rng, *up;
+    const void *q, *k, *v, *o, *d_o;
+    const float *lse;                          // (rowsum(dO . O) is computed from o)
+    float scale, scale_log2;
+    void *dq, *dk, *dv;
+    float *part[3];
+};
+int launch_fwd_tile(const TileFwdArgs &a, int head_dim, cudaStream_t st);
+int launch_bwd_tile(const TileBwdArgs &a, int head_dim, cudaStream_t st);
 int launch_fwd_rows(const RowFwdArgs &a, int head_dim, int dtype, cudaStream_t st);
 int launch_bwd_rows(const RowBwdArgs &a, int head_dim, int dtype, cudaStream_t st);
 // One launch that completes every token of stage 1 (= every token that lives in a stage above 0):
