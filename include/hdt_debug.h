@@ -49,6 +49,9 @@ extern "C" {
  *                    of the stage-1 kernel itself (the default where a family of stage 1 is longer than
  *                    a block); bit 1: the stage-1 kernel does it there too; bit 2: the backward's
  *                    stage-1 kernel does the completion (off by default).
+ *   "no_rows"        1: no row-wise kernels (short families above stage 0, batches of tiny families, fp32
+ *                    stage 0 with its keys in shared memory); the other options that choose a kernel
+ *                    for the stages above 0 switch them off too.
  *   "no_overlap"     1: the stages above 0 run after stage 0 on the caller's stream instead of
  *                    beside it on an internal stream.
  *   "no_graph"       accepted and without effect (the index build is two launches; there is no graph to leave out).

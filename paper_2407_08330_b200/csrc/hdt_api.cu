@@ -74,7 +74,6 @@ static int g_no_self_beside = 0;
 static int g_no_fused_delta = 0;
 static int g_no_fold = 0;
 static int g_no_rows = 0;
-static long long g_rows_lim[5] = {400000, 40000, 10, 10, 4000000};
 
 int get_side(Side **out) {
     int dev = -1;
@@ -186,7 +185,6 @@ extern "C" int hdt_set_option(const char *name, int32_t value) {
     if (name && std::strcmp(name, "no_multi_upper") == 0) { g_no_multi_upper = value; return HDT_OK; }
     if (name && std::strcmp(name, "no_self_beside") == 0) { g_no_self_beside = value; return HDT_OK; }
     if (name && std::strcmp(name, "no_rows") == 0) { g_no_rows = value; return HDT_OK; }
-    if (name && std::strncmp(name, "rows_lim", 8) == 0) { g_rows_lim[name[8] - '0'] = value; return HDT_OK; }
     return set_error(HDT_ERR_INVALID_ARG, "hdt_set_option: unknown option");
 }
 
@@ -241,18 +239,26 @@ extern "C" int hdt_profile_read(int32_t id, int64_t *launches, double *total_ms,
 static bool rows_allowed() {
     return !g_no_rows && !g_force_simt && !g_simt_upper && !g_no_overlap && !g_no_fold && !g_no_multi_upper && g_no_persistent == 0;
 }
-// All stages row by row.
-static bool rows_all(const hdt_index *ix, int dtype) {
-    return rows_allowed() && ix->nnz <= g_rows_lim[dtype == HDT_F32 ? 3 : 2] * ix->total_tokens;
+// All stages row by row: families so small that a tile kernel's 128 x 128 products are nearly all padding
+// (expression trees have six keys a row, documents forty; at ten the two cost the same), and small fp32 calls, whose
+// rows all fit on the SMs in a wave or two (2935 tokens, 12 x 64, forward: 83 us a call against 88 on the
+// shared-memory kernels; 4096: 107 against 88).
+static bool rows_all(const hdt_index *ix, int heads, int head_dim, int dtype) {
+    const bool few = dtype == HDT_F32 && (long long)ix->total_tokens * heads * (head_dim / 64) <= 40000;
+    return rows_allowed() && ix->nnz <= (few ? 64 : 10) * ix->real;
 }
-// fp32 calls: stage 0 on the kernels that stage its keys in shared memory.
-static bool tile_f32(int dtype) { return dtype == HDT_F32 && !g_no_rows && !g_force_simt; }
-static bool tile_walk(const hdt_index *ix, int heads, int head_dim) {
-    return ix->n_stages == 1 || (rows_allowed() && ix->nnz_upper * heads * (head_dim / 64) <= g_rows_lim[4]);
-}
-// The stages above 0 row by row.
+// The stages above 0 row by row, in one launch behind stage 0, while their pairs are few; beyond, the tile
+// kernels' launches beside stage 0 and the merge behind it cost less.  The lines lie where the two met on
+// documents of 200 to 90 000 tokens (forward: 4 x 8192 tokens and 12 heads, 215 000, lost 2 us of 219; backward,
+// four times the work a pair: gains of 5 to 10 us of 60 to 150 below 30 000, a loss of 2 at 97 000).
 static bool rows_upper(const hdt_index *ix, int heads, int head_dim, int bwd) {
-    return rows_allowed() && ix->n_stages > 1 && ix->nnz_upper * heads * (head_dim / 64) <= g_rows_lim[bwd];
+    return rows_allowed() && ix->n_stages > 1 && ix->nnz_upper * heads * (head_dim / 64) <= (bwd ? 40000 : 200000);
+}
+// fp32 calls: stage 0 on the kernels that stage its keys in shared memory; the stages above it row by row unless
+// their families are long (the SIMT tile kernels read such a family's rows once per block).
+static bool tile_f32(int dtype) { return dtype == HDT_F32 && !g_no_rows && !g_force_simt; }
+static bool tile_f32_rows(const hdt_index *ix, int heads, int head_dim) {
+    return ix->n_stages == 1 || (rows_allowed() && ix->nnz_upper * heads * (head_dim / 64) <= 4000000);
 }
 static void row_stages(const hdt_index *ix, RowStage *st) {
     for (int s = 0; s < ix->n_stages; ++s) st[s] = RowStage{ix->st[s].tok, ix->st[s].rng, ix->st[s].up};
@@ -319,12 +325,12 @@ extern "C" int hdt_attn_fwd(const hdt_index_t *ix, const void *q, const void *k,
     rc = check_common(ix, heads, head_dim, dtype, workspace, workspace_bytes, L.total, "hdt_attn_fwd");
     if (rc) return rc;
     if (ix->total_tokens == 0) return HDT_OK;
-    const bool all_rows = !early && rows_all(ix, dtype);
+    const bool all_rows = !early && rows_all(ix, heads, head_dim, dtype);
     const bool up_rows = all_rows || rows_upper(ix, heads, head_dim, 0);
     auto upper_rows = [&](int first) {      // the elements of stage `first` with everything above it
         RowFwdArgs a{};
         a.n = ix->desc[first].n; a.H = heads; a.T = ix->total_tokens; a.first = first; a.dirs = ix->directions;
-        a.keys = (float)(first ? ix->nnz_upper : ix->nnz) / (float)(a.n > 0 ? a.n : 1);
+        a.keys = first ? (float)ix->nnz_upper / (float)(a.n > 0 ? a.n : 1) : (float)ix->nnz / (float)(ix->real > 0 ? ix->real : 1);
         a.q = q; a.k = k; a.v = v; a.o = o; a.lse = lse;
         a.scale_log2 = scale * 1.4426950408889634f;
         if (first) { a.base_o = (const float *)(ws + L.part[1][0]); a.base_lse = (const float *)(ws + L.part[1][1]); }
@@ -343,7 +349,7 @@ extern "C" int hdt_attn_fwd(const hdt_index_t *ix, const void *q, const void *k,
         ProfScope ps(PROF_FWD_STAGE0, s_);
         return launch_fwd_tile(a, head_dim, s_);
     };
-    if (tile_f32(dtype) && tile_walk(ix, heads, head_dim)) {
+    if (tile_f32(dtype) && tile_f32_rows(ix, heads, head_dim)) {
         rc = tile_stage0(st);
         return rc || ix->n_stages == 1 ? rc : upper_rows(1);
     }
@@ -521,11 +527,11 @@ extern "C" int hdt_attn_bwd(const hdt_index_t *ix, const void *q, const void *k,
     int *status = device_status_ptr();
     if (!status) return HDT_ERR_CUDA;
     const bool overlap = ix->n_stages > 1 && !g_no_overlap;
-    const bool all_rows = rows_all(ix, dtype), up_rows = all_rows || rows_upper(ix, heads, head_dim, 1);
+    const bool all_rows = rows_all(ix, heads, head_dim, dtype), up_rows = all_rows || rows_upper(ix, heads, head_dim, 1);
     auto upper_rows = [&](int first, const float *delta_) {      // (see hdt_attn_fwd)
         RowBwdArgs a{};
         a.n = ix->desc[first].n; a.H = heads; a.T = ix->total_tokens; a.first = first; a.dirs = ix->directions;
-        a.keys = (float)(first ? ix->nnz_upper : ix->nnz) / (float)(a.n > 0 ? a.n : 1);
+        a.keys = first ? (float)ix->nnz_upper / (float)(a.n > 0 ? a.n : 1) : (float)ix->nnz / (float)(ix->real > 0 ? ix->real : 1);
         a.q = q; a.k = k; a.v = v; a.o = o; a.d_o = d_o; a.lse = lse; a.delta = delta_;
         a.scale = scale; a.scale_log2 = scale * 1.4426950408889634f;
         a.dq = dq; a.dk = dk; a.dv = dv;
@@ -583,7 +589,7 @@ extern "C" int hdt_attn_bwd(const hdt_index_t *ix, const void *q, const void *k,
         ProfScope ps(PROF_BWD_STAGE0, st);
         return launch_bwd_tile(a, head_dim, st);
     };
-    if (tile_f32(dtype) && tile_walk(ix, heads, head_dim)) {
+    if (tile_f32(dtype) && tile_f32_rows(ix, heads, head_dim)) {
         rc = tile_stage0();
         return rc || ix->n_stages == 1 ? rc : upper_rows(1, nullptr);
     }

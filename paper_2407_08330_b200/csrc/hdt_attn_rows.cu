@@ -7,6 +7,11 @@
 //   - all stages of batches whose families are tiny throughout (expression trees: six keys a row).
 // All arithmetic is fp32 (P and dS are not rounded).
 //
+// What bounds them: the latency of a row's chain of loads at the occupancy their registers leave, then instruction
+// issue (200 trees: 55 us forward at 44 % of the issue slots).  Whole calls before and after (build, forward and,
+// with b, backward): 200 trees 807 -> 260 us b, one tree 280 -> 82 b, 12 layers of 1 x 4096 tokens 389 -> 295,
+// 2 x 220 tokens fp32 133 -> 46 b, 8 x 2048 padded 56 -> 51.
+//
 // Lanes: D / 8 lanes hold 8 dimensions each; a chunk of C keys is a C-fold load of 16 (bf16) or 32 (fp32)
 // bytes per lane, all in flight together.  The C dot products are summed over the lanes by a reduce-scatter
 // (C - 1 shuffles instead of 3 C or 4 C), which leaves one key's score per lane: one exponential per key
@@ -249,7 +254,7 @@ __device__ __forceinline__ void fwd_walk(const Args &a, const Raw<BF16, D / 8> &
 }
 
 template <int D, bool BF16, int KP, int C>
-__global__ void __launch_bounds__(ROW_THREADS) k_fwd_rows(const RowFwdArgs a) {
+__global__ void __launch_bounds__(ROW_THREADS, KP == 1 && C == 4 && BF16 ? 8 : 4) k_fwd_rows(const RowFwdArgs a) {
     constexpr int LPK = D / 8, G = LPK * KP;
     using R = Raw<BF16, LPK>;
     const int lane = threadIdx.x & 31, sub = lane % G, g = sub % LPK, kp = sub / LPK;
@@ -389,7 +394,7 @@ __device__ __forceinline__ void bwd_walk(const Args &a, RowGrad<BF16, D / 8> &S,
 
 template <int D, bool BF16, int KP, bool DELTA>
 __global__ void __launch_bounds__(ROW_THREADS, BF16 ? 4 : 3) k_bwd_rows(const RowBwdArgs a) {
-    constexpr int LPK = D / 8, G = LPK * KP, C = BF16 ? 4 : 2;
+    constexpr int LPK = D / 8, G = LPK * KP, C = 2;
     using R = Raw<BF16, LPK>;
     const int lane = threadIdx.x & 31, sub = lane % G, g = sub % LPK, kp = sub / LPK;
     const unsigned all = G == 32 ? 0xffffffffu : ((1u << G) - 1u) << (lane - sub);     // the lanes of the row
@@ -434,7 +439,7 @@ __global__ void __launch_bounds__(ROW_THREADS, BF16 ? 4 : 3) k_bwd_rows(const Ro
 // A CTA takes 32 (head_dim 64) or 16 (128) rows of a block and the keys of their ranges, in pieces of KT; a
 // row is owned by D / 8 lanes as above.  The elements that live on leave their partial result in stage 1's
 // buffers.  What bounds it is the chain of a key chunk (loads, products, reduction, exponential, broadcast) at the
-// six warps a scheduler holds: 2 x 2048 tokens, 12 x 64, FWD_US us forward and BWD_US backward, against 100 and 191 for
+// six warps a scheduler holds: 2 x 2048 tokens, 12 x 64, 53 us forward and 141 backward, against 100 and 191 for
 // the kernels that give 16 dimensions to a lane and walk a whole block's span in step.  Measured and not kept: a row
 // on 2 (forward) or 4 (backward) lanes (49 and 173 us: fewer warps, twice the registers), four and two rows to
 // eight lanes, so that a key read from shared memory serves several (58 and 213), going on to the
@@ -692,7 +697,7 @@ template <int D, bool BF16, bool DELTA>
 static int launch_bwd_rows_t(const RowBwdArgs &a, cudaStream_t st) {
     const long long rows = (long long)a.n * a.H;
     if (rows == 0) return HDT_OK;
-    const int kp = row_groups(rows, D, a.keys, BF16 ? 4 : 2, BF16 ? 16 : 12);
+    const int kp = row_groups(rows, D, a.keys, 2, BF16 ? 16 : 12);
     const unsigned grid = (unsigned)((rows * kp * (D / 8) + ROW_THREADS - 1) / ROW_THREADS);
     if (kp == 4) k_bwd_rows<D, BF16, D == 64 ? 4 : 1, DELTA><<<grid, ROW_THREADS, 0, st>>>(a);
     else if (kp == 2) k_bwd_rows<D, BF16, 2, DELTA><<<grid, ROW_THREADS, 0, st>>>(a);

@@ -36,7 +36,7 @@ struct SeqInfo {
     int stages;                // stages this sequence's own hierarchy needs (at least 1)
     int res;                   // elements it still has in any later stage of the batch: its root, or nothing
     int err, err_pos;          // structure error, 0 = none
-    int more, pad;             // elements were left after the last allowed stage
+    int more, real;            // elements were left after the last allowed stage; tokens that are not PAD
     long long nnz, nnz_upper, visited;
 };
 
@@ -181,7 +181,7 @@ struct SeqArgs {
 struct SeqShared {
     int bst0[SB0], bst[SBU];
     int wtot[32], wtotu[32], ctot[SEQ_CLUSTER];
-    int err, err_pos, flag0, flag, nb0, nb, nf0, ne0, nf, ne;
+    int err, err_pos, real, flag0, flag, nb0, nb, nf0, ne0, nf, ne;
     int ns[HDT_MAX_STAGES], bsw[16][SBW], nfs[16], nes[16];     // (seq_upper_all)
     unsigned long long nnz, nnz_upper, vis;
 };
@@ -366,7 +366,7 @@ __device__ __forceinline__ void seq_stage0(const SeqArgs &a, SeqShared &sh, SeqS
     }
     seq_sync(c.cs);
     const int k = seg_shift(c.ne, nw);
-    int run = 0, next = 0;
+    int run = 0, next = 0, nreal = 0;
     long long deg = 0;
     for (int i0 = w << k; i0 < min((w + 1) << k, c.ne); i0 += 32) {
         const int i = i0 + lane, e = c.e0 + i, g = c.s0 + e;
@@ -378,6 +378,7 @@ __device__ __forceinline__ void seq_stage0(const SeqArgs &a, SeqShared &sh, SeqS
             const bool child = elem_range<E>(e, p, y[i], p != E::NONE ? Y.get(p) : 0u, e == 0 && root_real, lo, hi);
             if (child && !((int)p < e && e < (int)hi)) seq_fail(sh0, g);
             kp = real && !child;
+            nreal += real;
             fpos[e] = child ? (uint8_t)min(e - (int)p, 255) : 0;
             deg += row_pairs(e, (int)lo, (int)hi, a.dirs);
             if (kp && p != E::NONE) next = 1;
@@ -388,8 +389,10 @@ __device__ __forceinline__ void seq_stage0(const SeqArgs &a, SeqShared &sh, SeqS
     }
     for (int o = 16; o; o >>= 1) deg += __shfl_xor_sync(0xffffffffu, deg, o);
     next = __any_sync(0xffffffffu, next);
+    nreal = __reduce_add_sync(0xffffffffu, nreal);
     if (lane == 0) {
         sh.wtot[w] = run;
+        if (nreal) atomicAdd(&sh0->real, nreal);
         if (deg) atomicAdd(&sh0->nnz, (unsigned long long)deg);
         if (next) sh0->flag0 = 1;
     }
@@ -662,7 +665,7 @@ __global__ void __launch_bounds__(512) k_seq(const SeqArgs a) {
     c.ne = min(1 << c.sl, c.L - c.e0);
     const bool first = c.rank == 0;
     if (t == 0) {
-        sh.err = 0; sh.err_pos = 0; sh.flag0 = 0; sh.nf0 = 0; sh.ne0 = 0; sh.nnz = 0; sh.nnz_upper = 0; sh.vis = 0;
+        sh.err = 0; sh.err_pos = 0; sh.real = 0; sh.flag0 = 0; sh.nf0 = 0; sh.ne0 = 0; sh.nnz = 0; sh.nnz_upper = 0; sh.vis = 0;
         if (first) {
             if (c1 < c0 || c0 < 0 || c1 > a.T || (b == 0 && c0 != 0) || (b == a.B - 1 && c1 != a.T)) seq_fail(&sh, b);
             a.scu[b] = c0;
@@ -763,7 +766,7 @@ __global__ void __launch_bounds__(512) k_seq(const SeqArgs a) {
             p[0] = res; p[q] = res; p[2 * q] = 0; p[3 * q] = res;
         }
         SeqInfo f;
-        f.stages = stages; f.res = res; f.err = sh.err; f.err_pos = sh.err_pos; f.more = more; f.pad = 0;
+        f.stages = stages; f.res = res; f.err = sh.err; f.err_pos = sh.err_pos; f.more = more; f.real = sh.real;
         f.nnz = (long long)(sh.nnz + sh.nnz_upper); f.nnz_upper = (long long)sh.nnz_upper; f.visited = (long long)sh.vis;
         a.info[b] = f;
     }
@@ -814,8 +817,8 @@ __device__ __forceinline__ void row_sums(int rows, int m, int w, int nw, int lan
 __device__ void finish_header(const FinishArgs &f, int S) {
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     __shared__ int s_err, s_more;
-    __shared__ long long s_sum[3];
-    if (t == 0) { s_err = 0x7fffffff; s_more = 0; s_sum[0] = s_sum[1] = s_sum[2] = 0; }
+    __shared__ long long s_sum[4];
+    if (t == 0) { s_err = 0x7fffffff; s_more = 0; s_sum[0] = s_sum[1] = s_sum[2] = s_sum[3] = 0; }
     __syncthreads();
     const size_t q = (size_t)f.ms * f.B;
     row_sums(4 * S, f.B, w, FT / 32, lane, [&](int i) { return f.counts + (i & 3) * q + (size_t)(i >> 2) * f.B; },
@@ -827,15 +830,15 @@ __device__ void finish_header(const FinishArgs &f, int S) {
                  *pd = v;
                  *reinterpret_cast<volatile int *>(ph) = v;
              });
-    long long nnz = 0, vis = 0, nup = 0;
+    long long nnz = 0, vis = 0, nup = 0, real = 0;
     for (int b = t; b < f.B; b += FT) {
         const SeqInfo &x = f.info[b];
-        nnz += x.nnz; vis += x.visited; nup += x.nnz_upper;
+        nnz += x.nnz; vis += x.visited; nup += x.nnz_upper; real += x.real;
         if (x.err) atomicMin(&s_err, b);
         if (x.more) s_more = 1;
     }
-    nnz = warp_sum(nnz); vis = warp_sum(vis); nup = warp_sum(nup);
-    if (lane == 0) { atomicAdd((unsigned long long *)&s_sum[0], (unsigned long long)nnz); atomicAdd((unsigned long long *)&s_sum[1], (unsigned long long)vis); atomicAdd((unsigned long long *)&s_sum[2], (unsigned long long)nup); }
+    nnz = warp_sum(nnz); vis = warp_sum(vis); nup = warp_sum(nup); real = warp_sum(real);
+    if (lane == 0) { atomicAdd((unsigned long long *)&s_sum[0], (unsigned long long)nnz); atomicAdd((unsigned long long *)&s_sum[1], (unsigned long long)vis); atomicAdd((unsigned long long *)&s_sum[2], (unsigned long long)nup); atomicAdd((unsigned long long *)&s_sum[3], (unsigned long long)real); }
     __syncthreads();
     if (t <= HDT_MAX_STAGES) {
         const int more = (t + 1 < S) || (t + 1 == S && s_more);
@@ -853,8 +856,8 @@ __device__ void finish_header(const FinishArgs &f, int S) {
         if (f.B == 0) { f.st[0].scu[0] = f.cu[0]; if (f.cu[0] != 0 || f.T != 0) err = HDT_ERR_BAD_HIERARCHY; }
         else if (s_err != 0x7fffffff) { err = f.info[s_err].err; pos = f.info[s_err].err_pos; }
         volatile DevHeader *h = f.host;
-        f.hdr->status = err; f.hdr->err_pos = pos; f.hdr->nnz = s_sum[0]; f.hdr->visited = s_sum[1]; f.hdr->nnz_upper = s_sum[2]; f.hdr->tail = 0;
-        h->status = err; h->err_pos = pos; h->nnz = s_sum[0]; h->visited = s_sum[1]; h->nnz_upper = s_sum[2];
+        f.hdr->status = err; f.hdr->err_pos = pos; f.hdr->nnz = s_sum[0]; f.hdr->visited = s_sum[1]; f.hdr->nnz_upper = s_sum[2]; f.hdr->real = s_sum[3]; f.hdr->tail = 0;
+        h->status = err; h->err_pos = pos; h->nnz = s_sum[0]; h->visited = s_sum[1]; h->nnz_upper = s_sum[2]; h->real = s_sum[3];
     }
     __threadfence_system();
     __syncthreads();
@@ -1258,6 +1261,7 @@ int index_ready(const hdt_index *cix) {
                 ix->nnz = h.nnz;
                 ix->visited = h.visited;
                 ix->nnz_upper = h.nnz_upper;
+                ix->real = h.real;
                 for (int s = 0; s <= HDT_MAX_STAGES; ++s) ix->desc[s] = h.st[s];
             }
         }

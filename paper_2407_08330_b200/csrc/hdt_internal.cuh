@@ -23,6 +23,7 @@ struct DevHeader {
     int err_pos;             // element / sequence where it was detected
     long long nnz;           // unmasked pairs
     long long nnz_upper;     // those of the stages above 0
+    long long real;          // tokens that are not PAD
     long long visited;       // sum over blocks of rows x span
     StageDesc st[HDT_MAX_STAGES + 1];
     int tail;                // always 0 on the device: the last word of the header to arrive on the host
@@ -38,7 +39,7 @@ struct StagePtrs {
 struct hdt_index {
     int batch, total_tokens, block_m, block_m_upper, n_stages;
     int directions;   // bits 1 | 2 | 4: child->parent, sibling<->sibling, parent->child entries kept (7 = full rule)
-    long long nnz, nnz_upper, visited;
+    long long nnz, nnz_upper, real, visited;
     hdt::StageDesc desc[HDT_MAX_STAGES + 1];
     hdt::StagePtrs st[HDT_MAX_STAGES];
     void *workspace;
