@@ -96,8 +96,17 @@ __global__ void __launch_bounds__(128) k_fwd_tc(const __grid_constant__ CUtensor
                            : (a.rest_only ? a.queue_split[a.n_fused + blockIdx.x] : a.queue[blockIdx.x]);
     const int h = blockIdx.y, H = a.H;
     const int *rec = a.blocks + 5 * (size_t)blk;
-    const int r0 = rec[0], r1 = rec[1], ka = rec[2], kb = rec[3], fl = rec[4];
+    const int r0 = rec[0], r1 = rec[1], fl = rec[4];
+    int ka = rec[2], kb = rec[3];
     const float NEG = -INFINITY, LN2 = 0.6931471805599453f;
+    if constexpr (GATHER) {
+        if (r1 <= r0) return;               // a block slot that is not in use
+        if (a.splits > 1) {                 // this CTA's share of the key span, whole chunks
+            const int per = ((kb - ka + 127) / 128 + a.splits - 1) / a.splits * 128;
+            ka += (int)blockIdx.z * per;
+            kb = min(kb, ka + per);
+        }
+    }
 
     if (tid == 0) {
         mbar_init(bar_tma, 1);
@@ -134,7 +143,7 @@ __global__ void __launch_bounds__(128) k_fwd_tc(const __grid_constant__ CUtensor
             }
         }
     }
-    const bool empty = (fl & HDT_BLK_EMPTY) != 0;
+    const bool empty = (fl & HDT_BLK_EMPTY) != 0 || ka >= kb;
     const bool dead = (*abort_flag != 0);   // same value in every thread: read after the barrier
 
     if (!empty && !dead) {
@@ -374,7 +383,8 @@ __global__ void __launch_bounds__(128) k_fwd_tc(const __grid_constant__ CUtensor
             if (warp == 0) tmem_dealloc(tmem, TM_COLS);
             return;
         }
-        float *own = inb ? a.own_o + ((size_t)row * H + h) * D : nullptr;
+        const size_t zrow = (size_t)blockIdx.z * a.split_rows + row;
+        float *own = inb ? a.own_o + (zrow * H + h) * D : nullptr;
 #pragma unroll
         for (int k = 0; k < D / 32; ++k) {
             uint32_t r[32];
@@ -397,7 +407,7 @@ __global__ void __launch_bounds__(128) k_fwd_tc(const __grid_constant__ CUtensor
                 }
             }
         }
-        if (inb) a.own_lse[(size_t)row * H + h] = lse;
+        if (inb) a.own_lse[zrow * H + h] = lse;
         tc_fence_before();
         __syncthreads();
         if (warp == 0) tmem_dealloc(tmem, TM_COLS);
@@ -1541,7 +1551,7 @@ static int launch_fwd_tc_upper_t(const FwdStageArgs &a, cudaStream_t st) {
         }
         k_fwd_tc<D, true, true><<<dim3(a.nb, a.H), 128, smem_1, st>>>(tq, tq, tq, b);
     } else
-        k_fwd_tc<D, false, true><<<dim3(a.nb, a.H), 128, smem, st>>>(tq, tq, tq, b);
+        k_fwd_tc<D, false, true><<<dim3(a.nb, a.H, a.splits > 1 ? a.splits : 1), 128, smem, st>>>(tq, tq, tq, b);
     count_launch();
     HDT_CUDA_CHECK(cudaGetLastError());
     return HDT_OK;

@@ -147,10 +147,30 @@ __global__ void __launch_bounds__(256) k_bwd_tc(const __grid_constant__ CUtensor
 
     const int tid = threadIdx.x, warp = tid >> 5, rl = tid & 127, hf = tid >> 7;
     // rest_only: take the blocks after the first n_fused entries of queue_split
-    const int blk = a.rest_only ? a.queue_split[a.n_fused + blockIdx.x] : a.queue[blockIdx.x];
+    int qi = blockIdx.x, split = 0;
+    if (GATHER && a.phase_split > 0 && a.splits > 1) {      // (the phase-1 blocks come first, `splits` CTAs each)
+        const int n1 = a.phase_split * a.splits;
+        if (qi < n1) { split = qi % a.splits; qi /= a.splits; }
+        else qi -= n1 - a.phase_split;
+    }
+    const int blk = a.rest_only ? a.queue_split[a.n_fused + qi] : a.queue[qi];
     const int h = blockIdx.y, H = a.H;
     const int *rec = a.blocks + 5 * (size_t)blk;
-    const int r0 = rec[0], r1 = rec[1], ka = rec[2], kb = rec[3], fl = rec[4];
+    const int r0 = rec[0], r1 = rec[1], fl = rec[4];
+    int ka = rec[2], kb = rec[3];
+    int phases = a.phases, final_merge = a.final_merge;
+    if constexpr (GATHER) {
+        if (r1 <= r0) return;               // a block slot that is not in use
+        if (a.phase_split > 0) {
+            phases = qi < a.phase_split ? 1 : 2;
+            if (phases == 1 && a.splits > 1) {      // this CTA's share of the key span, whole tiles
+                final_merge = 0;
+                const int per = ((kb - ka + 127) / 128 + a.splits - 1) / a.splits * 128;
+                ka += split * per;
+                kb = min(kb, ka + per);
+            }
+        }
+    }
     const int nrows = r1 - r0;
     const float LOG2E = 1.4426950408889634f;
 
@@ -167,7 +187,7 @@ __global__ void __launch_bounds__(256) k_bwd_tc(const __grid_constant__ CUtensor
     const uint32_t tmem = *slot;
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
     const bool dead = (*abort_flag != 0);
-    const bool empty = (fl & HDT_BLK_EMPTY) != 0;
+    const bool empty = (fl & HDT_BLK_EMPTY) != 0 || ka >= kb;
     const bool self = (fl & HDT_BLK_SELF) != 0;
     const bool fused = self && !empty && !dead;   // one pass yields dQ, dK and dV
     const uint32_t TM_DK = (D == 64) ? 320u : (fused ? 128u : 256u);
@@ -422,9 +442,9 @@ __global__ void __launch_bounds__(256) k_bwd_tc(const __grid_constant__ CUtensor
     const bool inb = row < r1;
     float *cq = nullptr, *ck = nullptr, *cv = nullptr;
     if constexpr (GATHER) {
-        if (inb && !a.final_merge) {      // the drains write the own gradients here; the staged bf16 copies are not used
-            if (a.phases != 2) cq = a.own_dq + ((size_t)row * H + h) * D;
-            if (a.phases != 1) {
+        if (inb && !final_merge) {      // the drains write the own gradients here; the staged bf16 copies are not used
+            if (phases != 2) cq = a.own_dq + (((size_t)split * a.split_rows + row) * H + h) * D;
+            if (phases != 1) {
                 ck = a.own_dk + ((size_t)row * H + h) * D;
                 cv = a.own_dv + ((size_t)row * H + h) * D;
             }
@@ -439,17 +459,17 @@ __global__ void __launch_bounds__(256) k_bwd_tc(const __grid_constant__ CUtensor
     }
 
     // final_merge: where this row's three gradients go and what is added to them
-    const bool fin = GATHER && a.final_merge;
+    const bool fin = GATHER && final_merge != 0;
     const float *fb[3] = {nullptr, nullptr, nullptr}, *fn[3] = {nullptr, nullptr, nullptr};
     __nv_bfloat16 *fo[3] = {nullptr, nullptr, nullptr};
     if constexpr (GATHER) {
         if (fin && inb) {
             const size_t tk = (size_t)a.tok[row];
             const size_t ob = ((size_t)row * H + h) * D;
-            if (a.final_merge == 1) { fb[0] = a.carry_dq + ob; fb[1] = a.carry_dk + ob; fb[2] = a.carry_dv + ob; }
+            if (final_merge == 1) { fb[0] = a.carry_dq + ob; fb[1] = a.carry_dk + ob; fb[2] = a.carry_dv + ob; }
             // (final_merge = 2: nothing to add; a launch that walks one side only writes that side's gradients only)
-            if (a.final_merge == 1 || a.phases != 2) fo[0] = reinterpret_cast<__nv_bfloat16 *>(a.dq) + (tk * H + h) * D;
-            if (a.final_merge == 1 || a.phases != 1) {
+            if (final_merge == 1 || phases != 2) fo[0] = reinterpret_cast<__nv_bfloat16 *>(a.dq) + (tk * H + h) * D;
+            if (final_merge == 1 || phases != 1) {
                 fo[1] = reinterpret_cast<__nv_bfloat16 *>(a.dk) + (tk * H + h) * D;
                 fo[2] = reinterpret_cast<__nv_bfloat16 *>(a.dv) + (tk * H + h) * D;
             }
@@ -477,7 +497,7 @@ __global__ void __launch_bounds__(256) k_bwd_tc(const __grid_constant__ CUtensor
             drain(TM_DV, true, 1.f, cv, sQ);
         }
     } else {
-        if (run && (!GATHER || a.phases != 2)) {
+        if (run && (!GATHER || phases != 2)) {
             // this block as query rows: dQ over the key span
             load(true, r0, false, 0);
             for (int c0 = ka; c0 < kb; c0 += 128) {
@@ -493,7 +513,7 @@ __global__ void __launch_bounds__(256) k_bwd_tc(const __grid_constant__ CUtensor
         tc_fence_after();
         if constexpr (!GATHER) copy_out(sP, a.dq);
         __syncthreads();
-        if (run && (!GATHER || a.phases != 1)) {
+        if (run && (!GATHER || phases != 1)) {
             // this block as keys: dK, dV over the same span taken as query rows
             load(false, 0, true, r0);
             for (int c0 = ka; c0 < kb; c0 += 128) {
@@ -1430,7 +1450,7 @@ static int launch_bwd_tc_upper_t(const BwdStageArgs &a, cudaStream_t st) {
     BwdStageArgs b = a;
     b.rest_only = 0;
     if (a.dirs != 7) k_bwd_tc<D, true, true><<<dim3(a.nb, a.H), 256, smem, st>>>(tq, tq, tq, tq, b);      // direction bits
-    else k_bwd_tc<D, true><<<dim3(a.nb, a.H), 256, smem, st>>>(tq, tq, tq, tq, b);
+    else k_bwd_tc<D, true><<<dim3(a.nb + (a.splits > 1 ? (a.splits - 1) * a.phase_split : 0), a.H), 256, smem, st>>>(tq, tq, tq, tq, b);
     count_launch();
     HDT_CUDA_CHECK(cudaGetLastError());
     return HDT_OK;

@@ -4,36 +4,57 @@
 // Encoder and Decoder Stacks").  Within the chosen subset it is plain softmax attention between
 // the decoder rows of a document and the chosen encoder rows of the same document.
 //
-// The chosen rows are never copied.  Every call builds (count, scan, fill: three small kernels,
-// 32 CTAs per document, no host wait) one element space for both sides: elements 0 .. Tq-1 are
-// the decoder rows (token map = identity, into Q / dO / O), elements Tq .. Tq+ns-1 the chosen
-// encoder tokens in order (token map = their index, into K / V); a decoder row's key range is its
-// document's slice of the second part, a chosen token's range the document's decoder rows.  The
-// attention kernels of the hierarchical path take any (row blocks, per-row range, token map)
-// description, so they serve as they are:
+// The chosen rows are never copied.
+//   few decoder rows a document (a step of autoregressive decoding): k_cross_decode reads levels, K and V once, the
+//         tokens of a document dealt to many CTAs, and k_cross_combine merges their partial results.  No index.
+//   otherwise one kernel (k_cross_index) builds one element space for both sides: elements 0 .. Tq-1 are
+//         the decoder rows (token map = identity, into Q / dO / O), elements Tq .. Tq+ns-1 the chosen
+//         encoder tokens in order (token map = their index, into K / V); a decoder row's key range is its
+//         document's slice of the second part, a chosen token's range the document's decoder rows.  The
+//         attention kernels of the hierarchical path take any (row blocks, per-row range, token map)
+//         description, so they serve as they are:
 //   bf16  the gathering tcgen05 kernels (128-row blocks): forward over the decoder-row blocks;
-//         backward once over the decoder-row blocks (dQ) and once over the blocks of chosen
+//         backward in one launch over the decoder-row blocks (dQ) and the blocks of chosen
 //         tokens (dK, dV); their epilogues round to bf16 and write each element's rows at its token in
-//         the caller's tensors (no fp32 buffers, no convert pass);
+//         the caller's tensors.  Long key lists are split over CTAs, whose fp32 partial results
+//         k_cross_combine merges;
 //   fp32  the SIMT kernels (32-row blocks), which write the caller's tensors directly.
-// Encoder rows outside the subset get zero dK, dV (cleared first).  Block slots are assigned
-// without a scan: document b owns the slots from start / rows_per_block + b on, unused slots stay
+// Encoder rows outside the subset get zero dK, dV from a kernel of their own beside the others.  Block slots are
+// assigned without a scan: document b owns the slots from start / rows_per_block + b on, unused slots stay
 // empty (r0 == r1).
 #include <cuda_bf16.h>
 
 #include "hdt_internal.cuh"
+#include "hdt_rows.cuh"
 
 namespace hdt {
 
-constexpr int XC = 32;      // CTAs (contiguous chunks) per document in the selection kernels
+constexpr int XC = 32;      // CTAs (contiguous chunks) per document in the index kernel
 
 struct CrossLayout {
-    size_t cnt, cntc, cu_sel, tokx, rngx, blocks_q, blocks_k, queue, delta, total;
+    size_t tokx, rngx, blocks, queue, delta, part, part_lse, total;
     int nbq, nbk, xr;
-    size_t zero_bytes;      // cnt .. tokx is cleared at the start of every call
 };
 
 static size_t al256c(size_t v) { return (v + 255) & ~size_t(255); }
+
+// Decoding: few decoder rows a document on average.  At 16 rows the 128-row tile of the other path is an eighth
+// full and the two cost the same per document.
+static bool cross_decode(int B, int Tq) { return (long long)Tq <= 4LL * B; }
+// CTAs a document's tokens are dealt to in the decode kernel: four per SM over all documents, 32 tokens each at least.
+static int decode_splits(int B, int T) {
+    const long long mean = B > 0 ? (T + B - 1) / B : 0;
+    return (int)max(1LL, min((mean + 31) / 32, (148LL * 4 + B - 1) / max(B, 1)));
+}
+// CTAs a row block's keys are dealt to in the tile kernels: enough to fill the SMs (`per_sm` CTAs each), pieces of
+// four chunks at least.  level_mask < 0: every level (for the workspace size).  Without the token level the keys are
+// the anchors, some thirtieth of the tokens.
+static int tile_splits(int B, int T, int Tq, int H, int level_mask, int per_sm) {
+    if (B <= 0 || Tq <= 0) return 1;
+    const long long mean = (T + B - 1) / B, keys = (level_mask < 0 || (level_mask >> 3)) ? mean : mean / 16;
+    const long long ctas = (long long)B * ((Tq + 128LL * B - 1) / (128LL * B)) * H;
+    return (int)max(1LL, min((keys + 511) / 512, (148LL * per_sm + ctas - 1) / ctas));
+}
 
 // tc: bf16 on the tensor-core kernels (128-row blocks)
 static CrossLayout cross_layout(int B, int T, int Tq, int H, int D, bool tc, int bwd) {
@@ -43,106 +64,83 @@ static CrossLayout cross_layout(int B, int T, int Tq, int H, int D, bool tc, int
     L.nbk = T / L.xr + B + 1;
     const size_t n = (size_t)Tq + T;
     size_t o = 0;
-    L.cnt = o; o += al256c(sizeof(int) * (size_t)(B + 1));
-    L.cntc = o; o += al256c(sizeof(int) * (size_t)(B + 1) * XC);
-    L.cu_sel = o; o += al256c(sizeof(int) * (size_t)(B + 2));
-    L.blocks_q = o; o += al256c(sizeof(int) * 5 * (size_t)L.nbq);
-    L.blocks_k = o; o += al256c(sizeof(int) * 5 * (size_t)L.nbk);
+    L.blocks = o; o += al256c(sizeof(int) * 5 * (size_t)(L.nbq + L.nbk));       // blocks of the decoder rows, then of the chosen tokens
     L.tokx = o; o += al256c(sizeof(int) * max(n, (size_t)1));
-    L.zero_bytes = o;
     L.rngx = o; o += al256c(sizeof(int) * 2 * max(n, (size_t)1));
-    L.queue = o; o += al256c(sizeof(int) * (size_t)max(L.nbq, L.nbk));
+    L.queue = o; o += al256c(sizeof(int) * (size_t)(L.nbq + L.nbk));
     L.delta = o; if (bwd) o += al256c(sizeof(float) * (size_t)H * max(Tq, 1));
+    // partial results [splits, Tq, H, D] and, in the forward, their LSE
+    const size_t splits = !bwd && cross_decode(B, Tq) ? decode_splits(B, T) : tile_splits(B, T, Tq, H, -1, bwd ? 8 : 2);
+    L.part = o; o += al256c(sizeof(float) * splits * Tq * H * D);
+    L.part_lse = o; if (!bwd) o += al256c(sizeof(float) * splits * Tq * H);
     L.total = o + 256;
     return L;
 }
 
-__device__ __forceinline__ int chosen(const int8_t *level, int i, int level_mask) {
-    const int lv = level[i];
-    return (lv >= 0 && lv < 31 && ((level_mask >> lv) & 1)) ? 1 : 0;
-}
+__device__ __forceinline__ int chosen_level(int lv, int level_mask) { return (lv >= 0 && lv < 31 && ((level_mask >> lv) & 1)) ? 1 : 0; }
+__device__ __forceinline__ int chosen(const int8_t *level, int i, int level_mask) { return chosen_level(level[i], level_mask); }
 
-// cnt[b] = chosen tokens of document b; cntc[b][y] = those in its y-th chunk (XC equal chunks)
-__global__ void k_cross_count(const int8_t *__restrict__ level, const int32_t *__restrict__ cu_k, int level_mask,
-                              int *cnt, int *cntc) {
-    __shared__ int s_c;
-    const int b = blockIdx.x, y = blockIdx.y;
-    const int k0 = cu_k[b], k1 = cu_k[b + 1], cs = (k1 - k0 + XC - 1) / XC;
-    const int c0 = k0 + y * cs, c1 = min(k1, c0 + cs);
-    if (threadIdx.x == 0) s_c = 0;
-    __syncthreads();
-    int c = 0;
-    for (int i = c0 + threadIdx.x; i < c1; i += blockDim.x) c += chosen(level, i, level_mask);
-    for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-    if ((threadIdx.x & 31) == 0 && c) atomicAdd(&s_c, c);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        cntc[b * XC + y] = s_c;
-        if (s_c) atomicAdd(&cnt[b], s_c);
-    }
-}
+struct CrossIndexArgs {
+    const int8_t *level;
+    const int32_t *cu_k, *cu_q;
+    int B, T, Tq, level_mask, xr, nbq, nbk;
+    int *tokx, *rngx, *blocks, *queue;
+};
 
-// cu_sel = exclusive scan of cnt (one CTA); queue = identity
-__global__ void __launch_bounds__(1024) k_cross_scan(const int *__restrict__ cnt, int B, int *cu_sel, int *queue, int nq) {
-    __shared__ int s_w[32];
-    __shared__ int s_carry;
-    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    if (t == 0) s_carry = 0;
-    __syncthreads();
-    for (int base = 0; base < B; base += 1024) {
-        const int b = base + t;
-        const int c = (b < B) ? cnt[b] : 0;
-        int v = c;
-        for (int o = 1; o < 32; o <<= 1) { const int x = __shfl_up_sync(0xffffffffu, v, o); if (lane >= o) v += x; }
-        if (lane == 31) s_w[w] = v;
-        __syncthreads();
-        if (w == 0) {
-            int x = s_w[lane];
-            for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(0xffffffffu, x, o); if (lane >= o) x += y; }
-            s_w[lane] = x;
-        }
-        __syncthreads();
-        if (b < B) cu_sel[b] = s_carry + (w ? s_w[w - 1] : 0) + v - c;
-        __syncthreads();
-        if (t == 0) s_carry += s_w[31];
-        __syncthreads();
-    }
-    if (t == 0) cu_sel[B] = s_carry;
-    for (int i = t; i < nq; i += 1024) queue[i] = i;
-}
-
-// Chunk y of document b: its part of the ordered list of chosen tokens (elements KO + position, with
-// their row ranges) and its share of the document's decoder rows (elements = row numbers: token
-// map, key range) and of the block records of both sides.  xr = rows per block.
-__global__ void __launch_bounds__(256) k_cross_fill(const int8_t *__restrict__ level, const int32_t *__restrict__ cu_k,
-                                                    const int32_t *__restrict__ cu_q, int level_mask,
-                                                    const int *__restrict__ cu_sel, const int *__restrict__ cntc, int KO,
-                                                    int xr, int *tokx, int *rngx, int *blocks_q, int *blocks_k) {
-    __shared__ int s_w[8];
+// Chunk y of document b: its part of the ordered list of chosen tokens (elements Tq + position, with their row
+// ranges) and its share of the document's decoder rows and of the block records of both sides.  Where
+// its part starts is counted over the levels of all tokens before it by the CTA itself: a byte a token, read by
+// every CTA, costs less than the launches of a count and a scan kernel (four launches with a clear, 14 us of every call).
+__global__ void __launch_bounds__(256) k_cross_index(const CrossIndexArgs a) {
+    pdl_launch_dependents();
+    __shared__ int s_w[8], s_n[4];
     __shared__ int s_carry;
     const int b = blockIdx.x, y = blockIdx.y, t = threadIdx.x, lane = t & 31, w = t >> 5;
-    const int k0 = cu_k[b], k1 = cu_k[b + 1], q0 = cu_q[b], q1 = cu_q[b + 1], s0 = cu_sel[b], s1 = cu_sel[b + 1];
-    const int cs = (k1 - k0 + XC - 1) / XC, c0 = k0 + y * cs, c1 = min(k1, c0 + cs);
-    if (w == 0) {       // chosen tokens of the chunks before this one
-        int v = (lane < y) ? cntc[b * XC + lane] : 0;       // XC == 32: one lane per chunk
-        for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) s_carry = v;
+    const int8_t *level = a.level;
+    const int KO = a.Tq, xr = a.xr, mask = a.level_mask;
+    const int k0 = a.cu_k[b], k1 = a.cu_k[b + 1], q0 = a.cu_q[b], q1 = a.cu_q[b + 1];
+    const int cs = (k1 - k0 + XC - 1) / XC, c0 = min(k1, k0 + y * cs), c1 = min(k1, c0 + cs);
+    if (t < 4) s_n[t] = 0;
+    __syncthreads();
+    {   // chosen tokens below k0, c0, k1 and in all
+        int n0 = 0, n1 = 0, n2 = 0, n3 = 0;
+        const bool vec = ((uintptr_t)level & 15) == 0;
+        const int units = vec ? a.T / 16 : 0;
+        for (int u = t; u < units; u += 256) {
+            const uint4 x = reinterpret_cast<const uint4 *>(level)[u];
+            const uint32_t xs[4] = {x.x, x.y, x.z, x.w};
+            const int i0 = 16 * u;
+            unsigned bits = 0;
+#pragma unroll
+            for (int j = 0; j < 16; ++j) bits |= (unsigned)chosen_level((int8_t)(xs[j >> 2] >> (8 * (j & 3))), mask) << j;
+            auto below = [&](int lim) { const int d = lim - i0; return d <= 0 ? 0 : __popc(d >= 16 ? bits : bits & ((1u << d) - 1u)); };
+            n0 += below(k0); n1 += below(c0); n2 += below(k1); n3 += __popc(bits);
+        }
+        for (int i = units * 16 + t; i < a.T; i += 256) {
+            const int f = chosen(level, i, mask);
+            n0 += f & (i < k0); n1 += f & (i < c0); n2 += f & (i < k1); n3 += f;
+        }
+        n0 = __reduce_add_sync(0xffffffffu, n0); n1 = __reduce_add_sync(0xffffffffu, n1);
+        n2 = __reduce_add_sync(0xffffffffu, n2); n3 = __reduce_add_sync(0xffffffffu, n3);
+        if (lane == 0) { atomicAdd(&s_n[0], n0); atomicAdd(&s_n[1], n1); atomicAdd(&s_n[2], n2); atomicAdd(&s_n[3], n3); }
     }
+    __syncthreads();
+    const int s0 = s_n[0], s1 = s_n[2], total = s_n[3];
+    if (t == 0) s_carry = s_n[1];
     __syncthreads();
     for (int base = c0; base < c1; base += 256) {
         const int i = base + t;
-        const int f = (i < c1) ? chosen(level, i, level_mask) : 0;
-        int v = f;
-        for (int o = 1; o < 32; o <<= 1) { const int x = __shfl_up_sync(0xffffffffu, v, o); if (lane >= o) v += x; }
-        if (lane == 31) s_w[w] = v;
+        const int f = (i < c1) ? chosen(level, i, mask) : 0;
+        const unsigned m = __ballot_sync(0xffffffffu, f);
+        if (lane == 0) s_w[w] = __popc(m);
         __syncthreads();
         int before = s_carry;
         for (int j = 0; j < w; ++j) before += s_w[j];
         if (f) {
-            const int e = KO + s0 + before + v - 1;
-            tokx[e] = i;
-            rngx[2 * e] = q0;
-            rngx[2 * e + 1] = q1;
+            const int e = KO + before + __popc(m & ((1u << lane) - 1u));
+            a.tokx[e] = i;
+            a.rngx[2 * e] = q0;
+            a.rngx[2 * e + 1] = q1;
         }
         __syncthreads();
         if (t == 0) { int tot = 0; for (int j = 0; j < 8; ++j) tot += s_w[j]; s_carry += tot; }
@@ -150,35 +148,235 @@ __global__ void __launch_bounds__(256) k_cross_fill(const int8_t *__restrict__ l
     }
     // decoder rows and block records: spread over the document's chunks
     const int nt = XC * 256, gt = y * 256 + t;
-    for (int r = q0 + gt; r < q1; r += nt) { tokx[r] = r; rngx[2 * r] = KO + s0; rngx[2 * r + 1] = KO + s1; }
+    for (int r = q0 + gt; r < q1; r += nt) { a.tokx[r] = r; a.rngx[2 * r] = KO + s0; a.rngx[2 * r + 1] = KO + s1; }
     const int live = (s1 > s0 && q1 > q0) ? 0 : HDT_BLK_EMPTY;
-    const int slot_q = q0 / xr + b, nbq = (q1 - q0 + xr - 1) / xr;
-    for (int j = gt; j < nbq; j += nt) {
-        int *rec = blocks_q + 5 * (size_t)(slot_q + j);
-        rec[0] = q0 + j * xr; rec[1] = min(q1, q0 + (j + 1) * xr); rec[2] = KO + s0; rec[3] = KO + s1; rec[4] = live;
-    }
-    const int slot_k = s0 / xr + b, nbk = (s1 - s0 + xr - 1) / xr;
-    for (int j = gt; j < nbk; j += nt) {
-        int *rec = blocks_k + 5 * (size_t)(slot_k + j);
-        rec[0] = KO + s0 + j * xr; rec[1] = KO + min(s1, s0 + (j + 1) * xr); rec[2] = q0; rec[3] = q1; rec[4] = live;
+    const bool last = b == a.B - 1;
+    auto put = [&](int slot, int next, int x0, int x1, int off, int ka, int kb) {      // slots [slot, next): this document's
+        for (int j = gt; j < next - slot; j += nt) {
+            int *rec = a.blocks + 5 * (size_t)(slot + j);
+            const int r0 = min(x1, x0 + j * xr);
+            rec[0] = off + r0; rec[1] = off + min(x1, r0 + xr); rec[2] = ka; rec[3] = kb; rec[4] = live;
+        }
+    };
+    put(q0 / xr + b, last ? a.nbq : q1 / xr + b + 1, q0, q1, 0, KO + s0, KO + s1);
+    put(a.nbq + s0 / xr + b, a.nbq + (last ? a.nbk : s1 / xr + b + 1), s0, s1, KO, q0, q1);
+    // tiles of the gathering kernels reach past the elements in use: element 0 is a valid row of every tensor
+    const int all = a.B * nt, ga = b * nt + gt;
+    for (int e = KO + total + ga; e < KO + a.T; e += all) a.tokx[e] = 0;
+    for (int i = ga; i < a.nbq + a.nbk; i += all) a.queue[i] = i;
+}
+
+// Zero dK, dV rows of the encoder tokens that no decoder row attends to.  n16: 16-byte pieces of a token's row.
+__global__ void __launch_bounds__(256) k_cross_zero(const int8_t *__restrict__ level, const int32_t *__restrict__ cu_k, const int32_t *__restrict__ cu_q, int B,
+                                                    int T, int level_mask, int n16, uint4 *dk, uint4 *dv) {
+    const int per = 256 / 32, lane = threadIdx.x & 31;
+    for (int i = blockIdx.x * per + (threadIdx.x >> 5); i < T; i += gridDim.x * per) {
+        if (chosen(level, i, level_mask)) {
+            int lo = 0, hi = B;          // its document: the last b with cu_k[b] <= i
+            while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (cu_k[mid] <= i) lo = mid; else hi = mid; }
+            if (cu_q[lo + 1] > cu_q[lo]) continue;
+        }
+        for (int j = lane; j < n16; j += 32) {
+            dk[(size_t)i * n16 + j] = make_uint4(0, 0, 0, 0);
+            dv[(size_t)i * n16 + j] = make_uint4(0, 0, 0, 0);
+        }
     }
 }
 
-static int cross_build(const CrossLayout &L, char *ws, const int8_t *level, const int32_t *cu_k, const int32_t *cu_q,
-                       int B, int Tq, int level_mask, cudaStream_t st) {
-    // the token map is cleared as a whole: tiles of the gathering kernels reach past the elements
-    // in use, and element 0 is a valid row of every tensor
-    HDT_CUDA_CHECK(cudaMemsetAsync(ws, 0, L.zero_bytes, st));
-    if (B > 0) {
-        static_assert(XC == 32, "k_cross_fill sums the chunk counts with one lane per chunk");
-        k_cross_count<<<dim3(B, XC), 256, 0, st>>>(level, cu_k, level_mask, (int *)(ws + L.cnt), (int *)(ws + L.cntc));
-        k_cross_scan<<<1, 1024, 0, st>>>((const int *)(ws + L.cnt), B, (int *)(ws + L.cu_sel), (int *)(ws + L.queue),
-                                         max(L.nbq, L.nbk));
-        k_cross_fill<<<dim3(B, XC), 256, 0, st>>>(level, cu_k, cu_q, level_mask, (const int *)(ws + L.cu_sel),
-                                                  (const int *)(ws + L.cntc), Tq, L.xr, (int *)(ws + L.tokx),
-                                                  (int *)(ws + L.rngx), (int *)(ws + L.blocks_q), (int *)(ws + L.blocks_k));
-        count_launch(3);
+// ---- decoding ------------------------------------------------------------------------------------
+// CTA (y, b, z): the y-th share of document b's tokens, heads z * HC ..., every decoder row of the document in
+// turn.  Thread (slot, head, lane): D / 8 lanes per (key, head), the heads of a token next to one another, so that a
+// CTA reads whole token rows.  The bound is reading K and V once (4 x 8192 tokens, 12 x 64: 101 MB, 15 us at the
+// copy rate): four keys a thread in flight and four CTAs an SM; the tile kernel took 352 us here, one CTA per
+// document and head walking 64 chunks with one row of 128 in use.
+struct DecodeArgs {
+    const int8_t *level;
+    const int32_t *cu_k, *cu_q;
+    int level_mask, H, HC, KS, Tq, splits;
+    const void *q, *k, *v;
+    float scale_log2;
+    void *o;
+    float *lse, *part_o, *part_lse;       // splits > 1: [splits, Tq, H, D], [splits, Tq, H]
+};
+static constexpr int DEC_LIST = 1024;
+
+template <int D, bool BF16>
+__global__ void __launch_bounds__(512, 2) k_cross_decode(const DecodeArgs a) {
+    pdl_launch_dependents();
+    constexpr int LPK = D / 8, C = 4;
+    using W = Raw<BF16, LPK>;
+    extern __shared__ float s_red[];                 // [KS][HC][D + 2]
+    __shared__ int s_list[DEC_LIST];
+    __shared__ int s_n;
+    const int b = blockIdx.y, t = threadIdx.x, lane = t & 31, g = t % LPK, src = lane - g;
+    const unsigned mask = ((1u << LPK) - 1u) << src;
+    const int pair = t / LPK, hl = pair % a.HC, ks = pair / a.HC, h = blockIdx.z * a.HC + hl;
+    const bool on = ks < a.KS && h < a.H;
+    const int k0 = a.cu_k[b], k1 = a.cu_k[b + 1], q0 = a.cu_q[b], q1 = a.cu_q[b + 1];
+    const int per = (k1 - k0 + a.splits - 1) / a.splits, c0 = min(k1, k0 + (int)blockIdx.x * per), c1 = min(k1, c0 + per);
+    for (int row = q0; row < q1; ++row) {
+        RowSoftmax S;
+        S.clear();
+        W q;
+        if (on) q.load(a.q, (unsigned)row * a.H + h, g);
+        for (int p0 = c0; p0 < c1; p0 += DEC_LIST) {
+            const int p1 = min(c1, p0 + DEC_LIST);
+            if (row == q0 || c1 - c0 > DEC_LIST) {           // the chosen tokens of this piece, in order
+                __syncthreads();
+                if (t < 32) {
+                    int n = 0;
+                    for (int i0 = p0; i0 < p1; i0 += 32) {
+                        const bool f = i0 + lane < p1 && chosen(a.level, i0 + lane, a.level_mask);
+                        const unsigned m = __ballot_sync(0xffffffffu, f);
+                        if (f) s_list[n + __popc(m & ((1u << lane) - 1u))] = i0 + lane;
+                        n += __popc(m);
+                    }
+                    if (lane == 0) s_n = n;
+                }
+                __syncthreads();
+            }
+            const int n = s_n;
+            if (!on) continue;
+            for (int i0 = ks * C; i0 < n; i0 += a.KS * C) {
+                W x[C], y[C];
+#pragma unroll
+                for (int c = 0; c < C; ++c) {
+                    const unsigned r = (unsigned)s_list[min(i0 + c, n - 1)] * a.H + h;      // (past the end: the last key, weight 0)
+                    x[c].load(a.k, r, g);
+                    y[c].load(a.v, r, g);
+                }
+                float sc[C];
+                dots<C>(q, x, sc);
+                const float s = reduce_scatter<C, LPK>(sc, g, mask) * a.scale_log2;
+                const float p = S.add<C>(i0 + (g & (C - 1)) < n ? s : -INFINITY, mask);
+                axpys<C>(S.acc, p, y, mask, src);
+            }
+        }
+        // the slots of a head: one after the other through shared memory
+        if (on) {
+#pragma unroll
+            for (int o = 1; o < C; o *= 2) S.l += __shfl_xor_sync(mask, S.l, o);
+            float *d = s_red + (size_t)(ks * a.HC + hl) * (D + 2);
+            const float lse = S.finish();
+#pragma unroll
+            for (int u = 0; u < 4; ++u) unpack2(S.acc[u], d[8 * g + 2 * u], d[8 * g + 2 * u + 1]);
+            if (g == 0) d[D] = lse;
+        }
+        __syncthreads();
+        if (on && ks == 0) {
+            RowSoftmax R;
+            R.clear();
+            for (int i = 0; i < a.KS; ++i) {
+                const float *d = s_red + (size_t)(i * a.HC + hl) * (D + 2);
+                f2 x[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) x[u] = pack2(d[8 * g + 2 * u], d[8 * g + 2 * u + 1]);
+                R.merge(d[D] * 1.4426950408889634f, d[D] > -INFINITY ? 1.f : 0.f, x);
+            }
+            const float lse = R.finish();
+            if (a.splits == 1) {
+                W::store(a.o, (unsigned)row * a.H + h, g, R.acc);
+                if (g == 0) a.lse[(size_t)h * a.Tq + row] = lse;
+            } else {
+                const size_t r = ((size_t)blockIdx.x * a.Tq + row) * a.H + h;
+                W::store_f32(a.part_o, r, g, R.acc);
+                if (g == 0) a.part_lse[r] = lse;
+            }
+        }
+        __syncthreads();
     }
+}
+
+// Merge of partial results over `splits`, a CTA per (row, head).  Forward (lse given): log-sum-exp merge of
+// normalised rows; backward: sum.
+template <int D, bool BF16>
+__global__ void __launch_bounds__(128) k_cross_combine(int splits, int Tq, int H, const float *part, const float *part_lse, void *out, float *lse) {
+    pdl_wait();
+    constexpr int LPK = D / 8, G = 128 / LPK;
+    using W = Raw<BF16, LPK>;
+    __shared__ float s_red[G][D + 2];
+    const int row = blockIdx.x, h = blockIdx.y, g = threadIdx.x % LPK, i = threadIdx.x / LPK;
+    RowSoftmax R;
+    R.clear();
+#pragma unroll 4
+    for (int s = i; s < splits; s += G) {
+        const size_t r = ((size_t)s * Tq + row) * H + h;
+        f2 x[4];
+        W::load_f32(part, r, g, x);
+        if (part_lse != nullptr) {
+            const float L = part_lse[r];
+            R.merge(L * 1.4426950408889634f, L > -INFINITY ? 1.f : 0.f, x);
+        } else {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) R.acc[u] = add2(R.acc[u], x[u]);
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) unpack2(R.acc[u], s_red[i][8 * g + 2 * u], s_red[i][8 * g + 2 * u + 1]);
+    if (g == 0) { s_red[i][D] = R.m; s_red[i][D + 1] = R.l; }
+    __syncthreads();
+    if (i != 0) return;
+    for (int j = 1; j < min(G, splits); ++j) {
+        f2 x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = pack2(s_red[j][8 * g + 2 * u], s_red[j][8 * g + 2 * u + 1]);
+        if (part_lse != nullptr) R.merge(s_red[j][D], s_red[j][D + 1], x);
+        else
+#pragma unroll
+            for (int u = 0; u < 4; ++u) R.acc[u] = add2(R.acc[u], x[u]);
+    }
+    if (part_lse != nullptr) {
+        const float L = R.finish();
+        if (g == 0) lse[(size_t)h * Tq + row] = L;
+    }
+    W::store(out, (unsigned)row * H + h, g, R.acc);
+}
+
+template <class... P, class... A>
+static cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = g_no_pdl ? 0 : 1;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    count_launch();
+    return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
+static int launch_combine(int splits, int Tq, int H, int D, int dtype, const float *part, const float *part_lse, void *out, float *lse, cudaStream_t st) {
+    const dim3 grid(Tq, H);
+    cudaError_t e;
+    if (D == 64) e = dtype == HDT_BF16 ? launch_dependent(k_cross_combine<64, true>, grid, 128, 0, st, splits, Tq, H, part, part_lse, out, lse)
+                                       : launch_dependent(k_cross_combine<64, false>, grid, 128, 0, st, splits, Tq, H, part, part_lse, out, lse);
+    else e = dtype == HDT_BF16 ? launch_dependent(k_cross_combine<128, true>, grid, 128, 0, st, splits, Tq, H, part, part_lse, out, lse)
+                               : launch_dependent(k_cross_combine<128, false>, grid, 128, 0, st, splits, Tq, H, part, part_lse, out, lse);
+    if (e != cudaSuccess) return set_error(HDT_ERR_CUDA, "launch of the combining kernel failed: %s", cudaGetErrorString(e));
+    return HDT_OK;
+}
+
+template <int D, bool BF16>
+static int launch_decode_t(DecodeArgs a, int B, cudaStream_t st) {
+    constexpr int LPK = D / 8;
+    a.HC = min(a.H, 512 / LPK);
+    a.KS = max(1, min(16, 384 / (a.HC * LPK)));
+    const int threads = (a.HC * LPK * a.KS + 31) / 32 * 32;
+    const size_t smem = sizeof(float) * (size_t)a.KS * a.HC * (D + 2);
+    k_cross_decode<D, BF16><<<dim3(a.splits, B, (a.H + a.HC - 1) / a.HC), threads, smem, st>>>(a);
+    count_launch();
+    HDT_CUDA_CHECK(cudaGetLastError());
+    return HDT_OK;
+}
+
+static int cross_build(const CrossLayout &L, char *ws, const int8_t *level, const int32_t *cu_k, const int32_t *cu_q, int B, int T, int Tq, int level_mask,
+                       cudaStream_t st) {
+    if (B <= 0) return HDT_OK;
+    CrossIndexArgs a{};
+    a.level = level; a.cu_k = cu_k; a.cu_q = cu_q; a.B = B; a.T = T; a.Tq = Tq; a.level_mask = level_mask;
+    a.xr = L.xr; a.nbq = L.nbq; a.nbk = L.nbk;
+    a.tokx = (int *)(ws + L.tokx); a.rngx = (int *)(ws + L.rngx); a.blocks = (int *)(ws + L.blocks); a.queue = (int *)(ws + L.queue);
+    k_cross_index<<<dim3(B, XC), 256, 0, st>>>(a);
+    count_launch();
     HDT_CUDA_CHECK(cudaGetLastError());
     return HDT_OK;
 }
@@ -220,26 +418,47 @@ extern "C" int hdt_cross_attn_fwd(const int8_t *level, const int32_t *cu_seqlens
     if (total_q == 0) return HDT_OK;
     if (!q || !o || !lse || (total_tokens > 0 && (!k || !v)))
         return set_error(HDT_ERR_INVALID_ARG, "hdt_cross_attn_fwd: null tensor pointer");
+    if (batch == 0) return HDT_OK;
     const bool tc = cross_tc(dtype);
     const CrossLayout L = cross_layout(batch, total_tokens, total_q, heads, head_dim, tc, 0);
     cudaStream_t st = (cudaStream_t)stream;
     char *ws = (char *)workspace;
-    rc = cross_build(L, ws, level, cu_seqlens_k, cu_seqlens_q, batch, total_q, level_mask, st);
-    if (rc) return rc;
     const float scale = softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf((float)head_dim);
+    float *part = (float *)(ws + L.part), *part_lse = (float *)(ws + L.part_lse);
+    if (cross_decode(batch, total_q) && !g_force_simt) {
+        DecodeArgs a{};
+        a.level = level; a.cu_k = cu_seqlens_k; a.cu_q = cu_seqlens_q; a.level_mask = level_mask; a.H = heads; a.Tq = total_q;
+        a.splits = decode_splits(batch, total_tokens);
+        a.q = q; a.k = k; a.v = v; a.scale_log2 = scale * 1.4426950408889634f;
+        a.o = o; a.lse = lse; a.part_o = part; a.part_lse = part_lse;
+        if (head_dim == 64) rc = dtype == HDT_BF16 ? launch_decode_t<64, true>(a, batch, st) : launch_decode_t<64, false>(a, batch, st);
+        else rc = dtype == HDT_BF16 ? launch_decode_t<128, true>(a, batch, st) : launch_decode_t<128, false>(a, batch, st);
+        if (rc || a.splits == 1) return rc;
+        return launch_combine(a.splits, total_q, heads, head_dim, dtype, part, part_lse, o, lse, st);
+    }
+    rc = cross_build(L, ws, level, cu_seqlens_k, cu_seqlens_q, batch, total_tokens, total_q, level_mask, st);
+    if (rc) return rc;
     FwdStageArgs a{};
     a.n = total_q + total_tokens; a.nb = L.nbq; a.H = heads; a.T = total_q;
     a.tok = (const int *)(ws + L.tokx);
     a.tok_rows = a.tok;
-    a.rng = (const int *)(ws + L.rngx); a.blocks = (const int *)(ws + L.blocks_q);
+    a.rng = (const int *)(ws + L.rngx); a.blocks = (const int *)(ws + L.blocks);
     a.queue = (const int *)(ws + L.queue); a.queue_split = a.queue;
     a.q = q; a.k = k; a.v = v; a.o = o; a.lse = lse;
     a.scale_log2 = scale * 1.4426950408889634f;
     a.status = device_status_ptr();
     a.block_rows = L.xr; a.dirs = 7;
     if (!tc) return launch_fwd_simt(a, head_dim, dtype, st);
-    a.final_merge = 2;       // the kernel's epilogue writes the bf16 rows and the LSE of the decoder rows itself
-    return launch_fwd_tc_upper(a, head_dim, st);
+    a.splits = tile_splits(batch, total_tokens, total_q, heads, level_mask, head_dim == 64 ? 2 : 1);
+    if (a.splits == 1) {
+        a.final_merge = 2;       // the kernel's epilogue writes the bf16 rows and the LSE of the decoder rows itself
+        return launch_fwd_tc_upper(a, head_dim, st);
+    }
+    a.split_rows = total_q;
+    a.own_o = part; a.own_lse = part_lse;
+    rc = launch_fwd_tc_upper(a, head_dim, st);
+    if (rc) return rc;
+    return launch_combine(a.splits, total_q, heads, head_dim, dtype, part, part_lse, o, lse, st);
 }
 
 extern "C" int hdt_cross_attn_bwd(const int8_t *level, const int32_t *cu_seqlens_k, const int32_t *cu_seqlens_q,
@@ -254,48 +473,74 @@ extern "C" int hdt_cross_attn_bwd(const int8_t *level, const int32_t *cu_seqlens
     if (rc) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     const size_t esz = dtype == HDT_BF16 ? 2 : 4;
-    if (total_tokens > 0) {
-        if (!dk || !dv) return set_error(HDT_ERR_INVALID_ARG, "hdt_cross_attn_bwd: null tensor pointer");
-        // encoder rows outside the subset (and of documents without decoder rows) get zero gradients
+    if (total_tokens > 0 && (!dk || !dv)) return set_error(HDT_ERR_INVALID_ARG, "hdt_cross_attn_bwd: null tensor pointer");
+    if (total_q > 0 && (!q || !o || !lse || !d_o || !dq || (total_tokens > 0 && (!k || !v))))
+        return set_error(HDT_ERR_INVALID_ARG, "hdt_cross_attn_bwd: null tensor pointer");
+    // Encoder rows outside the subset (and of documents without decoder rows) get zero gradients: writes of
+    // their own, beside the other kernels.
+    Side *sd = nullptr;
+    if (total_tokens > 0 && batch == 0) {
         HDT_CUDA_CHECK(cudaMemsetAsync(dk, 0, (size_t)total_tokens * heads * head_dim * esz, st));
         HDT_CUDA_CHECK(cudaMemsetAsync(dv, 0, (size_t)total_tokens * heads * head_dim * esz, st));
+    } else if (total_tokens > 0) {
+        cudaStream_t sz = st;
+        if (total_q > 0 && !g_no_overlap) {
+            rc = get_side(&sd);
+            if (rc) return rc;
+            HDT_CUDA_CHECK(cudaEventRecord(sd->fork, st));
+            HDT_CUDA_CHECK(cudaStreamWaitEvent(sd->s, sd->fork, 0));
+            sz = sd->s;
+        }
+        k_cross_zero<<<min((total_tokens + 7) / 8, 148 * 8), 256, 0, sz>>>(level, cu_seqlens_k, cu_seqlens_q, batch, total_tokens, level_mask,
+                                                                        (int)(heads * head_dim * esz / 16), (uint4 *)dk, (uint4 *)dv);
+        count_launch();
+        HDT_CUDA_CHECK(cudaGetLastError());
+        if (sd) HDT_CUDA_CHECK(cudaEventRecord(sd->join, sd->s));
     }
-    if (total_q == 0) return HDT_OK;
-    if (!q || !o || !lse || !d_o || !dq || (total_tokens > 0 && (!k || !v)))
-        return set_error(HDT_ERR_INVALID_ARG, "hdt_cross_attn_bwd: null tensor pointer");
-    const bool tc = cross_tc(dtype);
-    const CrossLayout L = cross_layout(batch, total_tokens, total_q, heads, head_dim, tc, 1);
-    char *ws = (char *)workspace;
-    rc = cross_build(L, ws, level, cu_seqlens_k, cu_seqlens_q, batch, total_q, level_mask, st);
-    if (rc) return rc;
-    float *delta = (float *)(ws + L.delta);
-    rc = launch_delta(o, d_o, delta, total_q, heads, head_dim, dtype, st);
-    if (rc) return rc;
-    const float scale = softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf((float)head_dim);
-    BwdStageArgs a{};
-    a.n = total_q + total_tokens; a.H = heads; a.T = total_q;
-    a.tok = (const int *)(ws + L.tokx); a.tok_rows = a.tok;
-    a.rng = (const int *)(ws + L.rngx);
-    a.queue = (const int *)(ws + L.queue); a.queue_split = a.queue;
-    a.q = q; a.k = k; a.v = v; a.d_o = d_o; a.lse = lse; a.delta = delta;
-    a.scale = scale; a.scale_log2 = scale * 1.4426950408889634f;
-    a.dq = dq; a.dk = dk; a.dv = dv;
-    a.status = device_status_ptr();
-    a.block_rows = L.xr; a.dirs = 7;
-    a.gather_end_q = total_q;                       // Q, dO have total_q rows
-    a.gather_end_k = total_q + total_tokens;
-    BwdStageArgs aq = a, ak = a;
-    aq.nb = L.nbq; aq.phases = 1; aq.blocks = (const int *)(ws + L.blocks_q);   // decoder rows as queries: dQ
-    ak.nb = L.nbk; ak.phases = 2; ak.blocks = (const int *)(ws + L.blocks_k);   // chosen tokens as keys: dK, dV
-    if (!tc) {
-        rc = launch_bwd_simt(aq, head_dim, dtype, st);
-        if (rc) return rc;
-        return launch_bwd_simt(ak, head_dim, dtype, st);
-    }
-    // the epilogues write bf16 rows at the element's token: dq from the first launch (decoder rows, token =
-    // row), dk and dv from the second (chosen tokens, token = their encoder row)
-    aq.final_merge = 2; ak.final_merge = 2;
-    rc = launch_bwd_tc_upper(aq, head_dim, st);
-    if (rc) return rc;
-    return launch_bwd_tc_upper(ak, head_dim, st);
+    if (total_q == 0 || batch == 0) return HDT_OK;
+    auto attend = [&]() -> int {
+        const bool tc = cross_tc(dtype);
+        const CrossLayout L = cross_layout(batch, total_tokens, total_q, heads, head_dim, tc, 1);
+        char *ws = (char *)workspace;
+        int r = cross_build(L, ws, level, cu_seqlens_k, cu_seqlens_q, batch, total_tokens, total_q, level_mask, st);
+        if (r) return r;
+        const float scale = softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf((float)head_dim);
+        BwdStageArgs a{};
+        a.n = total_q + total_tokens; a.H = heads; a.T = total_q;
+        a.tok = (const int *)(ws + L.tokx); a.tok_rows = a.tok;
+        a.rng = (const int *)(ws + L.rngx);
+        a.queue = (const int *)(ws + L.queue); a.queue_split = a.queue;
+        a.blocks = (const int *)(ws + L.blocks);
+        a.q = q; a.k = k; a.v = v; a.d_o = d_o; a.o = o; a.lse = lse;
+        a.scale = scale; a.scale_log2 = scale * 1.4426950408889634f;
+        a.dq = dq; a.dk = dk; a.dv = dv;
+        a.status = device_status_ptr();
+        a.block_rows = L.xr; a.dirs = 7;
+        if (!tc) {
+            float *delta = (float *)(ws + L.delta);
+            r = launch_delta(o, d_o, delta, total_q, heads, head_dim, dtype, st);
+            if (r) return r;
+            a.delta = delta;
+            BwdStageArgs aq = a, ak = a;
+            aq.nb = L.nbq; aq.phases = 1;                                            // decoder rows as queries: dQ
+            ak.nb = L.nbk; ak.phases = 2; ak.blocks = a.blocks + 5 * (size_t)L.nbq;   // chosen tokens as keys: dK, dV
+            r = launch_bwd_simt(aq, head_dim, dtype, st);
+            return r ? r : launch_bwd_simt(ak, head_dim, dtype, st);
+        }
+        // One launch over the blocks of both sides: the decoder rows' leave dq, the chosen tokens' dk and dv, as
+        // bf16 rows at the element's token (decoder rows: token = row).  dO . O comes from the rows as they are gathered.
+        a.gather_end_q = total_q;                       // Q, dO have total_q rows
+        a.gather_end_k = total_q + total_tokens;
+        a.nb = L.nbq + L.nbk; a.phase_split = L.nbq;
+        a.final_merge = 2;
+        a.splits = tile_splits(batch, total_tokens, total_q, heads, level_mask, 8);
+        a.split_rows = total_q;
+        a.own_dq = (float *)(ws + L.part);
+        r = launch_bwd_tc_upper(a, head_dim, st);
+        if (r || a.splits == 1) return r;
+        return launch_combine(a.splits, total_q, heads, head_dim, dtype, a.own_dq, nullptr, dq, nullptr, st);
+    };
+    rc = attend();
+    if (sd) HDT_CUDA_CHECK(cudaStreamWaitEvent(st, sd->join, 0));
+    return rc;
 }

@@ -199,6 +199,9 @@ struct FwdStageArgs {
     // bf16 rows and LSE straight to the element's token, no partial buffers.
     int final_merge;
     const float *next_own_o, *next_own_lse;
+    // Gathering kernel in own-partial mode: splits > 1 gives the key span of a block to that many CTAs (grid.z), each with
+    // a partial result of its own (own_o / own_lse hold splits x split_rows rows).
+    int splits, split_rows;
     const DevHeader *hdr; // set: the index build is still in flight; the looping kernel reads n_fused and stage 1's size here
     size_t ws_bytes;      // with hdr: bytes behind part_o (the caller's workspace)
     int n_empty;          // EMPTY blocks of the stage (0 where the caller does not know): when they are all that is left
@@ -239,6 +242,10 @@ struct BwdStageArgs {
     int n_empty;                                  // EMPTY blocks of the stage (-1: unknown)
     void *self_stream;                            // stage 0 with dq_acc: stream (cudaStream_t, already forked from the caller's) for the kernel of the
                                                   // self-contained blocks, which then runs beside the one-walk kernel of the others (nullptr: behind it)
+    // Gathering kernel: with phase_split > 0 the blocks before it take phase 1 and the others phase 2 (both sides of a
+    // cross-attention in one launch); splits > 1 gives a phase-1 block's key span to that many CTAs, each with
+    // a partial dQ of its own (own_dq holds splits x split_rows rows; phase 2 still writes the final rows).
+    int phase_split, splits, split_rows;
     int gather_end_q, gather_end_k;               // gathering kernel: elements at or beyond these read as zero rows on the Q/dO and the K/V side (0: n)
 };
 
