@@ -106,6 +106,8 @@ __global__ void __launch_bounds__(ROW_THREADS, KP == 1 && C == 4 && BF16 ? 8 : 4
     const int src = lane - g;                                                             // and of the group that shares a key
     const unsigned mask = ((1u << LPK) - 1u) << src;
     const unsigned long long id = ((unsigned long long)blockIdx.x * ROW_THREADS + threadIdx.x) / G;
+    pdl_launch_dependents();
+    if (a.first == 0) pdl_wait();     // (else: only what stage 0 leaves is waited for, behind the walk)
     if (id >= (unsigned long long)a.n * a.H) return;
     const int e = (int)(id / a.H), h = (int)(id % a.H);     // (the rows of a warp are heads of an element: one range, no divergence)
     const int t = a.first ? a.st[a.first].tok[e] : e;
@@ -127,6 +129,7 @@ __global__ void __launch_bounds__(ROW_THREADS, KP == 1 && C == 4 && BF16 ? 8 : 4
         S.merge(m2, l2, acc2);
     }
     if (kp != 0) return;
+    if (a.first != 0) pdl_wait();
     if (a.base_o != nullptr) {              // stage 0's partial result, normalised, as one more key
         f2 o0[4];
         R::load_f32(a.base_o, (size_t)e * a.H + h, g, o0);
@@ -245,6 +248,8 @@ __global__ void __launch_bounds__(ROW_THREADS, BF16 ? 4 : 3) k_bwd_rows(const Ro
     const int src = lane - g;                                                             // and of the group that shares a key
     const unsigned mask = ((1u << LPK) - 1u) << src;
     const unsigned long long id = ((unsigned long long)blockIdx.x * ROW_THREADS + threadIdx.x) / G;
+    pdl_launch_dependents();
+    if (a.first == 0) pdl_wait();     // (else: only what stage 0 leaves is waited for, behind the walk)
     if (id >= (unsigned long long)a.n * a.H) return;
     const int e = (int)(id / a.H), h = (int)(id % a.H);     // (the rows of a warp are heads of an element: one range, no divergence)
     const int t = a.first ? a.st[a.first].tok[e] : e;
@@ -261,6 +266,7 @@ __global__ void __launch_bounds__(ROW_THREADS, BF16 ? 4 : 3) k_bwd_rows(const Ro
         }
     }
     if (kp != 0) return;
+    if (a.first != 0) pdl_wait();
     S.scale(a.scale);
     if (a.base[0] != nullptr) {         // stage 0's partial gradients
         f2 y[4];
@@ -326,6 +332,8 @@ template <int D>
 __global__ void __launch_bounds__(TILE_THREADS, 3) k_fwd_tile(const TileFwdArgs a) {
     constexpr int LPK = D / 8, ROWS = TileShape<D>::ROWS, KT = TileShape<D>::KT, C = 4, U = D / 4;
     using R = Raw<false, LPK>;
+    pdl_wait();
+    pdl_launch_dependents();
     extern __shared__ float4 s_tile[];
     __shared__ int s_ab[2];
     float4 *sK = s_tile, *sV = sK + KT * U;
@@ -399,6 +407,8 @@ template <int D>
 __global__ void __launch_bounds__(TILE_THREADS, 2) k_bwd_tile(const TileBwdArgs a) {
     constexpr int LPK = D / 8, ROWS = TileShape<D>::ROWS, KT = TileShape<D>::KT, C = 2, U = D / 4;
     using R = Raw<false, LPK>;
+    pdl_wait();
+    pdl_launch_dependents();
     extern __shared__ float4 s_tile[];
     __shared__ int s_ab[2];
     __shared__ float s_lse[KT], s_delta[KT];
@@ -479,9 +489,7 @@ static int launch_fwd_tile_t(const TileFwdArgs &a, cudaStream_t st) {
         once.set();
     }
     constexpr int ROWS = TileShape<D>::ROWS;
-    k_fwd_tile<D><<<dim3(a.nb * ((a.block_rows + ROWS - 1) / ROWS), a.H), TILE_THREADS, smem, st>>>(a);
-    count_launch();
-    HDT_CUDA_CHECK(cudaGetLastError());
+    HDT_CUDA_CHECK(launch_dependent(k_fwd_tile<D>, true, dim3(a.nb * ((a.block_rows + ROWS - 1) / ROWS), a.H), TILE_THREADS, smem, st, a));
     return HDT_OK;
 }
 template <int D>
@@ -494,9 +502,7 @@ static int launch_bwd_tile_t(const TileBwdArgs &a, cudaStream_t st) {
         once.set();
     }
     constexpr int ROWS = TileShape<D>::ROWS;
-    k_bwd_tile<D><<<dim3(a.nb * ((a.block_rows + ROWS - 1) / ROWS), a.H), TILE_THREADS, smem, st>>>(a);
-    count_launch();
-    HDT_CUDA_CHECK(cudaGetLastError());
+    HDT_CUDA_CHECK(launch_dependent(k_bwd_tile<D>, true, dim3(a.nb * ((a.block_rows + ROWS - 1) / ROWS), a.H), TILE_THREADS, smem, st, a));
     return HDT_OK;
 }
 int launch_fwd_tile(const TileFwdArgs &a, int D, cudaStream_t st) {
@@ -529,12 +535,8 @@ static int launch_fwd_rows_t(const RowFwdArgs &a, cudaStream_t st) {
     if (rows == 0) return HDT_OK;
     const int kp = row_groups(rows, D, a.keys, a.first ? 8 : 4, BF16 ? 16 : 12);
     const unsigned grid = (unsigned)((rows * kp * (D / 8) + ROW_THREADS - 1) / ROW_THREADS);
-    if (kp == 4) k_fwd_rows<D, BF16, D == 64 ? 4 : 1, 8><<<grid, ROW_THREADS, 0, st>>>(a);
-    else if (kp == 2) k_fwd_rows<D, BF16, 2, 8><<<grid, ROW_THREADS, 0, st>>>(a);
-    else if (a.first) k_fwd_rows<D, BF16, 1, 8><<<grid, ROW_THREADS, 0, st>>>(a);
-    else k_fwd_rows<D, BF16, 1, 4><<<grid, ROW_THREADS, 0, st>>>(a);
-    count_launch();
-    HDT_CUDA_CHECK(cudaGetLastError());
+    auto *kern = kp == 4 ? k_fwd_rows<D, BF16, D == 64 ? 4 : 1, 8> : kp == 2 ? k_fwd_rows<D, BF16, 2, 8> : a.first ? k_fwd_rows<D, BF16, 1, 8> : k_fwd_rows<D, BF16, 1, 4>;
+    HDT_CUDA_CHECK(launch_dependent(kern, true, dim3(grid), ROW_THREADS, 0, st, a));
     return HDT_OK;
 }
 template <int D, bool BF16, bool DELTA>
@@ -543,11 +545,8 @@ static int launch_bwd_rows_t(const RowBwdArgs &a, cudaStream_t st) {
     if (rows == 0) return HDT_OK;
     const int kp = row_groups(rows, D, a.keys, 2, BF16 ? 16 : 12);
     const unsigned grid = (unsigned)((rows * kp * (D / 8) + ROW_THREADS - 1) / ROW_THREADS);
-    if (kp == 4) k_bwd_rows<D, BF16, D == 64 ? 4 : 1, DELTA><<<grid, ROW_THREADS, 0, st>>>(a);
-    else if (kp == 2) k_bwd_rows<D, BF16, 2, DELTA><<<grid, ROW_THREADS, 0, st>>>(a);
-    else k_bwd_rows<D, BF16, 1, DELTA><<<grid, ROW_THREADS, 0, st>>>(a);
-    count_launch();
-    HDT_CUDA_CHECK(cudaGetLastError());
+    auto *kern = kp == 4 ? k_bwd_rows<D, BF16, D == 64 ? 4 : 1, DELTA> : kp == 2 ? k_bwd_rows<D, BF16, 2, DELTA> : k_bwd_rows<D, BF16, 1, DELTA>;
+    HDT_CUDA_CHECK(launch_dependent(kern, true, dim3(grid), ROW_THREADS, 0, st, a));
     return HDT_OK;
 }
 int launch_fwd_rows(const RowFwdArgs &a, int D, int dtype, cudaStream_t st) {

@@ -413,6 +413,8 @@ __global__ void __launch_bounds__(NTHREADS) k_bwd_simt_multi(const MultiBwdArgs 
 // one 16-byte load each per tensor (8 bf16 or 4 fp32 values), so a warp covers 32 / LPR rows.
 template <int D, bool BF16>
 __global__ void __launch_bounds__(256) k_delta(const void *o, const void *d_o, float *delta, int T, int H) {
+    pdl_wait();
+    pdl_launch_dependents();
     constexpr int VPL = BF16 ? 8 : 4;          // values per lane
     constexpr int LPR = D / VPL;               // lanes per row: 8 (bf16, D=64) ... 32 (fp32, D=128)
     const long long gtid = (long long)blockIdx.x * blockDim.x + threadIdx.x;

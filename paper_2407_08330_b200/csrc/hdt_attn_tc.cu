@@ -91,6 +91,7 @@ __global__ void __launch_bounds__(128) k_fwd_tc(const __grid_constant__ CUtensor
     volatile int *abort_flag = (volatile int *)(slot + 1);
 
     const int tid = threadIdx.x, warp = tid >> 5;
+    if constexpr (GATHER) pdl_wait();
     // SINGLE: the first n_fused entries of queue_split; rest_only: the blocks after them
     const int blk = SINGLE ? a.queue_split[blockIdx.x]
                            : (a.rest_only ? a.queue_split[a.n_fused + blockIdx.x] : a.queue[blockIdx.x]);
@@ -498,6 +499,7 @@ __global__ void __launch_bounds__(128) k_fwd_tc_loop(const __grid_constant__ CUt
     // S (N <= 128 columns); P (bf16, two per column) is written over its first half as the rows are
     // exponentiated and is the A operand of O = P V; O lies beside it
     constexpr uint32_t TM_O = (D == 64) ? 64 : 128, TM_COLS = (D == 64) ? 128 : 256;
+    pdl_wait();                   // (a programmatic dependent: what it reads is complete from here on)
     extern __shared__ uint8_t smem_raw[];
     uint8_t *sm = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t *sQ = sm, *sK = sQ + NSUB * SUB, *sV = sK + NSUB * SUB;
@@ -569,6 +571,7 @@ __global__ void __launch_bounds__(128) k_fwd_tc_loop(const __grid_constant__ CUt
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_launch_dependents();      // (behind the TMEM allocation: a successor that becomes resident now takes none this CTA waits for)
     const uint32_t tmem = *slot;
     const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
     const bool dead = (*abort_flag != 0);
@@ -1454,10 +1457,7 @@ static int launch_fwd_tc_t(const FwdStageArgs &a, cudaStream_t st) {
         int n_sm_e = 0;
         if (const int rc_ = sm_count(&n_sm_e)) return rc_;
         const int grid = n_sm_e * (D == 64 ? 4 : 2);
-        if (dirs) k_fwd_tc_loop<D, true><<<grid, 128, smem_1, st>>>(tq, tk, tv, om, a);
-        else k_fwd_tc_loop<D><<<grid, 128, smem_1, st>>>(tq, tk, tv, om, a);
-        count_launch();
-        HDT_CUDA_CHECK(cudaGetLastError());
+        HDT_CUDA_CHECK(launch_dependent(dirs ? k_fwd_tc_loop<D, true> : k_fwd_tc_loop<D>, true, dim3(grid), 128, smem_1, st, tq, tk, tv, om, a));
         return HDT_OK;
     }
     FwdStageArgs b = a;
@@ -1475,16 +1475,19 @@ static int launch_fwd_tc_t(const FwdStageArgs &a, cudaStream_t st) {
             if (const int rc_ = sm_count(&n_sm)) return rc_;
             const long long items = (long long)a.n_fused * a.H;
             k_fwd_tc_p<<<(int)(items < n_sm ? items : n_sm), 512, smem_p, st>>>(tq, tk, tv, a);
+            count_launch();
         } else
 #endif
         if (a.no_persistent == 3 && !dirs) {       // option: one CTA per (block, head), no loop
             k_fwd_tc<D, true><<<dim3(a.n_fused, a.H), 128, smem_1, st>>>(tq, tk, tv, a);
+            count_launch();
         } else {
             int n_sm = 0;
             if (const int rc_ = sm_count(&n_sm)) return rc_;
             const long long items = (long long)a.n_fused * a.H;
             const long long slots = (long long)n_sm * (D == 64 ? 4 : 2);
-            if (dirs) k_fwd_tc_loop<D, true><<<(int)(items < slots ? items : slots), 128, smem_1, st>>>(tq, tk, tv, om, a);
+            const dim3 grid_l((unsigned)(items < slots ? items : slots));
+            if (dirs) HDT_CUDA_CHECK(launch_dependent(k_fwd_tc_loop<D, true>, true, grid_l, 128, smem_1, st, tq, tk, tv, om, a));
 #ifdef HDT_WORKBENCH
             else if (g_phase_stamps == 1 && D == 64) {
                 static DevOnce attr_s;
@@ -1493,11 +1496,11 @@ static int launch_fwd_tc_t(const FwdStageArgs &a, cudaStream_t st) {
                     attr_s.set();
                 }
                 k_fwd_tc_loop<64, false, true><<<(int)(items < slots ? items : slots), 128, 3 * SUB + 1024 + 64, st>>>(tq, tk, tv, om, a);
+                count_launch();
             }
 #endif
-            else k_fwd_tc_loop<D><<<(int)(items < slots ? items : slots), 128, smem_1, st>>>(tq, tk, tv, om, a);
+            else HDT_CUDA_CHECK(launch_dependent(k_fwd_tc_loop<D>, true, grid_l, 128, smem_1, st, tq, tk, tv, om, a));
         }
-        count_launch();
         HDT_CUDA_CHECK(cudaGetLastError());
         b.rest_only = 1;
         n_general = a.nb - a.n_fused;
@@ -1549,10 +1552,9 @@ static int launch_fwd_tc_upper_t(const FwdStageArgs &a, cudaStream_t st) {
             HDT_CUDA_CHECK(cudaFuncSetAttribute(k_fwd_tc<D, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_1));
             attr_1.set();
         }
-        k_fwd_tc<D, true, true><<<dim3(a.nb, a.H), 128, smem_1, st>>>(tq, tq, tq, b);
+        HDT_CUDA_CHECK(launch_dependent(k_fwd_tc<D, true, true>, a.pdl != 0, dim3(a.nb, a.H), 128, smem_1, st, tq, tq, tq, b));
     } else
-        k_fwd_tc<D, false, true><<<dim3(a.nb, a.H, a.splits > 1 ? a.splits : 1), 128, smem, st>>>(tq, tq, tq, b);
-    count_launch();
+        HDT_CUDA_CHECK(launch_dependent(k_fwd_tc<D, false, true>, a.pdl != 0, dim3(a.nb, a.H, a.splits > 1 ? a.splits : 1), 128, smem, st, tq, tq, tq, b));
     HDT_CUDA_CHECK(cudaGetLastError());
     return HDT_OK;
 }

@@ -146,32 +146,7 @@ __global__ void __launch_bounds__(256) k_bwd_tc(const __grid_constant__ CUtensor
     float *s_delta = (float *)(bar_tma + 8);     // gathering kernel without a delta pass: dO . O of the query-side rows
 
     const int tid = threadIdx.x, warp = tid >> 5, rl = tid & 127, hf = tid >> 7;
-    // rest_only: take the blocks after the first n_fused entries of queue_split
-    int qi = blockIdx.x, split = 0;
-    if (GATHER && a.phase_split > 0 && a.splits > 1) {      // (the phase-1 blocks come first, `splits` CTAs each)
-        const int n1 = a.phase_split * a.splits;
-        if (qi < n1) { split = qi % a.splits; qi /= a.splits; }
-        else qi -= n1 - a.phase_split;
-    }
-    const int blk = a.rest_only ? a.queue_split[a.n_fused + qi] : a.queue[qi];
     const int h = blockIdx.y, H = a.H;
-    const int *rec = a.blocks + 5 * (size_t)blk;
-    const int r0 = rec[0], r1 = rec[1], fl = rec[4];
-    int ka = rec[2], kb = rec[3];
-    int phases = a.phases, final_merge = a.final_merge;
-    if constexpr (GATHER) {
-        if (r1 <= r0) return;               // a block slot that is not in use
-        if (a.phase_split > 0) {
-            phases = qi < a.phase_split ? 1 : 2;
-            if (phases == 1 && a.splits > 1) {      // this CTA's share of the key span, whole tiles
-                final_merge = 0;
-                const int per = ((kb - ka + 127) / 128 + a.splits - 1) / a.splits * 128;
-                ka += split * per;
-                kb = min(kb, ka + per);
-            }
-        }
-    }
-    const int nrows = r1 - r0;
     const float LOG2E = 1.4426950408889634f;
 
     if (tid == 0) {
@@ -187,12 +162,43 @@ __global__ void __launch_bounds__(256) k_bwd_tc(const __grid_constant__ CUtensor
     const uint32_t tmem = *slot;
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
     const bool dead = (*abort_flag != 0);
+    uint32_t ph_tma = 0, ph_mma = 0;
+
+    if constexpr (GATHER) pdl_wait();
+    // One block; with phase_split, where most block slots may be unused (the host does not know how many tokens a
+    // level subset has), as many as the grid leaves to this CTA.
+    const int n_items = (GATHER && a.phase_split > 0) ? a.phase_split * (a.splits - 1) + a.nb : (int)blockIdx.x + 1;
+    for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+    // rest_only: take the blocks after the first n_fused entries of queue_split
+    int qi = item, split = 0;
+    if (GATHER && a.phase_split > 0) {      // (the phase-1 blocks come first, `splits` items each)
+        const int n1 = a.phase_split * a.splits;
+        if (qi < n1) { split = qi % a.splits; qi /= a.splits; }
+        else qi -= n1 - a.phase_split;
+    }
+    const int blk = a.rest_only ? a.queue_split[a.n_fused + qi] : a.queue[qi];
+    const int *rec = a.blocks + 5 * (size_t)blk;
+    const int r0 = rec[0], r1 = rec[1], fl = rec[4];
+    int ka = rec[2], kb = rec[3];
+    int phases = a.phases, final_merge = a.final_merge;
+    if constexpr (GATHER) {
+        if (r1 <= r0) continue;             // a block slot that is not in use
+        if (a.phase_split > 0) {
+            phases = qi < a.phase_split ? 1 : 2;
+            if (phases == 1 && a.splits > 1) {      // this item's share of the key span, whole tiles
+                final_merge = 0;
+                const int per = ((kb - ka + 127) / 128 + a.splits - 1) / a.splits * 128;
+                ka += split * per;
+                kb = min(kb, ka + per);
+            }
+        }
+    }
+    const int nrows = r1 - r0;
     const bool empty = (fl & HDT_BLK_EMPTY) != 0 || ka >= kb;
     const bool self = (fl & HDT_BLK_SELF) != 0;
     const bool fused = self && !empty && !dead;   // one pass yields dQ, dK and dV
     const uint32_t TM_DK = (D == 64) ? 320u : (fused ? 128u : 256u);
     const uint32_t TM_DV = (D == 64) ? 384u : (fused ? 0u : 384u);
-    uint32_t ph_tma = 0, ph_mma = 0;
     bool ok = true;
 
     // One tile pass.  q_row0 / k_row0: first token row of the query-side / key-side tile;
@@ -537,6 +543,8 @@ __global__ void __launch_bounds__(256) k_bwd_tc(const __grid_constant__ CUtensor
         copy_out(sDS, a.dk);
         copy_out(sQ, a.dv);
     }
+    tc_fence_after();
+    }
     if (warp == 0) tmem_dealloc(tmem, TM_COLS);
 }
 
@@ -560,6 +568,7 @@ __global__ void __launch_bounds__(256, 1) k_bwd_tc_loop(const __grid_constant__ 
                                                         const __grid_constant__ StoreMaps sm_out, const BwdStageArgs a) {
     constexpr int NSUB = D / 64;
     constexpr uint32_t TM_S = 0, TM_DP = 128, TM_DV = 0, TM_DK = 128, TM_DQ = 256, TM_COLS = 512;
+    pdl_wait();                   // (a programmatic dependent: what it reads is complete from here on)
     extern __shared__ uint8_t smem_raw[];
     uint8_t *sm = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t *sQ = sm, *sDO = sQ + NSUB * SUB, *sK = sDO + NSUB * SUB, *sV = sK + NSUB * SUB;
@@ -588,6 +597,7 @@ __global__ void __launch_bounds__(256, 1) k_bwd_tc_loop(const __grid_constant__ 
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_launch_dependents();      // (behind the TMEM allocation: a successor that becomes resident now takes none this CTA waits for)
     const uint32_t tmem = *slot;
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
     const bool dead = (*abort_flag != 0);
@@ -1402,10 +1412,9 @@ static int launch_bwd_tc_t(const BwdStageArgs &a, cudaStream_t st) {
         const long long items = (long long)a.n_fused * a.H;
         if (a.delta == nullptr) {      // no delta pass ran: the kernel computes dO . O of its rows itself
             if (a.o == nullptr) return set_error(HDT_ERR_INVALID_ARG, "launch_bwd_tc: the fused-delta kernel needs o");
-            k_bwd_tc_loop<D, true><<<(int)(items < n_sm_l ? items : n_sm_l), 256, smem_l, st>>>(tq, tk, tv, tdo, outs, a);
-        } else k_bwd_tc_loop<D><<<(int)(items < n_sm_l ? items : n_sm_l), 256, smem_l, st>>>(tq, tk, tv, tdo, outs, a);
-        count_launch();
-        HDT_CUDA_CHECK(cudaGetLastError());
+        }
+        HDT_CUDA_CHECK(launch_dependent(a.delta == nullptr ? k_bwd_tc_loop<D, true> : k_bwd_tc_loop<D>, true, dim3((unsigned)(items < n_sm_l ? items : n_sm_l)), 256,
+                                        smem_l, st, tq, tk, tv, tdo, outs, a));
         b.rest_only = 1;
         n_general = a.nb - a.n_fused;
     }
@@ -1449,8 +1458,15 @@ static int launch_bwd_tc_upper_t(const BwdStageArgs &a, cudaStream_t st) {
     }
     BwdStageArgs b = a;
     b.rest_only = 0;
+    if (b.splits < 1) b.splits = 1;
+    // (phase_split: the blocks of the queries, and of the others two CTAs per SM; an unused slot costs its CTA two loads)
+    int grid_x = a.nb;
+    if (a.phase_split > 0) grid_x = min(a.phase_split * (b.splits - 1) + a.nb, a.phase_split * b.splits + (2 * 148 + a.H - 1) / a.H);
     if (a.dirs != 7) k_bwd_tc<D, true, true><<<dim3(a.nb, a.H), 256, smem, st>>>(tq, tq, tq, tq, b);      // direction bits
-    else k_bwd_tc<D, true><<<dim3(a.nb + (a.splits > 1 ? (a.splits - 1) * a.phase_split : 0), a.H), 256, smem, st>>>(tq, tq, tq, tq, b);
+    else {
+        HDT_CUDA_CHECK(launch_dependent(k_bwd_tc<D, true>, a.pdl != 0, dim3(grid_x, a.H), 256, smem, st, tq, tq, tq, tq, b));
+        return HDT_OK;
+    }
     count_launch();
     HDT_CUDA_CHECK(cudaGetLastError());
     return HDT_OK;

@@ -68,6 +68,7 @@ __global__ void __maxnreg__(120) k_bwd_tc_t(const __grid_constant__ CUtensorMap 
                                                      const __grid_constant__ StoreMaps sm_out, const BwdStageArgs a) {
     constexpr int D = 64;
     constexpr uint32_t TM_S = 0, TM_DP = 128, TM_DV = 32, TM_DK = 128, TM_DQ = 192, TM_COLS = 256;
+    pdl_wait();                   // (a programmatic dependent: what it reads is complete from here on)
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t *sQ = smem_raw, *sDO = sQ + SUB, *sK = sDO + SUB, *sV = sK + SUB;
     uint8_t *sDS = sV + SUB;              // dS^T: sub-tile u = queries 64u..64u+63, row = key; later staging of dQ, dK
@@ -121,6 +122,7 @@ __global__ void __maxnreg__(120) k_bwd_tc_t(const __grid_constant__ CUtensorMap 
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_launch_dependents();      // (behind the TMEM allocation: a successor that becomes resident now takes none this CTA waits for)
     const uint32_t tmem = *slot;
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
     const bool dead = (*abort_flag != 0);
@@ -395,9 +397,11 @@ int launch_bwd_tc_fused64(const BwdStageArgs &a, const CUtensorMap &tq, const CU
         else k_bwd_tc_t<false, true><<<grid, 256, smem, st>>>(tq, tk, tv, tdo, outs, a);
     } else
 #endif
-    if (a.dirs != 7) k_bwd_tc_t<true><<<grid, 256, smem, st>>>(tq, tk, tv, tdo, outs, a);
-    else if (fd) k_bwd_tc_t<false, false, true><<<grid, 256, smem, st>>>(tq, tk, tv, tdo, outs, a);
-    else k_bwd_tc_t<false><<<grid, 256, smem, st>>>(tq, tk, tv, tdo, outs, a);
+    {
+        auto *kern = a.dirs != 7 ? k_bwd_tc_t<true> : fd ? k_bwd_tc_t<false, false, true> : k_bwd_tc_t<false>;
+        HDT_CUDA_CHECK(launch_dependent(kern, true, dim3(grid), 256, smem, st, tq, tk, tv, tdo, outs, a));
+        return HDT_OK;
+    }
     count_launch();
     HDT_CUDA_CHECK(cudaGetLastError());
     return HDT_OK;

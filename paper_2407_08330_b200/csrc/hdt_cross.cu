@@ -92,6 +92,7 @@ struct CrossIndexArgs {
 // its part starts is counted over the levels of all tokens before it by the CTA itself: a byte a token, read by
 // every CTA, costs less than the launches of a count and a scan kernel (four launches with a clear, 14 us of every call).
 __global__ void __launch_bounds__(256) k_cross_index(const CrossIndexArgs a) {
+    pdl_wait();
     pdl_launch_dependents();
     __shared__ int s_w[8], s_n[4];
     __shared__ int s_carry;
@@ -106,15 +107,21 @@ __global__ void __launch_bounds__(256) k_cross_index(const CrossIndexArgs a) {
         int n0 = 0, n1 = 0, n2 = 0, n3 = 0;
         const bool vec = ((uintptr_t)level & 15) == 0;
         const int units = vec ? a.T / 16 : 0;
-        for (int u = t; u < units; u += 256) {
-            const uint4 x = reinterpret_cast<const uint4 *>(level)[u];
+        for (int u0 = t; u0 < units; u0 += 4 * 256) {
+            uint4 x4[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) x4[k] = u0 + 256 * k < units ? reinterpret_cast<const uint4 *>(level)[u0 + 256 * k] : make_uint4(~0u, ~0u, ~0u, ~0u);
+#pragma unroll 1
+            for (int k = 0; k < 4; ++k) {
+            const uint4 x = k == 0 ? x4[0] : k == 1 ? x4[1] : k == 2 ? x4[2] : x4[3];
             const uint32_t xs[4] = {x.x, x.y, x.z, x.w};
-            const int i0 = 16 * u;
+            const int i0 = 16 * (u0 + 256 * k);
             unsigned bits = 0;
 #pragma unroll
             for (int j = 0; j < 16; ++j) bits |= (unsigned)chosen_level((int8_t)(xs[j >> 2] >> (8 * (j & 3))), mask) << j;
             auto below = [&](int lim) { const int d = lim - i0; return d <= 0 ? 0 : __popc(d >= 16 ? bits : bits & ((1u << d) - 1u)); };
             n0 += below(k0); n1 += below(c0); n2 += below(k1); n3 += __popc(bits);
+            }
         }
         for (int i = units * 16 + t; i < a.T; i += 256) {
             const int f = chosen(level, i, mask);
@@ -202,6 +209,7 @@ static constexpr int DEC_LIST = 1024;
 
 template <int D, bool BF16>
 __global__ void __launch_bounds__(512, 2) k_cross_decode(const DecodeArgs a) {
+    pdl_wait();
     pdl_launch_dependents();
     constexpr int LPK = D / 8, C = 4;
     using W = Raw<BF16, LPK>;
@@ -292,6 +300,7 @@ __global__ void __launch_bounds__(512, 2) k_cross_decode(const DecodeArgs a) {
 template <int D, bool BF16>
 __global__ void __launch_bounds__(128) k_cross_combine(int splits, int Tq, int H, const float *part, const float *part_lse, void *out, float *lse) {
     pdl_wait();
+    pdl_launch_dependents();
     constexpr int LPK = D / 8, G = 128 / LPK;
     using W = Raw<BF16, LPK>;
     __shared__ float s_red[G][D + 2];
@@ -332,25 +341,13 @@ __global__ void __launch_bounds__(128) k_cross_combine(int splits, int Tq, int H
     W::store(out, (unsigned)row * H + h, g, R.acc);
 }
 
-template <class... P, class... A>
-static cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = g_no_pdl ? 0 : 1;
-    cfg.attrs = at; cfg.numAttrs = 1;
-    count_launch();
-    return cudaLaunchKernelEx(&cfg, kern, P(args)...);
-}
-
 static int launch_combine(int splits, int Tq, int H, int D, int dtype, const float *part, const float *part_lse, void *out, float *lse, cudaStream_t st) {
     const dim3 grid(Tq, H);
     cudaError_t e;
-    if (D == 64) e = dtype == HDT_BF16 ? launch_dependent(k_cross_combine<64, true>, grid, 128, 0, st, splits, Tq, H, part, part_lse, out, lse)
-                                       : launch_dependent(k_cross_combine<64, false>, grid, 128, 0, st, splits, Tq, H, part, part_lse, out, lse);
-    else e = dtype == HDT_BF16 ? launch_dependent(k_cross_combine<128, true>, grid, 128, 0, st, splits, Tq, H, part, part_lse, out, lse)
-                               : launch_dependent(k_cross_combine<128, false>, grid, 128, 0, st, splits, Tq, H, part, part_lse, out, lse);
+    if (D == 64) e = dtype == HDT_BF16 ? launch_dependent(k_cross_combine<64, true>, true, grid, 128, 0, st, splits, Tq, H, part, part_lse, out, lse)
+                                       : launch_dependent(k_cross_combine<64, false>, true, grid, 128, 0, st, splits, Tq, H, part, part_lse, out, lse);
+    else e = dtype == HDT_BF16 ? launch_dependent(k_cross_combine<128, true>, true, grid, 128, 0, st, splits, Tq, H, part, part_lse, out, lse)
+                               : launch_dependent(k_cross_combine<128, false>, true, grid, 128, 0, st, splits, Tq, H, part, part_lse, out, lse);
     if (e != cudaSuccess) return set_error(HDT_ERR_CUDA, "launch of the combining kernel failed: %s", cudaGetErrorString(e));
     return HDT_OK;
 }
@@ -362,9 +359,7 @@ static int launch_decode_t(DecodeArgs a, int B, cudaStream_t st) {
     a.KS = max(1, min(16, 384 / (a.HC * LPK)));
     const int threads = (a.HC * LPK * a.KS + 31) / 32 * 32;
     const size_t smem = sizeof(float) * (size_t)a.KS * a.HC * (D + 2);
-    k_cross_decode<D, BF16><<<dim3(a.splits, B, (a.H + a.HC - 1) / a.HC), threads, smem, st>>>(a);
-    count_launch();
-    HDT_CUDA_CHECK(cudaGetLastError());
+    HDT_CUDA_CHECK(launch_dependent(k_cross_decode<D, BF16>, true, dim3(a.splits, B, (a.H + a.HC - 1) / a.HC), threads, smem, st, a));
     return HDT_OK;
 }
 
@@ -375,9 +370,7 @@ static int cross_build(const CrossLayout &L, char *ws, const int8_t *level, cons
     a.level = level; a.cu_k = cu_k; a.cu_q = cu_q; a.B = B; a.T = T; a.Tq = Tq; a.level_mask = level_mask;
     a.xr = L.xr; a.nbq = L.nbq; a.nbk = L.nbk;
     a.tokx = (int *)(ws + L.tokx); a.rngx = (int *)(ws + L.rngx); a.blocks = (int *)(ws + L.blocks); a.queue = (int *)(ws + L.queue);
-    k_cross_index<<<dim3(B, XC), 256, 0, st>>>(a);
-    count_launch();
-    HDT_CUDA_CHECK(cudaGetLastError());
+    HDT_CUDA_CHECK(launch_dependent(k_cross_index, true, dim3(B, XC), 256, 0, st, a));
     return HDT_OK;
 }
 
@@ -450,6 +443,7 @@ extern "C" int hdt_cross_attn_fwd(const int8_t *level, const int32_t *cu_seqlens
     a.block_rows = L.xr; a.dirs = 7;
     if (!tc) return launch_fwd_simt(a, head_dim, dtype, st);
     a.splits = tile_splits(batch, total_tokens, total_q, heads, level_mask, head_dim == 64 ? 2 : 1);
+    a.pdl = 1;
     if (a.splits == 1) {
         a.final_merge = 2;       // the kernel's epilogue writes the bf16 rows and the LSE of the decoder rows itself
         return launch_fwd_tc_upper(a, head_dim, st);
@@ -536,6 +530,7 @@ extern "C" int hdt_cross_attn_bwd(const int8_t *level, const int32_t *cu_seqlens
         a.splits = tile_splits(batch, total_tokens, total_q, heads, level_mask, 8);
         a.split_rows = total_q;
         a.own_dq = (float *)(ws + L.part);
+        a.pdl = 1;
         r = launch_bwd_tc_upper(a, head_dim, st);
         if (r || a.splits == 1) return r;
         return launch_combine(a.splits, total_q, heads, head_dim, dtype, a.own_dq, nullptr, dq, nullptr, st);

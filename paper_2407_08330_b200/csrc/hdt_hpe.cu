@@ -183,17 +183,20 @@ __global__ void __launch_bounds__(384, 2) k_hpe_eval_vec(const int8_t *__restric
     }
 }
 
-// x += HPE(p) as a bulk-copy pipeline (d_model % 8 == 0, three levels): a resident CTA walks tiles
-// of HPE_R tokens; one thread keeps up to HPE_NS - 1 tiles of x rows, p-vectors and levels in
-// flight as bulk copies into shared memory, the CTA adds the encoding in place there and the same
-// thread sends the tile back with a bulk store.  Thread (g, y) owns frequencies 4g..4g+3 of the
-// HPE_R / 4 consecutive tokens y * HPE_R / 4 ... of each tile.  Along such a run the section and
-// sentence numbers rarely change and the token number mostly grows by one, so the thread keeps
-// the sum of the first two levels, re-evaluates a sine/cosine only for a level whose p changed,
-// and advances the third level by the rotation (sin, cos)(a + w) from (sin, cos)(a) and
-// (sin, cos)(w) when p grew by exactly one.  A run is at most HPE_R / 4 tokens long and restarts
-// from a full evaluation, so the rotations add at most a few 1e-7 of error.
-constexpr int HPE_R = 32, HPE_NS = 4;     // tokens per tile; most stages a CTA keeps
+// x += HPE(p) or x = HPE(p) as a bulk-copy pipeline (d_model % 8 == 0, three levels).  Resident CTAs walk tiles of R
+// tokens; a warp of its own keeps `ns` tiles in flight: it requests the x rows as a bulk copy into shared memory,
+// walks the tile's tokens up their ancestors (a lane per token) while the copy is under way, and sends a tile the other
+// warps have finished back with a bulk store; the two sides meet at an mbarrier per stage and direction.
+// Thread (g, y) of the others owns frequencies 4g..4g+3 of the R / 4 consecutive tokens y * R / 4 ... of each
+// tile.  Along such a run the section and sentence numbers rarely change and the token number mostly grows
+// by one, so the thread keeps the sum of the first two levels, re-evaluates a sine/cosine only for a level
+// whose p changed, and advances the third level by the rotation (sin, cos)(a + w) from (sin, cos)(a) and
+// (sin, cos)(w) when p grew by exactly one.  A run is at most 8 tokens long and restarts from a full
+// evaluation, so the rotations add at most a few 1e-7 of error.
+// The bound is HBM: x read and written (4 x 8192 tokens, d_model 768, bf16: 101 MB, 15.4 us at the copy rate;
+// 20 us, against 29 with a kernel for the numbers in front of a pipeline that stopped at a CTA barrier per tile).
+// R: 32 tokens, 8 where that would leave SMs without a tile.
+constexpr int HPE_R = 32, HPE_R_SMALL = 8, HPE_NS = 8;     // tokens per tile; most stages a CTA keeps
 
 // (sin, cos)(p w) with p w carried as a float pair and reduced by 2 pi in two steps
 __device__ __forceinline__ void hpe_sincos(float pf, float wh, float wl, float &sn, float &cs) {
@@ -205,38 +208,69 @@ __device__ __forceinline__ void hpe_sincos(float pf, float wh, float wl, float &
     __sincosf(a, &sn, &cs);
 }
 
-template <bool BF16>
-__global__ void __launch_bounds__(512, 1) k_hpe_acc_bulk(const int8_t *__restrict__ level, const int *__restrict__ pvec,
-                                                         int n_tiles, int d_model, int ns, void *x, int *status) {
+template <bool BF16, bool ACC>
+__global__ void __launch_bounds__(544, 1) k_hpe_stream(const int8_t *__restrict__ level, const int *__restrict__ par, const int *__restrict__ rank, int T, int R,
+                                                       int tx, int d_model, int ns, void *x, int *status) {
+    pdl_wait();
+    pdl_launch_dependents();
     using namespace sm100;
-    constexpr int L = 3, ESZ = BF16 ? 2 : 4, NV = BF16 ? 1 : 2, TPT = HPE_R / 4;
+    constexpr int ESZ = BF16 ? 2 : 4, NV = BF16 ? 1 : 2;
     extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ uint64_t full[HPE_NS];
+    __shared__ uint64_t full[HPE_NS], done[HPE_NS];
     __shared__ int abort_flag;
-    const uint32_t row_bytes = (uint32_t)d_model * ESZ;
-    const uint32_t x_bytes = HPE_R * row_bytes, p_bytes = HPE_R * L * 4, l_bytes = HPE_R;
-    const uint32_t stage_bytes = x_bytes + p_bytes + l_bytes;        // multiple of 16
-    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+    const uint32_t row_bytes = (uint32_t)d_model * ESZ, stage_bytes = (uint32_t)R * (row_bytes + 16);
+    const int tid = threadIdx.x, lane = tid & 31, n_compute = tx * 4;
     if (tid == 0) {
-        for (int i = 0; i < HPE_NS; ++i) mbar_init(&full[i], 1);
+        for (int i = 0; i < ns; ++i) { mbar_init(&full[i], ACC ? 2 : 1); mbar_init(&done[i], n_compute / 32); }
         abort_flag = 0;
         fence_mbar_init();
     }
     __syncthreads();
-    const int n_mine = blockIdx.x < n_tiles ? (n_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
-    auto issue = [&](int i) {       // thread 0: fetch my i-th tile into stage i % ns
-        const int tile = blockIdx.x + i * gridDim.x;
-        unsigned char *st = smem + (size_t)(i % ns) * stage_bytes;
-        uint64_t *bar = &full[i % ns];
-        mbar_expect_tx(bar, stage_bytes);
-        bulk_load(st, reinterpret_cast<const char *>(x) + (size_t)tile * x_bytes, x_bytes, bar);
-        bulk_load(st + x_bytes, pvec + (size_t)tile * HPE_R * L, p_bytes, bar);
-        bulk_load(st + x_bytes + p_bytes, level + (size_t)tile * HPE_R, l_bytes, bar);
-    };
-    if (tid == 0)
-        for (int i = 0; i < ns - 1 && i < n_mine; ++i) issue(i);
-
-    const int G = d_model >> 3, g = threadIdx.x;      // blockDim.x >= G: one frequency group per thread
+    const int n_tiles = (T + R - 1) / R;
+    const int n_mine = (int)blockIdx.x < n_tiles ? (n_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
+    if (tid >= n_compute) {          // ---- the copying warp ----
+        auto issue = [&](int i) {
+            const int t0 = (blockIdx.x + i * gridDim.x) * R, n = min(R, T - t0);
+            unsigned char *st = smem + (size_t)(i % ns) * stage_bytes;
+            if (ACC && lane == 0) {
+                mbar_expect_tx(&full[i % ns], n * row_bytes);
+                bulk_load(st, reinterpret_cast<const char *>(x) + (size_t)t0 * row_bytes, n * row_bytes, &full[i % ns]);
+            }
+            if (lane < n) {              // p of level 1, 2, 3 and the token's own level
+                int node = t0 + lane, p[3] = {0, 0, 0};
+                const int lv = level[node];
+                for (int l = lv; l >= 1; --l) {          // PAD (-1) and the root (0) keep all zeros
+                    const int up = par[node];
+                    if (l <= 3) p[l - 1] = rank[node];
+                    node = up;
+                }
+                *reinterpret_cast<int4 *>(st + R * row_bytes + lane * 16) = make_int4(p[0], p[1], p[2], lv);
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&full[i % ns]);
+        };
+        for (int i = 0; i < min(ns, n_mine); ++i) issue(i);
+        for (int i = 0; i < n_mine; ++i) {
+            const bool ok = mbar_wait(&done[i % ns], (i / ns) & 1, &abort_flag, 2000000000LL);
+            if (!__all_sync(0xffffffffu, ok)) break;
+            if (lane == 0) {
+                const int t0 = (blockIdx.x + i * gridDim.x) * R, n = min(R, T - t0);
+                bulk_store(reinterpret_cast<char *>(x) + (size_t)t0 * row_bytes, smem + (size_t)(i % ns) * stage_bytes, n * row_bytes);
+                bulk_commit();
+            }
+            if (i >= 1 && i - 1 + ns < n_mine) {
+                if (lane == 0) bulk_wait_read_1();     // the stage refilled now was stored one tile ago
+                __syncwarp();
+                issue(i - 1 + ns);
+            }
+        }
+        if (lane == 0) {
+            bulk_wait_all();
+            if (abort_flag) atomicCAS(status, 0, (int)HDT_ERR_TIMEOUT);
+        }
+        return;
+    }
+    const int G = d_model >> 3, g = tid % tx, y = tid / tx, TPT = R / 4;      // tx >= G: one frequency group per thread
     float wh[4], wl[4], sw[4], cw[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -248,8 +282,8 @@ __global__ void __launch_bounds__(512, 1) k_hpe_acc_bulk(const int8_t *__restric
     for (int i = 0; i < n_mine; ++i) {
         unsigned char *st = smem + (size_t)(i % ns) * stage_bytes;
         if (!mbar_wait(&full[i % ns], (i / ns) & 1, &abort_flag, 2000000000LL)) break;
-        const int *sp = reinterpret_cast<const int *>(st + x_bytes);
-        const int8_t *sl = reinterpret_cast<const int8_t *>(st + x_bytes + p_bytes);
+        const int n = min(R, T - (int)(blockIdx.x + i * gridDim.x) * R);
+        const int4 *sp = reinterpret_cast<const int4 *>(st + R * row_bytes);
         if (g < G) {
             // p = 0 on every level: sin 0 = 0, cos 0 = 1
             int pc0 = 0, pc1 = 0, pc2 = 0;
@@ -263,9 +297,17 @@ __global__ void __launch_bounds__(512, 1) k_hpe_acc_bulk(const int8_t *__restric
             }
 #pragma unroll 2
             for (int u = 0; u < TPT; ++u) {
-                const int r = threadIdx.y * TPT + u;
-                if (sl[r] < 0) continue;                    // PAD rows pass through unchanged
-                const int p0 = sp[r * L], p1 = sp[r * L + 1], p2 = sp[r * L + 2];
+                const int r = y * TPT + u;
+                if (r >= n) break;
+                const int4 pv = sp[r];
+                uint4 *cell = reinterpret_cast<uint4 *>(st + (size_t)r * row_bytes + (size_t)g * 8 * ESZ);
+                if (pv.w < 0) {                             // PAD rows: unchanged, or zero
+                    if (!ACC)
+#pragma unroll
+                        for (int q = 0; q < NV; ++q) cell[q] = make_uint4(0, 0, 0, 0);
+                    continue;
+                }
+                const int p0 = pv.x, p1 = pv.y, p2 = pv.z;
                 if (p0 != pc0 || p1 != pc1) {
                     if (p0 != pc0) {
 #pragma unroll
@@ -292,9 +334,8 @@ __global__ void __launch_bounds__(512, 1) k_hpe_acc_bulk(const int8_t *__restric
                     for (int j = 0; j < 4; ++j) hpe_sincos((float)p2, wh[j], wl[j], s2[j], c2[j]);
                 }
                 pc2 = p2;
-                uint4 *cell = reinterpret_cast<uint4 *>(st + (size_t)r * row_bytes + (size_t)g * 8 * ESZ);
                 if constexpr (BF16) {
-                    uint4 v = cell[0];
+                    uint4 v = ACC ? cell[0] : make_uint4(0, 0, 0, 0);
                     __nv_bfloat162 *h = reinterpret_cast<__nv_bfloat162 *>(&v);
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
@@ -305,7 +346,7 @@ __global__ void __launch_bounds__(512, 1) k_hpe_acc_bulk(const int8_t *__restric
                 } else {
 #pragma unroll
                     for (int q = 0; q < NV; ++q) {
-                        float4 f = *reinterpret_cast<float4 *>(&cell[q]);
+                        float4 f = ACC ? *reinterpret_cast<float4 *>(&cell[q]) : make_float4(0.f, 0.f, 0.f, 0.f);
                         f.x += bs[2 * q] + s2[2 * q];
                         f.y += bc[2 * q] + c2[2 * q];
                         f.z += bs[2 * q + 1] + s2[2 * q + 1];
@@ -316,20 +357,8 @@ __global__ void __launch_bounds__(512, 1) k_hpe_acc_bulk(const int8_t *__restric
             }
         }
         fence_proxy_async_smem();       // the tile was written through the generic proxy
-        __syncthreads();
-        if (tid == 0) {
-            const int tile = blockIdx.x + i * gridDim.x;
-            bulk_store(reinterpret_cast<char *>(x) + (size_t)tile * x_bytes, st, x_bytes);
-            bulk_commit();
-            if (i + ns - 1 < n_mine) {
-                bulk_wait_read_1();     // the stage refilled next was stored one tile ago
-                issue(i + ns - 1);
-            }
-        }
-    }
-    if (tid == 0) {
-        bulk_wait_all();
-        if (abort_flag) atomicCAS(status, 0, (int)HDT_ERR_TIMEOUT);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&done[i % ns]);
     }
 }
 
@@ -363,44 +392,42 @@ extern "C" int hdt_hpe(const hdt_index_t *ix, const int8_t *level, const int32_t
         return set_error(HDT_ERR_INVALID_ARG, "hdt_hpe: workspace must be 256-byte, x 8-byte aligned");
     cudaStream_t st = (cudaStream_t)stream;
     const int *rank = ix->rank;
+    const bool x16 = ((uintptr_t)x & 15) == 0;
+    if (d_model % 8 == 0 && x16 && n_levels == 3 && d_model <= 1024) {
+        const int R = T < 148 * 64 ? HPE_R_SMALL : HPE_R;
+        const size_t stage = (size_t)R * (d_model * (dtype == HDT_BF16 ? 2 : 4) + 16);
+        const int n_tiles = (T + R - 1) / R, per_sm = stage * 4 <= 100 * 1024 ? 2 : 1;
+        const int ns = (int)max((size_t)1, min((size_t)HPE_NS, (size_t)(per_sm == 2 ? 104 : 208) * 1024 / stage));
+        if (ns >= 2) {
+            const int tx = (d_model / 8 + 31) / 32 * 32, nb = min(n_tiles, 148 * per_sm);
+            int *status = device_status_ptr();
+            if (!status) return HDT_ERR_CUDA;
+            const int b16 = dtype == HDT_BF16;
+            auto *kern = b16 ? (accumulate ? k_hpe_stream<true, true> : k_hpe_stream<true, false>)
+                             : (accumulate ? k_hpe_stream<false, true> : k_hpe_stream<false, false>);
+            static DevOnce once[2][2];
+            if (!once[b16][accumulate ? 1 : 0].done()) {
+                HDT_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 208 * 1024));
+                once[b16][accumulate ? 1 : 0].set();
+            }
+            HDT_CUDA_CHECK(launch_dependent(kern, true, dim3(nb), tx * 4 + 32, stage * ns, st, level, ix->st[0].par, rank, T, R, tx, d_model, ns, x, status));
+            return HDT_OK;
+        }
+    }
     int *pvec = (int *)workspace;
     k_hpe_pvec<<<(T + 255) / 256, 256, 0, st>>>(level, parent, cu_seqlens, B, T, n_levels, rank, pvec);
     count_launch();
-    const bool x16 = ((uintptr_t)x & 15) == 0;
     if (d_model % 8 == 0 && x16) {
         // threads.x covers the 8-element groups of a row (whole warps), threads.y token runs
         const int G = d_model / 8;
-        int t_begin = 0;
-        const size_t esz = dtype == HDT_BF16 ? 2 : 4;
-        const size_t stage = (size_t)HPE_R * d_model * esz + HPE_R * 3 * 4 + HPE_R;
-        const int ns = (int)min((size_t)HPE_NS, (size_t)(220 * 1024) / stage);
-        if (accumulate && n_levels == 3 && G <= 128 && ns >= 2 && T >= HPE_R && ((uintptr_t)level & 15) == 0) {
-            // whole tiles through the bulk-copy pipeline, the ragged tail through the register kernel
-            const int n_tiles = T / HPE_R;
-            const int tx = ((G + 31) / 32) * 32;
-            const size_t smem = stage * ns;
-            const int per_sm = (int)max((size_t)1, min((size_t)2, (size_t)(220 * 1024) / (smem + 1024)));
-            const int nb = min(n_tiles, 148 * per_sm);
-            int *status = device_status_ptr();
-            static DevOnce attr_done;
-            if (!attr_done.done()) {
-                HDT_CUDA_CHECK(cudaFuncSetAttribute(k_hpe_acc_bulk<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-                HDT_CUDA_CHECK(cudaFuncSetAttribute(k_hpe_acc_bulk<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-                attr_done.set();
-            }
-            if (dtype == HDT_BF16) k_hpe_acc_bulk<true><<<nb, dim3(tx, 4), smem, st>>>(level, pvec, n_tiles, d_model, ns, x, status);
-            else k_hpe_acc_bulk<false><<<nb, dim3(tx, 4), smem, st>>>(level, pvec, n_tiles, d_model, ns, x, status);
-            count_launch();
-            t_begin = n_tiles * HPE_R;
-        }
-        if (t_begin < T) {
+        {
         const int tx = min(384, ((G + 31) / 32) * 32), ty = max(1, 384 / tx);
         int run = 16;
-        const int Tr = T - t_begin;
+        const int Tr = T;
         while ((long long)((Tr + run - 1) / run + ty - 1) / ty > 148LL * 64) run *= 2;
         const int nb = ((Tr + run - 1) / run + ty - 1) / ty;
         const dim3 blk(tx, ty);
-#define HPE_LAUNCH(BF, LL) k_hpe_eval_vec<BF, LL><<<nb, blk, 0, st>>>(level, pvec, t_begin, T, n_levels, d_model, accumulate, run, x)
+#define HPE_LAUNCH(BF, LL) k_hpe_eval_vec<BF, LL><<<nb, blk, 0, st>>>(level, pvec, 0, T, n_levels, d_model, accumulate, run, x)
         if (dtype == HDT_BF16) {
             if (n_levels == 3) HPE_LAUNCH(true, 3); else if (n_levels == 2) HPE_LAUNCH(true, 2); else HPE_LAUNCH(true, 0);
         } else {

@@ -649,6 +649,7 @@ __device__ __forceinline__ bool seq_upper_all(const SeqArgs &a, SeqShared &sh, c
 // Shared memory: 6 bytes per token of the slice (parents, counts, prefix sums), `pool` for the upper stages, one
 // per token of `cap` for the walk.
 __global__ void __launch_bounds__(512) k_seq(const SeqArgs a) {
+    pdl_wait();
     pdl_launch_dependents();
     extern __shared__ __align__(16) uint16_t s_dyn[];
     __shared__ SeqShared sh;
@@ -1184,11 +1185,13 @@ extern "C" int hdt_build_index(const int8_t *level, const int32_t *parent, const
             cfg.blockDim = dim3(threads);
             cfg.dynamicSmemBytes = smem;
             cfg.stream = st;
-            cudaLaunchAttribute at[1];
+            cudaLaunchAttribute at[2];
             at[0].id = cudaLaunchAttributeClusterDimension;
             at[0].val.clusterDim.x = cs; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+            at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            at[1].val.programmaticStreamSerializationAllowed = g_no_pdl ? 0 : 1;
             cfg.attrs = at;
-            cfg.numAttrs = 1;
+            cfg.numAttrs = 2;
             e = cudaLaunchKernelEx(&cfg, k_seq, a);
             count_launch();
         }

@@ -119,6 +119,18 @@ extern int g_no_fwd_mc;    // option "no_fwd_mc": blocks that are not self-conta
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 extern int g_no_pdl;       // option "no_pdl"
+// Launch as a programmatic dependent of the kernel before it on the stream (`dependent`; the kernel calls pdl_wait).
+template <class... P, class... A>
+inline cudaError_t launch_dependent(void (*kern)(P...), bool dependent, dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid; cfg.blockDim = dim3((unsigned)threads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = (dependent && !g_no_pdl) ? 1 : 0;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    count_launch();
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
 extern int g_bwd_walk;     // option "bwd_walk": families longer than a row block in the head_dim 64 backward: 0 = one walk on the
                            // warp-specialised kernel, 1 = two walks (no dQ buffer, deterministic), 2 = one walk on the lockstep kernel
 
@@ -202,6 +214,7 @@ struct FwdStageArgs {
     // Gathering kernel in own-partial mode: splits > 1 gives the key span of a block to that many CTAs (grid.z), each with
     // a partial result of its own (own_o / own_lse hold splits x split_rows rows).
     int splits, split_rows;
+    int pdl;              // gathering kernel: launched as a programmatic dependent of the kernel before it on the stream
     const DevHeader *hdr; // set: the index build is still in flight; the looping kernel reads n_fused and stage 1's size here
     size_t ws_bytes;      // with hdr: bytes behind part_o (the caller's workspace)
     int n_empty;          // EMPTY blocks of the stage (0 where the caller does not know): when they are all that is left
@@ -246,6 +259,7 @@ struct BwdStageArgs {
     // cross-attention in one launch); splits > 1 gives a phase-1 block's key span to that many CTAs, each with
     // a partial dQ of its own (own_dq holds splits x split_rows rows; phase 2 still writes the final rows).
     int phase_split, splits, split_rows;
+    int pdl;                                      // as in FwdStageArgs
     int gather_end_q, gather_end_k;               // gathering kernel: elements at or beyond these read as zero rows on the Q/dO and the K/V side (0: n)
 };
 

@@ -1,0 +1,62 @@
+"""Split key lists and the decoding kernel of the cross-attention, the streaming positional encoding: the sizes where
+their splits change, against the oracles."""
+import numpy as np
+import pytest
+
+import gen
+from oracle import cross_oracle, hpe_oracle
+from tests.gpu_util import check_close, dev_struct, dev_tensor, host
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dtype,d", [("bf16", 64), ("bf16", 128), ("f32", 64)])
+@pytest.mark.parametrize("lengths,rows,mask", [
+    ([40], [1], 15), ([700, 33], [4, 4], 15), ([700, 33, 1], [1, 0, 1], 6), ([60], [4], 2),      # decoding: one and several splits, no key
+    ([1500, 90], [130, 5], 15), ([600], [20], 15), ([2100], [7], 15),                            # tiles with split key lists
+])
+def test_cross_splits(dtype, d, lengths, rows, mask):
+    import torch
+    import paper_2407_08330_b200 as P
+    rng = np.random.default_rng(11)
+    b = gen.pack([gen.gen_fill(rng, n, (2, 6), (2, 8), (3, 20))[:2] for n in lengths])
+    H, T, Tq = 3, b.total_tokens, sum(rows)
+    cu_q = np.concatenate([[0], np.cumsum(rows)]).astype(np.int32)
+    t = gen.make_tensors(3, T, H, d, dtype, names=("k", "v"))
+    tq = gen.make_tensors(4, Tq, H, d, dtype, names=("q", "do"))
+    level, _, cu = dev_struct(b)
+    q, do, k, v = (dev_tensor(x, dtype) for x in (tq["q"], tq["do"], t["k"], t["v"]))
+    cq = torch.from_numpy(cu_q).cuda()
+    o, lse = P.hdt_cross_attn_fwd(level, cu, cq, mask, q, k, v)
+    g = P.hdt_cross_attn_bwd(level, cu, cq, mask, q, k, v, o, lse, do)
+    torch.cuda.synchronize()
+    P.hdt_device_status()
+    o_r, lse_r = cross_oracle.forward(b.level, b.cu_seqlens, mask, cu_q, tq["q"], t["k"], t["v"])
+    g_r = cross_oracle.backward(b.level, b.cu_seqlens, mask, cu_q, tq["q"], t["k"], t["v"], tq["do"])
+    check_close(host(o), o_r, dtype, "O", out_rounding=True)
+    check_close(lse.cpu().numpy(), lse_r, dtype, "LSE")
+    for x, r, what in zip(g, g_r, ("dQ", "dK", "dV")):
+        check_close(host(x), r, dtype, what, out_rounding=True, row_rel=2.0 ** -8)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("accumulate", [True, False])
+@pytest.mark.parametrize("T,d_model", [(1, 8), (31, 1024), (33, 256), (9473, 64), (9999, 264)])
+def test_hpe_stream(T, d_model, dtype, accumulate):
+    import torch
+    import paper_2407_08330_b200 as P
+    rng = np.random.default_rng(T)
+    n = max(1, T - T // 10)
+    lv, pa = gen.gen_fill(rng, n, (4, 24), (3, 20), (5, 60))[:2]
+    b = gen.pack([gen.fit(lv, pa, T, pad=True)])
+    level, parent, cu = dev_struct(b)
+    idx = P.hdt_build_index(level, parent, cu)
+    x0 = gen.make_tensors(1, T, 1, d_model, dtype, names=("x",))["x"][:, 0]
+    x = dev_tensor(x0, dtype)
+    P.hdt_hpe(idx, level, parent, cu, d_model, x=x, accumulate=accumulate)
+    torch.cuda.synchronize()
+    P.hdt_device_status()
+    want = hpe_oracle.hpe(b.level, b.parent, b.cu_seqlens, d_model, 3)
+    if accumulate:
+        want = want + x0
+    check_close(host(x), want, dtype, "x", out_rounding=True)
