@@ -2,6 +2,7 @@
 from __future__ import annotations
 
 import ctypes as C
+import functools
 import os
 import re
 
@@ -63,6 +64,24 @@ def lib():
                                                        C.c_void_p, C.c_size_t, C.c_void_p]
         L.hdt_last_error.restype = C.c_char_p
         L.hdt_launch_count.restype = C.c_int64
+        L.hdt_attn_fwd_static_max_bytes.restype = C.c_size_t
+        L.hdt_attn_fwd_static.restype = C.c_int
+        L.hdt_attn_fwd_static.argtypes = [C.c_void_p] * 6 + [C.c_int32, C.c_int32, C.c_int32, C.c_float, C.c_void_p]
+        L.hdt_hpe_workspace_bytes.restype = C.c_size_t
+        L.hdt_hpe_workspace_bytes.argtypes = [C.c_void_p, C.c_int32]
+        L.hdt_hpe.restype = C.c_int
+        L.hdt_hpe.argtypes = [C.c_void_p] * 4 + [C.c_int32] * 4 + [C.c_void_p, C.c_void_p, C.c_size_t, C.c_void_p]
+        L.hdt_cross_workspace_bytes.restype = C.c_size_t
+        L.hdt_cross_workspace_bytes.argtypes = [C.c_int32] * 7
+        L.hdt_cross_attn_fwd.restype = C.c_int
+        L.hdt_cross_attn_fwd.argtypes = [C.c_void_p] * 3 + [C.c_int32] * 4 + [C.c_void_p] * 5 + [C.c_int32] * 3 + \
+                                        [C.c_float, C.c_void_p, C.c_size_t, C.c_void_p]
+        L.hdt_cross_attn_bwd.restype = C.c_int
+        L.hdt_cross_attn_bwd.argtypes = [C.c_void_p] * 3 + [C.c_int32] * 4 + [C.c_void_p] * 9 + [C.c_int32] * 3 + \
+                                        [C.c_float, C.c_void_p, C.c_size_t, C.c_void_p]
+        L.hdt_set_option.restype = C.c_int
+        L.hdt_device_status.restype = C.c_int
+        L.hdt_device_status.argtypes = [C.c_void_p]
         _lib = L
     return _lib
 
@@ -86,26 +105,25 @@ def _check(rc):
         raise HdtError(rc, lib().hdt_last_error().decode())
 
 
-def _ptr(t):
-    return C.c_void_p(t.data_ptr()) if t is not None else C.c_void_p(0)
-
-
 def _stream():
-    # the raw handle of the current stream without building a torch.cuda.Stream object
-    return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+    # the raw handle of the current stream without building a torch.cuda.Stream object (0: the default stream)
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
+@functools.lru_cache(maxsize=64)
 def _params(block_m, max_stages, block_m_upper=0, directions=7, deferred=False):
+    """A parameter block and its address (the library only reads it)."""
     p = _Params()
     p.block_m, p.max_stages, p.block_m_upper = int(block_m), int(max_stages), int(block_m_upper)
     p.mask_off = (~int(directions)) & 7
     p.deferred = 1 if deferred else 0
-    return p
+    return p, C.addressof(p)
 
 
+@functools.lru_cache(maxsize=256)
 def hdt_index_workspace_bytes(batch, total_tokens, block_m=0, max_stages=0, block_m_upper=0) -> int:
-    p = _params(block_m, max_stages, block_m_upper)
-    return int(lib().hdt_index_workspace_bytes(batch, total_tokens, C.cast(C.byref(p), C.c_void_p)))
+    p, addr = _params(block_m, max_stages, block_m_upper)
+    return int(lib().hdt_index_workspace_bytes(batch, total_tokens, addr))
 
 
 class HdtIndex:
@@ -115,6 +133,7 @@ class HdtIndex:
         self._h, self._ws = handle, workspace
         self.batch, self.total_tokens = batch, total_tokens
         self._info = None
+        self._ws_bytes = {}        # attention workspace sizes, by (heads, head_dim, dtype, bwd)
 
     def _get_info(self):
         if self._info is None:
@@ -177,39 +196,48 @@ def hdt_build_index(level, parent, cu_seqlens, block_m=0, max_stages=0, workspac
     assert level.dtype == torch.int8 and parent.dtype == torch.int32 and cu_seqlens.dtype == torch.int32
     level, parent, cu_seqlens = level.contiguous(), parent.contiguous(), cu_seqlens.contiguous()
     T, B = level.numel(), cu_seqlens.numel() - 1
-    p = _params(block_m, max_stages, block_m_upper, directions, deferred)
-    need = int(lib().hdt_index_workspace_bytes(B, T, C.cast(C.byref(p), C.c_void_p)))
+    need = hdt_index_workspace_bytes(B, T, block_m, max_stages, block_m_upper)
     if need == 0:
         raise HdtError(-1, "invalid index parameters")
+    _, addr = _params(block_m, max_stages, block_m_upper, directions, deferred)
     if workspace is None:
         workspace = torch.empty(need, dtype=torch.uint8, device=level.device)
     h = C.c_void_p()
-    _check(lib().hdt_build_index(_ptr(level), _ptr(parent), _ptr(cu_seqlens), B, T, C.cast(C.byref(p), C.c_void_p),
-                                 _ptr(workspace), workspace.numel(), _stream(), C.byref(h)))
+    rc = (_lib or lib()).hdt_build_index(level.data_ptr(), parent.data_ptr(), cu_seqlens.data_ptr(), B, T, addr,
+                                         workspace.data_ptr(), workspace.numel(), _stream(), C.byref(h))
+    if rc:
+        _check(rc)
     return HdtIndex(h, workspace, B, T)
 
 
 def hdt_attn_workspace_bytes(index: HdtIndex, heads, head_dim, dtype, bwd) -> int:
-    return int(lib().hdt_attn_workspace_bytes(index.handle, heads, head_dim, _DTYPES[dtype], int(bwd)))
+    key = (heads, head_dim, dtype, bwd)
+    n = index._ws_bytes.get(key)
+    if n is None:
+        n = int(lib().hdt_attn_workspace_bytes(index.handle, heads, head_dim, _DTYPES[dtype], int(bwd)))
+        if n:                      # (0: nothing needed, or an index whose build failed)
+            index._ws_bytes[key] = n
+    return n
 
 
 def _ws(index, heads, head_dim, dtype, bwd, device, workspace):
     if workspace is not None:      # the library checks the size itself
-        return workspace, None
-    need = hdt_attn_workspace_bytes(index, heads, head_dim, dtype, bwd)
-    return torch.empty(max(need, 256), dtype=torch.uint8, device=device), need
+        return workspace
+    return torch.empty(max(hdt_attn_workspace_bytes(index, heads, head_dim, dtype, bwd), 256), dtype=torch.uint8, device=device)
 
 
 def hdt_attn_fwd(index: HdtIndex, q, k, v, softmax_scale=0.0, out=None, lse=None, workspace=None):
     """q, k, v: CUDA [T, H, d] float32 or bfloat16, contiguous.  Returns (O, LSE [H, T])."""
     T, H, d = q.shape
-    assert q.is_contiguous() and k.is_contiguous() and v.is_contiguous() and q.dtype == k.dtype == v.dtype
+    dt = q.dtype
+    assert q.is_contiguous() and k.is_contiguous() and v.is_contiguous() and dt == k.dtype == v.dtype
     o = torch.empty_like(q) if out is None else out
     lse = torch.empty((H, T), dtype=torch.float32, device=q.device) if lse is None else lse
-    workspace, need = _ws(index, H, d, q.dtype, 0, q.device, workspace)
-    _check(lib().hdt_attn_fwd(index.handle, _ptr(q), _ptr(k), _ptr(v), _ptr(o), _ptr(lse), H, d,
-                              _DTYPES[q.dtype], float(softmax_scale), _ptr(workspace), workspace.numel(),
-                              _stream()))
+    workspace = _ws(index, H, d, dt, 0, q.device, workspace)
+    rc = (_lib or lib()).hdt_attn_fwd(index._h, q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), lse.data_ptr(), H, d,
+                                      _DTYPES[dt], float(softmax_scale), workspace.data_ptr(), workspace.numel(), _stream())
+    if rc:
+        _check(rc)
     return o, lse
 
 
@@ -217,20 +245,22 @@ def hdt_attn_bwd(index: HdtIndex, q, k, v, o, lse, d_o, softmax_scale=0.0, dq=No
                  workspace=None):
     """Returns (dQ, dK, dV) with the shape and dtype of q."""
     T, H, d = q.shape
+    dt = q.dtype
     for t in (q, k, v, o, d_o):
-        assert t.is_contiguous() and t.dtype == q.dtype
+        assert t.is_contiguous() and t.dtype == dt
     dq = torch.empty_like(q) if dq is None else dq
     dk = torch.empty_like(q) if dk is None else dk
     dv = torch.empty_like(q) if dv is None else dv
-    workspace, need = _ws(index, H, d, q.dtype, 1, q.device, workspace)
-    _check(lib().hdt_attn_bwd(index.handle, _ptr(q), _ptr(k), _ptr(v), _ptr(o), _ptr(lse), _ptr(d_o),
-                              _ptr(dq), _ptr(dk), _ptr(dv), H, d, _DTYPES[q.dtype], float(softmax_scale),
-                              _ptr(workspace), workspace.numel(), _stream()))
+    workspace = _ws(index, H, d, dt, 1, q.device, workspace)
+    rc = (_lib or lib()).hdt_attn_bwd(index._h, q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), lse.data_ptr(),
+                                      d_o.data_ptr(), dq.data_ptr(), dk.data_ptr(), dv.data_ptr(), H, d, _DTYPES[dt],
+                                      float(softmax_scale), workspace.data_ptr(), workspace.numel(), _stream())
+    if rc:
+        _check(rc)
     return dq, dk, dv
 
 
 def hdt_attn_fwd_static_max_bytes() -> int:
-    lib().hdt_attn_fwd_static_max_bytes.restype = C.c_size_t
     return int(lib().hdt_attn_fwd_static_max_bytes())
 
 
@@ -243,18 +273,13 @@ def hdt_attn_fwd_static(index: HdtIndex, q, k, v, softmax_scale=0.0, out=None, l
     assert q.is_contiguous() and k.is_contiguous() and v.is_contiguous() and q.dtype == k.dtype == v.dtype
     o = torch.empty_like(q) if out is None else out
     lse = torch.empty((H, T), dtype=torch.float32, device=q.device) if lse is None else lse
-    f = lib().hdt_attn_fwd_static
-    f.restype = C.c_int
-    f.argtypes = [C.c_void_p] * 6 + [C.c_int32, C.c_int32, C.c_int32, C.c_float, C.c_void_p]
-    _check(f(index.handle, _ptr(q), _ptr(k), _ptr(v), _ptr(o), _ptr(lse), H, d, _DTYPES[q.dtype],
-             float(softmax_scale), _stream()))
+    _check(lib().hdt_attn_fwd_static(index.handle, q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), lse.data_ptr(), H, d,
+                                     _DTYPES[q.dtype], float(softmax_scale), _stream()))
     return o, lse
 
 
 def hdt_hpe_workspace_bytes(index: HdtIndex, n_levels=3) -> int:
     L = lib()
-    L.hdt_hpe_workspace_bytes.restype = C.c_size_t
-    L.hdt_hpe_workspace_bytes.argtypes = [C.c_void_p, C.c_int32]
     return int(L.hdt_hpe_workspace_bytes(index.handle, n_levels))
 
 
@@ -262,26 +287,20 @@ def hdt_hpe(index: HdtIndex, level, parent, cu_seqlens, d_model, n_levels=3, dty
             accumulate=False, workspace=None):
     """Hierarchical positional encoding [T, d_model]; with `x` and accumulate=True it is added to x."""
     L = lib()
-    L.hdt_hpe_workspace_bytes.restype = C.c_size_t
-    L.hdt_hpe_workspace_bytes.argtypes = [C.c_void_p, C.c_int32]
-    L.hdt_hpe.restype = C.c_int
-    L.hdt_hpe.argtypes = [C.c_void_p] * 4 + [C.c_int32] * 4 + [C.c_void_p, C.c_void_p, C.c_size_t, C.c_void_p]
     T = level.numel()
     if x is None:
         x = torch.empty((T, d_model), dtype=dtype, device=level.device)
     assert x.is_contiguous() and x.shape == (T, d_model)
-    need = int(L.hdt_hpe_workspace_bytes(index.handle, n_levels))
     if workspace is None:
-        workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=level.device)
-    _check(L.hdt_hpe(index.handle, _ptr(level), _ptr(parent), _ptr(cu_seqlens), n_levels, d_model, _DTYPES[x.dtype],
-                     int(bool(accumulate)), _ptr(x), _ptr(workspace), workspace.numel(), _stream()))
+        workspace = torch.empty(max(hdt_hpe_workspace_bytes(index, n_levels), 256), dtype=torch.uint8, device=level.device)
+    _check(L.hdt_hpe(index.handle, level.data_ptr(), parent.data_ptr(), cu_seqlens.data_ptr(), n_levels, d_model, _DTYPES[x.dtype],
+                     int(bool(accumulate)), x.data_ptr(), workspace.data_ptr(), workspace.numel(), _stream()))
     return x
 
 
+@functools.lru_cache(maxsize=256)
 def hdt_cross_workspace_bytes(batch, total_tokens, total_q, heads, head_dim, dtype, bwd) -> int:
     L = lib()
-    L.hdt_cross_workspace_bytes.restype = C.c_size_t
-    L.hdt_cross_workspace_bytes.argtypes = [C.c_int32] * 7
     return int(L.hdt_cross_workspace_bytes(batch, total_tokens, total_q, heads, head_dim, _DTYPES[dtype], int(bwd)))
 
 
@@ -298,21 +317,17 @@ def hdt_cross_attn_fwd(level, cu_seqlens_k, cu_seqlens_q, level_mask, q, k, v, s
     """Decoder rows q [Tq,H,d] attend to the encoder rows of k, v [T,H,d] whose level bit is set in
     level_mask.  Returns (O [Tq,H,d], LSE [H,Tq])."""
     L = lib()
-    L.hdt_cross_attn_fwd.restype = C.c_int
-    L.hdt_cross_attn_fwd.argtypes = [C.c_void_p] * 3 + [C.c_int32] * 4 + [C.c_void_p] * 5 + [C.c_int32] * 3 + \
-                                    [C.c_float, C.c_void_p, C.c_size_t, C.c_void_p]
     B, T, Tq, H, d = _cross_common(level, cu_seqlens_k, cu_seqlens_q, q, k)
     assert q.is_contiguous() and k.is_contiguous() and v.is_contiguous()
     if out is None:
         out = torch.empty_like(q)
     if lse is None:
         lse = torch.empty((H, Tq), dtype=torch.float32, device=q.device)
-    need = hdt_cross_workspace_bytes(B, T, Tq, H, d, q.dtype, 0)
     if workspace is None:
-        workspace = torch.empty(need, dtype=torch.uint8, device=q.device)
-    _check(L.hdt_cross_attn_fwd(_ptr(level), _ptr(cu_seqlens_k), _ptr(cu_seqlens_q), B, T, Tq, int(level_mask), _ptr(q),
-                                _ptr(k), _ptr(v), _ptr(out), _ptr(lse), H, d, _DTYPES[q.dtype], float(softmax_scale),
-                                _ptr(workspace), workspace.numel(), _stream()))
+        workspace = torch.empty(hdt_cross_workspace_bytes(B, T, Tq, H, d, q.dtype, 0), dtype=torch.uint8, device=q.device)
+    _check(L.hdt_cross_attn_fwd(level.data_ptr(), cu_seqlens_k.data_ptr(), cu_seqlens_q.data_ptr(), B, T, Tq, int(level_mask), q.data_ptr(),
+                                k.data_ptr(), v.data_ptr(), out.data_ptr(), lse.data_ptr(), H, d, _DTYPES[q.dtype], float(softmax_scale),
+                                workspace.data_ptr(), workspace.numel(), _stream()))
     return out, lse
 
 
@@ -320,31 +335,25 @@ def hdt_cross_attn_bwd(level, cu_seqlens_k, cu_seqlens_q, level_mask, q, k, v, o
                        dk=None, dv=None, workspace=None):
     """Gradients (dQ [Tq,H,d], dK, dV [T,H,d]) of hdt_cross_attn_fwd."""
     L = lib()
-    L.hdt_cross_attn_bwd.restype = C.c_int
-    L.hdt_cross_attn_bwd.argtypes = [C.c_void_p] * 3 + [C.c_int32] * 4 + [C.c_void_p] * 9 + [C.c_int32] * 3 + \
-                                    [C.c_float, C.c_void_p, C.c_size_t, C.c_void_p]
     B, T, Tq, H, d = _cross_common(level, cu_seqlens_k, cu_seqlens_q, q, k)
     assert all(x.is_contiguous() for x in (q, k, v, o, do))
     dq = torch.empty_like(q) if dq is None else dq
     dk = torch.empty_like(k) if dk is None else dk
     dv = torch.empty_like(v) if dv is None else dv
-    need = hdt_cross_workspace_bytes(B, T, Tq, H, d, q.dtype, 1)
     if workspace is None:
-        workspace = torch.empty(need, dtype=torch.uint8, device=q.device)
-    _check(L.hdt_cross_attn_bwd(_ptr(level), _ptr(cu_seqlens_k), _ptr(cu_seqlens_q), B, T, Tq, int(level_mask), _ptr(q),
-                                _ptr(k), _ptr(v), _ptr(o), _ptr(lse), _ptr(do), _ptr(dq), _ptr(dk), _ptr(dv), H, d,
-                                _DTYPES[q.dtype], float(softmax_scale), _ptr(workspace), workspace.numel(), _stream()))
+        workspace = torch.empty(hdt_cross_workspace_bytes(B, T, Tq, H, d, q.dtype, 1), dtype=torch.uint8, device=q.device)
+    _check(L.hdt_cross_attn_bwd(level.data_ptr(), cu_seqlens_k.data_ptr(), cu_seqlens_q.data_ptr(), B, T, Tq, int(level_mask), q.data_ptr(),
+                                k.data_ptr(), v.data_ptr(), o.data_ptr(), lse.data_ptr(), do.data_ptr(), dq.data_ptr(), dk.data_ptr(), dv.data_ptr(), H, d,
+                                _DTYPES[q.dtype], float(softmax_scale), workspace.data_ptr(), workspace.numel(), _stream()))
     return dq, dk, dv
 
 
 def hdt_set_option(name: str, value: int) -> None:
-    lib().hdt_set_option.restype = C.c_int
     _check(lib().hdt_set_option(C.c_char_p(name.encode()), C.c_int32(int(value))))
 
 
 def hdt_device_status() -> None:
     """Wait for the current stream and raise if a kernel recorded a device-side failure."""
-    lib().hdt_device_status.restype = C.c_int
     _check(lib().hdt_device_status(_stream()))
 
 

@@ -52,10 +52,15 @@ ProfScope::~ProfScope() {
 __device__ int g_device_status[4] = {0, 0, 0, 0};  // [0] first failure recorded by a kernel (hdt_status_t), 0 = none; [1] where (kernel << 8 | wait site), [2] its loop count
 
 int *device_status_ptr() {
-    int *p = nullptr;
-    if (cudaGetSymbolAddress((void **)&p, g_device_status) != cudaSuccess) {
-        set_error(HDT_ERR_CUDA, "cudaGetSymbolAddress(g_device_status) failed");
-        return nullptr;
+    static std::atomic<int *> cache[64];        // per device ordinal
+    const int dev = DevOnce::cur();
+    int *p = cache[dev].load(std::memory_order_relaxed);
+    if (!p) {
+        if (cudaGetSymbolAddress((void **)&p, g_device_status) != cudaSuccess) {
+            set_error(HDT_ERR_CUDA, "cudaGetSymbolAddress(g_device_status) failed");
+            return nullptr;
+        }
+        cache[dev].store(p, std::memory_order_relaxed);
     }
     return p;
 }
@@ -292,14 +297,19 @@ extern "C" int hdt_attn_fwd(const hdt_index_t *ix, const void *q, const void *k,
     // queued before the host waits for the counts (it reads them on the device), so the GPU goes
     // from the build straight into the attention.  The stream is forked first: what the host
     // launches on the side streams after its wait still runs beside that kernel, not behind it.
-    bool early = false;
+    bool early = false, forked = false;
     std::unique_ptr<ProfScope> ps_early;      // stage 0's time when a kernel goes ahead: from its start to the end of the stage's other kernel
     if (ix->pending && ix->total_tokens > 0 && dtype == HDT_BF16 && !g_force_simt && g_no_persistent == 0 &&
         !g_no_overlap && ix->max_stages <= 8 && (workspace == nullptr || ((uintptr_t)workspace & 255) == 0)) {
-        Side *sd = nullptr;
-        rc = get_side(&sd);
-        if (rc) return rc;
-        HDT_CUDA_CHECK(cudaEventRecord(sd->fork, st));
+        // (A small batch will most likely need no side stream: its stages above 0 go row by row.  An event recorded
+        // between the build and this kernel would keep them from overlapping as programmatic dependents.)
+        if ((long long)ix->total_tokens * heads * (head_dim / 64) > 300000) {
+            Side *sd = nullptr;
+            rc = get_side(&sd);
+            if (rc) return rc;
+            HDT_CUDA_CHECK(cudaEventRecord(sd->fork, st));
+            forked = true;
+        }
         const StagePtrs &P = ix->st[0];
         FwdStageArgs a{};
         a.n = ix->total_tokens; a.H = heads; a.T = ix->total_tokens;
@@ -382,18 +392,20 @@ extern "C" int hdt_attn_fwd(const hdt_index_t *ix, const void *q, const void *k,
     // The stages above 0 do not depend on stage 0 until their results are merged: compute them on
     // the side stream while stage 0 runs, then finish each with an element-wise merge.
     const bool overlap = (ix->n_stages > 1 && !g_no_overlap) || early;
+    // Stage 0's blocks that are not self-contained, and whether their kernel runs beside the looping kernel (see below).
+    const int rest0 = ix->desc[0].nb - ix->desc[0].n_fused;
     if (overlap) {
         Side *sd = nullptr;
         rc = get_side(&sd);
         if (rc) return rc;
-        if (!early) HDT_CUDA_CHECK(cudaEventRecord(sd->fork, st));
+        if (!forked && (!up_rows || rest0 > 0)) HDT_CUDA_CHECK(cudaEventRecord(sd->fork, st));
         if (!up_rows) HDT_CUDA_CHECK(cudaStreamWaitEvent(sd->s, sd->fork, 0));
         const bool tc0 = dtype == HDT_BF16 && !g_force_simt;
         // Stage 0's blocks that are not self-contained (split families, EMPTY blocks) have a kernel of
         // their own.  Where the split families are the smaller part it runs on the second side stream beside the
         // looping kernel (measured: a batch of padded documents gains 7 %); where split families
         // dominate, one kernel after the other is faster (the skewed batch loses 3 % side by side).
-        const bool rest_beside = early || (tc0 && 2 * (ix->desc[0].nb - ix->desc[0].n_fused - ix->desc[0].n_empty) <= ix->desc[0].nb);
+        const bool rest_beside = rest0 > 0 && (early || (tc0 && 2 * (ix->desc[0].nb - ix->desc[0].n_fused - ix->desc[0].n_empty) <= ix->desc[0].nb));
         const bool two = ix->n_stages > 2 && !up_rows;
         if (two) HDT_CUDA_CHECK(cudaStreamWaitEvent(sd->s2, sd->fork, 0));
         // Stages above 0 of bf16 calls run on the gathering tensor-core kernels, whatever the depth of the
@@ -633,12 +645,12 @@ extern "C" int hdt_attn_bwd(const hdt_index_t *ix, const void *q, const void *k,
         Side *sd = nullptr;
         rc = get_side(&sd);
         if (rc) return rc;
-        HDT_CUDA_CHECK(cudaEventRecord(sd->fork, st));
-        if (!up_rows) HDT_CUDA_CHECK(cudaStreamWaitEvent(sd->s, sd->fork, 0));
         // (with the one-walk kernel the self-contained blocks' kernel goes to the second side stream: its CTAs take
         // the SMs that the one-walk kernel's CTAs leave first, and it shares HBM with the pass that converts dQ)
         const bool self_beside = dq_acc != nullptr && ix->desc[0].n_fused > 0 && !g_no_self_beside;
         const bool two = (ix->n_stages > 2 && !up_rows) || self_beside;
+        if (!up_rows || two) HDT_CUDA_CHECK(cudaEventRecord(sd->fork, st));
+        if (!up_rows) HDT_CUDA_CHECK(cudaStreamWaitEvent(sd->s, sd->fork, 0));
         if (two) HDT_CUDA_CHECK(cudaStreamWaitEvent(sd->s2, sd->fork, 0));
         ChainArgs c{};
         c.n1 = ix->desc[1].n; c.H = heads; c.T = ix->total_tokens; c.n_stages = ix->n_stages; c.nt = 3;

@@ -26,8 +26,9 @@ inline EncodeTiledFn encode_fn() {
 }
 
 // A tensor map is a function of (address, extents, box) only, and a training loop comes back with the
-// same tensors step after step: each host thread keeps the maps it made in a small direct-mapped
-// table (a call of the attention makes some thirty of them).
+// same tensors step after step: each host thread keeps the maps it made in a direct-mapped table (a call of the
+// attention makes ten to thirty of them; encoding one costs the host about 0.4 us.  1024 entries: a dozen layers
+// with tensors of their own collided in 128).
 struct TmapEntry {
     alignas(64) CUtensorMap map;
     const void *base;
@@ -35,10 +36,10 @@ struct TmapEntry {
     int D, H, box_rows, kind;      // kind: 1 = bf16 [T, H, D], 2 = fp32 accumulation buffer; 0 = empty
 };
 inline TmapEntry *tmap_slot(const void *base, int D, int H, long long T, int box_rows, int kind, bool *hit) {
-    static thread_local TmapEntry table[128];
+    static thread_local TmapEntry table[1024];
     const uintptr_t a = (uintptr_t)base;
     const unsigned h = (unsigned)((a >> 8) * 0x9E3779B1u) ^ ((unsigned)box_rows * 0x85EBCA6Bu) ^ ((unsigned)kind << 5) ^ (unsigned)D;
-    TmapEntry *e = &table[(h ^ (h >> 15)) & 127u];
+    TmapEntry *e = &table[(h ^ (h >> 15)) & 1023u];
     *hit = e->kind == kind && e->base == base && e->T == T && e->D == D && e->H == H && e->box_rows == box_rows;
     return e;
 }
