@@ -394,18 +394,21 @@ extern "C" int hdt_attn_fwd(const hdt_index_t *ix, const void *q, const void *k,
     const bool overlap = (ix->n_stages > 1 && !g_no_overlap) || early;
     // Stage 0's blocks that are not self-contained, and whether their kernel runs beside the looping kernel (see below).
     const int rest0 = ix->desc[0].nb - ix->desc[0].n_fused;
+    // Nothing but EMPTY blocks (padded batches) in front of the row-wise kernel: their zero rows are written by a
+    // programmatic dependent of the looping kernel on the caller's stream, beside its last CTAs.
+    const bool rest_main = up_rows && rest0 > 0 && rest0 == ix->desc[0].n_empty && dtype == HDT_BF16 && !g_force_simt && !g_no_fwd_mc;
     if (overlap) {
         Side *sd = nullptr;
         rc = get_side(&sd);
         if (rc) return rc;
-        if (!forked && (!up_rows || rest0 > 0)) HDT_CUDA_CHECK(cudaEventRecord(sd->fork, st));
+        if (!forked && (!up_rows || (rest0 > 0 && !rest_main))) HDT_CUDA_CHECK(cudaEventRecord(sd->fork, st));
         if (!up_rows) HDT_CUDA_CHECK(cudaStreamWaitEvent(sd->s, sd->fork, 0));
         const bool tc0 = dtype == HDT_BF16 && !g_force_simt;
         // Stage 0's blocks that are not self-contained (split families, EMPTY blocks) have a kernel of
         // their own.  Where the split families are the smaller part it runs on the second side stream beside the
         // looping kernel (measured: a batch of padded documents gains 7 %); where split families
         // dominate, one kernel after the other is faster (the skewed batch loses 3 % side by side).
-        const bool rest_beside = rest0 > 0 && (early || (tc0 && 2 * (ix->desc[0].nb - ix->desc[0].n_fused - ix->desc[0].n_empty) <= ix->desc[0].nb));
+        const bool rest_beside = rest0 > 0 && !rest_main && (early || (tc0 && 2 * (ix->desc[0].nb - ix->desc[0].n_fused - ix->desc[0].n_empty) <= ix->desc[0].nb));
         const bool two = ix->n_stages > 2 && !up_rows;
         if (two) HDT_CUDA_CHECK(cudaStreamWaitEvent(sd->s2, sd->fork, 0));
         // Stages above 0 of bf16 calls run on the gathering tensor-core kernels, whatever the depth of the
@@ -473,7 +476,7 @@ extern "C" int hdt_attn_fwd(const hdt_index_t *ix, const void *q, const void *k,
         {   // stage 0 after the small side kernels are queued: they take their SM share first (the
             // stage-0 kernel would otherwise fill every SM and push them behind itself)
             FwdStageArgs a = stage_args(0);
-            a.part = rest_beside ? 1 : 0;
+            a.part = rest_beside || rest_main ? 1 : 0;
             if (!early) {                    // (early: already queued)
                 ProfScope ps(PROF_FWD_STAGE0, st);
                 if (tc0) rc = launch_fwd_tc(a, head_dim, st);
@@ -481,6 +484,13 @@ extern "C" int hdt_attn_fwd(const hdt_index_t *ix, const void *q, const void *k,
                 else rc = launch_fwd_simt(a, head_dim, dtype, st);
                 if (rc) return rc;
             }
+        }
+        if (rest_main) {
+            FwdStageArgs a = stage_args(0);
+            a.part = 2;
+            a.pdl = 1;
+            rc = launch_fwd_tc(a, head_dim, st);
+            if (rc) return rc;
         }
         if (ix->n_stages == 1) {             // (early only) nothing to merge: wait for the other blocks' kernel
             if (two) HDT_CUDA_CHECK(cudaStreamWaitEvent(st, sd->join2, 0));

@@ -147,28 +147,81 @@ __global__ void __launch_bounds__(128) k_fwd_tc(const __grid_constant__ CUtensor
     const bool empty = (fl & HDT_BLK_EMPTY) != 0 || ka >= kb;
     const bool dead = (*abort_flag != 0);   // same value in every thread: read after the barrier
 
+    // A gathering walk over several chunks keeps one ahead in registers: its K and V rows are requested before a
+    // chunk's S and stored behind its P V, their token numbers one chunk earlier, so no chunk waits for global memory.
+    // Thread t holds 16-byte chunk t % 8 of rows t / 8 + 16 p.
+    constexpr bool AHEAD = GATHER && !SINGLE;
+    const int g_c = tid & 7, g_r = tid >> 3;
+    int tk_n[AHEAD ? 8 : 1];
+    uint4 k_n[AHEAD ? NSUB : 1][AHEAD ? 8 : 1], v_n[AHEAD ? NSUB : 1][AHEAD ? 8 : 1];
+    auto ahead_tok = [&](int row0) {
+#pragma unroll
+        for (int p = 0; p < 8; ++p) {
+            const int e = row0 + g_r + 16 * p;
+            tk_n[p] = e < kb ? a.tok[e] : -1;
+        }
+    };
+    auto ahead_rows = [&](const void *src, auto &v) {
+        const __nv_bfloat16 *g = reinterpret_cast<const __nv_bfloat16 *>(src);
+#pragma unroll
+        for (int t = 0; t < NSUB; ++t)
+#pragma unroll
+            for (int p = 0; p < 8; ++p) {
+                v[t][p] = make_uint4(0u, 0u, 0u, 0u);
+                if (tk_n[p] >= 0) v[t][p] = *reinterpret_cast<const uint4 *>(g + ((size_t)tk_n[p] * H + h) * D + t * 64 + g_c * 8);
+            }
+    };
+    auto put_rows = [&](uint8_t *dst, const auto &v) {
+#pragma unroll
+        for (int t = 0; t < NSUB; ++t)
+#pragma unroll
+            for (int p = 0; p < 8; ++p) *reinterpret_cast<uint4 *>(dst + t * SUB + swz(g_r + 16 * p, g_c)) = v[t][p];
+    };
+    const bool own_keys = ka == r0 && kb == r1;      // keys = the block's own rows: one round of loads for all three tensors
+    if constexpr (AHEAD) {
+        if (!empty && !dead && !own_keys) {
+            ahead_tok(ka);
+            ahead_rows(a.k, k_n);
+            ahead_rows(a.v, v_n);
+            if (ka + 128 < kb) ahead_tok(ka + 128);
+        }
+    }
+
     if (!empty && !dead) {
         for (int c0 = ka; c0 < kb; c0 += 128) {
             const int nvalid = min(128, kb - c0);
             const int Nc = (nvalid + 15) & ~15;
             const bool first = (c0 == ka);
             if constexpr (GATHER) {
-                if (first && ka == r0 && kb == r1) {     // keys = the block's own rows: one round of loads for all three
+                if (own_keys) {
                     uint8_t *const d3[3] = {sQ, sK, sV};
                     const void *const s3[3] = {a.q, a.k, a.v};
                     gather_tiles<D, 128, 3>(d3, s3, a.tok, r0, r1, H, h, tid);
-                } else {
+                } else if constexpr (AHEAD) {
                     if (first) {
                         uint8_t *const dq_[1] = {sQ};
                         const void *const sq_[1] = {a.q};
                         gather_tiles<D, 128, 1>(dq_, sq_, a.tok, r0, r1, H, h, tid);
                     }
+                    put_rows(sK, k_n);
+                    put_rows(sV, v_n);
+                } else {
+                    uint8_t *const dq_[1] = {sQ};
+                    const void *const sq_[1] = {a.q};
+                    gather_tiles<D, 128, 1>(dq_, sq_, a.tok, r0, r1, H, h, tid);
                     uint8_t *const dkv[2] = {sK, sV};
                     const void *const skv[2] = {a.k, a.v};
                     gather_tiles<D, 128, 2>(dkv, skv, a.tok, c0, kb, H, h, tid);
                 }
                 fence_proxy_async_smem();     // generic-proxy writes, read by the MMA
                 __syncthreads();
+                if constexpr (AHEAD) {
+                    if (c0 + 128 < kb) {
+                        ahead_rows(a.k, k_n);
+                        ahead_rows(a.v, v_n);
+                        if (c0 + 256 < kb) ahead_tok(c0 + 256);
+                    }
+                }
             } else if constexpr (PIPE) {
                 const int ci = (c0 - ka) >> 7;
                 if (tid == 0 && !*abort_flag) {   // after a failed wait nothing new is issued
@@ -201,7 +254,7 @@ __global__ void __launch_bounds__(128) k_fwd_tc(const __grid_constant__ CUtensor
                 if (!mbar_wait(bar_tma, ph_tma, abort_flag, WAIT_CYCLES)) { ok = false; if (a.status[1] == 0) a.status[1] = (1 << 8) | 2; }
                 ph_tma ^= 1;
             }
-            if (tid == 0 && !*abort_flag) {
+            if (warp == 0 && !*abort_flag && elect_one()) {
                 tc_fence_after();
                 const uint32_t idesc = idesc_bf16(Nc, false, false);
 #pragma unroll
@@ -292,7 +345,7 @@ __global__ void __launch_bounds__(128) k_fwd_tc(const __grid_constant__ CUtensor
             fence_proxy_async_smem();
             tc_fence_before();
             __syncthreads();
-            if (tid == 0 && !*abort_flag) {
+            if (warp == 0 && !*abort_flag && elect_one()) {
                 tc_fence_after();
                 const uint32_t idesc = idesc_bf16(D, false, true);
                 for (int kk = 0; kk < Nc / 16; ++kk) {
@@ -1396,9 +1449,13 @@ __global__ void __launch_bounds__(256, 2) k_fwd_tc_mc(const __grid_constant__ CU
 // SM's TMEM and most of its shared memory).  Blocks of the list that are not EMPTY are skipped.
 template <int D>
 __global__ void __launch_bounds__(128) k_fwd_empty(const FwdStageArgs a) {
+    if (a.pdl) pdl_launch_dependents();
     const int blk = a.rest_only ? a.queue_split[a.n_fused + blockIdx.x] : a.queue[blockIdx.x];
     const int *rec = a.blocks + 5 * (size_t)blk;
-    if (!(rec[4] & HDT_BLK_EMPTY)) return;
+    if (!(rec[4] & HDT_BLK_EMPTY)) {
+        if (a.pdl) pdl_wait();
+        return;
+    }
     const int r0 = rec[0], nrows = rec[1] - r0, h = blockIdx.y, H = a.H;
     __nv_bfloat16 *og = reinterpret_cast<__nv_bfloat16 *>(a.o);
     const uint4 z4 = make_uint4(0u, 0u, 0u, 0u);
@@ -1418,6 +1475,7 @@ __global__ void __launch_bounds__(128) k_fwd_empty(const FwdStageArgs a) {
             }
         }
     }
+    if (a.pdl) pdl_wait();      // (it depends on nothing the kernel before it does, but what follows takes its end for that kernel's end too)
 }
 
 template <int D>
@@ -1508,7 +1566,7 @@ static int launch_fwd_tc_t(const FwdStageArgs &a, cudaStream_t st) {
     if (a.part == 1 && split_launch) n_general = 0;     // the caller launches the other blocks separately
     if (n_general > 0) {
         dim3 grid(n_general, a.H);
-        if (a.n_empty == n_general && !g_no_fwd_mc) k_fwd_empty<D><<<grid, 128, 0, st>>>(b);   // nothing but EMPTY blocks left
+        if (a.n_empty == n_general && !g_no_fwd_mc) HDT_CUDA_CHECK(launch_dependent(k_fwd_empty<D>, b.pdl != 0, grid, 128, 0, st, b));   // nothing but EMPTY blocks left
         else if (dirs) k_fwd_tc<D, false, false, true><<<grid, 128, smem, st>>>(tq, tk, tv, b);
 #ifdef HDT_WORKBENCH
         else if (D == 64 && !g_no_fwd_mc && g_phase_stamps == 2) k_fwd_tc_mc<true><<<grid, 256, smem_mc, st>>>(tq, tk, tv, b);

@@ -180,7 +180,8 @@ __global__ void __launch_bounds__(256) k_bwd_tc(const __grid_constant__ CUtensor
     const int *rec = a.blocks + 5 * (size_t)blk;
     const int r0 = rec[0], r1 = rec[1], fl = rec[4];
     int ka = rec[2], kb = rec[3];
-    int phases = a.phases, final_merge = a.final_merge;
+    int phases = a.phases;
+    int final_merge = a.final_merge;
     if constexpr (GATHER) {
         if (r1 <= r0) continue;             // a block slot that is not in use
         if (a.phase_split > 0) {
@@ -197,17 +198,37 @@ __global__ void __launch_bounds__(256) k_bwd_tc(const __grid_constant__ CUtensor
     const bool empty = (fl & HDT_BLK_EMPTY) != 0 || ka >= kb;
     const bool self = (fl & HDT_BLK_SELF) != 0;
     const bool fused = self && !empty && !dead;   // one pass yields dQ, dK and dV
+    if constexpr (GATHER) {
+        if (gridDim.z == 2) {               // the two walks of a block in two CTAs
+            if (!self && !empty) phases = (int)blockIdx.z + 1;
+            else if (blockIdx.z) continue;
+        }
+    }
     const uint32_t TM_DK = (D == 64) ? 320u : (fused ? 128u : 256u);
     const uint32_t TM_DV = (D == 64) ? 384u : (fused ? 0u : 384u);
     bool ok = true;
 
+    // Key range, LSE and delta of query-side row e (token tk).
+    struct Stat { int lo, hi; float lse2, dl; };
+    auto stat_of = [&](int e, int end, int tk) {
+        Stat t{0, 0, 0.f, 0.f};
+        if (e < end) {
+            t.lo = a.rng[2 * e];
+            t.hi = a.rng[2 * e + 1];
+            t.lse2 = a.lse[(size_t)h * a.T + tk] * LOG2E;
+            if (a.delta != nullptr) t.dl = a.delta[(size_t)h * a.T + tk];
+        }
+        return t;
+    };
+    auto token_of = [&](int e, int end) { return e < end ? (GATHER ? a.tok[e] : e) : 0; };
+
     // One tile pass.  q_row0 / k_row0: first token row of the query-side / key-side tile;
-    // q_end / k_end: end of the valid rows of each side.
+    // q_end / k_end: end of the valid rows of each side; stat(): the statistics of this thread's query-side row.
     auto tile_pass = [&](int q_row0, int q_end, int k_row0, int k_end, bool want_dq, bool want_dkdv, bool acc_q,
-                         bool acc_kv) {
+                         bool acc_kv, auto stat) {
         const int nq = min(128, q_end - q_row0), nk = min(128, k_end - k_row0);
         const int Nc = (nk + 15) & ~15, Kr = (nq + 15) & ~15;
-        if (tid == 0 && !*abort_flag) {
+        if (warp == 0 && !*abort_flag && elect_one()) {
             tc_fence_after();
             const uint32_t idesc = idesc_bf16(Nc, false, false);
 #pragma unroll
@@ -227,18 +248,9 @@ __global__ void __launch_bounds__(256) k_bwd_tc(const __grid_constant__ CUtensor
         // row statistics of this thread's query-side row while the MMAs run
         const int e = q_row0 + rl;
         const bool inq = e < q_end;
-        int lo = 0, hi = 0;
-        float lse2 = 0.f, dl = 0.f;
-        if (inq) {
-            lo = a.rng[2 * e];
-            hi = a.rng[2 * e + 1];
-            if (hi > lo) {
-                const int tk = GATHER ? a.tok[e] : e;
-                lse2 = a.lse[(size_t)h * a.T + tk] * LOG2E;
-                if (a.delta != nullptr) dl = a.delta[(size_t)h * a.T + tk];
-                else dl = s_delta[rl];      // no delta pass ran: left by the gather of the query-side rows
-            }
-        }
+        const Stat rs_ = stat();
+        const int lo = rs_.lo, hi = rs_.hi;
+        const float lse2 = rs_.lse2, dl = (GATHER && a.delta == nullptr) ? s_delta[rl] : rs_.dl;   // (no delta pass ran: left by the gather of the query-side rows)
         const int jl = max(lo - k_row0, 0), jh = min(hi - k_row0, nk);
         const bool has = inq && jh > jl;
         // direction bits: column of the row itself, of its parent (none for a head row), and
@@ -289,7 +301,7 @@ __global__ void __launch_bounds__(256) k_bwd_tc(const __grid_constant__ CUtensor
         fence_proxy_async_smem();
         tc_fence_before();
         __syncthreads();
-        if (tid == 0 && !*abort_flag) {
+        if (warp == 0 && !*abort_flag && elect_one()) {
             tc_fence_after();
             const uint32_t idesc_kv = idesc_bf16(D, true, true);   // A = P^T / dS^T, B = dO / Q (both MN-major)
             const uint32_t idesc_q = idesc_bf16(D, false, true);   // A = dS (K-major), B = K (MN-major)
@@ -489,9 +501,39 @@ __global__ void __launch_bounds__(256) k_bwd_tc(const __grid_constant__ CUtensor
         }
     }
 
+    // The walks of the gathering kernel keep one tile ahead in registers: its rows are requested before a tile pass
+    // and stored behind it, their token numbers one tile earlier, so no pass waits for global memory.
+    // Thread t holds 16-byte chunk t % 8 of rows t / 8 + 32 p of both tensors of a side.
+    const int g_c = tid & 7, g_r = tid >> 3;
+    auto ahead_tok = [&](int row0, int end, int (&tk)[4]) {
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+            const int e = row0 + g_r + 32 * p;
+            tk[p] = e < end ? a.tok[e] : -1;
+        }
+    };
+    auto ahead_rows = [&](const void *src, const int (&tk)[4], uint4 (&v)[NSUB][4]) {
+        const __nv_bfloat16 *g = reinterpret_cast<const __nv_bfloat16 *>(src);
+#pragma unroll
+        for (int t = 0; t < NSUB; ++t)
+#pragma unroll
+            for (int p = 0; p < 4; ++p) {
+                v[t][p] = make_uint4(0u, 0u, 0u, 0u);
+                if (tk[p] >= 0) v[t][p] = *reinterpret_cast<const uint4 *>(g + ((size_t)tk[p] * H + h) * D + t * 64 + g_c * 8);
+            }
+    };
+    auto put_rows = [&](uint8_t *dst, const uint4 (&v)[NSUB][4]) {
+#pragma unroll
+        for (int t = 0; t < NSUB; ++t)
+#pragma unroll
+            for (int p = 0; p < 4; ++p) *reinterpret_cast<uint4 *>(dst + t * SUB + swz(g_r + 32 * p, g_c)) = v[t][p];
+    };
+
     if (fused) {
+        Stat st{};
+        if constexpr (GATHER) st = stat_of(row, r1, token_of(row, r1));      // (in flight beside the gather)
         load(true, r0, true, r0);
-        tile_pass(r0, r1, r0, r1, true, true, false, false);
+        tile_pass(r0, r1, r0, r1, true, true, false, false, [&]() { return GATHER ? st : stat_of(row, r1, token_of(row, r1)); });
         if (!ok && tid == 0) atomicCAS(a.status, 0, HDT_ERR_TIMEOUT);
         if (fin) {
             drain_final(TM_DQ, true, a.scale, fb[0], fn[0], fo[0]);
@@ -505,14 +547,39 @@ __global__ void __launch_bounds__(256) k_bwd_tc(const __grid_constant__ CUtensor
     } else {
         if (run && (!GATHER || phases != 2)) {
             // this block as query rows: dQ over the key span
-            load(true, r0, false, 0);
-            for (int c0 = ka; c0 < kb; c0 += 128) {
-                load(false, 0, true, c0);
-                tile_pass(r0, r1, c0, kb, true, false, c0 > ka, false);
+            if constexpr (GATHER) {
+                const int end_k = a.gather_end_k ? a.gather_end_k : a.n;
+                int tk[4];
+                uint4 v0[NSUB][4], v1[NSUB][4];
+                ahead_tok(ka, end_k, tk);
+                const int tkr = token_of(row, r1);
+                ahead_rows(a.k, tk, v0);
+                ahead_rows(a.v, tk, v1);
+                if (ka + 128 < kb) ahead_tok(ka + 128, end_k, tk);
+                const Stat st = stat_of(row, r1, tkr);
+                load(true, r0, false, 0);
+                for (int c0 = ka; c0 < kb; c0 += 128) {
+                    put_rows(sK, v0);
+                    put_rows(sV, v1);
+                    fence_proxy_async_smem();     // generic-proxy writes, read by the MMAs
+                    __syncthreads();
+                    if (c0 + 128 < kb) {
+                        ahead_rows(a.k, tk, v0);
+                        ahead_rows(a.v, tk, v1);
+                        if (c0 + 256 < kb) ahead_tok(c0 + 256, end_k, tk);
+                    }
+                    tile_pass(r0, r1, c0, kb, true, false, c0 > ka, false, [&]() { return st; });
+                }
+            } else {
+                load(true, r0, false, 0);
+                for (int c0 = ka; c0 < kb; c0 += 128) {
+                    load(false, 0, true, c0);
+                    tile_pass(r0, r1, c0, kb, true, false, c0 > ka, false, [&]() { return stat_of(row, r1, row); });
+                }
             }
         }
         if (fin) drain_final(TM_DQ, run, a.scale, fb[0], fn[0], fo[0]);
-        else drain(TM_DQ, run, a.scale, cq, sP);
+        else if (!GATHER || phases != 2) drain(TM_DQ, run, a.scale, cq, sP);
         // dQ leaves now: the second walk reuses sP and (at D = 128) the dQ columns of TMEM
         tc_fence_before();
         __syncthreads();
@@ -521,10 +588,61 @@ __global__ void __launch_bounds__(256) k_bwd_tc(const __grid_constant__ CUtensor
         __syncthreads();
         if (run && (!GATHER || phases != 1)) {
             // this block as keys: dK, dV over the same span taken as query rows
-            load(false, 0, true, r0);
-            for (int c0 = ka; c0 < kb; c0 += 128) {
-                load(true, c0, false, 0);
-                tile_pass(c0, kb, r0, r1, false, true, false, c0 > ka);
+            if constexpr (GATHER) {
+                const int end_q = a.gather_end_q ? a.gather_end_q : a.n;
+                const bool need_delta = a.delta == nullptr;
+                int tk[4];
+                uint4 v0[NSUB][4], v1[NSUB][4], vo[NSUB][4];
+                ahead_tok(ka, end_q, tk);
+                int tkr = token_of(ka + rl, kb);
+                ahead_rows(a.q, tk, v0);
+                ahead_rows(a.d_o, tk, v1);
+                if (need_delta) ahead_rows(a.o, tk, vo);
+                if (ka + 128 < kb) ahead_tok(ka + 128, end_q, tk);
+                Stat st = stat_of(ka + rl, kb, tkr);
+                tkr = token_of(ka + 128 + rl, kb);
+                load(false, 0, true, r0);
+                for (int c0 = ka; c0 < kb; c0 += 128) {
+                    put_rows(sQ, v0);
+                    put_rows(sDO, v1);
+                    if (need_delta) {
+#pragma unroll
+                        for (int p = 0; p < 4; ++p) {
+                            float x = 0.f;
+#pragma unroll
+                            for (int t = 0; t < NSUB; ++t) {
+                                const uint32_t xs[4] = {vo[t][p].x, vo[t][p].y, vo[t][p].z, vo[t][p].w}, ys[4] = {v1[t][p].x, v1[t][p].y, v1[t][p].z, v1[t][p].w};
+#pragma unroll
+                                for (int w = 0; w < 4; ++w) {
+                                    x = fmaf(__uint_as_float(xs[w] << 16), __uint_as_float(ys[w] << 16), x);
+                                    x = fmaf(__uint_as_float(xs[w] & 0xffff0000u), __uint_as_float(ys[w] & 0xffff0000u), x);
+                                }
+                            }
+                            x += __shfl_xor_sync(0xffffffffu, x, 1);
+                            x += __shfl_xor_sync(0xffffffffu, x, 2);
+                            x += __shfl_xor_sync(0xffffffffu, x, 4);
+                            if (g_c == 0) s_delta[g_r + 32 * p] = x;
+                        }
+                    }
+                    fence_proxy_async_smem();
+                    __syncthreads();
+                    const Stat cur = st;
+                    if (c0 + 128 < kb) {
+                        ahead_rows(a.q, tk, v0);
+                        ahead_rows(a.d_o, tk, v1);
+                        if (need_delta) ahead_rows(a.o, tk, vo);
+                        if (c0 + 256 < kb) ahead_tok(c0 + 256, end_q, tk);
+                        st = stat_of(c0 + 128 + rl, kb, tkr);
+                        tkr = token_of(c0 + 256 + rl, kb);
+                    }
+                    tile_pass(c0, kb, r0, r1, false, true, false, c0 > ka, [&]() { return cur; });
+                }
+            } else {
+                load(false, 0, true, r0);
+                for (int c0 = ka; c0 < kb; c0 += 128) {
+                    load(true, c0, false, 0);
+                    tile_pass(c0, kb, r0, r1, false, true, false, c0 > ka, [&]() { return stat_of(c0 + rl, kb, c0 + rl); });
+                }
             }
             if (!ok && tid == 0) atomicCAS(a.status, 0, HDT_ERR_TIMEOUT);
         }
@@ -1462,9 +1580,11 @@ static int launch_bwd_tc_upper_t(const BwdStageArgs &a, cudaStream_t st) {
     // (phase_split: the blocks of the queries, and of the others two CTAs per SM; an unused slot costs its CTA two loads)
     int grid_x = a.nb;
     if (a.phase_split > 0) grid_x = min(a.phase_split * (b.splits - 1) + a.nb, a.phase_split * b.splits + (2 * 148 + a.H - 1) / a.H);
-    if (a.dirs != 7) k_bwd_tc<D, true, true><<<dim3(a.nb, a.H), 256, smem, st>>>(tq, tq, tq, tq, b);      // direction bits
+    // (families longer than a block: the dQ walk and the dK / dV walk of such a block in CTAs of their own)
+    const unsigned grid_z = a.phase_split == 0 && a.phases == 0 && !a.final_merge && a.n_fused + a.n_empty < a.nb ? 2u : 1u;
+    if (a.dirs != 7) k_bwd_tc<D, true, true><<<dim3(a.nb, a.H, grid_z), 256, smem, st>>>(tq, tq, tq, tq, b);      // direction bits
     else {
-        HDT_CUDA_CHECK(launch_dependent(k_bwd_tc<D, true>, a.pdl != 0, dim3(grid_x, a.H), 256, smem, st, tq, tq, tq, tq, b));
+        HDT_CUDA_CHECK(launch_dependent(k_bwd_tc<D, true>, a.pdl != 0, dim3(grid_x, a.H, grid_z), 256, smem, st, tq, tq, tq, tq, b));
         return HDT_OK;
     }
     count_launch();
