@@ -158,7 +158,7 @@ __device__ __forceinline__ void count_children(const A &cnt, unsigned p, int lan
 
 static constexpr int SEQ_CAP_MAX = 32768;   // tokens of a sequence held in shared memory (15-bit counts)
 static constexpr int UC_MAX = 4096;         // elements of an upper stage held there
-static constexpr int SB0 = 1024, SBU = 256, SBW = 64; // block starts of stage 0 / an upper stage (by the CTA, by a warp) held there
+static constexpr int SB0 = 1024, SBU = 256, SBA = 1024; // block starts of stage 0 / an upper stage / all upper stages held there
 static constexpr int SEQ_CLUSTER = 8;       // CTAs of a long sequence
 
 struct SeqArgs {
@@ -182,7 +182,7 @@ struct SeqShared {
     int bst0[SB0], bst[SBU];
     int wtot[32], wtotu[32], ctot[SEQ_CLUSTER];
     int err, err_pos, real, flag0, flag, nb0, nb, nf0, ne0, nf, ne;
-    int ns[HDT_MAX_STAGES], bsw[16][SBW], nfs[16], nes[16];     // (seq_upper_all)
+    int ns[HDT_MAX_STAGES], nbs[HDT_MAX_STAGES], bso[HDT_MAX_STAGES], nfs[HDT_MAX_STAGES], nes[HDT_MAX_STAGES], bsu[SBA];     // (seq_upper_all)
     unsigned long long nnz, nnz_upper, vis;
 };
 
@@ -192,9 +192,10 @@ __device__ __forceinline__ void seq_fail(SeqShared *sh, int pos) {
 
 // Barrier of the warps that build the upper stages (with one CTA per sequence its last warp meanwhile walks stage 0's blocks).
 __device__ __forceinline__ void bar_upper(int n) { asm volatile("bar.sync 1, %0;" ::"r"(n) : "memory"); }
+__device__ __forceinline__ void cluster_arrive() { __syncwarp(); asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { __syncwarp(); asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void seq_sync(unsigned cs) {
-    __syncwarp();
-    if (cs > 1) asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (cs > 1) { cluster_arrive(); cluster_wait(); }
     else __syncthreads();
 }
 
@@ -233,16 +234,17 @@ __device__ __forceinline__ int walk_blocks(const uint8_t *fpos, int n, int bm, i
     return nb;
 }
 
-// Records of the blocks i = i0, i0 + di, ... < i1 of a stage with nb blocks and n elements, one warp per block.
-// get(e, lo, hi) gives the range of an element and returns whether it lives on.  (The loops stay rolled: nearly
+// Records of the blocks block(v), v = v0, v0 + dv, ... < v1, of a stage with nb blocks and n elements, one warp per
+// block.  get(e, lo, hi) gives the range of an element and returns whether it lives on.  (The loops stay rolled: nearly
 // every instruction of this kernel is executed once or twice by a warp, and fetching it costs more than that.)
-template <class Get>
-__device__ __forceinline__ void make_records(Get get, int n, int nb, const int *bst, int nbst, int4 *rec, int i0, int i1, int di, int lane, int *nf,
-                                             int *ne, unsigned long long *vis_out) {
+template <class Get, class Block>
+__device__ __forceinline__ void make_records(Get get, int n, int nb, const int *bst, int nbst, int4 *rec, int v0, int v1, int dv, Block block, int lane,
+                                             int *nf, int *ne, unsigned long long *vis_out) {
     long long vis = 0;
     int mf = 0, me = 0;
 #pragma unroll 1
-    for (int i = i0; i < i1; i += di) {
+    for (int v = v0; v < v1; v += dv) {
+        const int i = block(v);
         const int r0 = i < nbst ? bst[i] : rec[i].x;
         const int r1 = (i + 1 < nb) ? (i + 1 < nbst ? bst[i + 1] : rec[i + 1].x) : n;
         // a block is dense where all its rows have one range
@@ -507,7 +509,7 @@ __device__ __forceinline__ void seq_upper(const SeqArgs &a, SeqShared &sh, J *pa
                          lo = (int)l; hi = (int)h;
                          return !child;
                      },
-                     n, sh.nb, sh.bst, SBU, rec, w, sh.nb, nw, lane, &sh.nf, &sh.ne, &sh.vis);
+                     n, sh.nb, sh.bst, SBU, rec, w, sh.nb, nw, [](int v) { return v; }, lane, &sh.nf, &sh.ne, &sh.vis);
         bar_upper(tu);
         if (t == 0) {
             int *c = a.counts + (size_t)s * a.B + b;
@@ -616,28 +618,34 @@ __device__ __forceinline__ bool seq_upper_all(const SeqArgs &a, SeqShared &sh, c
     for (int o = 16; o; o >>= 1) deg += __shfl_xor_sync(0xffffffffu, deg, o);
     if (lane == 0 && deg) atomicAdd(&sh.nnz_upper, (unsigned long long)deg);
     bar_upper(tu);
-    for (int s = 1 + w; s < S; s += nw) {          // a warp per stage: its blocks
-        int4 *rec = a.recs + (size_t)s * a.capnb + slot;
+    for (int s = 1 + w; s < S; s += nw) {          // a warp per stage: where its blocks start
+        if (lane == 0) {
+            int o = 0;
+            for (int i = 1; i < s; ++i) o += 2 * (sh.ns[i] / a.bmu) + 2;
+            sh.bso[s] = o;
+            sh.nbs[s] = walk_blocks(fp + s * (size_t)n2, sh.ns[s], a.bmu, sh.bsu + min(o, SBA), max(SBA - o, 0), a.recs + (size_t)s * a.capnb + slot);
+            sh.nfs[s] = 0; sh.nes[s] = 0;
+        }
+    }
+    bar_upper(tu);
+    const int split = max(nw / max(S - 1, 1), 1);     // warps that share a stage
+#pragma unroll 1
+    for (int s = 1 + w / split; s < S; s += nw / split) {
         const int4 *el = a.el + (size_t)(s - 1) * a.T + s0;
         const int *upl = a.upl + (size_t)(s - 1) * a.T + s0;
-        const int ns = sh.ns[s];
-        int *bst = sh.bsw[w];
-        int nb = 0;
-        if (lane == 0) nb = walk_blocks(fp + s * (size_t)n2, ns, a.bmu, bst, SBW, rec);
-        nb = __shfl_sync(0xffffffffu, nb, 0);
-        if (lane == 0) { sh.nfs[w] = 0; sh.nes[w] = 0; }
-        __syncwarp();
+        const int nb = sh.nbs[s], o = sh.bso[s];
         make_records([&](int e, int &lo, int &hi) {
             const int4 x = el[e];
             lo = x.z; hi = x.w;
             return upl[e] >= 0;
-        }, ns, nb, bst, SBW, rec, 0, nb, 1, lane, &sh.nfs[w], &sh.nes[w], &sh.vis);
-        if (lane == 0) {
-            int *c = a.counts + (size_t)s * a.B + b;
-            const size_t q = (size_t)a.ms * a.B;
-            c[0] = ns; c[q] = nb; c[2 * q] = sh.nfs[w]; c[3 * q] = sh.nes[w];
-        }
-        __syncwarp();
+        }, sh.ns[s], nb, sh.bsu + min(o, SBA), max(SBA - o, 0), a.recs + (size_t)s * a.capnb + slot, w % split, nb, split,
+           [](int v) { return v; }, lane, &sh.nfs[s], &sh.nes[s], &sh.vis);
+    }
+    bar_upper(tu);
+    for (int s = 1 + t; s < S; s += tu) {
+        int *c = a.counts + (size_t)s * a.B + b;
+        const size_t q = (size_t)a.ms * a.B;
+        c[0] = sh.ns[s]; c[q] = sh.nbs[s]; c[2 * q] = sh.nfs[s]; c[3 * q] = sh.nes[s];
     }
     return true;
 }
@@ -706,6 +714,10 @@ __global__ void __launch_bounds__(512) k_seq(const SeqArgs a) {
     seq_sync(c.cs);
     int stages = 1, res = n1, more = 0;
     const int nwu = c.cs > 1 ? nw : nw - 1;
+    // In a cluster the first CTA builds the stages above 0 beside stage 0's records, which the others make: it only
+    // arrives at the barrier behind the walk, and waits for it when it is done.
+    const bool apart = c.cs > 1 && next;
+    if (apart && first) cluster_arrive();
     if (c.rank == wr && w == nw - 1) {
         if (lane == 0) sh.nb0 = walk_blocks(f0, c.L, a.bm, sh.bst0, SB0, a.recs + slot);
     } else if (first && next) {
@@ -715,13 +727,14 @@ __global__ void __launch_bounds__(512) k_seq(const SeqArgs a) {
         else if (up_smem) seq_upper<uint16_t>(a, sh, U, U + a.uc, U + 2 * a.uc, U + 3 * a.uc, U + 4 * a.uc, U + 5 * a.uc, fu, b, c.s0, slot, n1, nwu, stages, res, more);
         else seq_upper<uint32_t>(a, sh, G[3], G[4], G[5], G[6], G[7], G[8], reinterpret_cast<uint8_t *>(a.glob + a.glob_stride * 10) + c.s0, b, c.s0, slot, n1, nwu, stages, res, more);
     }
-    seq_sync(c.cs);
+    if (apart && first) cluster_wait();
+    else seq_sync(c.cs);
     const SeqShared *shw = c.cs > 1 ? map_rank(&sh, wr) : &sh;
     const int nb0 = shw->nb0;
     if (c.rank != wr)
         for (int i = t; i < min(nb0, SB0); i += blockDim.x) sh.bst0[i] = shw->bst0[i];
     __syncthreads();
-    int i0 = 0, i1 = nb0, di = nw;      // the blocks that start in this slice
+    int i0 = 0, i1 = nb0, n0 = 0;       // the blocks that start in this slice; those of the first slice that its CTA leaves to the others
     if (c.cs > 1 && nb0 <= SB0) {
         auto before = [&](int e) {      // blocks that start before element e
             int lo = 0, hi = nb0;
@@ -730,10 +743,14 @@ __global__ void __launch_bounds__(512) k_seq(const SeqArgs a) {
         };
         i0 = before(c.e0);
         i1 = c.rank + 1 == c.cs ? nb0 : before(c.e0 + c.ne);
+        if (apart) n0 = before(min(1 << c.sl, c.L));
     } else if (c.cs > 1) {
-        i0 = c.rank * nw;
-        di = c.cs * nw;
+        i0 = i1 = n0 = 0;
+        n0 = nb0;                       // (more than fit there: dealt to all CTAs but the first)
     }
+    // the blocks of this CTA: its slice's, then every (cs - 1)th of the n0
+    const int own = i1 - i0, spread = c.cs > 1 ? (int)c.cs - 1 : 1, left = (int)c.rank - 1;
+    const int mine = (c.cs > 1 && first) ? (apart || nb0 > SB0 ? 0 : own) : own + (n0 - left + spread - 1) / spread * (n0 > 0);
     // (the elements' arrays are written here, not where they are first known: a cluster barrier waits for the
     // CTA's outstanding stores, and the blocks cover every token)
     auto records = [&](const auto &par, const auto &cnt, const auto &pre) {
@@ -753,7 +770,8 @@ __global__ void __launch_bounds__(512) k_seq(const SeqArgs a) {
             a.up[g] = kept ? (int)pre.get(e) + sh.ctot[e >> c.sl] : -1;
             if (child) a.rank[g] = e - (int)p;       // the token's number among its siblings (hierarchical positions)
             return kept;
-        }, c.L, nb0, sh.bst0, SB0, a.recs + slot, i0 + w, i1, di, lane, &sh0->nf0, &sh0->ne0, &sh0->vis);
+        }, c.L, nb0, sh.bst0, SB0, a.recs + slot, w, mine, nw, [&](int v) { return v < own ? i0 + v : left + (v - own) * spread; }, lane, &sh0->nf0,
+           &sh0->ne0, &sh0->vis);
     };
     if (in_smem) records(X, Y, Z);
     else records(GX, GY, GZ);
@@ -782,7 +800,8 @@ struct FinishArgs {
     const int4 *recs, *el;
     const int *upl;
     long long *keys;
-    DevHeader *hdr, *host;         // host: pinned landing buffer (its words are not 0 at `tail` before)
+    DevHeader *hdr;
+    HostHeader *host;              // pinned landing buffer
 };
 
 static constexpr int FT = 256;     // threads of k_finish
@@ -813,8 +832,7 @@ __device__ __forceinline__ void row_sums(int rows, int m, int w, int nw, int lan
 }
 
 // Header: totals over the sequences.  The words go to the workspace (kernels read them there) and
-// straight to the host's pinned buffer, the tail word last and behind a system-wide fence: the host
-// watches for it, so no copy has to be queued behind the build.
+// straight to the host's pinned buffer, which the host watches, so no copy has to be queued behind the build.
 __device__ void finish_header(const FinishArgs &f, int S) {
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     __shared__ int s_err, s_more;
@@ -822,14 +840,14 @@ __device__ void finish_header(const FinishArgs &f, int S) {
     if (t == 0) { s_err = 0x7fffffff; s_more = 0; s_sum[0] = s_sum[1] = s_sum[2] = s_sum[3] = 0; }
     __syncthreads();
     const size_t q = (size_t)f.ms * f.B;
+    volatile HostHeader *host = f.host;
     row_sums(4 * S, f.B, w, FT / 32, lane, [&](int i) { return f.counts + (i & 3) * q + (size_t)(i >> 2) * f.B; },
              [&](int i, int v) {
-                 StageDesc &d = f.hdr->st[i >> 2], &h = f.host->st[i >> 2];
+                 StageDesc &d = f.hdr->st[i >> 2];
                  const int c = i & 3;
                  int *pd = c == 0 ? &d.n : c == 1 ? &d.nb : c == 2 ? &d.n_fused : &d.n_empty;
-                 int *ph = c == 0 ? &h.n : c == 1 ? &h.nb : c == 2 ? &h.n_fused : &h.n_empty;
                  *pd = v;
-                 *reinterpret_cast<volatile int *>(ph) = v;
+                 host->st[i >> 2][c] = v;
              });
     long long nnz = 0, vis = 0, nup = 0, real = 0;
     for (int b = t; b < f.B; b += FT) {
@@ -844,25 +862,22 @@ __device__ void finish_header(const FinishArgs &f, int S) {
     if (t <= HDT_MAX_STAGES) {
         const int more = (t + 1 < S) || (t + 1 == S && s_more);
         f.hdr->st[t].has_next = more;
-        *reinterpret_cast<volatile int *>(&f.host->st[t].has_next) = more;
+        if (t < f.ms) host->st[t][4] = more;
         if (t >= S) {
             StageDesc &d = f.hdr->st[t];
             d.n = d.nb = d.n_fused = d.n_empty = 0;
-            volatile StageDesc *h = &f.host->st[t];
-            h->n = 0; h->nb = 0; h->n_fused = 0; h->n_empty = 0;
+            if (t < f.ms) for (int c = 0; c < 4; ++c) host->st[t][c] = 0;
         }
     }
     if (t == 0) {
         int err = 0, pos = 0;
         if (f.B == 0) { f.st[0].scu[0] = f.cu[0]; if (f.cu[0] != 0 || f.T != 0) err = HDT_ERR_BAD_HIERARCHY; }
         else if (s_err != 0x7fffffff) { err = f.info[s_err].err; pos = f.info[s_err].err_pos; }
-        volatile DevHeader *h = f.host;
-        f.hdr->status = err; f.hdr->err_pos = pos; f.hdr->nnz = s_sum[0]; f.hdr->visited = s_sum[1]; f.hdr->nnz_upper = s_sum[2]; f.hdr->real = s_sum[3]; f.hdr->tail = 0;
-        h->status = err; h->err_pos = pos; h->nnz = s_sum[0]; h->visited = s_sum[1]; h->nnz_upper = s_sum[2]; h->real = s_sum[3];
+        f.hdr->status = err; f.hdr->err_pos = pos; f.hdr->nnz = s_sum[0]; f.hdr->visited = s_sum[1]; f.hdr->nnz_upper = s_sum[2]; f.hdr->real = s_sum[3];
+        host->status = err; host->err_pos = pos;
+        for (int i = 0; i < HostHeader::TOTALS; ++i)
+            for (int k = 0; k < 3; ++k) host->total[i][k] = (int)((s_sum[i] >> (30 * k)) & 0x3fffffff);
     }
-    __threadfence_system();
-    __syncthreads();
-    if (t == 0) *reinterpret_cast<volatile int *>(&f.host->tail) = 0;
 }
 
 // Rank sort of a stage's blocks: queue[rank] = block id, cost descending, id ascending.  queue_split:
@@ -941,15 +956,18 @@ __global__ void __launch_bounds__(FT) k_finish(const FinishArgs f) {
     const size_t q = (size_t)f.ms * f.B;
     if (t == 0) { s_stages = 1; s_bad = 0; }
     __syncthreads();
+    int s0 = 0, L = 0;
+    if (seq) {                        // (the caller's array: k_seq, which let this kernel start, had waited for all before it)
+        s0 = f.cu[b];
+        L = f.cu[b + 1] - s0;
+    }
     pdl_wait();
     // One round of loads: the stages of the batch and its errors; in a sequence's CTA also the sums over the
     // sequences before it (elements and blocks of every stage) and its own numbers.
-    int m = 1, bad = 0, s0 = 0, L = 0;
+    int m = 1, bad = 0;
     SeqInfo info{};
     if (seq) {
         info = f.info[b];
-        s0 = f.cu[b];
-        L = f.cu[b + 1] - s0;
         if (t < f.ms) {
             s_cn[t] = f.counts[(size_t)t * f.B + b];
             s_cb[t] = f.counts[q + (size_t)t * f.B + b];
@@ -1061,26 +1079,25 @@ extern "C" size_t hdt_index_workspace_bytes(int32_t batch, int32_t total_tokens,
 
 // Pinned landing buffers for index headers: a small pool shared by all host threads (an index keeps
 // its buffer until the header has been read).
-static const int kUnset = 0x7fffffff;
 static std::mutex g_pinned_mu;
-static std::vector<DevHeader *> g_pinned_free;
-static DevHeader *pinned_acquire() {
+static std::vector<HostHeader *> g_pinned_free;
+static HostHeader *pinned_acquire() {
     {
         std::lock_guard<std::mutex> lk(g_pinned_mu);
         if (!g_pinned_free.empty()) {
-            DevHeader *p = g_pinned_free.back();
+            HostHeader *p = g_pinned_free.back();
             g_pinned_free.pop_back();
             return p;
         }
     }
-    DevHeader *p = nullptr;
-    if (cudaHostAlloc((void **)&p, sizeof(DevHeader), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+    HostHeader *p = nullptr;
+    if (cudaHostAlloc((void **)&p, sizeof(HostHeader), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
         (void)cudaGetLastError();
         return nullptr;
     }
     return p;
 }
-static void pinned_release(DevHeader *p) {
+static void pinned_release(HostHeader *p) {
     if (!p) return;
     std::lock_guard<std::mutex> lk(g_pinned_mu);
     g_pinned_free.push_back(p);
@@ -1133,9 +1150,9 @@ extern "C" int hdt_build_index(const int8_t *level, const int32_t *parent, const
         HDT_CUDA_CHECK(cudaFuncSetAttribute(k_seq, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
         attr_done.set();
     }
-    DevHeader *hp = pinned_acquire();
+    HostHeader *hp = pinned_acquire();
     if (!hp) return set_error(HDT_ERR_CUDA, "hdt_build_index: no pinned host memory for the index header");
-    hp->tail = kUnset;
+    for (int i = 0; i < HostHeader::words(ms); ++i) reinterpret_cast<int *>(hp)[i] = HostHeader::UNSET;
 
     hdt_index *ix = new hdt_index();
     ix->batch = B; ix->total_tokens = T; ix->block_m = bm; ix->block_m_upper = bmu; ix->n_stages = 0;
@@ -1230,15 +1247,20 @@ namespace hdt {
 int index_ready(const hdt_index *cix) {
     hdt_index *ix = const_cast<hdt_index *>(cix);
     if (ix->pending) {
-        // The host watches the tail word of the pinned header, which the device writes last, behind a
-        // system-wide fence.  After a bounded number of looks it waits for the stream instead.
-        DevHeader *hp = ix->h_pinned;
-        volatile int *p_tail = &hp->tail;
-        for (long long spin = 0; spin < 20000000LL && *p_tail == kUnset; ++spin) {}
+        // The host watches the words of the pinned header.  After a bounded number of looks it waits for the stream instead.
+        HostHeader *hp = ix->h_pinned;
+        const volatile int *words = reinterpret_cast<const volatile int *>(hp);
+        const int n_words = HostHeader::words(ix->max_stages);
+        int got = 0;
+        auto look = [&]() {
+            while (got < n_words && words[got] != HostHeader::UNSET) ++got;
+            return got == n_words;
+        };
+        for (long long spin = 0; spin < 20000000LL && !look(); ++spin) {}
         cudaError_t e_ = cudaSuccess;
-        if (*p_tail == kUnset) {
+        if (!look()) {
             e_ = cudaStreamSynchronize(ix->stream);
-            if (e_ == cudaSuccess && *p_tail == kUnset) e_ = cudaErrorUnknown;
+            if (e_ == cudaSuccess && !look()) e_ = cudaErrorUnknown;
         }
         ix->pending = 0;
         ix->h_pinned = nullptr;
@@ -1249,23 +1271,29 @@ int index_ready(const hdt_index *cix) {
             return set_error(HDT_ERR_CUDA, "waiting for the index build failed: %s", cudaGetErrorString(e_));
         }
         std::atomic_thread_fence(std::memory_order_acquire);
-        const DevHeader h = *hp;
+        const HostHeader h = *hp;
         pinned_release(hp);
         ix->failed = h.status;
         ix->err_pos = h.err_pos;
         if (h.status == 0) {
             int ns = 1;
-            while (ns < ix->max_stages && h.st[ns].n > 0) ++ns;
-            if (h.st[ns - 1].has_next && ns == ix->max_stages) {
+            while (ns < ix->max_stages && h.st[ns][0] > 0) ++ns;
+            if (h.st[ns - 1][4] && ns == ix->max_stages) {
                 ix->failed = HDT_ERR_BAD_HIERARCHY;
                 ix->err_pos = -1;
             } else {
                 ix->n_stages = ns;
-                ix->nnz = h.nnz;
-                ix->visited = h.visited;
-                ix->nnz_upper = h.nnz_upper;
-                ix->real = h.real;
-                for (int s = 0; s <= HDT_MAX_STAGES; ++s) ix->desc[s] = h.st[s];
+                auto total = [&](int i) { return (int64_t)h.total[i][0] | (int64_t)h.total[i][1] << 30 | (int64_t)h.total[i][2] << 60; };
+                ix->nnz = total(0);
+                ix->visited = total(1);
+                ix->nnz_upper = total(2);
+                ix->real = total(3);
+                for (int s = 0; s <= HDT_MAX_STAGES; ++s) {
+                    StageDesc &d = ix->desc[s];
+                    d = StageDesc{};
+                    if (s >= ix->max_stages) continue;
+                    d.n = h.st[s][0]; d.nb = h.st[s][1]; d.n_fused = h.st[s][2]; d.n_empty = h.st[s][3]; d.has_next = h.st[s][4];
+                }
             }
         }
     }

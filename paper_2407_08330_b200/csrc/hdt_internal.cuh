@@ -26,7 +26,17 @@ struct DevHeader {
     long long real;          // tokens that are not PAD
     long long visited;       // sum over blocks of rows x span
     StageDesc st[HDT_MAX_STAGES + 1];
-    int tail;                // always 0 on the device: the last word of the header to arrive on the host
+};
+
+// The header as it lands in pinned host memory: 32-bit words in any order, none of which ever is UNSET (totals go
+// in pieces of 30 bits).  The host fills the words with UNSET before the build and has the header when none is
+// left: the device sends them without a fence, which would hold up the end of its kernel by a trip to the host.
+struct HostHeader {
+    static constexpr int UNSET = 0x7fffffff, TOTALS = 4;
+    int status, err_pos;
+    int total[TOTALS][3];    // nnz, visited, nnz_upper, real
+    int st[HDT_MAX_STAGES][5];    // n, nb, n_fused, n_empty, has_next
+    static int words(int stages) { return 2 + 3 * TOTALS + 5 * stages; }
 };
 
 // Host-side pointers to one stage's arrays inside the workspace.
@@ -50,7 +60,7 @@ struct hdt_index {
     int pending;                      // 1 until the header has been read
     int failed;                       // hdt_status_t found in the header (or by its check), 0 = fine
     int err_pos, max_stages;
-    hdt::DevHeader *h_pinned;         // pinned landing buffer (from a pool), nullptr once released
+    hdt::HostHeader *h_pinned;         // pinned landing buffer (from a pool), nullptr once released
     const hdt::DevHeader *hdr_dev;    // the header in the index workspace
     cudaStream_t stream;              // stream of the build
 };
