@@ -181,8 +181,11 @@ struct SeqArgs {
 struct SeqShared {
     int bst0[SB0], bst[SBU];
     int wtot[32], wtotu[32], ctot[SEQ_CLUSTER];
-    int err, err_pos, real, flag0, flag, nb0, nb, nf0, ne0, nf, ne;
-    int ns[HDT_MAX_STAGES], nbs[HDT_MAX_STAGES], bso[HDT_MAX_STAGES], nfs[HDT_MAX_STAGES], nes[HDT_MAX_STAGES], bsu[SBA];     // (seq_upper_all)
+    int err, err_pos, real, flag0, flag, nb, nf, ne;
+    int ns[HDT_MAX_STAGES], nbs[HDT_MAX_STAGES], bso[HDT_MAX_STAGES], nfs[HDT_MAX_STAGES], nes[HDT_MAX_STAGES], bsu[SBA], bsu_n;     // (seq_upper_all)
+    uint32_t seg[2][4][128], slice[2][128], slices[SEQ_CLUSTER][128];     // (walk_slice)
+    int bstf[SB0];                         // block starts of the first slice
+    int own[2], own_end[2], base;          // blocks of this slice and of the first one, ends of their last ones; blocks before this slice
     unsigned long long nnz, nnz_upper, vis;
 };
 
@@ -234,19 +237,24 @@ __device__ __forceinline__ int walk_blocks(const uint8_t *fpos, int n, int bm, i
     return nb;
 }
 
-// Records of the blocks block(v), v = v0, v0 + dv, ... < v1, of a stage with nb blocks and n elements, one warp per
-// block.  get(e, lo, hi) gives the range of an element and returns whether it lives on.  (The loops stay rolled: nearly
+// Rows of block i of a stage with nb blocks and n elements: its first nbst starts are in bst, the others in the records.
+__device__ __forceinline__ void block_rows(const int *bst, int nbst, const int4 *rec, int i, int nb, int n, int &r0, int &r1) {
+    r0 = i < nbst ? bst[i] : rec[i].x;
+    r1 = i + 1 < nb ? (i + 1 < nbst ? bst[i + 1] : rec[i + 1].x) : n;
+}
+
+// Records of the blocks i0, i0 + di, ... < i1, one warp per block.  rows(i, r0, r1) gives the rows of a block,
+// get(e, lo, hi) the range of an element and returns whether it lives on.  (The loops stay rolled: nearly
 // every instruction of this kernel is executed once or twice by a warp, and fetching it costs more than that.)
-template <class Get, class Block>
-__device__ __forceinline__ void make_records(Get get, int n, int nb, const int *bst, int nbst, int4 *rec, int v0, int v1, int dv, Block block, int lane,
-                                             int *nf, int *ne, unsigned long long *vis_out) {
+template <class Get, class Rows>
+__device__ __forceinline__ void make_records(Get get, Rows rows, int4 *rec, int i0, int i1, int di, int lane, int *nf, int *ne,
+                                             unsigned long long *vis_out) {
     long long vis = 0;
     int mf = 0, me = 0;
 #pragma unroll 1
-    for (int v = v0; v < v1; v += dv) {
-        const int i = block(v);
-        const int r0 = i < nbst ? bst[i] : rec[i].x;
-        const int r1 = (i + 1 < nb) ? (i + 1 < nbst ? bst[i + 1] : rec[i + 1].x) : n;
+    for (int i = i0; i < i1; i += di) {
+        int r0, r1;
+        rows(i, r0, r1);
         // a block is dense where all its rows have one range
         int a = INT_MAX, bb = INT_MIN, a2 = INT_MIN, bb2 = INT_MAX;
         bool carry = false, none = false;
@@ -310,6 +318,69 @@ struct Slice {
     unsigned rank, cs, sl;     // CTA in the cluster, its size, log2 of the slice length
     int s0, L, e0, ne;         // sequence start and length; first element of the slice and their number
 };
+
+// The walk of a sequence whose slices lie in the CTAs of a cluster.  A walk enters a stretch of the array at one of bm
+// offsets, and where it leaves the stretch depends on nothing else: so a thread per offset walks each quarter of a
+// slice (seg: offset behind it | blocks << 8), the quarters are composed, then the slices, and four threads
+// repeat the walk that was the right one.  One thread for the whole sequence took 120 cycles a block: 11 000 cycles of the
+// build of 8192 tokens, 37 000 of 32768.  fpos(e): see walk_blocks.
+template <class F>
+__device__ __forceinline__ int next_block(F fpos, int pos, int bm, int n) {
+    int end = min(pos + bm, n);
+    if (end < n) {
+        const int f = fpos(end);
+        if (f < end - pos) end -= f;
+    }
+    return end;
+}
+template <class F>
+__device__ __forceinline__ void walk_slice(F fpos, int bm, SeqShared &sh, const Slice &c, unsigned rank, int at) {
+    const int t = threadIdx.x, g = t >> 7, o = t & 127, len = 1 << (c.sl - 2);
+    const int a = (int)(rank << c.sl) + g * len, b = a + len;
+    int pos = a + o, k = 0;
+    while (pos < min(b, c.L)) { pos = next_block(fpos, pos, bm, c.L); ++k; }
+    sh.seg[at][g][o] = (uint32_t)min(max(pos - b, 0), 127) | (uint32_t)k << 8;
+    __syncthreads();
+    if (t < 128) {
+        unsigned x = t, n = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) { const uint32_t v = sh.seg[at][i][x]; x = v & 255u; n += v >> 8; }
+        sh.slice[at][t] = x | n << 8;
+    }
+}
+// Behind a cluster barrier, in every CTA but the first: the block starts of its slice (bst0) and of the first one (bstf),
+// the first SB0 of each (the others' in the records).  nb: the number of all.
+template <class F>
+__device__ __forceinline__ void walk_starts(F fpos, int bm, SeqShared &sh, const Slice &c, int4 *rec, int *nb) {
+    const int t = threadIdx.x;
+    for (int i = t; i < (int)c.cs * 128; i += blockDim.x) {
+        const int r = i >> 7, k = i & 127;
+        sh.slices[r][k] = *map_rank(&sh.slice[r ? 0 : 1][k], r ? r : 1);
+    }
+    __syncthreads();
+    const int f = t >> 5, q = t & 31;          // warp 0: this slice, warp 1: the first one; a lane per quarter
+    if (f < 2 && q < 4) {
+        unsigned x = 0, n = 0;
+        for (unsigned r = 0; r < (f ? 0u : c.rank); ++r) { const uint32_t v = sh.slices[r][x]; x = v & 255u; n += v >> 8; }
+        const SeqShared *shs = f ? map_rank(&sh, 1) : &sh;
+        unsigned m = 0;
+        for (int i = 0; i < q; ++i) { const uint32_t v = shs->seg[f][i][x]; x = v & 255u; m += v >> 8; }
+        const int len = 1 << (c.sl - 2), a = (f ? 0 : (int)(c.rank << c.sl)) + q * len, b = min(a + len, c.L);
+        int *bst = f ? sh.bstf : sh.bst0;
+        int pos = a + (int)x;
+        for (; pos < b; ++m) {
+            if (m < SB0) bst[m] = pos; else rec[n + m].x = pos;
+            pos = next_block(fpos, pos, bm, c.L);
+        }
+        if (q == 3) {
+            sh.own[f] = (int)m;
+            sh.own_end[f] = min(max(pos, a), c.L);
+            if (!f) sh.base = (int)n;
+            if (!f && c.rank + 1 == c.cs) *nb = (int)(n + m);
+        }
+    }
+    __syncthreads();
+}
 
 // Stage 0 of one slice up to the keep flags: X parents, Y counts, Z levels and then the number of kept
 // elements before each kept one, relative to the slice.  sh: this CTA's, sh0: the first CTA's shared state.
@@ -381,7 +452,7 @@ __device__ __forceinline__ void seq_stage0(const SeqArgs &a, SeqShared &sh, SeqS
             if (child && !((int)p < e && e < (int)hi)) seq_fail(sh0, g);
             kp = real && !child;
             nreal += real;
-            fpos[e] = child ? (uint8_t)min(e - (int)p, 255) : 0;
+            fpos[i] = child ? (uint8_t)min(e - (int)p, 255) : 0;
             deg += row_pairs(e, (int)lo, (int)hi, a.dirs);
             if (kp && p != E::NONE) next = 1;
         }
@@ -509,7 +580,7 @@ __device__ __forceinline__ void seq_upper(const SeqArgs &a, SeqShared &sh, J *pa
                          lo = (int)l; hi = (int)h;
                          return !child;
                      },
-                     n, sh.nb, sh.bst, SBU, rec, w, sh.nb, nw, [](int v) { return v; }, lane, &sh.nf, &sh.ne, &sh.vis);
+                     [&](int i, int &r0, int &r1) { block_rows(sh.bst, SBU, rec, i, sh.nb, n, r0, r1); }, rec, w, sh.nb, nw, lane, &sh.nf, &sh.ne, &sh.vis);
         bar_upper(tu);
         if (t == 0) {
             int *c = a.counts + (size_t)s * a.B + b;
@@ -584,7 +655,7 @@ __device__ __forceinline__ bool seq_upper_all(const SeqArgs &a, SeqShared &sh, c
         }
         if (lane == 0) sh.ns[s] = run;
     }
-    if (t == 0) sh.ns[1] = n;
+    if (t == 0) { sh.ns[1] = n; sh.bsu_n = 0; }
     bar_upper(tu);
     long long deg = 0;
     for (int i = w; i < nch * (S - 1); i += nw) {
@@ -620,8 +691,7 @@ __device__ __forceinline__ bool seq_upper_all(const SeqArgs &a, SeqShared &sh, c
     bar_upper(tu);
     for (int s = 1 + w; s < S; s += nw) {          // a warp per stage: where its blocks start
         if (lane == 0) {
-            int o = 0;
-            for (int i = 1; i < s; ++i) o += 2 * (sh.ns[i] / a.bmu) + 2;
+            const int o = atomicAdd(&sh.bsu_n, 2 * (sh.ns[s] / a.bmu) + 2);
             sh.bso[s] = o;
             sh.nbs[s] = walk_blocks(fp + s * (size_t)n2, sh.ns[s], a.bmu, sh.bsu + min(o, SBA), max(SBA - o, 0), a.recs + (size_t)s * a.capnb + slot);
             sh.nfs[s] = 0; sh.nes[s] = 0;
@@ -633,13 +703,15 @@ __device__ __forceinline__ bool seq_upper_all(const SeqArgs &a, SeqShared &sh, c
     for (int s = 1 + w / split; s < S; s += nw / split) {
         const int4 *el = a.el + (size_t)(s - 1) * a.T + s0;
         const int *upl = a.upl + (size_t)(s - 1) * a.T + s0;
-        const int nb = sh.nbs[s], o = sh.bso[s];
+        int4 *rec = a.recs + (size_t)s * a.capnb + slot;
+        const int nb = sh.nbs[s], ns = sh.ns[s], o = sh.bso[s], held = max(SBA - o, 0);
+        const int *bst = sh.bsu + min(o, SBA);
         make_records([&](int e, int &lo, int &hi) {
             const int4 x = el[e];
             lo = x.z; hi = x.w;
             return upl[e] >= 0;
-        }, sh.ns[s], nb, sh.bsu + min(o, SBA), max(SBA - o, 0), a.recs + (size_t)s * a.capnb + slot, w % split, nb, split,
-           [](int v) { return v; }, lane, &sh.nfs[s], &sh.nes[s], &sh.vis);
+        }, [&](int i, int &r0, int &r1) { block_rows(bst, held, rec, i, nb, ns, r0, r1); }, rec, w % split, nb, split, lane, &sh.nfs[s], &sh.nes[s],
+           &sh.vis);
     }
     bar_upper(tu);
     for (int s = 1 + t; s < S; s += tu) {
@@ -652,10 +724,10 @@ __device__ __forceinline__ bool seq_upper_all(const SeqArgs &a, SeqShared &sh, c
 
 // A sequence's stages, by one CTA or, for long sequences, a cluster of SEQ_CLUSTER CTAs: stage 0 a slice per CTA
 // (one SM issues about 1500 instructions per 32 tokens of it: 25 us of an 8192-token sequence on one CTA), then
-// the stages above it on the first CTA while a thread of the second one walks stage 0's blocks, then the
-// records of stage 0's blocks, each by the CTA that holds its first row.
-// Shared memory: 6 bytes per token of the slice (parents, counts, prefix sums), `pool` for the upper stages, one
-// per token of `cap` for the walk.
+// the stages above it on the first CTA beside the records of stage 0's blocks on the others, each by the CTA that
+// holds its first row.
+// Shared memory: 7 bytes per token of the slice (parents, counts, prefix sums, places in the family), `pool` for the
+// upper stages.
 __global__ void __launch_bounds__(512) k_seq(const SeqArgs a) {
     pdl_wait();
     pdl_launch_dependents();
@@ -674,9 +746,13 @@ __global__ void __launch_bounds__(512) k_seq(const SeqArgs a) {
     c.ne = min(1 << c.sl, c.L - c.e0);
     const bool first = c.rank == 0;
     if (t == 0) {
-        sh.err = 0; sh.err_pos = 0; sh.real = 0; sh.flag0 = 0; sh.nf0 = 0; sh.ne0 = 0; sh.nnz = 0; sh.nnz_upper = 0; sh.vis = 0;
+        sh.err = 0; sh.err_pos = 0; sh.real = 0; sh.flag0 = 0; sh.nnz = 0; sh.nnz_upper = 0; sh.vis = 0;
         if (first) {
             if (c1 < c0 || c0 < 0 || c1 > a.T || (b == 0 && c0 != 0) || (b == a.B - 1 && c1 != a.T)) seq_fail(&sh, b);
+            int *p = a.counts + b;          // stage 0's sums over the CTAs: cleared behind two barriers, added to at the end
+            const size_t q = (size_t)a.ms * a.B;
+            p[2 * q] = 0; p[3 * q] = 0;
+            a.info[b].visited = 0;
             a.scu[b] = c0;
             if (b == a.B - 1) a.scu[a.B] = c1;
         }
@@ -686,13 +762,12 @@ __global__ void __launch_bounds__(512) k_seq(const SeqArgs a) {
     const int piece = a.cap / c.cs;
     uint16_t *U = s_dyn + 3 * piece;
     uint8_t *fu = reinterpret_cast<uint8_t *>(U + 6 * a.uc), *f0 = reinterpret_cast<uint8_t *>(U) + a.pool;
-    const unsigned wr = c.cs > 1 ? 1 : 0;          // CTA of the walk
     const bool in_smem = c.L <= a.cap;
     const Sliced X{s_dyn, c.sl, c.rank}, Y{s_dyn + piece, c.sl, c.rank}, Z{s_dyn + 2 * piece, c.sl, c.rank};
     uint32_t *G[NGLOB];
     for (int i = 0; i < NGLOB; ++i) G[i] = a.glob + a.glob_stride * i + c.s0;
     if (!in_smem) f0 = reinterpret_cast<uint8_t *>(a.glob + a.glob_stride * 9) + c.s0;
-    uint8_t *fw = (in_smem && c.cs > 1) ? map_rank(f0, wr) : f0;
+    uint8_t *fw = in_smem ? f0 : f0 + c.e0;
     const Flat<uint32_t> GX{G[0]}, GY{G[1]}, GZ{G[2]};
     bool root_real = false;
     if (in_smem) seq_stage0(a, sh, sh0, X, Y, Z, c, fw, root_real);
@@ -711,15 +786,38 @@ __global__ void __launch_bounds__(512) k_seq(const SeqArgs a) {
     else if (in_smem) seq_compact0(a, X, Z, sh.ctot, G[3], G[4], c);
     else if (up_smem) seq_compact0(a, GX, GZ, sh.ctot, P0, T0, c);
     else seq_compact0(a, GX, GZ, sh.ctot, G[3], G[4], c);
+    auto fpos = [&](int e) -> int {
+        if (!in_smem) return f0[e];
+        const unsigned r = (unsigned)e >> c.sl;
+        uint8_t *p = f0 + ((unsigned)e & ((1u << c.sl) - 1u));
+        return r == c.rank ? *p : *map_rank(p, r);
+    };
     seq_sync(c.cs);
     int stages = 1, res = n1, more = 0;
     const int nwu = c.cs > 1 ? nw : nw - 1;
-    // In a cluster the first CTA builds the stages above 0 beside stage 0's records, which the others make: it only
-    // arrives at the barrier behind the walk, and waits for it when it is done.
-    const bool apart = c.cs > 1 && next;
-    if (apart && first) cluster_arrive();
-    if (c.rank == wr && w == nw - 1) {
-        if (lane == 0) sh.nb0 = walk_blocks(f0, c.L, a.bm, sh.bst0, SB0, a.recs + slot);
+    int4 *rec = a.recs + slot;
+    int *cnt0 = a.counts + b;
+    const size_t q = (size_t)a.ms * a.B;
+    // In a cluster the first CTA builds the stages above 0; the others meanwhile walk stage 0 and make its records, the
+    // first slice's too (of which the second CTA makes the walk's table).  The first one only arrives at their
+    // barrier, and waits for it when it is done.
+    if (c.cs > 1) {
+        if (!first) {
+#pragma unroll 1
+            for (int at = 0; at < (c.rank == 1 ? 2 : 1); ++at) walk_slice(fpos, a.bm, sh, c, at ? 0u : c.rank, at);
+        }
+        cluster_arrive();
+        if (!first) {
+            cluster_wait();
+            walk_starts(fpos, a.bm, sh, c, rec, cnt0 + q);
+        }
+    }
+    if (c.cs == 1 && w == nw - 1) {
+        if (lane == 0) {
+            cnt0[q] = sh.own[0] = walk_blocks(f0, c.L, a.bm, sh.bst0, SB0, rec);
+            sh.own_end[0] = c.L;
+            sh.base = 0;
+        }
     } else if (first && next) {
         const bool done = up_smem && seq_upper_all(a, sh, U, U + a.uc, reinterpret_cast<uint32_t *>(U + 2 * a.uc), a.pool - 4 * (size_t)a.uc, b, c.s0, slot, n1,
                                                    nwu, stages, res, more);
@@ -727,33 +825,13 @@ __global__ void __launch_bounds__(512) k_seq(const SeqArgs a) {
         else if (up_smem) seq_upper<uint16_t>(a, sh, U, U + a.uc, U + 2 * a.uc, U + 3 * a.uc, U + 4 * a.uc, U + 5 * a.uc, fu, b, c.s0, slot, n1, nwu, stages, res, more);
         else seq_upper<uint32_t>(a, sh, G[3], G[4], G[5], G[6], G[7], G[8], reinterpret_cast<uint8_t *>(a.glob + a.glob_stride * 10) + c.s0, b, c.s0, slot, n1, nwu, stages, res, more);
     }
-    if (apart && first) cluster_wait();
-    else seq_sync(c.cs);
-    const SeqShared *shw = c.cs > 1 ? map_rank(&sh, wr) : &sh;
-    const int nb0 = shw->nb0;
-    if (c.rank != wr)
-        for (int i = t; i < min(nb0, SB0); i += blockDim.x) sh.bst0[i] = shw->bst0[i];
-    __syncthreads();
-    int i0 = 0, i1 = nb0, n0 = 0;       // the blocks that start in this slice; those of the first slice that its CTA leaves to the others
-    if (c.cs > 1 && nb0 <= SB0) {
-        auto before = [&](int e) {      // blocks that start before element e
-            int lo = 0, hi = nb0;
-            while (lo < hi) { const int mid = (lo + hi) >> 1; if (sh.bst0[mid] < e) lo = mid + 1; else hi = mid; }
-            return lo;
-        };
-        i0 = before(c.e0);
-        i1 = c.rank + 1 == c.cs ? nb0 : before(c.e0 + c.ne);
-        if (apart) n0 = before(min(1 << c.sl, c.L));
-    } else if (c.cs > 1) {
-        i0 = i1 = n0 = 0;
-        n0 = nb0;                       // (more than fit there: dealt to all CTAs but the first)
-    }
-    // the blocks of this CTA: its slice's, then every (cs - 1)th of the n0
-    const int own = i1 - i0, spread = c.cs > 1 ? (int)c.cs - 1 : 1, left = (int)c.rank - 1;
-    const int mine = (c.cs > 1 && first) ? (apart || nb0 > SB0 ? 0 : own) : own + (n0 - left + spread - 1) / spread * (n0 > 0);
+    if (c.cs == 1) __syncthreads();
+    else if (first) cluster_wait();
     // (the elements' arrays are written here, not where they are first known: a cluster barrier waits for the
     // CTA's outstanding stores, and the blocks cover every token)
-    auto records = [&](const auto &par, const auto &cnt, const auto &pre) {
+    auto records = [&](const auto &par, const auto &cnt, const auto &pre, int f, int i0, int di) {
+        const int base = f ? 0 : sh.base, nb = sh.own[f], end = sh.own_end[f];
+        const int *bst = f ? sh.bstf : sh.bst0;
         using E = Elem<typename std::remove_reference_t<decltype(par)>::I>;
         make_records([&](int e, int &lo, int &hi) {
             const unsigned p = par.get(e);
@@ -770,25 +848,34 @@ __global__ void __launch_bounds__(512) k_seq(const SeqArgs a) {
             a.up[g] = kept ? (int)pre.get(e) + sh.ctot[e >> c.sl] : -1;
             if (child) a.rank[g] = e - (int)p;       // the token's number among its siblings (hierarchical positions)
             return kept;
-        }, c.L, nb0, sh.bst0, SB0, a.recs + slot, w, mine, nw, [&](int v) { return v < own ? i0 + v : left + (v - own) * spread; }, lane, &sh0->nf0,
-           &sh0->ne0, &sh0->vis);
+        }, [&](int i, int &r0, int &r1) { block_rows(bst, SB0, rec + base, i - base, nb, end, r0, r1); }, rec, base + i0, base + nb, di, lane,
+           cnt0 + 2 * q, cnt0 + 3 * q, reinterpret_cast<unsigned long long *>(&a.info[b].visited));
     };
-    if (in_smem) records(X, Y, Z);
-    else records(GX, GY, GZ);
-    seq_sync(c.cs);
+    if (c.cs == 1 || !first) {
+#pragma unroll 1
+        for (int f = 0; f < (c.cs > 1 ? 2 : 1); ++f) {
+            // (the first slice's: to the warps that have none of their own, one CTA after the other)
+            const int i0 = f ? (nw - 1 - w) * (int)(c.cs - 1) + (int)c.rank - 1 : w, di = f ? (int)(c.cs - 1) * nw : nw;
+            if (in_smem) records(X, Y, Z, f, i0, di);
+            else records(GX, GY, GZ, f, i0, di);
+        }
+    }
     if (first && t == 0) {
-        const size_t q = (size_t)a.ms * a.B;
-        int *p = a.counts + b;
-        p[0] = c.L; p[q] = nb0; p[2 * q] = sh.nf0; p[3 * q] = sh.ne0;
+        int *p = cnt0;
+        p[0] = c.L;
         for (int s = stages; s < a.ms; ++s) {          // beyond its own stages: its root in a block of its own
             p = a.counts + (size_t)s * a.B + b;
             p[0] = res; p[q] = res; p[2 * q] = 0; p[3 * q] = res;
         }
-        SeqInfo f;
+        SeqInfo &f = a.info[b];
         f.stages = stages; f.res = res; f.err = sh.err; f.err_pos = sh.err_pos; f.more = more; f.real = sh.real;
-        f.nnz = (long long)(sh.nnz + sh.nnz_upper); f.nnz_upper = (long long)sh.nnz_upper; f.visited = (long long)sh.vis;
-        a.info[b] = f;
+        f.nnz = (long long)(sh.nnz + sh.nnz_upper); f.nnz_upper = (long long)sh.nnz_upper;
+        if (sh.vis) atomicAdd(reinterpret_cast<unsigned long long *>(&f.visited), sh.vis);
     }
+    // (nothing passes between the CTAs here: the others' shared memory has been read.  A barrier with release
+    // semantics would wait for the outstanding stores of all of them, 3000 cycles)
+    __syncwarp();
+    if (c.cs > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
 }
 
 struct FinishArgs {
@@ -1143,8 +1230,8 @@ extern "C" int hdt_build_index(const int8_t *level, const int32_t *parent, const
     a.cap = cap;
     a.uc = min(cap, UC_MAX);
     a.pool = (cap <= 2048 ? 32 : 16) * a.uc;       // (13 at least, for the stages one by one)
-    const size_t smem = 6 * (size_t)(cap / cs) + a.pool + cap;
-    static constexpr size_t kSmemMax = 6 * 8192 + 16 * UC_MAX + SEQ_CAP_MAX;
+    const size_t smem = 7 * (size_t)(cap / cs) + a.pool;
+    static constexpr size_t kSmemMax = 7 * 4096 + 16 * UC_MAX;
     static DevOnce attr_done;
     if (!attr_done.done()) {
         HDT_CUDA_CHECK(cudaFuncSetAttribute(k_seq, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
