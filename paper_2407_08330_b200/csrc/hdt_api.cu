@@ -93,8 +93,6 @@ int get_side(Side **out) {
         HDT_CUDA_CHECK(cudaEventCreateWithFlags(&sd.fork, cudaEventDisableTiming));
         HDT_CUDA_CHECK(cudaEventCreateWithFlags(&sd.join, cudaEventDisableTiming));
         HDT_CUDA_CHECK(cudaEventCreateWithFlags(&sd.join2, cudaEventDisableTiming));
-        HDT_CUDA_CHECK(cudaEventCreateWithFlags(&sd.fork0, cudaEventDisableTiming));
-        HDT_CUDA_CHECK(cudaEventCreateWithFlags(&sd.join0, cudaEventDisableTiming));
         sd.ready = true;
     }
     *out = &sd;
@@ -577,21 +575,14 @@ extern "C" int hdt_attn_bwd(const hdt_index_t *ix, const void *q, const void *k,
         (g_no_persistent == 0 || g_no_persistent == 4 || g_no_persistent == 6)) {
         dq_acc = (float *)(ws + L.dq_acc);
     }
-    // The buffer is cleared (writes) beside the delta pass (reads), on the second side stream: both are
-    // HBM-bound, one in each direction.  Stage 0 waits for it (join0).
-    Side *sd0 = nullptr;
-    const bool clear_beside = dq_acc != nullptr && !fused_delta && !g_no_overlap && get_side(&sd0) == HDT_OK && sd0 != nullptr;
+    // The delta pass, which every one-walk kernel needs, clears the buffer's rows of the blocks that are walked
+    // (k_bwd_tc_p, option "bwd_walk" = 2, walks the EMPTY blocks too).
+    DeltaClear clear{};
     if (dq_acc != nullptr) {
-        const size_t bytes = sizeof(float) * (size_t)ix->total_tokens * heads * 64;
-        if (clear_beside) {
-            HDT_CUDA_CHECK(cudaEventRecord(sd0->fork0, st));
-            HDT_CUDA_CHECK(cudaStreamWaitEvent(sd0->s2, sd0->fork0, 0));
-            HDT_CUDA_CHECK(cudaMemsetAsync(dq_acc, 0, bytes, sd0->s2));
-            HDT_CUDA_CHECK(cudaEventRecord(sd0->join0, sd0->s2));
-        } else {
-            ProfScope ps(PROF_BWD_STAGE0, st);
-            HDT_CUDA_CHECK(cudaMemsetAsync(dq_acc, 0, bytes, st));
-        }
+        clear.blocks = ix->st[0].blocks;
+        clear.list = ix->st[0].queue_split + ix->desc[0].n_fused;
+        clear.buf = dq_acc;
+        clear.n_ctas = DeltaClear::PARTS * (ix->desc[0].nb - ix->desc[0].n_fused - (g_bwd_walk == 2 ? 0 : ix->desc[0].n_empty));
     }
     if (all_rows) {
         {
@@ -617,10 +608,9 @@ extern "C" int hdt_attn_bwd(const hdt_index_t *ix, const void *q, const void *k,
     }
     if (!fused_delta) {
         ProfScope ps(PROF_DELTA, st);
-        rc = launch_delta(o, d_o, delta, ix->total_tokens, heads, head_dim, dtype, st);
+        rc = launch_delta(o, d_o, delta, ix->total_tokens, heads, head_dim, dtype, st, clear);
     }
     if (rc) return rc;
-    if (clear_beside) HDT_CUDA_CHECK(cudaStreamWaitEvent(st, sd0->join0, 0));
     auto stage_args = [&](int s) {
         const StagePtrs &P = ix->st[s];
         BwdStageArgs a{};

@@ -412,12 +412,25 @@ __global__ void __launch_bounds__(NTHREADS) k_bwd_simt_multi(const MultiBwdArgs 
 // delta[h, t] = sum_c dO[t,h,c] * O[t,h,c].  A (token, head) row is read by LPR adjacent lanes with
 // one 16-byte load each per tensor (8 bf16 or 4 fp32 values), so a warp covers 32 / LPR rows.
 template <int D, bool BF16>
-__global__ void __launch_bounds__(256) k_delta(const void *o, const void *d_o, float *delta, int T, int H) {
+__global__ void __launch_bounds__(256) k_delta(const void *o, const void *d_o, float *delta, int T, int H, const DeltaClear z) {
     pdl_wait();
     pdl_launch_dependents();
+    unsigned cta = blockIdx.x;
+    if (z.n_ctas > 0) {                        // clearing CTAs spread evenly among the others
+        const unsigned c0 = (unsigned)((unsigned long long)cta * z.n_ctas / gridDim.x), c1 = (unsigned)((unsigned long long)(cta + 1) * z.n_ctas / gridDim.x);
+        if (c1 > c0) {
+            const int *rec = z.blocks + 5 * (size_t)z.list[c0 / DeltaClear::PARTS];
+            const long long n4 = (long long)(rec[1] - rec[0]) * H * (64 / 4), per = (n4 + DeltaClear::PARTS - 1) / DeltaClear::PARTS;
+            float4 *g = reinterpret_cast<float4 *>(z.buf) + (size_t)rec[0] * H * (64 / 4);
+            const long long i0 = per * (c0 % DeltaClear::PARTS), i1 = min(n4, i0 + per);
+            for (long long i = i0 + threadIdx.x; i < i1; i += 256) g[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            return;
+        }
+        cta -= c0;
+    }
     constexpr int VPL = BF16 ? 8 : 4;          // values per lane
     constexpr int LPR = D / VPL;               // lanes per row: 8 (bf16, D=64) ... 32 (fp32, D=128)
-    const long long gtid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long long gtid = (long long)cta * blockDim.x + threadIdx.x;
     const long long row = gtid / LPR;
     const int sub = (int)(gtid % LPR);
     float acc = 0.f;
@@ -580,20 +593,20 @@ int launch_bwd_simt(const BwdStageArgs &a, int D, int dtype, cudaStream_t st) {
 }
 
 template <int D, bool BF16>
-static void launch_delta_t(const void *o, const void *d_o, float *delta, int T, int H, cudaStream_t st) {
+static void launch_delta_t(const void *o, const void *d_o, float *delta, int T, int H, const DeltaClear &z, cudaStream_t st) {
     constexpr int LPR = D / (BF16 ? 8 : 4);
     const long long threads = (long long)T * H * LPR;
-    k_delta<D, BF16><<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(o, d_o, delta, T, H);
+    k_delta<D, BF16><<<(unsigned)((threads + 255) / 256) + (unsigned)z.n_ctas, 256, 0, st>>>(o, d_o, delta, T, H, z);
 }
 
-int launch_delta(const void *o, const void *d_o, float *delta, int T, int H, int D, int dtype, cudaStream_t st) {
+int launch_delta(const void *o, const void *d_o, float *delta, int T, int H, int D, int dtype, cudaStream_t st, const DeltaClear &z) {
     if ((long long)T * H == 0) return HDT_OK;
     if (D == 64) {
-        if (dtype == HDT_BF16) launch_delta_t<64, true>(o, d_o, delta, T, H, st);
-        else launch_delta_t<64, false>(o, d_o, delta, T, H, st);
+        if (dtype == HDT_BF16) launch_delta_t<64, true>(o, d_o, delta, T, H, z, st);
+        else launch_delta_t<64, false>(o, d_o, delta, T, H, z, st);
     } else if (D == 128) {
-        if (dtype == HDT_BF16) launch_delta_t<128, true>(o, d_o, delta, T, H, st);
-        else launch_delta_t<128, false>(o, d_o, delta, T, H, st);
+        if (dtype == HDT_BF16) launch_delta_t<128, true>(o, d_o, delta, T, H, z, st);
+        else launch_delta_t<128, false>(o, d_o, delta, T, H, z, st);
     } else {
         return set_error(HDT_ERR_UNSUPPORTED, "head_dim %d not supported (64 or 128)", D);
     }

@@ -1412,17 +1412,27 @@ __global__ void __launch_bounds__(256) k_dq_finish(const BwdStageArgs a, int zer
         }
         return;
     }
-    for (int i = threadIdx.x; i < nrows * 16; i += 256) {
-        const int r = i >> 4, c = i & 15;
-        const size_t row = (size_t)(r0 + r);
-        const float4 x = *reinterpret_cast<const float4 *>(a.dq_acc + (row * H + h) * 64 + 4 * c);
-        const float4 y = make_float4(x.x * a.scale, x.y * a.scale, x.z * a.scale, x.w * a.scale);
+    // (all loads of a thread in flight together: a block has at most 128 rows)
+    float4 x[8];
+    int u[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const int i = threadIdx.x + 256 * k;
+        u[k] = -1;
+        if (i >= nrows * 16) continue;
+        const size_t row = (size_t)(r0 + (i >> 4));
+        x[k] = *reinterpret_cast<const float4 *>(a.dq_acc + (row * H + h) * 64 + 4 * (i & 15));
+        if (a.part_dq != nullptr) u[k] = a.up[row];
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const int i = threadIdx.x + 256 * k, c = i & 15;
+        if (i >= nrows * 16) break;
+        const size_t row = (size_t)(r0 + (i >> 4));
+        const float4 y = make_float4(x[k].x * a.scale, x[k].y * a.scale, x[k].z * a.scale, x[k].w * a.scale);
         *reinterpret_cast<uint2 *>(reinterpret_cast<__nv_bfloat16 *>(a.dq) + (row * H + h) * 64 + 4 * c) =
             make_uint2(pack_bf16(y.x, y.y), pack_bf16(y.z, y.w));
-        if (a.part_dq != nullptr) {
-            const int u = a.up[row];
-            if (u >= 0) *reinterpret_cast<float4 *>(a.part_dq + ((size_t)u * H + h) * 64 + 4 * c) = y;
-        }
+        if (u[k] >= 0) *reinterpret_cast<float4 *>(a.part_dq + ((size_t)u[k] * H + h) * 64 + 4 * c) = y;
     }
 }
 

@@ -113,7 +113,7 @@ int sm_count(int *n_sm);
 // on the main kernel of a call runs beside it.  fork / join are events for the two hand-overs.
 struct Side {
     cudaStream_t s, s2, s3;
-    cudaEvent_t fork, join, join2, join3, fork0, join0;      // fork0 / join0: a hand-over of their own for work that starts before `fork`
+    cudaEvent_t fork, join, join2, join3;
     bool ready;
 };
 int get_side(Side **out);
@@ -300,8 +300,17 @@ int read_bwd_t_timeline(long long *out2048);     // per CTA of the last instrume
 int read_fwd_phase_cycles(long long *out16);
 int read_fwd_timeline(long long *out4096);       // per CTA of the last instrumented looping forward: entry, first tiles in, end (ns), SM
 int launch_bwd_simt(const BwdStageArgs &a, int head_dim, int dtype, cudaStream_t st);
+// Rows of the listed blocks in the fp32 dQ buffer [T, H, 64] that the delta pass clears on its way: the pass only reads
+// and the clear only writes, so in one launch they share HBM (2 x 32768 skewed tokens: a clear of the whole buffer 34 us
+// and the pass 43, one after the other although on two streams; together, clearing only the rows that are added to, 57).
+struct DeltaClear {
+    static constexpr int PARTS = 8;        // CTAs of a block
+    const int *blocks, *list;
+    float *buf;
+    int n_ctas;                            // PARTS x listed blocks; 0 = nothing to clear
+};
 int launch_delta(const void *o, const void *d_o, float *delta, int T, int H, int head_dim, int dtype,
-                 cudaStream_t st);
+                 cudaStream_t st, const DeltaClear &clear = DeltaClear{});
 // Row-wise kernels (hdt_attn_rows.cu): the elements of stage `first` with all stages they live in from there on.
 struct RowStage { const int *tok, *rng, *up; };
 struct RowFwdArgs {
