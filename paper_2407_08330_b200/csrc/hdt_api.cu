@@ -251,11 +251,13 @@ static bool rows_all(const hdt_index *ix, int heads, int head_dim, int dtype) {
     return rows_allowed() && ix->nnz <= (few ? 64 : 10) * ix->real;
 }
 // The stages above 0 row by row, in one launch behind stage 0, while their pairs are few; beyond, the tile
-// kernels' launches beside stage 0 and the merge behind it cost less.  The lines lie where the two met on
-// documents of 200 to 90 000 tokens (forward: 4 x 8192 tokens and 12 heads, 215 000, lost 2 us of 219; backward,
-// four times the work a pair: gains of 5 to 10 us of 60 to 150 below 30 000, a loss of 2 at 97 000).
+// kernels' launches beside stage 0 and the merge behind it cost less.  The lines lie between the sizes where the two
+// were timed on documents of 200 to 90 000 tokens, the row-wise kernel as a programmatic dependent of stage 0.  Forward,
+// 12 heads x 64: 4 x 8192 tokens (215 000) 85.0 against 83.2 us, 8 x 8192 (430 000) 126.3 against 130.5.  Forward and
+// backward: 8 x 1024 tokens 90.5 against 82, 1 x 4096 with 16 heads x 128 (60 000) 117.5 against 106.4, 2 x 8192
+// (108 000) 130.8 against 132.4.
 static bool rows_upper(const hdt_index *ix, int heads, int head_dim, int bwd) {
-    return rows_allowed() && ix->n_stages > 1 && ix->nnz_upper * heads * (head_dim / 64) <= (bwd ? 40000 : 200000);
+    return rows_allowed() && ix->n_stages > 1 && ix->nnz_upper * heads * (head_dim / 64) <= (bwd ? 80000 : 300000);
 }
 // fp32 calls: stage 0 on the kernels that stage its keys in shared memory; the stages above it row by row unless
 // their families are long (the SIMT tile kernels read such a family's rows once per block).
