@@ -36,8 +36,9 @@
  *    by exact zeros, and 0 x NaN or 0 x inf would reach real rows of the same tile (zero-fill them,
  *    as a padded batch normally is; nothing checks this).
  *  - `stream` is a cudaStream_t passed as void* (NULL = default stream).  hdt_attn_fwd/bwd are
- *    asynchronous on it.  hdt_build_index enqueues its kernels on it and then waits for them,
- *    because it returns the sizes the attention calls need.
+ *    asynchronous on it.  hdt_build_index enqueues its kernels on it and then waits until they have
+ *    done all their reads and writes, because it returns the sizes the attention calls need.
+ *  - An index may be used on any stream and by several threads, whichever stream it was built on.
  *  - Every function returns an hdt_status_t (HDT_OK = 0, errors negative); nothing throws,
  *    aborts or traps the device.  hdt_last_error() gives a thread-local message.
  */
@@ -83,11 +84,15 @@ typedef struct {
                            the first call that needs the counts of the index on the host
                            (hdt_index_info, hdt_index_export, the workspace queries, the attention and
                            positional-encoding calls) waits instead and returns the structure error,
-                           if any; every later call on that index returns it too.  hdt_attn_fwd on a
-                           bf16 index still in flight queues its stage-0 kernel first (the kernel
-                           reads the counts on the device) and waits only then.  The structure
-                           arrays and the workspace must stay allocated until the stream has
-                           passed the build (as for any asynchronous call)                      */
+                           if any; every later call on that index returns it too.  Attention and
+                           positional-encoding calls on the stream of the build wait for the counts
+                           only, every other call until the build has ended.  hdt_attn_fwd on a
+                           bf16 index still in flight on its stream queues its stage-0 kernel first
+                           (the kernel reads the counts on the device) and waits only then.  The
+                           structure arrays and the workspace must stay allocated and unchanged until
+                           the stream has passed the build, the stream itself until a call has waited
+                           for its end.  A call captured into a graph on the stream of the build counts
+                           as one on that stream: replay it there, or ordered behind it          */
     int32_t reserved[3];
 } hdt_index_params_t;
 
@@ -138,7 +143,8 @@ size_t hdt_index_workspace_bytes(int32_t batch, int32_t total_tokens,
  *   workspace  device, >= hdt_index_workspace_bytes(...), 256-byte aligned; must stay allocated
  *              and untouched until hdt_index_destroy
  *   out        receives a host object (free with hdt_index_destroy)
- * Waits for the stream before returning (unless params->deferred is set: see there).  Errors:
+ * Returns when the stream has passed the build (unless params->deferred is set: see there): the index
+ * may then be used on any stream, and the structure arrays may change.  Errors:
  * HDT_ERR_BAD_HIERARCHY when a precondition on the structure arrays fails or the hierarchy needs
  * more than max_stages stages (no index is returned; a deferred build returns the index and the
  * error comes from the first call that uses it), HDT_ERR_WORKSPACE, HDT_ERR_INVALID_ARG,

@@ -299,7 +299,7 @@ extern "C" int hdt_attn_fwd(const hdt_index_t *ix, const void *q, const void *k,
     // launches on the side streams after its wait still runs beside that kernel, not behind it.
     bool early = false, forked = false;
     std::unique_ptr<ProfScope> ps_early;      // stage 0's time when a kernel goes ahead: from its start to the end of the stage's other kernel
-    if (ix->pending && ix->total_tokens > 0 && dtype == HDT_BF16 && !g_force_simt && g_no_persistent == 0 &&
+    if (ix->state.load(std::memory_order_acquire) == INDEX_QUEUED && index_on_stream(ix, st) && ix->total_tokens > 0 && dtype == HDT_BF16 && !g_force_simt && g_no_persistent == 0 &&
         !g_no_overlap && ix->max_stages <= 8 && (workspace == nullptr || ((uintptr_t)workspace & 255) == 0)) {
         // (A small batch will most likely need no side stream: its stages above 0 go row by row.  An event recorded
         // between the build and this kernel would keep them from overlapping as programmatic dependents.)
@@ -329,7 +329,7 @@ extern "C" int hdt_attn_fwd(const hdt_index_t *ix, const void *q, const void *k,
         if (rc) return rc;
         early = true;
     }
-    rc = index_ready(ix);
+    rc = index_ready(ix, st);
     if (rc) return rc;
     const AttnLayout L = attn_layout(ix, heads, head_dim, 0);
     rc = check_common(ix, heads, head_dim, dtype, workspace, workspace_bytes, L.total, "hdt_attn_fwd");
@@ -532,7 +532,7 @@ extern "C" int hdt_attn_bwd(const hdt_index_t *ix, const void *q, const void *k,
                             int32_t head_dim, int32_t dtype, float softmax_scale, void *workspace,
                             size_t workspace_bytes, void *stream) {
     if (!ix) return set_error(HDT_ERR_INVALID_ARG, "hdt_attn_bwd: null index");
-    if (const int rc0 = index_ready(ix)) return rc0;
+    if (const int rc0 = index_ready(ix, (cudaStream_t)stream)) return rc0;
     const AttnLayout L = attn_layout(ix, heads > 0 ? heads : 1, head_dim > 0 ? head_dim : 64, 1, dtype);
     int rc = check_common(ix, heads, head_dim, dtype, workspace, workspace_bytes, L.total, "hdt_attn_bwd");
     if (rc) return rc;
@@ -754,7 +754,7 @@ extern "C" int hdt_attn_fwd_static(const hdt_index_t *ix, const void *q, const v
                                    float *lse, int32_t heads, int32_t head_dim, int32_t dtype,
                                    float softmax_scale, void *stream) {
     if (!ix) return set_error(HDT_ERR_INVALID_ARG, "hdt_attn_fwd_static: null index");
-    if (const int rc0 = index_ready(ix)) return rc0;
+    if (const int rc0 = index_ready(ix, (cudaStream_t)stream)) return rc0;
     const AttnLayout L = attn_layout(ix, heads > 0 ? heads : 1, head_dim > 0 ? head_dim : 64, 0);
     if (L.total > (size_t)HDT_FWD_STATIC_SCRATCH_BYTES)
         return set_error(HDT_ERR_WORKSPACE,

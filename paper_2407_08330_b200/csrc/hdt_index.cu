@@ -172,6 +172,7 @@ struct SeqArgs {
     int *counts;               // [4][ms][B]: elements, blocks, SELF non-EMPTY blocks, EMPTY blocks
     int4 *recs;                // [ms][capnb]: r0, a, b, rows | flags << 8, relative to the sequence
     int capnb;
+    int *ticket;               // (see HostHeader::done) cleared here for k_finish
     int4 *el;                  // [ms - 1][T]: tok, par, lo, hi of the upper stages, relative to the sequence
     int *upl;                  // [ms - 1][T]: index in the next stage, -1 = removed
     uint32_t *glob;            // NGLOB arrays of glob_stride elements
@@ -754,7 +755,7 @@ __global__ void __launch_bounds__(512) k_seq(const SeqArgs a) {
             p[2 * q] = 0; p[3 * q] = 0;
             a.info[b].visited = 0;
             a.scu[b] = c0;
-            if (b == a.B - 1) a.scu[a.B] = c1;
+            if (b == a.B - 1) { a.scu[a.B] = c1; *a.ticket = 0; }
         }
     }
     SeqShared *sh0 = c.cs > 1 ? map_rank(&sh, 0) : &sh;
@@ -889,6 +890,7 @@ struct FinishArgs {
     long long *keys;
     DevHeader *hdr;
     HostHeader *host;              // pinned landing buffer
+    int tell;                      // 1: HostHeader::done is sent
 };
 
 static constexpr int FT = 256;     // threads of k_finish
@@ -918,16 +920,14 @@ __device__ __forceinline__ void row_sums(int rows, int m, int w, int nw, int lan
     }
 }
 
-// Header: totals over the sequences.  The words go to the workspace (kernels read them there) and
-// straight to the host's pinned buffer, which the host watches, so no copy has to be queued behind the build.
-__device__ void finish_header(const FinishArgs &f, int S) {
+// Header: totals over the sequences.  The words go to the workspace (kernels read them there) and to `host`.
+__device__ void finish_header(const FinishArgs &f, int S, volatile HostHeader *host) {
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     __shared__ int s_err, s_more;
     __shared__ long long s_sum[4];
     if (t == 0) { s_err = 0x7fffffff; s_more = 0; s_sum[0] = s_sum[1] = s_sum[2] = s_sum[3] = 0; }
     __syncthreads();
     const size_t q = (size_t)f.ms * f.B;
-    volatile HostHeader *host = f.host;
     row_sums(4 * S, f.B, w, FT / 32, lane, [&](int i) { return f.counts + (i & 3) * q + (size_t)(i >> 2) * f.B; },
              [&](int i, int v) {
                  StageDesc &d = f.hdr->st[i >> 2];
@@ -1031,8 +1031,7 @@ __device__ void finish_rank(const FinishArgs &f, int s, int part, int parts, lon
 
 // CTA 0: header; then r0 CTAs rank stage 0's blocks and r1 each those of the other stages; then gy
 // CTAs per sequence move its elements and block records to their place in the batch's arrays.
-__global__ void __launch_bounds__(FT) k_finish(const FinishArgs f) {
-    pdl_launch_dependents();
+__device__ __forceinline__ void finish_part(const FinishArgs &f, volatile HostHeader *host) {
     __shared__ long long s_keys[FKEYS];
     __shared__ int s_stages, s_bad;
     __shared__ int s_n[HDT_MAX_STAGES], s_b[HDT_MAX_STAGES], s_cn[HDT_MAX_STAGES], s_cb[HDT_MAX_STAGES];
@@ -1073,7 +1072,7 @@ __global__ void __launch_bounds__(FT) k_finish(const FinishArgs f) {
     __syncthreads();
     const int S = s_stages;
     int id = blockIdx.x;
-    if (id == 0) { finish_header(f, S); return; }
+    if (id == 0) { finish_header(f, S, host); return; }
     if (s_bad) return;               // (offsets of a broken hierarchy mean nothing)
     id -= 1;
     if (id < f.r0) { finish_rank(f, 0, id, f.r0, s_keys); return; }
@@ -1143,6 +1142,29 @@ __global__ void __launch_bounds__(FT) k_finish(const FinishArgs f) {
     }
 }
 
+// The header's words go straight to the host's pinned buffer, which the host watches, so no copy has to be queued behind
+// the build.  A build that is waited for also says when it has ended (`tell`): every CTA's fence and ticket stand behind
+// its writes, so the word of the CTA that is last stands behind all of them.  Its header leaves behind the ticket:
+// a fence behind words to the host waits for their trip.  That costs 2 us of a call that waits, which a deferred build, whose
+// kernel the attention waits for, does not pay.
+__global__ void __launch_bounds__(FT) k_finish(const FinishArgs f) {
+    pdl_launch_dependents();
+    __shared__ HostHeader s_host;
+    finish_part(f, f.tell ? &s_host : f.host);
+    if (!f.tell) return;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (gridDim.x == 1 || atomicAdd(&f.hdr->ticket, 1) == (int)gridDim.x - 1) {      // (alone: no sequences, no k_seq that cleared the ticket)
+            __threadfence_system();
+            *(volatile int *)&f.host->done = 1;
+        }
+    }
+    if (blockIdx.x != 0) return;
+    __syncthreads();
+    for (int i = threadIdx.x; i < HostHeader::words(f.ms); i += FT) (&f.host->status)[i] = (&s_host.status)[i];
+}
+
 }  // namespace hdt
 
 using namespace hdt;
@@ -1188,6 +1210,45 @@ static void pinned_release(HostHeader *p) {
     if (!p) return;
     std::lock_guard<std::mutex> lk(g_pinned_mu);
     g_pinned_free.push_back(p);
+}
+
+// Waits for all that is on the stream, also where another stream of this thread is being captured.  A stream that is being
+// captured itself takes no wait, and needs none: what is captured on it runs behind what it holds.
+static cudaError_t stream_passed(cudaStream_t st) {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaError_t e = cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) return e;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    e = cudaStreamIsCapturing(st, &cap);
+    if (e == cudaSuccess && cap == cudaStreamCaptureStatusNone) e = cudaStreamSynchronize(st);
+    const cudaError_t back = cudaThreadExchangeStreamCaptureMode(&mode);
+    return e != cudaSuccess ? e : back;
+}
+
+// The counts that attention calls need, from the header.
+static void index_counts(hdt_index *ix, const HostHeader &h) {
+    ix->failed = h.status;
+    ix->err_pos = h.err_pos;
+    if (h.status != 0) return;
+    int ns = 1;
+    while (ns < ix->max_stages && h.st[ns][0] > 0) ++ns;
+    if (h.st[ns - 1][4] && ns == ix->max_stages) {
+        ix->failed = HDT_ERR_BAD_HIERARCHY;
+        ix->err_pos = -1;
+        return;
+    }
+    ix->n_stages = ns;
+    auto total = [&](int i) { return (int64_t)h.total[i][0] | (int64_t)h.total[i][1] << 30 | (int64_t)h.total[i][2] << 60; };
+    ix->nnz = total(0);
+    ix->visited = total(1);
+    ix->nnz_upper = total(2);
+    ix->real = total(3);
+    for (int s = 0; s <= HDT_MAX_STAGES; ++s) {
+        StageDesc &d = ix->desc[s];
+        d = StageDesc{};
+        if (s >= ix->max_stages) continue;
+        d.n = h.st[s][0]; d.nb = h.st[s][1]; d.n_fused = h.st[s][2]; d.n_empty = h.st[s][3]; d.has_next = h.st[s][4];
+    }
 }
 
 extern "C" int hdt_build_index(const int8_t *level, const int32_t *parent, const int32_t *cu_seqlens,
@@ -1239,7 +1300,8 @@ extern "C" int hdt_build_index(const int8_t *level, const int32_t *parent, const
     }
     HostHeader *hp = pinned_acquire();
     if (!hp) return set_error(HDT_ERR_CUDA, "hdt_build_index: no pinned host memory for the index header");
-    for (int i = 0; i < HostHeader::words(ms); ++i) reinterpret_cast<int *>(hp)[i] = HostHeader::UNSET;
+    hp->done = HostHeader::UNSET;
+    for (int i = 0; i < HostHeader::words(ms); ++i) (&hp->status)[i] = HostHeader::UNSET;
 
     hdt_index *ix = new hdt_index();
     ix->batch = B; ix->total_tokens = T; ix->block_m = bm; ix->block_m_upper = bmu; ix->n_stages = 0;
@@ -1256,7 +1318,9 @@ extern "C" int hdt_build_index(const int8_t *level, const int32_t *parent, const
     ix->hdr_dev = (const DevHeader *)(ws + L.header);
     ix->stream = st;
     ix->max_stages = ms;
-    ix->pending = 1;
+    const bool deferred = params && params->deferred;
+    ix->tells = !deferred || st == cudaStreamPerThread;
+    ix->state.store(INDEX_QUEUED, std::memory_order_relaxed);
 
     a.level = level; a.parent = parent; a.cu = cu_seqlens;
     a.B = B; a.T = T; a.ms = ms; a.bm = bm; a.bmu = bmu; a.bmin = bmin; a.dirs = dirs;
@@ -1266,6 +1330,7 @@ extern "C" int hdt_build_index(const int8_t *level, const int32_t *parent, const
     a.counts = (int *)(ws + L.counts);
     a.recs = (int4 *)(ws + L.recs);
     a.capnb = L.capnb;
+    a.ticket = &((DevHeader *)(ws + L.header))->ticket;
     a.el = (int4 *)(ws + L.el);
     a.upl = (int *)(ws + L.upl);
     a.glob = (uint32_t *)(ws + L.glob);
@@ -1280,6 +1345,7 @@ extern "C" int hdt_build_index(const int8_t *level, const int32_t *parent, const
     f.keys = (long long *)(ws + L.keys);
     f.hdr = (DevHeader *)(ws + L.header);
     f.host = hp;
+    f.tell = ix->tells;
     cudaError_t e = cudaSuccess;
     {
         ProfScope ps(PROF_INDEX, st);
@@ -1302,7 +1368,7 @@ extern "C" int hdt_build_index(const int8_t *level, const int32_t *parent, const
         if (e == cudaSuccess) {
             // a programmatic dependent: its CTAs are scheduled while k_seq runs and wait for its end
             cudaLaunchConfig_t cfg{};
-            cfg.gridDim = dim3((unsigned)(1 + f.r0 + f.r1 * (ms - 1) + (size_t)B * f.gy));
+            cfg.gridDim = dim3(B > 0 ? (unsigned)(1 + f.r0 + f.r1 * (ms - 1) + (size_t)B * f.gy) : 1u);
             cfg.blockDim = dim3(FT);
             cfg.stream = st;
             cudaLaunchAttribute at[1];
@@ -1319,7 +1385,7 @@ extern "C" int hdt_build_index(const int8_t *level, const int32_t *parent, const
         delete ix;
         return set_error(HDT_ERR_CUDA, "hdt_build_index: launch failed: %s", cudaGetErrorString(e));
     }
-    if (!(params && params->deferred)) {
+    if (!deferred) {
         const int rc = index_ready(ix);
         if (rc) {
             delete ix;
@@ -1331,58 +1397,54 @@ extern "C" int hdt_build_index(const int8_t *level, const int32_t *parent, const
 }
 
 namespace hdt {
-int index_ready(const hdt_index *cix) {
+// (the per-thread default stream has one handle and is another stream in every thread)
+bool index_on_stream(const hdt_index *ix, cudaStream_t st) { return st == ix->stream && st != cudaStreamPerThread; }
+
+int index_wait(const hdt_index *cix, IndexState want) {
     hdt_index *ix = const_cast<hdt_index *>(cix);
-    if (ix->pending) {
-        // The host watches the words of the pinned header.  After a bounded number of looks it waits for the stream instead.
+    if (ix->state.load(std::memory_order_acquire) < want) {
+        std::lock_guard<std::mutex> lk(ix->mu);
         HostHeader *hp = ix->h_pinned;
-        const volatile int *words = reinterpret_cast<const volatile int *>(hp);
-        const int n_words = HostHeader::words(ix->max_stages);
-        int got = 0;
-        auto look = [&]() {
-            while (got < n_words && words[got] != HostHeader::UNSET) ++got;
-            return got == n_words;
+        // The host watches words of the pinned header.  After a bounded number of looks it waits for the stream instead.
+        auto watch = [&](int *first, int n) {
+            const volatile int *words = first;
+            int got = 0;
+            auto look = [&]() {
+                while (got < n && words[got] != HostHeader::UNSET) ++got;
+                return got == n;
+            };
+            for (long long spin = 0; spin < 20000000LL && !look(); ++spin) {}
+            cudaError_t e = cudaSuccess;
+            if (!look()) {
+                e = cudaStreamSynchronize(ix->stream);
+                if (e == cudaSuccess && !look()) e = cudaErrorUnknown;
+            }
+            std::atomic_thread_fence(std::memory_order_acquire);
+            return e;
         };
-        for (long long spin = 0; spin < 20000000LL && !look(); ++spin) {}
-        cudaError_t e_ = cudaSuccess;
-        if (!look()) {
-            e_ = cudaStreamSynchronize(ix->stream);
-            if (e_ == cudaSuccess && !look()) e_ = cudaErrorUnknown;
+        cudaError_t e = cudaSuccess;
+        int state = ix->state.load(std::memory_order_relaxed);
+        if (state == INDEX_QUEUED) {
+            e = watch(&hp->status, HostHeader::words(ix->max_stages));
+            if (e == cudaSuccess) index_counts(ix, *hp);
+            state = INDEX_COUNTED;
         }
-        ix->pending = 0;
-        ix->h_pinned = nullptr;
-        if (e_ != cudaSuccess) {
+        if (e == cudaSuccess && state == INDEX_COUNTED && want == INDEX_COMPLETE) {
+            if (ix->tells) e = watch(&hp->done, 1);
+            else e = stream_passed(ix->stream);
+            state = INDEX_COMPLETE;
+        }
+        if (e != cudaSuccess) {
             (void)cudaGetLastError();
             ix->failed = HDT_ERR_CUDA;
+            state = INDEX_COMPLETE;
+        }
+        if (hp != nullptr && (state == INDEX_COMPLETE || !ix->tells)) {      // nothing more comes
+            ix->h_pinned = nullptr;
             pinned_release(hp);
-            return set_error(HDT_ERR_CUDA, "waiting for the index build failed: %s", cudaGetErrorString(e_));
         }
-        std::atomic_thread_fence(std::memory_order_acquire);
-        const HostHeader h = *hp;
-        pinned_release(hp);
-        ix->failed = h.status;
-        ix->err_pos = h.err_pos;
-        if (h.status == 0) {
-            int ns = 1;
-            while (ns < ix->max_stages && h.st[ns][0] > 0) ++ns;
-            if (h.st[ns - 1][4] && ns == ix->max_stages) {
-                ix->failed = HDT_ERR_BAD_HIERARCHY;
-                ix->err_pos = -1;
-            } else {
-                ix->n_stages = ns;
-                auto total = [&](int i) { return (int64_t)h.total[i][0] | (int64_t)h.total[i][1] << 30 | (int64_t)h.total[i][2] << 60; };
-                ix->nnz = total(0);
-                ix->visited = total(1);
-                ix->nnz_upper = total(2);
-                ix->real = total(3);
-                for (int s = 0; s <= HDT_MAX_STAGES; ++s) {
-                    StageDesc &d = ix->desc[s];
-                    d = StageDesc{};
-                    if (s >= ix->max_stages) continue;
-                    d.n = h.st[s][0]; d.nb = h.st[s][1]; d.n_fused = h.st[s][2]; d.n_empty = h.st[s][3]; d.has_next = h.st[s][4];
-                }
-            }
-        }
+        ix->state.store(state, std::memory_order_release);
+        if (e != cudaSuccess) return set_error(HDT_ERR_CUDA, "waiting for the index build failed: %s", cudaGetErrorString(e));
     }
     if (ix->failed == 0) return HDT_OK;
     if (ix->failed == HDT_ERR_BAD_HIERARCHY && ix->err_pos < 0)
@@ -1417,7 +1479,7 @@ extern "C" int hdt_index_export(const hdt_index_t *ix, int32_t stage, hdt_stage_
 }
 
 extern "C" int hdt_index_destroy(hdt_index_t *ix) {
-    if (ix && ix->pending) (void)index_ready(ix);     // the header must not land in a recycled buffer
+    if (ix) (void)index_wait(ix, INDEX_COUNTED);     // the header must not land in a recycled buffer
     delete ix;
     return HDT_OK;
 }

@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <atomic>
+#include <mutex>
 
 #include "../../include/hdt.h"
 #include "../../include/hdt_debug.h"
@@ -19,6 +20,7 @@ struct StageDesc {
 };
 
 struct DevHeader {
+    int ticket;              // CTAs of the build's last kernel that are done
     int status;              // hdt_status_t, first error wins
     int err_pos;             // element / sequence where it was detected
     long long nnz;           // unmasked pairs
@@ -31,12 +33,16 @@ struct DevHeader {
 // The header as it lands in pinned host memory: 32-bit words in any order, none of which ever is UNSET (totals go
 // in pieces of 30 bits).  The host fills the words with UNSET before the build and has the header when none is
 // left: the device sends them without a fence, which would hold up the end of its kernel by a trip to the host.
+// The words may come while other CTAs of the build still write the index.  `done`, which a build that is waited for also
+// sends, comes from the last of these, behind all their reads and writes: from then on any stream or thread may
+// read the index or reuse the build's buffers.
 struct HostHeader {
     static constexpr int UNSET = 0x7fffffff, TOTALS = 4;
+    int done;
     int status, err_pos;
     int total[TOTALS][3];    // nnz, visited, nnz_upper, real
     int st[HDT_MAX_STAGES][5];    // n, nb, n_fused, n_empty, has_next
-    static int words(int stages) { return 2 + 3 * TOTALS + 5 * stages; }
+    static __host__ __device__ int words(int stages) { return 2 + 3 * TOTALS + 5 * stages; }     // (from `status` on)
 };
 
 // Host-side pointers to one stage's arrays inside the workspace.
@@ -55,11 +61,12 @@ struct hdt_index {
     void *workspace;
     size_t workspace_bytes;
     const int *rank;                  // device [total_tokens]: a token's number among its siblings (undefined for roots and PAD)
-    // Deferred build: the device header is on its way to h_pinned; hdt::index_ready() waits for it
-    // and fills n_stages, nnz, visited and desc.
-    int pending;                      // 1 until the header has been read
+    // The header of the build lands in h_pinned; hdt::index_wait() reads it there and fills n_stages, nnz, visited and desc.
+    std::atomic<int> state;           // what of the build has been waited for: hdt::IndexState
+    std::mutex mu;                    // held while the state changes: several threads may use one index
     int failed;                       // hdt_status_t found in the header (or by its check), 0 = fine
     int err_pos, max_stages;
+    int tells;                        // the build sends HostHeader::done (a deferred one does not: its stream is waited for)
     hdt::HostHeader *h_pinned;         // pinned landing buffer (from a pool), nullptr once released
     const hdt::DevHeader *hdr_dev;    // the header in the index workspace
     cudaStream_t stream;              // stream of the build
@@ -68,9 +75,19 @@ struct hdt_index {
 namespace hdt {
 
 int set_error(int code, const char *fmt, ...);
-// Waits (if the build was deferred) until the counts of the index are on the host; returns the
-// structure error of the build, if any.
-int index_ready(const hdt_index *ix);
+// INDEX_QUEUED: the build's kernels are on their stream.  INDEX_COUNTED: the counts are on the host; work that is queued
+// on the stream of the build may use the index.  INDEX_COMPLETE: the build has ended, any stream may.
+enum IndexState { INDEX_QUEUED = 0, INDEX_COUNTED, INDEX_COMPLETE };
+// Waits until the build has come to that state; returns the structure error of the build, if any.
+int index_wait(const hdt_index *ix, IndexState state);
+inline int index_ready(const hdt_index *ix) { return index_wait(ix, INDEX_COMPLETE); }
+// Whether `st` is the stream of the build, so that what is queued on it comes behind the build.
+bool index_on_stream(const hdt_index *ix, cudaStream_t st);
+// For work about to be queued on `st`.
+inline int index_ready(const hdt_index *ix, cudaStream_t st) {
+    if (ix->state.load(std::memory_order_acquire) == INDEX_COMPLETE) return index_wait(ix, INDEX_COMPLETE);
+    return index_wait(ix, index_on_stream(ix, st) ? INDEX_COUNTED : INDEX_COMPLETE);
+}
 int *device_status_ptr();  // device address of the failure word kernels report into
 extern std::atomic<long long> g_launches;
 inline void count_launch(int n = 1) { g_launches.fetch_add(n, std::memory_order_relaxed); }
