@@ -191,8 +191,8 @@ __global__ void __launch_bounds__(256) k_cross_zero(const int8_t *__restrict__ l
 }
 
 // ---- decoding ------------------------------------------------------------------------------------
-// CTA (y, b, z): the y-th share of document b's tokens, heads z * HC ..., every decoder row of the document in
-// turn.  Thread (slot, head, lane): D / 8 lanes per (key, head), the heads of a token next to one another, so that a
+// CTA (b, y, z): the y-th share of document b's tokens, heads z * HC ..., every decoder row of the document in
+// turn (a grid holds 2^31 documents along x, 65535 along y).  Thread (slot, head, lane): D / 8 lanes per (key, head), the heads of a token next to one another, so that a
 // CTA reads whole token rows.  The bound is reading K and V once (4 x 8192 tokens, 12 x 64: 101 MB, 15 us at the
 // copy rate): four keys a thread in flight and four CTAs an SM; the tile kernel took 352 us here, one CTA per
 // document and head walking 64 chunks with one row of 128 in use.
@@ -216,12 +216,12 @@ __global__ void __launch_bounds__(512, 2) k_cross_decode(const DecodeArgs a) {
     extern __shared__ float s_red[];                 // [KS][HC][D + 2]
     __shared__ int s_list[DEC_LIST];
     __shared__ int s_n;
-    const int b = blockIdx.y, t = threadIdx.x, lane = t & 31, g = t % LPK, src = lane - g;
+    const int b = blockIdx.x, t = threadIdx.x, lane = t & 31, g = t % LPK, src = lane - g;
     const unsigned mask = ((1u << LPK) - 1u) << src;
     const int pair = t / LPK, hl = pair % a.HC, ks = pair / a.HC, h = blockIdx.z * a.HC + hl;
     const bool on = ks < a.KS && h < a.H;
     const int k0 = a.cu_k[b], k1 = a.cu_k[b + 1], q0 = a.cu_q[b], q1 = a.cu_q[b + 1];
-    const int per = (k1 - k0 + a.splits - 1) / a.splits, c0 = min(k1, k0 + (int)blockIdx.x * per), c1 = min(k1, c0 + per);
+    const int per = (k1 - k0 + a.splits - 1) / a.splits, c0 = min(k1, k0 + (int)blockIdx.y * per), c1 = min(k1, c0 + per);
     for (int row = q0; row < q1; ++row) {
         RowSoftmax S;
         S.clear();
@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(512, 2) k_cross_decode(const DecodeArgs a) {
                 W::store(a.o, (unsigned)row * a.H + h, g, R.acc);
                 if (g == 0) a.lse[(size_t)h * a.Tq + row] = lse;
             } else {
-                const size_t r = ((size_t)blockIdx.x * a.Tq + row) * a.H + h;
+                const size_t r = ((size_t)blockIdx.y * a.Tq + row) * a.H + h;
                 W::store_f32(a.part_o, r, g, R.acc);
                 if (g == 0) a.part_lse[r] = lse;
             }
@@ -359,7 +359,7 @@ static int launch_decode_t(DecodeArgs a, int B, cudaStream_t st) {
     a.KS = max(1, min(16, 384 / (a.HC * LPK)));
     const int threads = (a.HC * LPK * a.KS + 31) / 32 * 32;
     const size_t smem = sizeof(float) * (size_t)a.KS * a.HC * (D + 2);
-    HDT_CUDA_CHECK(launch_dependent(k_cross_decode<D, BF16>, true, dim3(a.splits, B, (a.H + a.HC - 1) / a.HC), threads, smem, st, a));
+    HDT_CUDA_CHECK(launch_dependent(k_cross_decode<D, BF16>, true, dim3(B, a.splits, (a.H + a.HC - 1) / a.HC), threads, smem, st, a));
     return HDT_OK;
 }
 

@@ -39,6 +39,22 @@ def test_cross_splits(dtype, d, lengths, rows, mask):
         check_close(host(x), r, dtype, what, out_rounding=True, row_rel=2.0 ** -8)
 
 
+def test_cross_decode_many_documents():
+    """A decoding step for more documents than a grid has rows: one token and one decoder row each, so O is V and the
+    log-sum-exp the one score."""
+    import torch
+    import paper_2407_08330_b200 as P
+    B, H, d = 65537, 2, 64
+    g = torch.Generator(device="cuda").manual_seed(1)
+    q, k, v = (torch.randn(B, H, d, generator=g, device="cuda") for _ in range(3))
+    cu = torch.arange(B + 1, dtype=torch.int32, device="cuda")
+    o, lse = P.hdt_cross_attn_fwd(torch.zeros(B, dtype=torch.int8, device="cuda"), cu, cu, 1, q, k, v)
+    torch.cuda.synchronize()
+    P.hdt_device_status()
+    check_close(host(o), host(v), "f32", "O")
+    check_close(host(lse), host((q.double() * k.double()).sum(-1).T / d ** 0.5), "f32", "LSE")
+
+
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 @pytest.mark.parametrize("accumulate", [True, False])
 @pytest.mark.parametrize("T,d_model", [(1, 8), (31, 1024), (33, 256), (9473, 64), (9999, 264)])
