@@ -7,7 +7,7 @@
 // The chosen rows are never copied.
 //   few decoder rows a document (a step of autoregressive decoding): k_cross_decode reads levels, K and V once, the
 //         tokens of a document dealt to many CTAs, and k_cross_combine merges their partial results.  No index.
-//   otherwise one kernel (k_cross_index) builds one element space for both sides: elements 0 .. Tq-1 are
+//   otherwise k_cross_index (of large batches behind a count and a scan) builds one element space for both sides: elements 0 .. Tq-1 are
 //         the decoder rows (token map = identity, into Q / dO / O), elements Tq .. Tq+ns-1 the chosen
 //         encoder tokens in order (token map = their index, into K / V); a decoder row's key range is its
 //         document's slice of the second part, a chosen token's range the document's decoder rows.  The
@@ -32,7 +32,7 @@ namespace hdt {
 constexpr int XC = 32;      // CTAs (contiguous chunks) per document in the index kernel
 
 struct CrossLayout {
-    size_t tokx, rngx, blocks, queue, delta, part, part_lse, total;
+    size_t sel, tokx, rngx, blocks, queue, delta, part, part_lse, total;
     int nbq, nbk, xr;
 };
 
@@ -68,6 +68,7 @@ static CrossLayout cross_layout(int B, int T, int Tq, int H, int D, bool tc, int
     L.tokx = o; o += al256c(sizeof(int) * max(n, (size_t)1));
     L.rngx = o; o += al256c(sizeof(int) * 2 * max(n, (size_t)1));
     L.queue = o; o += al256c(sizeof(int) * (size_t)(L.nbq + L.nbk));
+    L.sel = o; o += al256c(sizeof(int) * (size_t)(B + 1));
     L.delta = o; if (bwd) o += al256c(sizeof(float) * (size_t)H * max(Tq, 1));
     // partial results [splits, Tq, H, D] and, in the forward, their LSE
     const size_t splits = !bwd && cross_decode(B, Tq) ? decode_splits(B, T) : tile_splits(B, T, Tq, H, -1, bwd ? 8 : 2);
@@ -84,13 +85,70 @@ struct CrossIndexArgs {
     const int8_t *level;
     const int32_t *cu_k, *cu_q;
     int B, T, Tq, level_mask, xr, nbq, nbk;
+    const int *sel;               // [B + 1] chosen tokens before each document and in all, or nullptr: counted by every CTA itself
     int *tokx, *rngx, *blocks, *queue;
 };
 
+// Which of 16 levels are chosen, one bit each.
+__device__ __forceinline__ unsigned chosen_bits(const uint4 &x, int level_mask) {
+    const uint32_t xs[4] = {x.x, x.y, x.z, x.w};
+    unsigned bits = 0;
+#pragma unroll
+    for (int j = 0; j < 16; ++j) bits |= (unsigned)chosen_level((int8_t)(xs[j >> 2] >> (8 * (j & 3))), level_mask) << j;
+    return bits;
+}
+// This thread's share (t of 256) of the number of chosen tokens in [lo, hi).
+__device__ __forceinline__ int count_chosen(const int8_t *level, int lo, int hi, int level_mask, int t) {
+    int n = 0;
+    const bool vec = ((uintptr_t)level & 15) == 0;
+    const int u1 = vec ? hi / 16 : 0, body = min(hi, (lo + 15) / 16 * 16);      // whole units: [body / 16, u1)
+    for (int u = body / 16 + t; u < u1; u += 256) n += __popc(chosen_bits(reinterpret_cast<const uint4 *>(level)[u], level_mask));
+    const int rest = max(body, 16 * u1);
+    for (int i = lo + t; i < body; i += 256) n += chosen(level, i, level_mask);
+    for (int i = rest + t; i < hi; i += 256) n += chosen(level, i, level_mask);
+    return n;
+}
+
+// Many tokens and documents (see cross_build): chosen tokens of each document, sel[b + 1], and their sums, sel[0] = 0.
+__global__ void __launch_bounds__(256) k_cross_count(const int8_t *level, const int32_t *cu_k, int level_mask, int *sel) {
+    pdl_wait();
+    pdl_launch_dependents();
+    __shared__ int s_n;
+    const int b = blockIdx.x, t = threadIdx.x;
+    if (t == 0) s_n = 0;
+    __syncthreads();
+    const int n = __reduce_add_sync(0xffffffffu, count_chosen(level, cu_k[b], cu_k[b + 1], level_mask, t));
+    if ((t & 31) == 0) atomicAdd(&s_n, n);
+    __syncthreads();
+    if (t == 0) sel[b + 1] = s_n;
+}
+__global__ void __launch_bounds__(1024) k_cross_scan(int *sel, int B) {
+    pdl_wait();
+    pdl_launch_dependents();
+    __shared__ int s_w[32];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    int run = 0;
+    if (t == 0) sel[0] = 0;
+    for (int b0 = 0; b0 < B; b0 += 1024) {
+        int v = b0 + t < B ? sel[b0 + t + 1] : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int x = __shfl_up_sync(0xffffffffu, v, o); if (lane >= o) v += x; }
+        if (lane == 31) s_w[w] = v;
+        __syncthreads();
+        int u = s_w[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int x = __shfl_up_sync(0xffffffffu, u, o); if (lane >= o) u += x; }
+        const int before = w ? __shfl_sync(0xffffffffu, u, w - 1) : 0;
+        if (b0 + t < B) sel[b0 + t + 1] = run + before + v;
+        run += __shfl_sync(0xffffffffu, u, 31);
+        __syncthreads();
+    }
+}
+
 // Chunk y of document b: its part of the ordered list of chosen tokens (elements Tq + position, with their row
 // ranges) and its share of the document's decoder rows and of the block records of both sides.  Where
-// its part starts is counted over the levels of all tokens before it by the CTA itself: a byte a token, read by
-// every CTA, costs less than the launches of a count and a scan kernel (four launches with a clear, 14 us of every call).
+// its part starts is counted over the levels of all tokens before it by the CTA itself while that costs less than the
+// launches of a count and a scan kernel; beyond, over those of its document (see cross_build).
 __global__ void __launch_bounds__(256) k_cross_index(const CrossIndexArgs a) {
     pdl_wait();
     pdl_launch_dependents();
@@ -103,7 +161,11 @@ __global__ void __launch_bounds__(256) k_cross_index(const CrossIndexArgs a) {
     const int cs = (k1 - k0 + XC - 1) / XC, c0 = min(k1, k0 + y * cs), c1 = min(k1, c0 + cs);
     if (t < 4) s_n[t] = 0;
     __syncthreads();
-    {   // chosen tokens below k0, c0, k1 and in all
+    if (a.sel != nullptr) {
+        const int n = __reduce_add_sync(0xffffffffu, count_chosen(level, k0, c0, mask, t));
+        if (lane == 0) atomicAdd(&s_n[1], n);
+        if (t == 0) { s_n[0] = a.sel[b]; s_n[2] = a.sel[b + 1]; s_n[3] = a.sel[a.B]; atomicAdd(&s_n[1], a.sel[b]); }
+    } else {   // chosen tokens below k0, c0, k1 and in all
         int n0 = 0, n1 = 0, n2 = 0, n3 = 0;
         const bool vec = ((uintptr_t)level & 15) == 0;
         const int units = vec ? a.T / 16 : 0;
@@ -113,14 +175,10 @@ __global__ void __launch_bounds__(256) k_cross_index(const CrossIndexArgs a) {
             for (int k = 0; k < 4; ++k) x4[k] = u0 + 256 * k < units ? reinterpret_cast<const uint4 *>(level)[u0 + 256 * k] : make_uint4(~0u, ~0u, ~0u, ~0u);
 #pragma unroll 1
             for (int k = 0; k < 4; ++k) {
-            const uint4 x = k == 0 ? x4[0] : k == 1 ? x4[1] : k == 2 ? x4[2] : x4[3];
-            const uint32_t xs[4] = {x.x, x.y, x.z, x.w};
-            const int i0 = 16 * (u0 + 256 * k);
-            unsigned bits = 0;
-#pragma unroll
-            for (int j = 0; j < 16; ++j) bits |= (unsigned)chosen_level((int8_t)(xs[j >> 2] >> (8 * (j & 3))), mask) << j;
-            auto below = [&](int lim) { const int d = lim - i0; return d <= 0 ? 0 : __popc(d >= 16 ? bits : bits & ((1u << d) - 1u)); };
-            n0 += below(k0); n1 += below(c0); n2 += below(k1); n3 += __popc(bits);
+                const unsigned bits = chosen_bits(k == 0 ? x4[0] : k == 1 ? x4[1] : k == 2 ? x4[2] : x4[3], mask);
+                const int i0 = 16 * (u0 + 256 * k);
+                auto below = [&](int lim) { const int d = lim - i0; return d <= 0 ? 0 : __popc(d >= 16 ? bits : bits & ((1u << d) - 1u)); };
+                n0 += below(k0); n1 += below(c0); n2 += below(k1); n3 += __popc(bits);
             }
         }
         for (int i = units * 16 + t; i < a.T; i += 256) {
@@ -363,6 +421,11 @@ static int launch_decode_t(DecodeArgs a, int B, cudaStream_t st) {
     return HDT_OK;
 }
 
+// Index of both sides.  Counting in every CTA reads a batch's levels 32 times per document, a time that grows with documents
+// times tokens; the count and scan kernels read them once more, for two launches.  The line lies between the
+// sizes timed (forward, 8 rows a document, 2 x 64): 4 x 8192 tokens (131 000) 23.2 us without them, 24.4 with; 8 x 8192
+// (524 000) 29.9 and 24.9; 256 x 1024 892 and 43; 1024 x 128 1806 and 138.
+static constexpr long long COUNT_LINE = 200000;
 static int cross_build(const CrossLayout &L, char *ws, const int8_t *level, const int32_t *cu_k, const int32_t *cu_q, int B, int T, int Tq, int level_mask,
                        cudaStream_t st) {
     if (B <= 0) return HDT_OK;
@@ -370,6 +433,12 @@ static int cross_build(const CrossLayout &L, char *ws, const int8_t *level, cons
     a.level = level; a.cu_k = cu_k; a.cu_q = cu_q; a.B = B; a.T = T; a.Tq = Tq; a.level_mask = level_mask;
     a.xr = L.xr; a.nbq = L.nbq; a.nbk = L.nbk;
     a.tokx = (int *)(ws + L.tokx); a.rngx = (int *)(ws + L.rngx); a.blocks = (int *)(ws + L.blocks); a.queue = (int *)(ws + L.queue);
+    if ((long long)B * T > COUNT_LINE) {
+        int *sel = (int *)(ws + L.sel);
+        a.sel = sel;
+        HDT_CUDA_CHECK(launch_dependent(k_cross_count, true, dim3(B), 256, 0, st, level, cu_k, level_mask, sel));
+        HDT_CUDA_CHECK(launch_dependent(k_cross_scan, true, dim3(1), 1024, 0, st, sel, B));
+    }
     HDT_CUDA_CHECK(launch_dependent(k_cross_index, true, dim3(B, XC), 256, 0, st, a));
     return HDT_OK;
 }

@@ -39,6 +39,41 @@ def test_cross_splits(dtype, d, lengths, rows, mask):
         check_close(host(x), r, dtype, what, out_rounding=True, row_rel=2.0 ** -8)
 
 
+@pytest.mark.parametrize("n,longest", [(40, 1500), (1100, 260)])        # (the scan takes 1024 documents at a time)
+def test_cross_index_counted(n, longest):
+    """More documents times tokens than every block of the index kernel counts itself, at odd places in the arrays."""
+    import torch
+    import paper_2407_08330_b200 as P
+    rng = np.random.default_rng(n)
+    docs = [gen.gen_fill(rng, int(k), (2, 6), (2, 8), (3, 20))[:2] for k in rng.integers(1, longest, n)]
+    docs[n // 2] = (np.zeros(0, np.int8), np.zeros(0, np.int32))
+    b = gen.pack(docs)
+    rows = rng.integers(0, 12, n)
+    rows[n // 3] = 150
+    H, d, T, Tq = 2, 64, b.total_tokens, int(rows.sum())
+    assert n * T > 200000 and Tq > 4 * n
+    cu_q = np.concatenate([[0], np.cumsum(rows)]).astype(np.int32)
+    t = gen.make_tensors(3, T, H, d, "bf16", names=("k", "v"))
+    tq = gen.make_tensors(4, Tq, H, d, "bf16", names=("q", "do"))
+    _, _, cu = dev_struct(b)
+    level = torch.empty(T + 1, dtype=torch.int8, device="cuda")
+    q, do, k, v = (dev_tensor(x, "bf16") for x in (tq["q"], tq["do"], t["k"], t["v"]))
+    cq = torch.from_numpy(cu_q).cuda()
+    for mask, shift in ((6, 0), (15, 0), (6, 1)):          # (levels at an odd address: no wide loads)
+        lv = level[shift:shift + T]
+        lv.copy_(torch.from_numpy(b.level))
+        o, lse = P.hdt_cross_attn_fwd(lv, cu, cq, mask, q, k, v)
+        g = P.hdt_cross_attn_bwd(lv, cu, cq, mask, q, k, v, o, lse, do)
+        torch.cuda.synchronize()
+        P.hdt_device_status()
+        o_r, lse_r = cross_oracle.forward(b.level, b.cu_seqlens, mask, cu_q, tq["q"], t["k"], t["v"])
+        g_r = cross_oracle.backward(b.level, b.cu_seqlens, mask, cu_q, tq["q"], t["k"], t["v"], tq["do"])
+        check_close(host(o), o_r, "bf16", "O", out_rounding=True)
+        check_close(lse.cpu().numpy(), lse_r, "bf16", "LSE")
+        for x, r, what in zip(g, g_r, ("dQ", "dK", "dV")):
+            check_close(host(x), r, "bf16", what, out_rounding=True, row_rel=2.0 ** -8)
+
+
 def test_cross_decode_many_documents():
     """A decoding step for more documents than a grid has rows: one token and one decoder row each, so O is V and the
     log-sum-exp the one score."""
