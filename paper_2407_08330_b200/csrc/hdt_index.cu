@@ -1,12 +1,13 @@
 // Device-side index builder: (level, parent, cu_seqlens) -> staged family ranges, row blocks,
 // work queues.  Integer work only; every array must equal the sequential definition bit for bit.
 //
-// Two launches, whatever the number of stages:
+// Two launches, whatever the number of stages (four for batches of many blocks, see many_blocks):
 //   k_seq     one CTA per sequence, its arrays in shared memory: validation, child counts, family
 //             ranges, compaction to the next stage, greedy packing of row blocks, block records - for
 //             all stages of the sequence, in sequence-relative numbers, beside the counts of the stage
 //   k_finish  adds the sequences' offsets (sums over the sequences before it), ranks the blocks of a
 //             stage by cost (longest first), and sends the header to the host
+//             (many blocks: with the offsets from k_offsets, the ranks from the runs that k_sort has sorted)
 // Per stage (array of n elements in document order):
 //   counts    cnt[p] = children of p, and whether one of them has children
 //   ranges    a node whose children are all childless heads a family; head and children get
@@ -21,6 +22,7 @@
 // (57 tokens, fp32, build and forward), 76 -> 56 (8 x 2048, build and forward), 1100 -> 807 (200 trees, build,
 // forward and backward).
 #include <cstdio>
+#include <climits>
 #include <cstring>
 #include <atomic>
 #include <mutex>
@@ -40,8 +42,16 @@ struct SeqInfo {
     long long nnz, nnz_upper, visited;
 };
 
+// Sums over the sequences of a batch of many (k_offsets).
+struct BatchSums {
+    int stages, first_err, more;         // stages of the batch; first sequence with an error, or NO_SEQ; SeqInfo::more of any
+    long long nnz, visited, nnz_upper, real;
+    int count[HDT_MAX_STAGES][4];        // of each stage: elements, blocks, SELF non-EMPTY blocks, EMPTY blocks
+};
+static constexpr int NO_SEQ = 0x7fffffff;
+
 struct Layout {
-    size_t header, info, counts, rank, recs, el, upl, glob, keys, stage0, stage_stride;
+    size_t header, info, sums, offs, counts, rank, recs, el, upl, glob, keys, before, stage0, stage_stride;
     size_t s_tok, s_par, s_rng, s_up, s_scu, s_blocks, s_queue, s_queue2;  // offsets inside a stage
     size_t total;
     int capnb;
@@ -57,10 +67,13 @@ static Layout make_layout(int B, int T, int bm, int max_stages) {   // bm: the s
     size_t o = 0;
     L.header = o; o += al(sizeof(DevHeader));
     L.info = o; o += al(sizeof(SeqInfo) * (size_t)B);
+    L.sums = o; o += al(sizeof(BatchSums));
+    L.offs = o; o += al(sizeof(int) * 2 * (size_t)max_stages * B);
     L.counts = o; o += al(sizeof(int) * 4 * (size_t)max_stages * B);
     L.rank = o; o += al(sizeof(int) * (size_t)T);
     L.recs = o; o += al(sizeof(int4) * (size_t)max_stages * L.capnb);
     L.keys = o; o += al(sizeof(long long) * (size_t)max_stages * L.capnb);
+    L.before = o; o += al(sizeof(int) * (size_t)max_stages * L.capnb);
     L.el = o; o += al(sizeof(int4) * (size_t)(max_stages - 1) * T);
     L.upl = o; o += al(sizeof(int) * (size_t)(max_stages - 1) * T);
     L.glob = o; o += NGLOB * al(sizeof(int) * (size_t)T);
@@ -885,9 +898,12 @@ struct FinishArgs {
     int B, T, ms, bm, bmu, bmin, capnb, gy, r0, r1;   // gy: CTAs of a sequence; r0 / r1: CTAs that rank the blocks of stage 0 / of another stage
     const SeqInfo *info;
     const int *counts;
+    const BatchSums *sums;         // set: k_offsets has run, and offs[2][ms][B] holds the elements and blocks before each sequence
+    const int *offs;
     const int4 *recs, *el;
     const int *upl;
     long long *keys;
+    int *before;
     DevHeader *hdr;
     HostHeader *host;              // pinned landing buffer
     int tell;                      // 1: HostHeader::done is sent
@@ -920,31 +936,92 @@ __device__ __forceinline__ void row_sums(int rows, int m, int w, int nw, int lan
     }
 }
 
+// Totals over the sequences by nt threads, added to sum[4] and merged into *err (the first sequence with one) and *more in
+// shared memory.
+__device__ __forceinline__ void seq_sums(const SeqInfo *info, int B, int t, int nt, long long *sum, int *err, int *more) {
+    long long v[4] = {0, 0, 0, 0};
+    for (int b = t; b < B; b += nt) {
+        const SeqInfo &x = info[b];
+        v[0] += x.nnz; v[1] += x.visited; v[2] += x.nnz_upper; v[3] += x.real;
+        if (x.err) atomicMin(err, b);
+        if (x.more) *more = 1;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        v[i] = warp_sum(v[i]);
+        if ((t & 31) == 0) atomicAdd((unsigned long long *)&sum[i], (unsigned long long)v[i]);
+    }
+}
+
+// Batches of many sequences (see hdt_build_index), between the two others: CTA i the sums and, of elements and blocks, the
+// offsets of count row i; the last CTA what is summed over SeqInfo.
+static constexpr int OT = 512;
+__global__ void __launch_bounds__(OT) k_offsets(const SeqInfo *info, const int *counts, int B, int ms, BatchSums *sums, int *offs) {
+    pdl_wait();
+    pdl_launch_dependents();
+    __shared__ int s_w[OT / 32], s_err, s_more, s_stages;
+    __shared__ long long s_sum[4];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    if ((int)blockIdx.x == 4 * ms) {
+        if (t == 0) { s_err = NO_SEQ; s_more = 0; s_stages = 1; s_sum[0] = s_sum[1] = s_sum[2] = s_sum[3] = 0; }
+        __syncthreads();
+        seq_sums(info, B, t, OT, s_sum, &s_err, &s_more);
+        int m = 1;
+        for (int b = t; b < B; b += OT) m = max(m, info[b].stages);
+        m = __reduce_max_sync(0xffffffffu, m);
+        if (lane == 0) atomicMax(&s_stages, m);
+        __syncthreads();
+        if (t == 0) {
+            sums->stages = s_stages; sums->first_err = s_err; sums->more = s_more;
+            sums->nnz = s_sum[0]; sums->visited = s_sum[1]; sums->nnz_upper = s_sum[2]; sums->real = s_sum[3];
+        }
+        return;
+    }
+    const int c = blockIdx.x & 3, s = blockIdx.x >> 2;
+    const int *row = counts + (size_t)c * ms * B + (size_t)s * B;
+    int *out = c < 2 ? offs + ((size_t)c * ms + s) * B : nullptr;
+    int run = 0;
+    for (int b0 = 0; b0 < B; b0 += OT) {
+        const int x = b0 + t < B ? row[b0 + t] : 0;
+        int v = x;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(0xffffffffu, v, o); if (lane >= o) v += y; }
+        if (lane == 31) s_w[w] = v;
+        __syncthreads();
+        int all;
+        const int before = __shfl_sync(0xffffffffu, warp_offsets(s_w, OT / 32, lane, all), w);
+        if (out != nullptr && b0 + t < B) out[b0 + t] = run + before + v - x;
+        run += all;
+        __syncthreads();
+    }
+    if (t == 0) sums->count[s][c] = run;
+}
+
 // Header: totals over the sequences.  The words go to the workspace (kernels read them there) and to `host`.
 __device__ void finish_header(const FinishArgs &f, int S, volatile HostHeader *host) {
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     __shared__ int s_err, s_more;
     __shared__ long long s_sum[4];
-    if (t == 0) { s_err = 0x7fffffff; s_more = 0; s_sum[0] = s_sum[1] = s_sum[2] = s_sum[3] = 0; }
+    if (t == 0) { s_err = NO_SEQ; s_more = 0; s_sum[0] = s_sum[1] = s_sum[2] = s_sum[3] = 0; }
     __syncthreads();
     const size_t q = (size_t)f.ms * f.B;
-    row_sums(4 * S, f.B, w, FT / 32, lane, [&](int i) { return f.counts + (i & 3) * q + (size_t)(i >> 2) * f.B; },
-             [&](int i, int v) {
-                 StageDesc &d = f.hdr->st[i >> 2];
-                 const int c = i & 3;
-                 int *pd = c == 0 ? &d.n : c == 1 ? &d.nb : c == 2 ? &d.n_fused : &d.n_empty;
-                 *pd = v;
-                 host->st[i >> 2][c] = v;
-             });
-    long long nnz = 0, vis = 0, nup = 0, real = 0;
-    for (int b = t; b < f.B; b += FT) {
-        const SeqInfo &x = f.info[b];
-        nnz += x.nnz; vis += x.visited; nup += x.nnz_upper; real += x.real;
-        if (x.err) atomicMin(&s_err, b);
-        if (x.more) s_more = 1;
+    auto put_count = [&](int i, int v) {
+        StageDesc &d = f.hdr->st[i >> 2];
+        const int c = i & 3;
+        int *pd = c == 0 ? &d.n : c == 1 ? &d.nb : c == 2 ? &d.n_fused : &d.n_empty;
+        *pd = v;
+        host->st[i >> 2][c] = v;
+    };
+    if (f.sums != nullptr) {
+        if (t < 4 * S) put_count(t, f.sums->count[t >> 2][t & 3]);
+        if (t == 0) {
+            s_err = f.sums->first_err; s_more = f.sums->more;
+            s_sum[0] = f.sums->nnz; s_sum[1] = f.sums->visited; s_sum[2] = f.sums->nnz_upper; s_sum[3] = f.sums->real;
+        }
+    } else {
+        row_sums(4 * S, f.B, w, FT / 32, lane, [&](int i) { return f.counts + (i & 3) * q + (size_t)(i >> 2) * f.B; }, put_count);
+        seq_sums(f.info, f.B, t, FT, s_sum, &s_err, &s_more);
     }
-    nnz = warp_sum(nnz); vis = warp_sum(vis); nup = warp_sum(nup); real = warp_sum(real);
-    if (lane == 0) { atomicAdd((unsigned long long *)&s_sum[0], (unsigned long long)nnz); atomicAdd((unsigned long long *)&s_sum[1], (unsigned long long)vis); atomicAdd((unsigned long long *)&s_sum[2], (unsigned long long)nup); atomicAdd((unsigned long long *)&s_sum[3], (unsigned long long)real); }
     __syncthreads();
     if (t <= HDT_MAX_STAGES) {
         const int more = (t + 1 < S) || (t + 1 == S && s_more);
@@ -959,11 +1036,109 @@ __device__ void finish_header(const FinishArgs &f, int S, volatile HostHeader *h
     if (t == 0) {
         int err = 0, pos = 0;
         if (f.B == 0) { f.st[0].scu[0] = f.cu[0]; if (f.cu[0] != 0 || f.T != 0) err = HDT_ERR_BAD_HIERARCHY; }
-        else if (s_err != 0x7fffffff) { err = f.info[s_err].err; pos = f.info[s_err].err_pos; }
+        else if (s_err != NO_SEQ) { err = f.info[s_err].err; pos = f.info[s_err].err_pos; }
         f.hdr->status = err; f.hdr->err_pos = pos; f.hdr->nnz = s_sum[0]; f.hdr->visited = s_sum[1]; f.hdr->nnz_upper = s_sum[2]; f.hdr->real = s_sum[3];
         host->status = err; host->err_pos = pos;
         for (int i = 0; i < HostHeader::TOTALS; ++i)
             for (int k = 0; k < 3; ++k) host->total[i][k] = (int)((s_sum[i] >> (30 * k)) & 0x3fffffff);
+    }
+}
+
+// cost << 1 | SELF non-EMPTY
+__device__ __forceinline__ long long block_key(const int4 &r) {
+    const int fl = r.w >> 8;
+    return ((long long)(r.w & 255) * (r.z - r.y)) * 2 + ((fl & HDT_BLK_SELF) && !(fl & HDT_BLK_EMPTY) ? 1 : 0);
+}
+
+// Large batches (see hdt_build_index): the blocks of a stage in runs of SORT_RUN, each sorted by one CTA.  keys: descending cost,
+// then id, as one ascending number (SORT_COST - cost) << 12 | place in the run << 1 | SELF non-EMPTY; before: how
+// many of the last kind come before an entry in its run.
+static constexpr int SORT_RUN = 1024, ST = 512;
+static constexpr long long SORT_COST = (1LL << 40) - 1;     // (128 rows x 2^31 keys at most)
+__global__ void __launch_bounds__(ST) k_sort(const FinishArgs f) {
+    pdl_wait();
+    pdl_launch_dependents();
+    __shared__ long long s_key[SORT_RUN];
+    __shared__ int s_w[ST / 32];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5, s = blockIdx.y, j0 = blockIdx.x * SORT_RUN;
+    const int nb = f.sums->count[s][1], n = min(SORT_RUN, nb - j0);
+    if (f.sums->first_err != NO_SEQ || s >= f.sums->stages || n <= 0) return;
+    const int *offs = f.offs + ((size_t)f.ms + s) * f.B;
+    for (int i = t; i < SORT_RUN; i += ST) {
+        long long k = LLONG_MAX;
+        if (i < n) {
+            int lo = 0, hi = f.B;        // its sequence is the last one that starts at or before it
+            while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (offs[mid] <= j0 + i) lo = mid; else hi = mid; }
+            k = 0;                       // (beyond its own stages a sequence has its root alone, in a block without keys: cost 0)
+            if (s < f.info[lo].stages)
+                k = block_key(f.recs[(size_t)s * f.capnb + block_slot(min(max(f.cu[lo], 0), f.T), lo, f.bmin) + (j0 + i - offs[lo])]);
+            k = (SORT_COST - (k >> 1)) << 12 | (long long)i << 1 | (k & 1);
+        }
+        s_key[i] = k;
+    }
+    __syncthreads();
+    for (int len = 2; len <= SORT_RUN; len *= 2)
+        for (int d = len / 2; d > 0; d /= 2) {
+            for (int i = t; i < SORT_RUN / 2; i += ST) {
+                const int a = 2 * i - (i & (d - 1)), b = a + d;
+                const long long x = s_key[a], y = s_key[b];
+                if ((x > y) == ((a & len) == 0)) { s_key[a] = y; s_key[b] = x; }
+            }
+            __syncthreads();
+        }
+    constexpr int PER = SORT_RUN / ST;
+    int c = 0;
+    for (int i = 0; i < PER; ++i) if (PER * t + i < n) c += (int)(s_key[PER * t + i] & 1);
+    int v = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(0xffffffffu, v, o); if (lane >= o) v += y; }
+    if (lane == 31) s_w[w] = v;
+    __syncthreads();
+    int all;
+    int run = __shfl_sync(0xffffffffu, warp_offsets(s_w, ST / 32, lane, all), w) + v - c;
+    const size_t base = (size_t)s * f.capnb + j0;
+    for (int i = PER * t; i < min(PER * t + PER, n); ++i) {
+        f.before[base + i] = run;
+        run += (int)(s_key[i] & 1);
+    }
+    for (int i = t; i < n; i += ST) f.keys[base + i] = s_key[i];
+}
+
+// The ranks from the sorted runs, eight lanes a block: its place in its own run and, by bisection, in the others.
+__device__ void finish_merge(const FinishArgs &f, int s, int part, int parts) {
+    const int t = threadIdx.x, sub = t & 7, nb = f.sums->count[s][1], n_fused = f.sums->count[s][2];
+    const int runs = (nb + SORT_RUN - 1) / SORT_RUN;
+    const long long *keys = f.keys + (size_t)s * f.capnb;
+    const int *before = f.before + (size_t)s * f.capnb;
+    for (int g0 = part * (FT / 8); g0 < nb; g0 += parts * (FT / 8)) {
+        const int g = g0 + (t >> 3), u = g / SORT_RUN;
+        int rank = 0, fused = 0;
+        long long key = 0;
+        if (g < nb) {
+            key = keys[g];
+            for (int r = sub; r < runs; r += 8) {
+                const int r0 = r * SORT_RUN, r1 = min(r0 + SORT_RUN, nb);
+                int p = g;
+                if (r != u) {        // entries of run r before this one: larger cost, or the same in an earlier run
+                    const long long bound = ((key >> 12) + (r < u ? 1 : 0)) << 12;
+                    int lo = r0, hi = r1;
+                    while (lo < hi) { const int mid = (lo + hi) >> 1; if (keys[mid] < bound) lo = mid + 1; else hi = mid; }
+                    p = lo;
+                }
+                rank += p - r0;
+                fused += p < r1 ? before[p] : before[r1 - 1] + (int)(keys[r1 - 1] & 1);
+            }
+        }
+#pragma unroll
+        for (int o = 1; o < 8; o *= 2) {
+            rank += __shfl_xor_sync(0xffffffffu, rank, o);
+            fused += __shfl_xor_sync(0xffffffffu, fused, o);
+        }
+        if (g < nb && sub == 0) {
+            const int id = u * SORT_RUN + (int)((key >> 1) & (SORT_RUN - 1));
+            f.st[s].queue[rank] = id;
+            f.st[s].queue_split[(key & 1) ? fused : n_fused + rank - fused] = id;
+        }
     }
 }
 
@@ -1000,13 +1175,7 @@ __device__ void finish_rank(const FinishArgs &f, int s, int part, int parts, lon
         for (int j = run + t; j < run + all; j += FT) {
             int lo = 0, hi = FT;
             while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (s_base[mid] <= j) lo = mid; else hi = mid; }
-            long long k = 0;
-            if (s_slot[lo] >= 0) {
-                const int4 r = f.recs[(size_t)s * f.capnb + s_slot[lo] + (j - s_base[lo])];
-                const int fl = r.w >> 8;
-                k = ((long long)(r.w & 255) * (r.z - r.y)) * 2 + ((fl & HDT_BLK_SELF) && !(fl & HDT_BLK_EMPTY) ? 1 : 0);
-            }
-            keys[j] = k;
+            keys[j] = s_slot[lo] >= 0 ? block_key(f.recs[(size_t)s * f.capnb + s_slot[lo] + (j - s_base[lo])]) : 0;
         }
         run += all;
         __syncthreads();
@@ -1059,8 +1228,17 @@ __device__ __forceinline__ void finish_part(const FinishArgs &f, volatile HostHe
             s_cb[t] = f.counts[q + (size_t)t * f.B + b];
         }
     }
-    for (int i = t; i < f.B; i += FT) { m = max(m, f.info[i].stages); bad |= f.info[i].err; }
-    if (seq)
+    if (f.sums != nullptr) {
+        m = f.sums->stages;
+        bad = f.sums->first_err != NO_SEQ;
+        if (seq && t < f.ms) {
+            s_n[t] = f.offs[(size_t)t * f.B + b];
+            s_b[t] = f.offs[q + (size_t)t * f.B + b];
+        }
+    } else {
+        for (int i = t; i < f.B; i += FT) { m = max(m, f.info[i].stages); bad |= f.info[i].err; }
+    }
+    if (seq && f.sums == nullptr)
         row_sums(2 * f.ms, b, w, nw, lane, [&](int i) { return f.counts + ((i & 1) ? q : 0) + (size_t)(i >> 1) * f.B; },
                  [&](int i, int v) {
                      if (i & 1) s_b[i >> 1] = v;
@@ -1075,9 +1253,13 @@ __device__ __forceinline__ void finish_part(const FinishArgs &f, volatile HostHe
     if (id == 0) { finish_header(f, S, host); return; }
     if (s_bad) return;               // (offsets of a broken hierarchy mean nothing)
     id -= 1;
-    if (id < f.r0) { finish_rank(f, 0, id, f.r0, s_keys); return; }
-    id -= f.r0;
-    if (!seq) { if (id / f.r1 + 1 < S) finish_rank(f, id / f.r1 + 1, id % f.r1, f.r1, s_keys); return; }
+    if (!seq) {
+        const int s = id < f.r0 ? 0 : (id - f.r0) / f.r1 + 1, parts = s ? f.r1 : f.r0, part = s ? (id - f.r0) % f.r1 : id;
+        if (s >= S) return;
+        if (f.sums != nullptr) finish_merge(f, s, part, parts);
+        else finish_rank(f, s, part, parts, s_keys);
+        return;
+    }
     const int step = FT * f.gy, me = y * FT + t;
     const int slot = block_slot(s0, b, f.bmin);
     {
@@ -1251,6 +1433,14 @@ static void index_counts(hdt_index *ix, const HostHeader &h) {
     }
 }
 
+// Batches whose offsets and ranks take two kernels more.  In k_finish alone every CTA of a sequence sums the counts of all
+// sequences before it and every block is compared with every other: work that grows with their squares.  The line is in
+// blocks (T / bm + B is about their number) and lies between the sizes timed, us without and with the two kernels: trees of
+// 370 tokens 200 (780) 49.8 and 57.0, 300 (1170) 81.6 and 59.7, 6400 14100 and 664; 8192 tokens 16 (1040) 43.1 and 48.2, 24
+// (1560) 57.7 and 49.0, 256 3540 and 289; 1024 tokens 64 (576) 40.4 and 45.5, 128 (1152) 81.3 and 72.3; 128 tokens 512 (1024)
+// 34.1 and 42.0, 768 (1540) 53.0 and 56.5, 1024 (2050) 71.2 and 66.5.
+static bool many_blocks(int B, int T, int bm) { return B > 0 && (long long)T / bm + B > 1100; }
+
 extern "C" int hdt_build_index(const int8_t *level, const int32_t *parent, const int32_t *cu_seqlens,
                                int32_t batch, int32_t total_tokens, const hdt_index_params_t *params,
                                void *workspace, size_t workspace_bytes, void *stream, hdt_index_t **out) {
@@ -1341,8 +1531,15 @@ extern "C" int hdt_build_index(const int8_t *level, const int32_t *parent, const
     f.gy = (int)min(16LL, max(1LL, mean / 2048));
     f.r0 = max(1, min(64, L.capnb / 16));
     f.r1 = ms > 4 ? max(1, min(8, L.capnb / 128)) : max(1, min(16, L.capnb / 64));
+    if (many_blocks(B, T, bmin)) {
+        f.sums = (const BatchSums *)(ws + L.sums);
+        f.offs = (const int *)(ws + L.offs);
+        f.r0 = max(f.r0, min(592, L.capnb / 64));
+        f.r1 = max(f.r1, min(ms > 4 ? 32 : 148, L.capnb / 512));
+    }
     f.info = a.info; f.counts = a.counts; f.recs = a.recs; f.el = a.el; f.upl = a.upl;
     f.keys = (long long *)(ws + L.keys);
+    f.before = (int *)(ws + L.before);
     f.hdr = (DevHeader *)(ws + L.header);
     f.host = hp;
     f.tell = ix->tells;
@@ -1365,6 +1562,10 @@ extern "C" int hdt_build_index(const int8_t *level, const int32_t *parent, const
             e = cudaLaunchKernelEx(&cfg, k_seq, a);
             count_launch();
         }
+        if (e == cudaSuccess && f.sums != nullptr)
+            e = launch_dependent(k_offsets, true, dim3(4 * ms + 1), OT, 0, st, a.info, a.counts, B, ms, (BatchSums *)(ws + L.sums), (int *)(ws + L.offs));
+        if (e == cudaSuccess && f.sums != nullptr)
+            e = launch_dependent(k_sort, true, dim3((L.capnb + SORT_RUN - 1) / SORT_RUN, ms), ST, 0, st, f);
         if (e == cudaSuccess) {
             // a programmatic dependent: its CTAs are scheduled while k_seq runs and wait for its end
             cudaLaunchConfig_t cfg{};
