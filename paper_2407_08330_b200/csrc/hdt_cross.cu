@@ -38,8 +38,12 @@ struct CrossLayout {
 
 static size_t al256c(size_t v) { return (v + 255) & ~size_t(255); }
 
-// Decoding: few decoder rows a document on average.  At 16 rows the 128-row tile of the other path is an eighth
-// full and the two cost the same per document.
+// Decoding: few decoder rows a document on average (the host knows no more; k_cross_decode deals a document's rows beyond
+// its first DEC_ROWS to CTAs of their own).  Every row reads its document's K and V again, while the other path's 128-row tile costs the
+// same up to 128 rows.  us a forward call of 1, 4, 5 and 8 rows a document, bf16, there and (in brackets) on the tiles: 4 x 8192 tokens with
+// 12 x 64 heads 24, 52, 63, 95 (84); 8 x 2048 12, 31, 38, 56 (52); 1 x 4096 with 16 x 128 14, 32, 38, 56 (35); 64 x 2048 88, 293, 363,
+// 568 (261); 4 x 8192, anchors alone, 14, 20, 25, 34 (21).  All rows of a batch of 4 a document on one of 64 x 2048
+// 182 (98), of 256 x 512 166 (71).  (fp32 tiles cost far more: 4 x 2048 at 8 rows 53 (574); the line stays where bf16 has it.)
 static bool cross_decode(int B, int Tq) { return (long long)Tq <= 4LL * B; }
 // CTAs a document's tokens are dealt to in the decode kernel: four per SM over all documents, 32 tokens each at least.
 static int decode_splits(int B, int T) {
@@ -249,21 +253,25 @@ __global__ void __launch_bounds__(256) k_cross_zero(const int8_t *__restrict__ l
 }
 
 // ---- decoding ------------------------------------------------------------------------------------
-// CTA (b, y, z): the y-th share of document b's tokens, heads z * HC ..., every decoder row of the document in
-// turn (a grid holds 2^31 documents along x, 65535 along y).  Thread (slot, head, lane): D / 8 lanes per (key, head), the heads of a token next to one another, so that a
+// CTA (group * splits + y, z): the y-th share of a document's tokens, heads z * HC ...  Group b < batch: the first DEC_ROWS decoder
+// rows of document b, in turn.  The groups behind take the rows beyond those, DEC_ROWS of all rows each, so that a
+// document that has most rows of the batch does not walk them on one CTA.  (All along x, where a grid has no limit that
+// matters; a document's CTAs follow one another, since some that lie a multiple of eight apart share a part of the
+// chip: 8 rows on one of 8 documents of 2048 tokens 28 us, so 19.)
+// Thread (slot, head, lane): D / 8 lanes per (key, head), the heads of a token next to one another, so that a
 // CTA reads whole token rows.  The bound is reading K and V once (4 x 8192 tokens, 12 x 64: 101 MB, 15 us at the
 // copy rate): four keys a thread in flight and four CTAs an SM; the tile kernel took 352 us here, one CTA per
 // document and head walking 64 chunks with one row of 128 in use.
 struct DecodeArgs {
     const int8_t *level;
     const int32_t *cu_k, *cu_q;
-    int level_mask, H, HC, KS, Tq, splits;
+    int B, level_mask, H, HC, KS, Tq, splits;
     const void *q, *k, *v;
     float scale_log2;
     void *o;
     float *lse, *part_o, *part_lse;       // splits > 1: [splits, Tq, H, D], [splits, Tq, H]
 };
-static constexpr int DEC_LIST = 1024;
+static constexpr int DEC_LIST = 1024, DEC_ROWS = 8;
 
 template <int D, bool BF16>
 __global__ void __launch_bounds__(512, 2) k_cross_decode(const DecodeArgs a) {
@@ -274,82 +282,103 @@ __global__ void __launch_bounds__(512, 2) k_cross_decode(const DecodeArgs a) {
     extern __shared__ float s_red[];                 // [KS][HC][D + 2]
     __shared__ int s_list[DEC_LIST];
     __shared__ int s_n;
-    const int b = blockIdx.x, t = threadIdx.x, lane = t & 31, g = t % LPK, src = lane - g;
+    const int t = threadIdx.x, lane = t & 31, g = t % LPK, src = lane - g;
     const unsigned mask = ((1u << LPK) - 1u) << src;
-    const int pair = t / LPK, hl = pair % a.HC, ks = pair / a.HC, h = blockIdx.z * a.HC + hl;
+    const int pair = t / LPK, hl = pair % a.HC, ks = pair / a.HC, h = blockIdx.y * a.HC + hl;
     const bool on = ks < a.KS && h < a.H;
-    const int k0 = a.cu_k[b], k1 = a.cu_k[b + 1], q0 = a.cu_q[b], q1 = a.cu_q[b + 1];
-    const int per = (k1 - k0 + a.splits - 1) / a.splits, c0 = min(k1, k0 + (int)blockIdx.y * per), c1 = min(k1, c0 + per);
-    for (int row = q0; row < q1; ++row) {
-        RowSoftmax S;
-        S.clear();
-        W q;
-        if (on) q.load(a.q, (unsigned)row * a.H + h, g);
-        for (int p0 = c0; p0 < c1; p0 += DEC_LIST) {
-            const int p1 = min(c1, p0 + DEC_LIST);
-            if (row == q0 || c1 - c0 > DEC_LIST) {           // the chosen tokens of this piece, in order
-                __syncthreads();
-                if (t < 32) {
-                    int n = 0;
-                    for (int i0 = p0; i0 < p1; i0 += 32) {
-                        const bool f = i0 + lane < p1 && chosen(a.level, i0 + lane, a.level_mask);
-                        const unsigned m = __ballot_sync(0xffffffffu, f);
-                        if (f) s_list[n + __popc(m & ((1u << lane) - 1u))] = i0 + lane;
-                        n += __popc(m);
+    const int group = blockIdx.x / a.splits, split = blockIdx.x % a.splits;
+    // Rows [row0, row1) of document b.
+    auto walk = [&](int b, int row0, int row1) {
+        const int k0 = a.cu_k[b], k1 = a.cu_k[b + 1];
+        const int per = (k1 - k0 + a.splits - 1) / a.splits, c0 = min(k1, k0 + split * per), c1 = min(k1, c0 + per);
+        for (int row = row0; row < row1; ++row) {
+            RowSoftmax S;
+            S.clear();
+            W q;
+            if (on) q.load(a.q, (unsigned)row * a.H + h, g);
+            for (int p0 = c0; p0 < c1; p0 += DEC_LIST) {
+                const int p1 = min(c1, p0 + DEC_LIST);
+                if (row == row0 || c1 - c0 > DEC_LIST) {         // the chosen tokens of this piece, in order
+                    __syncthreads();
+                    if (t < 32) {
+                        int n = 0;
+                        for (int i0 = p0; i0 < p1; i0 += 32) {
+                            const bool f = i0 + lane < p1 && chosen(a.level, i0 + lane, a.level_mask);
+                            const unsigned m = __ballot_sync(0xffffffffu, f);
+                            if (f) s_list[n + __popc(m & ((1u << lane) - 1u))] = i0 + lane;
+                            n += __popc(m);
+                        }
+                        if (lane == 0) s_n = n;
                     }
-                    if (lane == 0) s_n = n;
+                    __syncthreads();
                 }
-                __syncthreads();
-            }
-            const int n = s_n;
-            if (!on) continue;
-            for (int i0 = ks * C; i0 < n; i0 += a.KS * C) {
-                W x[C], y[C];
+                const int n = s_n;
+                if (!on) continue;
+                for (int i0 = ks * C; i0 < n; i0 += a.KS * C) {
+                    W x[C], y[C];
 #pragma unroll
-                for (int c = 0; c < C; ++c) {
-                    const unsigned r = (unsigned)s_list[min(i0 + c, n - 1)] * a.H + h;      // (past the end: the last key, weight 0)
-                    x[c].load(a.k, r, g);
-                    y[c].load(a.v, r, g);
+                    for (int c = 0; c < C; ++c) {
+                        const unsigned r = (unsigned)s_list[min(i0 + c, n - 1)] * a.H + h;      // (past the end: the last key, weight 0)
+                        x[c].load(a.k, r, g);
+                        y[c].load(a.v, r, g);
+                    }
+                    float sc[C];
+                    dots<C>(q, x, sc);
+                    const float s = reduce_scatter<C, LPK>(sc, g, mask) * a.scale_log2;
+                    const float p = S.add<C>(i0 + (g & (C - 1)) < n ? s : -INFINITY, mask);
+                    axpys<C>(S.acc, p, y, mask, src);
                 }
-                float sc[C];
-                dots<C>(q, x, sc);
-                const float s = reduce_scatter<C, LPK>(sc, g, mask) * a.scale_log2;
-                const float p = S.add<C>(i0 + (g & (C - 1)) < n ? s : -INFINITY, mask);
-                axpys<C>(S.acc, p, y, mask, src);
             }
-        }
-        // the slots of a head: one after the other through shared memory
-        if (on) {
+            // the slots of a head: one after the other through shared memory
+            if (on) {
 #pragma unroll
-            for (int o = 1; o < C; o *= 2) S.l += __shfl_xor_sync(mask, S.l, o);
-            float *d = s_red + (size_t)(ks * a.HC + hl) * (D + 2);
-            const float lse = S.finish();
+                for (int o = 1; o < C; o *= 2) S.l += __shfl_xor_sync(mask, S.l, o);
+                float *d = s_red + (size_t)(ks * a.HC + hl) * (D + 2);
+                const float lse = S.finish();
 #pragma unroll
-            for (int u = 0; u < 4; ++u) unpack2(S.acc[u], d[8 * g + 2 * u], d[8 * g + 2 * u + 1]);
-            if (g == 0) d[D] = lse;
-        }
-        __syncthreads();
-        if (on && ks == 0) {
-            RowSoftmax R;
-            R.clear();
-            for (int i = 0; i < a.KS; ++i) {
-                const float *d = s_red + (size_t)(i * a.HC + hl) * (D + 2);
-                f2 x[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) x[u] = pack2(d[8 * g + 2 * u], d[8 * g + 2 * u + 1]);
-                R.merge(d[D] * 1.4426950408889634f, d[D] > -INFINITY ? 1.f : 0.f, x);
+                for (int u = 0; u < 4; ++u) unpack2(S.acc[u], d[8 * g + 2 * u], d[8 * g + 2 * u + 1]);
+                if (g == 0) d[D] = lse;
             }
-            const float lse = R.finish();
-            if (a.splits == 1) {
-                W::store(a.o, (unsigned)row * a.H + h, g, R.acc);
-                if (g == 0) a.lse[(size_t)h * a.Tq + row] = lse;
-            } else {
-                const size_t r = ((size_t)blockIdx.y * a.Tq + row) * a.H + h;
-                W::store_f32(a.part_o, r, g, R.acc);
-                if (g == 0) a.part_lse[r] = lse;
+            __syncthreads();
+            if (on && ks == 0) {
+                RowSoftmax R;
+                R.clear();
+                for (int i = 0; i < a.KS; ++i) {
+                    const float *d = s_red + (size_t)(i * a.HC + hl) * (D + 2);
+                    f2 x[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) x[u] = pack2(d[8 * g + 2 * u], d[8 * g + 2 * u + 1]);
+                    R.merge(d[D] * 1.4426950408889634f, d[D] > -INFINITY ? 1.f : 0.f, x);
+                }
+                const float lse = R.finish();
+                if (a.splits == 1) {
+                    W::store(a.o, (unsigned)row * a.H + h, g, R.acc);
+                    if (g == 0) a.lse[(size_t)h * a.Tq + row] = lse;
+                } else {
+                    const size_t r = ((size_t)split * a.Tq + row) * a.H + h;
+                    W::store_f32(a.part_o, r, g, R.acc);
+                    if (g == 0) a.part_lse[r] = lse;
+                }
             }
+            __syncthreads();
         }
-        __syncthreads();
+    };
+    if (group < a.B) {
+        const int q0 = a.cu_q[group], q1 = a.cu_q[group + 1];
+        walk(group, q0, min(q1, q0 + DEC_ROWS));
+        return;
+    }
+    auto document_of = [&](int row) {                // the last one that starts at or before the row
+        int lo = 0, hi = a.B;
+        while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (a.cu_q[mid] <= row) lo = mid; else hi = mid; }
+        return lo;
+    };
+    const int first = DEC_ROWS * (group - a.B), end = min(a.Tq, first + DEC_ROWS);
+    if (!__syncthreads_or(t < end - first && first + t >= a.cu_q[document_of(first + t)] + DEC_ROWS)) return;
+    for (int row = first; row < end;) {
+        const int b = document_of(row), q1 = a.cu_q[b + 1];
+        walk(b, max(row, a.cu_q[b] + DEC_ROWS), min(end, q1));
+        row = q1 > row ? q1 : end;
     }
 }
 
@@ -415,9 +444,11 @@ static int launch_decode_t(DecodeArgs a, int B, cudaStream_t st) {
     constexpr int LPK = D / 8;
     a.HC = min(a.H, 512 / LPK);
     a.KS = max(1, min(16, 384 / (a.HC * LPK)));
+    a.B = B;
     const int threads = (a.HC * LPK * a.KS + 31) / 32 * 32;
+    const unsigned groups = B + (a.Tq > DEC_ROWS ? (a.Tq + DEC_ROWS - 1) / DEC_ROWS : 0);
     const size_t smem = sizeof(float) * (size_t)a.KS * a.HC * (D + 2);
-    HDT_CUDA_CHECK(launch_dependent(k_cross_decode<D, BF16>, true, dim3(B, a.splits, (a.H + a.HC - 1) / a.HC), threads, smem, st, a));
+    HDT_CUDA_CHECK(launch_dependent(k_cross_decode<D, BF16>, true, dim3(groups * a.splits, (a.H + a.HC - 1) / a.HC), threads, smem, st, a));
     return HDT_OK;
 }
 

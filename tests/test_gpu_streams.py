@@ -74,6 +74,27 @@ def test_cross_index_counted(n, longest):
             check_close(host(x), r, "bf16", what, out_rounding=True, row_rel=2.0 ** -8)
 
 
+@pytest.mark.parametrize("rows", [[0] * 9 + [57] + [0] * 5 + [1], [17] + [0] * 8, [1] * 12 + [33, 0, 18, 1] + [0] * 3, [16] * 2 + [0] * 10 + [20, 1]])
+def test_cross_decode_uneven(rows):
+    """Few decoder rows a document on average, most of them in one: its rows beyond those that one block walks."""
+    import torch
+    import paper_2407_08330_b200 as P
+    assert sum(rows) <= 4 * len(rows)
+    rng = np.random.default_rng(len(rows))
+    b = gen.pack([gen.gen_fill(rng, int(k), (2, 6), (2, 8), (3, 20))[:2] for k in rng.integers(1, 700, len(rows))])
+    H, d, T, Tq = 3, 64, b.total_tokens, sum(rows)
+    cu_q = np.concatenate([[0], np.cumsum(rows)]).astype(np.int32)
+    t = gen.make_tensors(3, T, H, d, "f32", names=("k", "v"))
+    q = gen.make_tensors(4, Tq, H, d, "f32", names=("q",))["q"]
+    level, _, cu = dev_struct(b)
+    o, lse = P.hdt_cross_attn_fwd(level, cu, torch.from_numpy(cu_q).cuda(), 15, *(dev_tensor(x, "f32") for x in (q, t["k"], t["v"])))
+    torch.cuda.synchronize()
+    P.hdt_device_status()
+    o_r, lse_r = cross_oracle.forward(b.level, b.cu_seqlens, 15, cu_q, q, t["k"], t["v"])
+    check_close(host(o), o_r, "f32", "O")
+    check_close(host(lse), lse_r, "f32", "LSE")
+
+
 def test_cross_decode_many_documents():
     """A decoding step for more documents than a grid has rows: one token and one decoder row each, so O is V and the
     log-sum-exp the one score."""
