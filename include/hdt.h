@@ -282,7 +282,10 @@ int hdt_hpe(const hdt_index_t *index, const int8_t *level, const int32_t *parent
  *                      head_dim, dtype, bwd), 256-byte aligned; holds the list of chosen tokens and
  *                      their block records, rebuilt by every call (and delta in the backward)
  * head_dim 64 or 128; softmax_scale <= 0 means 1/sqrt(head_dim).  Asynchronous on `stream`, no
- * host wait.  The chosen rows are read in place through the list (no gathered copy of K, V).
+ * host wait.  Bits of levels that no token has change nothing in the result.  How many blocks share a
+ * document's keys is chosen from the mask: with bit 3 or a higher one for every token, else for anchors
+ * (a sixteenth of the tokens), so hierarchies whose words lie on level 2 or 1 should set bit 3 beside
+ * the words' bit.  The chosen rows are read in place through the list (no gathered copy of K, V).
  */
 size_t hdt_cross_workspace_bytes(int32_t batch, int32_t total_tokens, int32_t total_q, int32_t heads,
                                  int32_t head_dim, int32_t dtype, int32_t bwd);

@@ -51,8 +51,12 @@ static int decode_splits(int B, int T) {
     return (int)max(1LL, min((mean + 31) / 32, (148LL * 4 + B - 1) / max(B, 1)));
 }
 // CTAs a row block's keys are dealt to in the tile kernels: enough to fill the SMs (`per_sm` CTAs each), pieces of
-// four chunks at least.  level_mask < 0: every level (for the workspace size).  Without the token level the keys are
-// the anchors, some thirtieth of the tokens.
+// four chunks at least.  level_mask < 0: every level (for the workspace size).  The host does not know how many tokens a level has:
+// a subset with level 3 or a deeper one is taken for all tokens, any other for the anchors of a [DOC]/[SEC]/[SENT]/token document and
+// put at a sixteenth of them (documents have a thirtieth; more pieces than needed cost a merge of mostly empty partial
+// results).  Where the words are on level 2, a subset with them is split too little, at worst not at all, as every subset was
+// before there were pieces: 1 x 4096 tokens, 64 decoder rows, forward 155 us and backward 137, with bit 3 set as well (a caller may: no
+// token has it) 31 and 61; 4 x 8192, 256 rows 310 and 597, so 191 and 516.
 static int tile_splits(int B, int T, int Tq, int H, int level_mask, int per_sm) {
     if (B <= 0 || Tq <= 0) return 1;
     const long long mean = (T + B - 1) / B, keys = (level_mask < 0 || (level_mask >> 3)) ? mean : mean / 16;
