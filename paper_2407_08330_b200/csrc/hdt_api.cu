@@ -244,18 +244,21 @@ static bool rows_allowed() {
 }
 // All stages row by row: families so small that a tile kernel's 128 x 128 products are nearly all padding
 // (expression trees have six keys a row, documents forty; at ten the two cost the same), and small fp32 calls, whose
-// rows all fit on the SMs in a wave or two (2935 tokens, 12 x 64, forward: 83 us a call against 88 on the
-// shared-memory kernels; 4096: 107 against 88).
+// rows all fit on the SMs in a wave or two (2935 tokens, 12 x 64, forward: 83 us a call, 88 on the
+// shared-memory kernels; 4096: 107 and 88).  The rules bound the mean, not the longest family, whose rows walk it key by key: that
+// costs little beside the other kernels.  us forward + backward, here and there: fp32, 38 000 tokens and one head, a family of 150
+// 101 and 111, of 600 389 and 360, of 1000 663 and 576; 2700 tokens, 12 heads, of 200 143 and 168, of 300 221 and 246; 200
+// expression trees, bf16, with a family of 300 268 and 773.
 static bool rows_all(const hdt_index *ix, int heads, int head_dim, int dtype) {
     const bool few = dtype == HDT_F32 && (long long)ix->total_tokens * heads * (head_dim / 64) <= 40000;
     return rows_allowed() && ix->nnz <= (few ? 64 : 10) * ix->real;
 }
 // The stages above 0 row by row, in one launch behind stage 0, while their pairs are few; beyond, the tile
 // kernels' launches beside stage 0 and the merge behind it cost less.  The lines lie between the sizes where the two
-// were timed on documents of 200 to 90 000 tokens, the row-wise kernel as a programmatic dependent of stage 0.  Forward,
-// 12 heads x 64: 4 x 8192 tokens (215 000) 85.0 against 83.2 us, 8 x 8192 (430 000) 126.3 against 130.5.  Forward and
-// backward: 8 x 1024 tokens 90.5 against 82, 1 x 4096 with 16 heads x 128 (60 000) 117.5 against 106.4, 2 x 8192
-// (108 000) 130.8 against 132.4.
+// were timed on documents of 200 to 90 000 tokens, the row-wise kernel as a programmatic dependent of stage 0.  us row by row, with the build, and in
+// brackets on the tile kernels.  Forward, 12 heads x 64: 4 x 8192 tokens (215 000 pairs) 83.2 (85.0), 8 x 8192 (430 000)
+// 130.5 (126.3).  Forward and backward: 8 x 1024 tokens 82 (90.5), 1 x 4096 with 16 heads x 128 (60 000) 106.4 (117.5), 2 x
+// 8192 (108 000) 132.4 (130.8).
 static bool rows_upper(const hdt_index *ix, int heads, int head_dim, int bwd) {
     return rows_allowed() && ix->n_stages > 1 && ix->nnz_upper * heads * (head_dim / 64) <= (bwd ? 80000 : 300000);
 }
