@@ -519,11 +519,11 @@ int launch_bwd_tile(const TileBwdArgs &a, int D, cudaStream_t st) {
 // Groups of lanes per row.  A row's time is its chain of chunks (about two round trips to L2 each), the launch's that
 // chain times the number of times the rows fill the SMs: take the split with the smallest product.  keys: mean
 // keys of a row, chunk: keys a group takes at a time, warps: warps resident on an SM.
-static int row_groups(long long rows, int D, float keys, int chunk, int warps) {
+static int row_groups(long long rows, int D, float keys, int chunk, int warps, int n_sm) {
     int best = 1;
     double least = 0;
     for (int kp = 1; kp <= 256 / D; kp *= 2) {
-        const double lanes = (double)rows * kp * (D / 8), waves = lanes / (148.0 * 32 * warps);
+        const double lanes = (double)rows * kp * (D / 8), waves = lanes / (32.0 * n_sm * warps);
         const double t = (waves < 1 ? 1 : waves) * (keys / (chunk * kp) + 2.5 + (kp > 1 ? 0.5 : 0));
         if (kp == 1 || t < least) { best = kp; least = t; }
     }
@@ -533,7 +533,9 @@ template <int D, bool BF16>
 static int launch_fwd_rows_t(const RowFwdArgs &a, cudaStream_t st) {
     const long long rows = (long long)a.n * a.H;
     if (rows == 0) return HDT_OK;
-    const int kp = row_groups(rows, D, a.keys, a.first ? 8 : 4, BF16 ? 16 : 12);
+    int n_sm = 0;
+    if (const int rc = sm_count(&n_sm)) return rc;
+    const int kp = row_groups(rows, D, a.keys, a.first ? 8 : 4, BF16 ? 16 : 12, n_sm);
     const unsigned grid = (unsigned)((rows * kp * (D / 8) + ROW_THREADS - 1) / ROW_THREADS);
     auto *kern = kp == 4 ? k_fwd_rows<D, BF16, D == 64 ? 4 : 1, 8> : kp == 2 ? k_fwd_rows<D, BF16, 2, 8> : a.first ? k_fwd_rows<D, BF16, 1, 8> : k_fwd_rows<D, BF16, 1, 4>;
     HDT_CUDA_CHECK(launch_dependent(kern, true, dim3(grid), ROW_THREADS, 0, st, a));
@@ -543,7 +545,9 @@ template <int D, bool BF16, bool DELTA>
 static int launch_bwd_rows_t(const RowBwdArgs &a, cudaStream_t st) {
     const long long rows = (long long)a.n * a.H;
     if (rows == 0) return HDT_OK;
-    const int kp = row_groups(rows, D, a.keys, 2, BF16 ? 16 : 12);
+    int n_sm = 0;
+    if (const int rc = sm_count(&n_sm)) return rc;
+    const int kp = row_groups(rows, D, a.keys, 2, BF16 ? 16 : 12, n_sm);
     const unsigned grid = (unsigned)((rows * kp * (D / 8) + ROW_THREADS - 1) / ROW_THREADS);
     auto *kern = kp == 4 ? k_bwd_rows<D, BF16, D == 64 ? 4 : 1, DELTA> : kp == 2 ? k_bwd_rows<D, BF16, 2, DELTA> : k_bwd_rows<D, BF16, 1, DELTA>;
     HDT_CUDA_CHECK(launch_dependent(kern, true, dim3(grid), ROW_THREADS, 0, st, a));

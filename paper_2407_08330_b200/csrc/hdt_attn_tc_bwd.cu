@@ -1589,7 +1589,11 @@ static int launch_bwd_tc_upper_t(const BwdStageArgs &a, cudaStream_t st) {
     if (b.splits < 1) b.splits = 1;
     // (phase_split: the blocks of the queries, and of the others two CTAs per SM; an unused slot costs its CTA two loads)
     int grid_x = a.nb;
-    if (a.phase_split > 0) grid_x = min(a.phase_split * (b.splits - 1) + a.nb, a.phase_split * b.splits + (2 * 148 + a.H - 1) / a.H);
+    if (a.phase_split > 0) {
+        int n_sm = 0;
+        if (const int rc_ = sm_count(&n_sm)) return rc_;
+        grid_x = min(a.phase_split * (b.splits - 1) + a.nb, a.phase_split * b.splits + (2 * n_sm + a.H - 1) / a.H);
+    }
     // (families longer than a block: the dQ walk and the dK / dV walk of such a block in CTAs of their own)
     const unsigned grid_z = a.phase_split == 0 && a.phases == 0 && !a.final_merge && a.n_fused + a.n_empty < a.nb ? 2u : 1u;
     if (a.dirs != 7) k_bwd_tc<D, true, true><<<dim3(a.nb, a.H, grid_z), 256, smem, st>>>(tq, tq, tq, tq, b);      // direction bits

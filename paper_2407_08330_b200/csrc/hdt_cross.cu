@@ -48,7 +48,7 @@ static bool cross_decode(int B, int Tq) { return (long long)Tq <= 4LL * B; }
 // CTAs a document's tokens are dealt to in the decode kernel: four per SM over all documents, 32 tokens each at least.
 static int decode_splits(int B, int T) {
     const long long mean = B > 0 ? (T + B - 1) / B : 0;
-    return (int)max(1LL, min((mean + 31) / 32, (148LL * 4 + B - 1) / max(B, 1)));
+    return (int)max(1LL, min((mean + 31) / 32, (4LL * PLAN_SMS + B - 1) / max(B, 1)));
 }
 // CTAs a row block's keys are dealt to in the tile kernels: enough to fill the SMs (`per_sm` CTAs each), pieces of
 // four chunks at least.  level_mask < 0: every level (for the workspace size).  The host does not know how many tokens a level has:
@@ -61,7 +61,7 @@ static int tile_splits(int B, int T, int Tq, int H, int level_mask, int per_sm) 
     if (B <= 0 || Tq <= 0) return 1;
     const long long mean = (T + B - 1) / B, keys = (level_mask < 0 || (level_mask >> 3)) ? mean : mean / 16;
     const long long ctas = (long long)B * ((Tq + 128LL * B - 1) / (128LL * B)) * H;
-    return (int)max(1LL, min((keys + 511) / 512, (148LL * per_sm + ctas - 1) / ctas));
+    return (int)max(1LL, min((keys + 511) / 512, ((long long)PLAN_SMS * per_sm + ctas - 1) / ctas));
 }
 
 // tc: bf16 on the tensor-core kernels (128-row blocks)
@@ -589,7 +589,9 @@ extern "C" int hdt_cross_attn_bwd(const int8_t *level, const int32_t *cu_seqlens
             HDT_CUDA_CHECK(cudaStreamWaitEvent(sd->s, sd->fork, 0));
             sz = sd->s;
         }
-        k_cross_zero<<<min((total_tokens + 7) / 8, 148 * 8), 256, 0, sz>>>(level, cu_seqlens_k, cu_seqlens_q, batch, total_tokens, level_mask,
+        int n_sm = 0;
+        if ((rc = sm_count(&n_sm))) return rc;
+        k_cross_zero<<<min((total_tokens + 7) / 8, 8 * n_sm), 256, 0, sz>>>(level, cu_seqlens_k, cu_seqlens_q, batch, total_tokens, level_mask,
                                                                         (int)(heads * head_dim * esz / 16), (uint4 *)dk, (uint4 *)dv);
         count_launch();
         HDT_CUDA_CHECK(cudaGetLastError());

@@ -393,8 +393,10 @@ extern "C" int hdt_hpe(const hdt_index_t *ix, const int8_t *level, const int32_t
     cudaStream_t st = (cudaStream_t)stream;
     const int *rank = ix->rank;
     const bool x16 = ((uintptr_t)x & 15) == 0;
+    int n_sm = 0;
+    if (const int rc0 = sm_count(&n_sm)) return rc0;
     if (d_model % 8 == 0 && x16 && n_levels == 3 && d_model <= 1024) {
-        int R = T < 148 * 64 ? HPE_R_SMALL : HPE_R;
+        int R = T < n_sm * 64 ? HPE_R_SMALL : HPE_R;
         // Tiles of fewer tokens where three of R do not fit (with two the producer waits for the store of the tile
         // before), but no more of them than three: a run of R / 4 tokens begins with a full evaluation.  Rows of which not
         // even two tiles fit get two.  fp32, 8 x 7394 tokens: d_model 768 83 -> 64 us (four tiles of 16: 69), 1024, on the
@@ -406,7 +408,7 @@ extern "C" int hdt_hpe(const hdt_index_t *ix, const int8_t *level, const int32_t
         const int n_tiles = (T + R - 1) / R, per_sm = stage * 4 <= 100 * 1024 ? 2 : 1;
         const int ns = (int)max((size_t)1, min((size_t)HPE_NS, (size_t)(per_sm == 2 ? 104 : 208) * 1024 / stage));
         if (ns >= 2) {
-            const int tx = (d_model / 8 + 31) / 32 * 32, nb = min(n_tiles, 148 * per_sm);
+            const int tx = (d_model / 8 + 31) / 32 * 32, nb = min(n_tiles, n_sm * per_sm);
             int *status = device_status_ptr();
             if (!status) return HDT_ERR_CUDA;
             const int b16 = dtype == HDT_BF16;
@@ -431,7 +433,7 @@ extern "C" int hdt_hpe(const hdt_index_t *ix, const int8_t *level, const int32_t
         const int tx = min(384, ((G + 31) / 32) * 32), ty = max(1, 384 / tx);
         int run = 16;
         const int Tr = T;
-        while ((long long)((Tr + run - 1) / run + ty - 1) / ty > 148LL * 64) run *= 2;
+        while ((long long)((Tr + run - 1) / run + ty - 1) / ty > 64LL * n_sm) run *= 2;
         const int nb = ((Tr + run - 1) / run + ty - 1) / ty;
         const dim3 blk(tx, ty);
 #define HPE_LAUNCH(BF, LL) k_hpe_eval_vec<BF, LL><<<nb, blk, 0, st>>>(level, pvec, 0, T, n_levels, d_model, accumulate, run, x)

@@ -1534,8 +1534,8 @@ extern "C" int hdt_build_index(const int8_t *level, const int32_t *parent, const
     if (many_blocks(B, T, bmin)) {
         f.sums = (const BatchSums *)(ws + L.sums);
         f.offs = (const int *)(ws + L.offs);
-        f.r0 = max(f.r0, min(592, L.capnb / 64));
-        f.r1 = max(f.r1, min(ms > 4 ? 32 : 148, L.capnb / 512));
+        f.r0 = max(f.r0, min(512, L.capnb / 64));
+        f.r1 = max(f.r1, min(ms > 4 ? 32 : 128, L.capnb / 512));
     }
     f.info = a.info; f.counts = a.counts; f.recs = a.recs; f.el = a.el; f.upl = a.upl;
     f.keys = (long long *)(ws + L.keys);

@@ -125,6 +125,8 @@ struct DevOnce {
 };
 // Number of SMs of the current device (cached per device ordinal).
 int sm_count(int *n_sm);
+// For sizes that a query without a device has to give as well (splits of the cross-attention's keys): SMs of a B200.
+constexpr int PLAN_SMS = 148;
 
 // Side stream (one per host thread and device, created on first use): work that does not depend
 // on the main kernel of a call runs beside it.  fork / join are events for the two hand-overs.
