@@ -578,8 +578,11 @@ __global__ void __launch_bounds__(256) k_bwd_tc(const __grid_constant__ CUtensor
                 }
             }
         }
-        if (fin) drain_final(TM_DQ, run, a.scale, fb[0], fn[0], fo[0]);
-        else if (!GATHER || phases != 2) drain(TM_DQ, run, a.scale, cq, sP);
+        // (a CTA that takes one walk only has nothing of the other one to drain)
+        if (!GATHER || phases != 2) {
+            if (fin) drain_final(TM_DQ, run, a.scale, fb[0], fn[0], fo[0]);
+            else drain(TM_DQ, run, a.scale, cq, sP);
+        }
         // dQ leaves now: the second walk reuses sP and (at D = 128) the dQ columns of TMEM
         tc_fence_before();
         __syncthreads();
@@ -646,12 +649,14 @@ __global__ void __launch_bounds__(256) k_bwd_tc(const __grid_constant__ CUtensor
             }
             if (!ok && tid == 0) atomicCAS(a.status, 0, HDT_ERR_TIMEOUT);
         }
-        if (fin) {
-            drain_final(TM_DK, run, a.scale, fb[1], fn[1], fo[1]);
-            drain_final(TM_DV, run, 1.f, fb[2], fn[2], fo[2]);
-        } else {
-            drain(TM_DK, run, a.scale, ck, sDS);
-            drain(TM_DV, run, 1.f, cv, sQ);
+        if (!GATHER || phases != 1) {
+            if (fin) {
+                drain_final(TM_DK, run, a.scale, fb[1], fn[1], fo[1]);
+                drain_final(TM_DV, run, 1.f, fb[2], fn[2], fo[2]);
+            } else {
+                drain(TM_DK, run, a.scale, ck, sDS);
+                drain(TM_DV, run, 1.f, cv, sQ);
+            }
         }
     }
     tc_fence_before();
