@@ -647,8 +647,8 @@ __global__ void __launch_bounds__(256) k_bwd_tc(const __grid_constant__ CUtensor
                     tile_pass(c0, kb, r0, r1, false, true, false, c0 > ka, [&]() { return stat_of(c0 + rl, kb, c0 + rl); });
                 }
             }
-            if (!ok && tid == 0) atomicCAS(a.status, 0, HDT_ERR_TIMEOUT);
         }
+        if (!ok && tid == 0) atomicCAS(a.status, 0, HDT_ERR_TIMEOUT);
         if (!GATHER || phases != 1) {
             if (fin) {
                 drain_final(TM_DK, run, a.scale, fb[1], fn[1], fo[1]);
