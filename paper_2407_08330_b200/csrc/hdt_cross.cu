@@ -499,8 +499,9 @@ static bool cross_tc(int dtype) { return dtype == HDT_BF16 && !g_force_simt; }
 extern "C" size_t hdt_cross_workspace_bytes(int32_t batch, int32_t total_tokens, int32_t total_q, int32_t heads,
                                             int32_t head_dim, int32_t dtype, int32_t bwd) {
     if (batch < 0 || total_tokens < 0 || total_q < 0 || heads < 1 || (head_dim != 64 && head_dim != 128)) return 0;
-    // sized for the tensor-core path whenever the dtype allows it (the larger of the two layouts)
-    return cross_layout(batch, total_tokens, total_q, heads, head_dim, dtype == HDT_BF16, bwd).total;
+    // for either path: the SIMT kernels' (fp32, option "force_simt") smaller blocks have more records
+    return max(cross_layout(batch, total_tokens, total_q, heads, head_dim, false, bwd).total,
+               cross_layout(batch, total_tokens, total_q, heads, head_dim, true, bwd).total);
 }
 
 extern "C" int hdt_cross_attn_fwd(const int8_t *level, const int32_t *cu_seqlens_k, const int32_t *cu_seqlens_q,

@@ -36,3 +36,14 @@ def test_oracle_and_cuda_path_share_nothing():
         if f.endswith((".py", ".c")):
             txt = open(os.path.join(ROOT, "oracle", f)).read()
             assert "paper_2407_08330_b200" not in txt and "libhdt.so" not in txt, f
+
+
+def test_cross_workspace_holds_either_path():
+    """A bf16 call runs on 128-row blocks or, with option force_simt, on 32-row blocks, whose records take more room."""
+    import torch
+    al = lambda n: (n + 255) // 256 * 256
+    for B, T, Tq, H in ((1, 1 << 20, 1, 1), (3, 50000, 7, 1), (1, 100, 4000, 2), (70, 9000, 0, 1)):
+        blocks = Tq // 32 + T // 32 + 2 * (B + 1)
+        for bwd in (0, 1):
+            need = al(20 * blocks) + 12 * (T + Tq) + 4 * blocks + (4 * H * Tq if bwd else 0)
+            assert P.hdt_cross_workspace_bytes(B, T, Tq, H, 64, torch.bfloat16, bwd) >= need, (B, T, Tq, H, bwd)
