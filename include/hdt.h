@@ -37,8 +37,9 @@
  *    as a padded batch normally is; nothing checks this).
  *  - `stream` is a cudaStream_t passed as void* (NULL = default stream).  hdt_attn_fwd/bwd are
  *    asynchronous on it.  hdt_build_index enqueues its kernels on it and then waits until they have
- *    done all their reads and writes, because it returns the sizes the attention calls need.
- *  - An index may be used on any stream and by several threads, whichever stream it was built on.
+ *    read the structure arrays and sent the sizes the attention calls need.
+ *  - An index may be used on any stream and by several threads, whichever stream it was built on:
+ *    hdt_index_export, and calls on another stream than the build's, wait until the build has ended.
  *  - Every function returns an hdt_status_t (HDT_OK = 0, errors negative); nothing throws,
  *    aborts or traps the device.  hdt_last_error() gives a thread-local message.
  */
@@ -84,15 +85,14 @@ typedef struct {
                            the first call that needs the counts of the index on the host
                            (hdt_index_info, hdt_index_export, the workspace queries, the attention and
                            positional-encoding calls) waits instead and returns the structure error,
-                           if any; every later call on that index returns it too.  Attention and
-                           positional-encoding calls on the stream of the build wait for the counts
-                           only, every other call until the build has ended.  hdt_attn_fwd on a
+                           if any; every later call on that index returns it too.  hdt_attn_fwd on a
                            bf16 index still in flight on its stream queues its stage-0 kernel first
                            (the kernel reads the counts on the device) and waits only then.  The
-                           structure arrays and the workspace must stay allocated and unchanged until
-                           the stream has passed the build, the stream itself until a call has waited
-                           for its end.  A call captured into a graph on the stream of the build counts
-                           as one on that stream: replay it there, or ordered behind it          */
+                           structure arrays must stay unchanged until the stream has passed the build or
+                           one of these calls has waited, the workspace until the stream has passed the
+                           build, and the stream itself must live until then.  A call captured into a
+                           graph on the stream of the build counts as one on that stream: replay it
+                           there, or ordered behind it                                          */
     int32_t reserved[3];
 } hdt_index_params_t;
 
@@ -143,8 +143,8 @@ size_t hdt_index_workspace_bytes(int32_t batch, int32_t total_tokens,
  *   workspace  device, >= hdt_index_workspace_bytes(...), 256-byte aligned; must stay allocated
  *              and untouched until hdt_index_destroy
  *   out        receives a host object (free with hdt_index_destroy)
- * Returns when the stream has passed the build (unless params->deferred is set: see there): the index
- * may then be used on any stream, and the structure arrays may change.  Errors:
+ * Waits for the stream, up to where the build has read the structure arrays, which may then change, and
+ * its sizes are known (unless params->deferred is set: see there).  Errors:
  * HDT_ERR_BAD_HIERARCHY when a precondition on the structure arrays fails or the hierarchy needs
  * more than max_stages stages (no index is returned; a deferred build returns the index and the
  * error comes from the first call that uses it), HDT_ERR_WORKSPACE, HDT_ERR_INVALID_ARG,
@@ -161,7 +161,7 @@ int hdt_index_info(const hdt_index_t *index, int32_t *n_stages, int64_t *nnz_pai
 /* Device views of stage `stage` (0 <= stage < n_stages) for inspection and parity tests. */
 int hdt_index_export(const hdt_index_t *index, int32_t stage, hdt_stage_view_t *view);
 
-/* Frees the host object only. */
+/* Frees the host object only.  Waits for a build that was not deferred to end: the workspace may be reused. */
 int hdt_index_destroy(hdt_index_t *index);
 
 /*

@@ -276,7 +276,7 @@ extern "C" size_t hdt_attn_workspace_bytes(const hdt_index_t *ix, int32_t heads,
                                            int32_t dtype, int32_t bwd) {
     (void)dtype;
     if (!ix || heads <= 0 || head_dim <= 0) return 0;
-    if (index_ready(ix)) return 0;
+    if (index_wait(ix, INDEX_COUNTED)) return 0;
     return attn_layout(ix, heads, head_dim, bwd, dtype).total;
 }
 

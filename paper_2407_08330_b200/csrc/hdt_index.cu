@@ -894,7 +894,7 @@ __global__ void __launch_bounds__(512) k_seq(const SeqArgs a) {
 
 struct FinishArgs {
     StagePtrs st[HDT_MAX_STAGES];
-    const int32_t *cu;
+    const int32_t *cu;             // the index's own copy (scu of stage 0): the caller's arrays are not read behind k_seq
     int B, T, ms, bm, bmu, bmin, capnb, gy, r0, r1;   // gy: CTAs of a sequence; r0 / r1: CTAs that rank the blocks of stage 0 / of another stage
     const SeqInfo *info;
     const int *counts;
@@ -997,8 +997,9 @@ __global__ void __launch_bounds__(OT) k_offsets(const SeqInfo *info, const int *
     if (t == 0) sums->count[s][c] = run;
 }
 
-// Header: totals over the sequences.  The words go to the workspace (kernels read them there) and to `host`.
-__device__ void finish_header(const FinishArgs &f, int S, volatile HostHeader *host) {
+// Header: totals over the sequences.  The words go to the workspace (kernels read them there) and to the host.
+__device__ void finish_header(const FinishArgs &f, int S) {
+    volatile HostHeader *host = f.host;
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     __shared__ int s_err, s_more;
     __shared__ long long s_sum[4];
@@ -1200,7 +1201,7 @@ __device__ void finish_rank(const FinishArgs &f, int s, int part, int parts, lon
 
 // CTA 0: header; then r0 CTAs rank stage 0's blocks and r1 each those of the other stages; then gy
 // CTAs per sequence move its elements and block records to their place in the batch's arrays.
-__device__ __forceinline__ void finish_part(const FinishArgs &f, volatile HostHeader *host) {
+__device__ __forceinline__ void finish_part(const FinishArgs &f) {
     __shared__ long long s_keys[FKEYS];
     __shared__ int s_stages, s_bad;
     __shared__ int s_n[HDT_MAX_STAGES], s_b[HDT_MAX_STAGES], s_cn[HDT_MAX_STAGES], s_cb[HDT_MAX_STAGES];
@@ -1212,16 +1213,14 @@ __device__ __forceinline__ void finish_part(const FinishArgs &f, volatile HostHe
     if (t == 0) { s_stages = 1; s_bad = 0; }
     __syncthreads();
     int s0 = 0, L = 0;
-    if (seq) {                        // (the caller's array: k_seq, which let this kernel start, had waited for all before it)
-        s0 = f.cu[b];
-        L = f.cu[b + 1] - s0;
-    }
     pdl_wait();
     // One round of loads: the stages of the batch and its errors; in a sequence's CTA also the sums over the
     // sequences before it (elements and blocks of every stage) and its own numbers.
     int m = 1, bad = 0;
     SeqInfo info{};
     if (seq) {
+        s0 = f.cu[b];
+        L = f.cu[b + 1] - s0;
         info = f.info[b];
         if (t < f.ms) {
             s_cn[t] = f.counts[(size_t)t * f.B + b];
@@ -1250,7 +1249,7 @@ __device__ __forceinline__ void finish_part(const FinishArgs &f, volatile HostHe
     __syncthreads();
     const int S = s_stages;
     int id = blockIdx.x;
-    if (id == 0) { finish_header(f, S, host); return; }
+    if (id == 0) { finish_header(f, S); return; }
     if (s_bad) return;               // (offsets of a broken hierarchy mean nothing)
     id -= 1;
     if (!seq) {
@@ -1326,25 +1325,18 @@ __device__ __forceinline__ void finish_part(const FinishArgs &f, volatile HostHe
 
 // The header's words go straight to the host's pinned buffer, which the host watches, so no copy has to be queued behind
 // the build.  A build that is waited for also says when it has ended (`tell`): every CTA's fence and ticket stand behind
-// its writes, so the word of the CTA that is last stands behind all of them.  Its header leaves behind the ticket:
-// a fence behind words to the host waits for their trip.  That costs 2 us of a call that waits, which a deferred build, whose
-// kernel the attention waits for, does not pay.
+// its writes, so the word of the CTA that is last stands behind all of them.  That makes the kernel 2 us longer, which
+// the host's way to the next call hides there, but not where the attention is queued behind it already (deferred builds).
 __global__ void __launch_bounds__(FT) k_finish(const FinishArgs f) {
     pdl_launch_dependents();
-    __shared__ HostHeader s_host;
-    finish_part(f, f.tell ? &s_host : f.host);
+    finish_part(f);
     if (!f.tell) return;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        if (gridDim.x == 1 || atomicAdd(&f.hdr->ticket, 1) == (int)gridDim.x - 1) {      // (alone: no sequences, no k_seq that cleared the ticket)
-            __threadfence_system();
-            *(volatile int *)&f.host->done = 1;
-        }
-    }
-    if (blockIdx.x != 0) return;
-    __syncthreads();
-    for (int i = threadIdx.x; i < HostHeader::words(f.ms); i += FT) (&f.host->status)[i] = (&s_host.status)[i];
+    if (threadIdx.x != 0) return;
+    __threadfence();
+    if (gridDim.x > 1 && atomicAdd(&f.hdr->ticket, 1) != (int)gridDim.x - 1) return;      // (alone: no sequences, no k_seq that cleared the ticket)
+    __threadfence_system();
+    *(volatile int *)&f.host->done = 1;
 }
 
 }  // namespace hdt
@@ -1527,7 +1519,7 @@ extern "C" int hdt_build_index(const int8_t *level, const int32_t *parent, const
     a.glob_stride = al(sizeof(int) * (size_t)T) / sizeof(int);
     FinishArgs f{};
     for (int s = 0; s < ms; ++s) f.st[s] = ix->st[s];
-    f.cu = cu_seqlens; f.B = B; f.T = T; f.ms = ms; f.bm = bm; f.bmu = bmu; f.bmin = bmin; f.capnb = L.capnb;
+    f.cu = B > 0 ? ix->st[0].scu : cu_seqlens; f.B = B; f.T = T; f.ms = ms; f.bm = bm; f.bmu = bmu; f.bmin = bmin; f.capnb = L.capnb;
     f.gy = (int)min(16LL, max(1LL, mean / 2048));
     f.r0 = max(1, min(64, L.capnb / 16));
     f.r1 = ms > 4 ? max(1, min(8, L.capnb / 128)) : max(1, min(16, L.capnb / 64));
@@ -1587,9 +1579,9 @@ extern "C" int hdt_build_index(const int8_t *level, const int32_t *parent, const
         return set_error(HDT_ERR_CUDA, "hdt_build_index: launch failed: %s", cudaGetErrorString(e));
     }
     if (!deferred) {
-        const int rc = index_ready(ix);
+        const int rc = index_wait(ix, INDEX_COUNTED);
         if (rc) {
-            delete ix;
+            (void)hdt_index_destroy(ix);
             return rc;
         }
     }
@@ -1657,7 +1649,7 @@ int index_wait(const hdt_index *cix, IndexState want) {
 
 extern "C" int hdt_index_info(const hdt_index_t *ix, int32_t *n_stages, int64_t *nnz, int64_t *visited) {
     if (!ix) return set_error(HDT_ERR_INVALID_ARG, "hdt_index_info: null index");
-    if (const int rc = index_ready(ix)) return rc;
+    if (const int rc = index_wait(ix, INDEX_COUNTED)) return rc;
     if (n_stages) *n_stages = ix->n_stages;
     if (nnz) *nnz = ix->nnz;
     if (visited) *visited = ix->visited;
@@ -1680,7 +1672,8 @@ extern "C" int hdt_index_export(const hdt_index_t *ix, int32_t stage, hdt_stage_
 }
 
 extern "C" int hdt_index_destroy(hdt_index_t *ix) {
-    if (ix) (void)index_wait(ix, INDEX_COUNTED);     // the header must not land in a recycled buffer
+    // The header must not land in a recycled buffer; the workspace is the caller's again (of a deferred build: behind its stream).
+    if (ix) (void)index_wait(ix, ix->tells ? INDEX_COMPLETE : INDEX_COUNTED);
     delete ix;
     return HDT_OK;
 }

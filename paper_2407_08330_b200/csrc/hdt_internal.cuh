@@ -33,9 +33,9 @@ struct DevHeader {
 // The header as it lands in pinned host memory: 32-bit words in any order, none of which ever is UNSET (totals go
 // in pieces of 30 bits).  The host fills the words with UNSET before the build and has the header when none is
 // left: the device sends them without a fence, which would hold up the end of its kernel by a trip to the host.
-// The words may come while other CTAs of the build still write the index.  `done`, which a build that is waited for also
-// sends, comes from the last of these, behind all their reads and writes: from then on any stream or thread may
-// read the index or reuse the build's buffers.
+// The words come behind the last read of the caller's structure arrays, while other CTAs of the build may still write the
+// index.  `done`, which a build that is waited for also sends, comes from the last of these, behind all their reads and
+// writes: from then on any stream may read the index, and the workspace may be reused.
 struct HostHeader {
     static constexpr int UNSET = 0x7fffffff, TOTALS = 4;
     int done;
@@ -75,8 +75,9 @@ struct hdt_index {
 namespace hdt {
 
 int set_error(int code, const char *fmt, ...);
-// INDEX_QUEUED: the build's kernels are on their stream.  INDEX_COUNTED: the counts are on the host; work that is queued
-// on the stream of the build may use the index.  INDEX_COMPLETE: the build has ended, any stream may.
+// INDEX_QUEUED: the build's kernels are on their stream.  INDEX_COUNTED: the counts are on the host and the caller's structure
+// arrays have been read; work that is queued on the stream of the build may use the index.  INDEX_COMPLETE: the build
+// has ended, any stream may.
 enum IndexState { INDEX_QUEUED = 0, INDEX_COUNTED, INDEX_COMPLETE };
 // Waits until the build has come to that state; returns the structure error of the build, if any.
 int index_wait(const hdt_index *ix, IndexState state);

@@ -1,6 +1,6 @@
-"""When a build may be relied on: a waiting build has ended when it returns, so that another stream may read the index or
-change the structure arrays at once; a deferred one has for every call that is not on its stream; several threads may
-make the first use of one index."""
+"""When a build may be relied on: a waiting build has read the structure arrays when it returns, so that another stream may
+change them; every call on another stream than the build's waits for its end, of a deferred build too; a destroyed
+index's workspace is free; several threads may make the first use of one index."""
 import threading
 
 import numpy as np
@@ -73,6 +73,25 @@ def test_structure_arrays_may_change_behind_the_wait():
                 x.fill_(-1)
         torch.cuda.synchronize()
         same(idx, want)
+
+
+def test_workspace_is_free_behind_destroy():
+    """A build into a workspace that the build before it, on another stream, has just left."""
+    import paper_2407_08330_b200 as P
+    b = many()
+    want = ix.build(b.level, b.parent, b.cu_seqlens)
+    st = dev_struct(b)
+    first, second = torch.cuda.Stream(), torch.cuda.Stream()
+    ws = torch.empty(P.hdt_index_workspace_bytes(b.batch, b.total_tokens), dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    for _ in range(4):
+        with torch.cuda.stream(first):
+            P.hdt_build_index(*st, workspace=ws).close()
+        with torch.cuda.stream(second):
+            ws.zero_()
+            idx = P.hdt_build_index(*st, workspace=ws)
+            same(idx, want)
+            idx.close()
 
 
 @pytest.mark.parametrize("deferred", [False, True])
