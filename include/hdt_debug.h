@@ -54,7 +54,7 @@ extern "C" {
  *                    for the stages above 0 switch them off too.
  *   "no_overlap"     1: the stages above 0 run after stage 0 on the caller's stream instead of
  *                    beside it on an internal stream.
- *   "no_graph"       accepted and without effect (the index build is two launches; there is no graph to leave out).
+ *   "no_graph"       accepted and without effect (the index build has no graph to leave out).
  *   "no_pdl"         1: the kernels of hdt_build_index are ordinary stream successors instead of
  *                    programmatic dependents.
  *   "phase_stamps"   (only in a library built with HDT_WORKBENCH defined; otherwise ignored)

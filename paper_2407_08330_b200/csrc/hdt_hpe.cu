@@ -194,7 +194,8 @@ __global__ void __launch_bounds__(384, 2) k_hpe_eval_vec(const int8_t *__restric
 // (sin, cos)(w) when p grew by exactly one.  A run is at most 8 tokens long and restarts from a full
 // evaluation, so the rotations add at most a few 1e-7 of error.
 // The bound is HBM: x read and written (4 x 8192 tokens, d_model 768, bf16: 101 MB, 15.4 us at the copy rate;
-// 20 us, against 29 with a kernel for the numbers in front of a pipeline that stopped at a CTA barrier per tile).
+// the kernel alone 22.6 us, the call 23.8; 29.6 with a kernel for the numbers in front of a pipeline that stopped at a CTA
+// barrier per tile).
 // R: 32 tokens, 8 where that would leave SMs without a tile.
 constexpr int HPE_R = 32, HPE_R_SMALL = 8, HPE_NS = 8;     // tokens per tile; most stages a CTA keeps
 

@@ -17,10 +17,10 @@
 // What bounds it: latency (about 40 bytes a token move; a chain of barriers and shared-memory round
 // trips per stage).  The stages of a sequence only meet the other sequences' in their offsets, so the
 // grid-wide steps (formerly nine launches for three stages and a hundred for twenty, each a launch
-// latency behind the one before) are one kernel boundary.  Device time: 57 tokens 15 us, 4 x 8192 tokens 25,
-// 2 x 32768 42, 200 trees of 20 stages 60; whole passes with the nine launches and with these: 81 -> 57 us
-// (57 tokens, fp32, build and forward), 76 -> 56 (8 x 2048, build and forward), 1100 -> 807 (200 trees, build,
-// forward and backward).
+// latency behind the one before) are one kernel boundary.  Device time from the first kernel's start to the second's end: 57
+// tokens 18 us, 8 x 2048 19, 4 x 8192 tokens 26, 16 documents of 131 000 tokens 43, 2 x 32768 43, 200 trees of 20 stages 58.  Of
+// whole passes their first form made, with all else as it was then: 81 -> 57 us (57 tokens, fp32, build and
+// forward), 76 -> 56 (8 x 2048, build and forward), 1100 -> 807 (200 trees, build, forward and backward).
 #include <cstdio>
 #include <climits>
 #include <cstring>

@@ -77,7 +77,7 @@ def test_deferred_index_is_bit_exact(P):
 
 def test_deferred_same_result_as_waiting_build_repeated(P):
     """The early kernel and the kernels the host launches after its wait write the same bytes as the
-    waiting path, call after call (graph replay of the build included)."""
+    waiting path, call after call."""
     b = batches()[0][1]
     H, d = 3, 64
     t = gen.make_tensors(9, b.total_tokens, H, d, "bf16")

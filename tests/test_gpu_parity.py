@@ -61,8 +61,8 @@ def test_index_generic_trees_and_degenerate(P):
 
 
 def test_index_graph_replay_with_new_contents(P):
-    """hdt_build_index replays a cached CUDA graph while buffers and sizes repeat: the second build
-    reuses every buffer of the first with another hierarchy of the same size written into them."""
+    """Nothing of a build outlives it: the second one reuses every buffer of the first with another hierarchy of the
+    same size written into them.  (Option no_graph, of the time when the build replayed a graph, is still accepted.)"""
     rng = np.random.default_rng(3)
     batches = [gen.pack([gen.gen_fill(rng, 700, (2, 6), (2, 9), (3, 30)) for _ in range(3)]) for _ in range(3)]
     lv, pa, cu = dev_struct(batches[0])
@@ -70,7 +70,7 @@ def test_index_graph_replay_with_new_contents(P):
     for no_graph in (0, 1):
         P.hdt_set_option("no_graph", no_graph)
         try:
-          with torch.cuda.stream(torch.cuda.Stream()):      # the default stream cannot be captured
+          with torch.cuda.stream(torch.cuda.Stream()):
             for b in batches:
                 lv.copy_(torch.from_numpy(b.level).cuda()); pa.copy_(torch.from_numpy(b.parent).cuda())
                 cu.copy_(torch.from_numpy(b.cu_seqlens).cuda())
@@ -87,9 +87,8 @@ def test_index_graph_replay_with_new_contents(P):
 
 
 def test_index_graph_cache_with_alternating_buffer_sets(P):
-    """Six buffer sets (structure arrays and workspace of their own) visited round-robin three times:
-    the build's graph cache holds fewer entries than that, so graphs are replayed, replaced and
-    captured again, and every build must still equal the oracle's index."""
+    """Six buffer sets (structure arrays and workspace of their own) visited in three orders: whatever is kept from one
+    build to the next (pinned headers), every build must equal the oracle's index."""
     rng = np.random.default_rng(5)
     sets = []
     for i in range(6):
@@ -111,7 +110,7 @@ def test_index_graph_cache_with_alternating_buffer_sets(P):
 
 
 def test_index_many_sequences(P):
-    """More sequences than the single-CTA upper-stage builder takes: the per-stage kernels run."""
+    """More sequences than offsets are summed for in one kernel: the scan and the sorted runs serve them."""
     rng = np.random.default_rng(12)
     seqs = [gen.gen_fill(rng, int(rng.integers(3, 40)), (1, 3), (1, 3), (0, 6))[:2] for _ in range(1100)]
     assert_index_equal(P, gen.pack(seqs), 128, max_stages=4)
