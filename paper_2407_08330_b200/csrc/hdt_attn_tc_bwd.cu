@@ -673,9 +673,9 @@ __global__ void __launch_bounds__(256) k_bwd_tc(const __grid_constant__ CUtensor
 
 
 // ---------------------------------------------------------------------------------------------
-// Looping backward for SELF, non-EMPTY blocks at D = 128 (the persistent kernel below covers
-// D = 64): the fused pass of k_bwd_tc (S, dP; P, dS; dV, dK, dQ over the dead S / dP columns), but
-// the CTA stays resident (one per SM: 224 KB of shared memory, all of TMEM), walks the items
+// Looping backward for SELF, non-EMPTY blocks (option "no_persistent" = 5, D = 64; head_dim 128 has k_bwd_tc_x):
+// the fused pass of k_bwd_tc (S, dP; P, dS; dV, dK, dQ over the dead S / dP columns), but
+// the CTA stays resident (one per SM, all of TMEM), walks the items
 // blockIdx.x, + gridDim.x, ... of queue_split x heads, and requests the four input tiles of the
 // next item as soon as the output MMAs of the current one have finished — the gradients are
 // staged in tiles of their own, so the loads fly while the CTA drains, stages and stores.
@@ -1531,7 +1531,13 @@ static int launch_bwd_tc_t(const BwdStageArgs &a, cudaStream_t st) {
         }
         n_general = 0;
     }
-    if (((D == 128 && !a.no_persistent) || (D == 64 && a.no_persistent == 5)) && a.n_fused > 0 && !dirs) {
+    if (D == 128 && !a.no_persistent && a.n_fused > 0 && !dirs) {      // self-contained blocks: the warp-specialised looping kernel
+        rc = launch_bwd_tc_fused128(a, tq, tk, tv, tdo, outs, st);
+        if (rc) return rc;
+        b.rest_only = 1;
+        n_general = a.nb - a.n_fused;
+    }
+    if constexpr (D == 64) if (a.no_persistent == 5 && a.n_fused > 0 && !dirs) {
         // self-contained blocks through the looping kernel, the rest through the general one
         constexpr int smem_l = (4 * (D / 64) + 4 + (D / 64)) * SUB + 1024 + 64 + 512;
         static DevOnce attr_l;

@@ -94,6 +94,10 @@ struct OutMaps { CUtensorMap m[7]; };     // the same for one tensor (the forwar
 int launch_bwd_tc_fused64(const BwdStageArgs &a, const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv,
                           const CUtensorMap &tdo, const StoreMaps &outs, cudaStream_t st);
 
+// The same at head_dim 128 (hdt_attn_tc_bwd_x.cu).
+int launch_bwd_tc_fused128(const BwdStageArgs &a, const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv,
+                           const CUtensorMap &tdo, const StoreMaps &outs, cudaStream_t st);
+
 // The blocks after the first n_fused of queue_split (pieces of families longer than a row block, and
 // EMPTY blocks) at head_dim 64 through the warp-specialised one-walk backward (hdt_attn_tc_bwd_w.cu):
 // dK, dV rows are written, dQ tiles are added to a.dq_acc through `tacc` (the caller converts the sums).
