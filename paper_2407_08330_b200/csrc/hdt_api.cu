@@ -89,6 +89,9 @@ int get_side(Side **out) {
         HDT_CUDA_CHECK(cudaStreamCreateWithFlags(&sd.s, cudaStreamNonBlocking));
         HDT_CUDA_CHECK(cudaStreamCreateWithFlags(&sd.s2, cudaStreamNonBlocking));
         HDT_CUDA_CHECK(cudaStreamCreateWithFlags(&sd.s3, cudaStreamNonBlocking));
+        int least = 0, greatest = 0;
+        HDT_CUDA_CHECK(cudaDeviceGetStreamPriorityRange(&least, &greatest));
+        HDT_CUDA_CHECK(cudaStreamCreateWithPriority(&sd.first, cudaStreamNonBlocking, greatest));
         HDT_CUDA_CHECK(cudaEventCreateWithFlags(&sd.join3, cudaEventDisableTiming));
         HDT_CUDA_CHECK(cudaEventCreateWithFlags(&sd.fork, cudaEventDisableTiming));
         HDT_CUDA_CHECK(cudaEventCreateWithFlags(&sd.join, cudaEventDisableTiming));

@@ -124,8 +124,9 @@ __device__ __forceinline__ void gather_tiles_delta(uint8_t *const (&dst)[NTEN], 
 // own gradients per element (fp32, indexed by element) for the chain merge.
 // DIRS = true: the index carries direction bits other than 7; entries of the row range that the
 // bits switch off are masked as well (dir_ok).
+// (At D = 64 240 registers at most: an SM has then as many left as a CTA of the cross-attention's zeroing kernel beside it takes)
 template <int D, bool GATHER = false, bool DIRS = false>
-__global__ void __launch_bounds__(256) k_bwd_tc(const __grid_constant__ CUtensorMap tm_q,
+__global__ void __maxnreg__(D == 64 ? 240 : 255) k_bwd_tc(const __grid_constant__ CUtensorMap tm_q,
                                                 const __grid_constant__ CUtensorMap tm_k,
                                                 const __grid_constant__ CUtensorMap tm_v,
                                                 const __grid_constant__ CUtensorMap tm_do, const BwdStageArgs a) {
@@ -149,6 +150,17 @@ __global__ void __launch_bounds__(256) k_bwd_tc(const __grid_constant__ CUtensor
     const int h = blockIdx.y, H = a.H;
     const float LOG2E = 1.4426950408889634f;
 
+    // One block; with phase_split, where most block slots may be unused (the host does not know how many tokens a
+    // level subset has, the index kernel leaves the number of slots in use), as many as the grid leaves to this CTA.  (Looking
+    // at every slot's record, 1.5 us each and seven a CTA, cost a backward of 4 x 8192 tokens and 256 rows 6 us.)
+    int n_items = (int)blockIdx.x + 1;
+    if constexpr (GATHER) {
+        if (a.phase_split > 0) {
+            pdl_wait();
+            n_items = a.phase_split * a.splits + min(a.nb - a.phase_split, *a.used_slots);
+            if ((int)blockIdx.x >= n_items) return;
+        }
+    }
     if (tid == 0) {
         mbar_init(bar_tma, 1);
         mbar_init(bar_mma, 1);
@@ -164,10 +176,7 @@ __global__ void __launch_bounds__(256) k_bwd_tc(const __grid_constant__ CUtensor
     const bool dead = (*abort_flag != 0);
     uint32_t ph_tma = 0, ph_mma = 0;
 
-    if constexpr (GATHER) pdl_wait();
-    // One block; with phase_split, where most block slots may be unused (the host does not know how many tokens a
-    // level subset has), as many as the grid leaves to this CTA.
-    const int n_items = (GATHER && a.phase_split > 0) ? a.phase_split * (a.splits - 1) + a.nb : (int)blockIdx.x + 1;
+    if constexpr (GATHER) { if (a.phase_split == 0) pdl_wait(); }
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
     // rest_only: take the blocks after the first n_fused entries of queue_split
     int qi = item, split = 0;

@@ -32,7 +32,7 @@ namespace hdt {
 constexpr int XC = 32;      // CTAs (contiguous chunks) per document in the index kernel
 
 struct CrossLayout {
-    size_t sel, tokx, rngx, blocks, queue, delta, part, part_lse, total;
+    size_t sel, used, tokx, rngx, blocks, queue, delta, part, part_lse, total;
     int nbq, nbk, xr;
 };
 
@@ -77,6 +77,7 @@ static CrossLayout cross_layout(int B, int T, int Tq, int H, int D, bool tc, int
     L.rngx = o; o += al256c(sizeof(int) * 2 * max(n, (size_t)1));
     L.queue = o; o += al256c(sizeof(int) * (size_t)(L.nbq + L.nbk));
     L.sel = o; o += al256c(sizeof(int) * (size_t)(B + 1));
+    L.used = o; o += 256;
     L.delta = o; if (bwd) o += al256c(sizeof(float) * (size_t)H * max(Tq, 1));
     // partial results [splits, Tq, H, D] and, in the forward, their LSE
     const size_t splits = !bwd && cross_decode(B, Tq) ? decode_splits(B, T) : tile_splits(B, T, Tq, H, -1, bwd ? 8 : 2);
@@ -94,7 +95,7 @@ struct CrossIndexArgs {
     const int32_t *cu_k, *cu_q;
     int B, T, Tq, level_mask, xr, nbq, nbk;
     const int *sel;               // [B + 1] chosen tokens before each document and in all, or nullptr: counted by every CTA itself
-    int *tokx, *rngx, *blocks, *queue;
+    int *tokx, *rngx, *blocks, *queue, *used;      // used: slots of the chosen tokens' blocks from the first to the last one in use
 };
 
 // Which of 16 levels are chosen, one bit each.
@@ -235,23 +236,31 @@ __global__ void __launch_bounds__(256) k_cross_index(const CrossIndexArgs a) {
     put(a.nbq + s0 / xr + b, a.nbq + (last ? a.nbk : s1 / xr + b + 1), s0, s1, KO, q0, q1);
     // tiles of the gathering kernels reach past the elements in use: element 0 is a valid row of every tensor
     const int all = a.B * nt, ga = b * nt + gt;
+    if (ga == 0) *a.used = total / xr + a.B;
     for (int e = KO + total + ga; e < KO + a.T; e += all) a.tokx[e] = 0;
     for (int i = ga; i < a.nbq + a.nbk; i += all) a.queue[i] = i;
 }
 
-// Zero dK, dV rows of the encoder tokens that no decoder row attends to.  n16: 16-byte pieces of a token's row.
-__global__ void __launch_bounds__(256) k_cross_zero(const int8_t *__restrict__ level, const int32_t *__restrict__ cu_k, const int32_t *__restrict__ cu_q, int B,
+// Zero dK, dV rows of the encoder tokens that no decoder row attends to.  n16: 16-byte pieces of a token's row.  A warp looks 32 tokens
+// over at a time, a lane each, then writes row after row.  CTAs of 128 threads have few enough registers to run beside those of
+// the tile kernel (which leaves 4096 an SM); see hdt_cross_attn_bwd.
+__global__ void __launch_bounds__(128) k_cross_zero(const int8_t *__restrict__ level, const int32_t *__restrict__ cu_k, const int32_t *__restrict__ cu_q, int B,
                                                     int T, int level_mask, int n16, uint4 *dk, uint4 *dv) {
-    const int per = 256 / 32, lane = threadIdx.x & 31;
-    for (int i = blockIdx.x * per + (threadIdx.x >> 5); i < T; i += gridDim.x * per) {
-        if (chosen(level, i, level_mask)) {
+    const int lane = threadIdx.x & 31, warps = gridDim.x * 4;
+    for (int i0 = (blockIdx.x * 4 + (threadIdx.x >> 5)) * 32; i0 < T; i0 += warps * 32) {
+        const int i = i0 + lane;
+        bool zero = i < T;
+        if (zero && chosen(level, i, level_mask)) {
             int lo = 0, hi = B;          // its document: the last b with cu_k[b] <= i
             while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (cu_k[mid] <= i) lo = mid; else hi = mid; }
-            if (cu_q[lo + 1] > cu_q[lo]) continue;
+            zero = cu_q[lo + 1] <= cu_q[lo];
         }
-        for (int j = lane; j < n16; j += 32) {
-            dk[(size_t)i * n16 + j] = make_uint4(0, 0, 0, 0);
-            dv[(size_t)i * n16 + j] = make_uint4(0, 0, 0, 0);
+        for (unsigned m = __ballot_sync(0xffffffffu, zero); m != 0u; m &= m - 1u) {
+            const size_t row = (size_t)(i0 + __ffs(m) - 1) * n16;
+            for (int j = lane; j < n16; j += 32) {
+                dk[row + j] = make_uint4(0, 0, 0, 0);
+                dv[row + j] = make_uint4(0, 0, 0, 0);
+            }
         }
     }
 }
@@ -468,6 +477,7 @@ static int cross_build(const CrossLayout &L, char *ws, const int8_t *level, cons
     a.level = level; a.cu_k = cu_k; a.cu_q = cu_q; a.B = B; a.T = T; a.Tq = Tq; a.level_mask = level_mask;
     a.xr = L.xr; a.nbq = L.nbq; a.nbk = L.nbk;
     a.tokx = (int *)(ws + L.tokx); a.rngx = (int *)(ws + L.rngx); a.blocks = (int *)(ws + L.blocks); a.queue = (int *)(ws + L.queue);
+    a.used = (int *)(ws + L.used);
     if ((long long)B * T > COUNT_LINE) {
         int *sel = (int *)(ws + L.sel);
         a.sel = sel;
@@ -576,7 +586,9 @@ extern "C" int hdt_cross_attn_bwd(const int8_t *level, const int32_t *cu_seqlens
     if (total_q > 0 && (!q || !o || !lse || !d_o || !dq || (total_tokens > 0 && (!k || !v))))
         return set_error(HDT_ERR_INVALID_ARG, "hdt_cross_attn_bwd: null tensor pointer");
     // Encoder rows outside the subset (and of documents without decoder rows) get zero gradients: writes of
-    // their own, beside the other kernels.
+    // their own, beside the other kernels, from one small CTA an SM on the stream of the highest priority.  On another it starts
+    // only when the last CTA of the tile kernel has (so a backward of 4 x 8192 tokens and 256 rows ended 8 us behind that
+    // kernel); half as many CTAs, so that the tile kernel has more of HBM, cost 1 us more, a quarter as many 5.
     Side *sd = nullptr;
     if (total_tokens > 0 && batch == 0) {
         HDT_CUDA_CHECK(cudaMemsetAsync(dk, 0, (size_t)total_tokens * heads * head_dim * esz, st));
@@ -587,16 +599,16 @@ extern "C" int hdt_cross_attn_bwd(const int8_t *level, const int32_t *cu_seqlens
             rc = get_side(&sd);
             if (rc) return rc;
             HDT_CUDA_CHECK(cudaEventRecord(sd->fork, st));
-            HDT_CUDA_CHECK(cudaStreamWaitEvent(sd->s, sd->fork, 0));
-            sz = sd->s;
+            HDT_CUDA_CHECK(cudaStreamWaitEvent(sd->first, sd->fork, 0));
+            sz = sd->first;
         }
         int n_sm = 0;
         if ((rc = sm_count(&n_sm))) return rc;
-        k_cross_zero<<<min((total_tokens + 7) / 8, 8 * n_sm), 256, 0, sz>>>(level, cu_seqlens_k, cu_seqlens_q, batch, total_tokens, level_mask,
+        k_cross_zero<<<min((total_tokens + 127) / 128, sd ? n_sm : 16 * n_sm), 128, 0, sz>>>(level, cu_seqlens_k, cu_seqlens_q, batch, total_tokens, level_mask,
                                                                         (int)(heads * head_dim * esz / 16), (uint4 *)dk, (uint4 *)dv);
         count_launch();
         HDT_CUDA_CHECK(cudaGetLastError());
-        if (sd) HDT_CUDA_CHECK(cudaEventRecord(sd->join, sd->s));
+        if (sd) HDT_CUDA_CHECK(cudaEventRecord(sd->join, sd->first));
     }
     if (total_q == 0 || batch == 0) return HDT_OK;
     auto attend = [&]() -> int {
@@ -638,6 +650,7 @@ extern "C" int hdt_cross_attn_bwd(const int8_t *level, const int32_t *cu_seqlens
         a.split_rows = total_q;
         a.own_dq = (float *)(ws + L.part);
         a.pdl = 1;
+        a.used_slots = (const int *)(ws + L.used);
         r = launch_bwd_tc_upper(a, head_dim, st);
         if (r || a.splits == 1) return r;
         return launch_combine(a.splits, total_q, heads, head_dim, dtype, a.own_dq, nullptr, dq, nullptr, st);

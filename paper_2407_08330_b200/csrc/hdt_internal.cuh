@@ -133,6 +133,7 @@ constexpr int PLAN_SMS = 148;
 // on the main kernel of a call runs beside it.  fork / join are events for the two hand-overs.
 struct Side {
     cudaStream_t s, s2, s3;
+    cudaStream_t first;      // of the highest priority: a kernel on it does not wait until every CTA of an earlier one elsewhere has started
     cudaEvent_t fork, join, join2, join3;
     bool ready;
 };
@@ -290,6 +291,7 @@ struct BwdStageArgs {
     // a partial dQ of its own (own_dq holds splits x split_rows rows; phase 2 still writes the final rows).
     int phase_split, splits, split_rows;
     int pdl;                                      // as in FwdStageArgs
+    const int *used_slots;                        // cross-attention (phase_split > 0): how many slots behind the phase-1 blocks are in use; only the device knows
     int gather_end_q, gather_end_k;               // gathering kernel: elements at or beyond these read as zero rows on the Q/dO and the K/V side (0: n)
 };
 
