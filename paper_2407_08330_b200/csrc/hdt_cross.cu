@@ -45,10 +45,24 @@ static size_t al256c(size_t v) { return (v + 255) & ~size_t(255); }
 // 568 (261); 4 x 8192, anchors alone, 14, 20, 25, 34 (21).  All rows of a batch of 4 a document on one of 64 x 2048
 // 182 (98), of 256 x 512 166 (71).  (fp32 tiles cost far more: 4 x 2048 at 8 rows 53 (574); the line stays where bf16 has it.)
 static bool cross_decode(int B, int Tq) { return (long long)Tq <= 4LL * B; }
-// CTAs a document's tokens are dealt to in the decode kernel: four per SM over all documents, 32 tokens each at least.
-static int decode_splits(int B, int T) {
-    const long long mean = B > 0 ? (T + B - 1) / B : 0;
-    return (int)max(1LL, min((mean + 31) / 32, (4LL * PLAN_SMS + B - 1) / max(B, 1)));
+// Shape of a CTA of the decode kernel: heads side by side (lanes of 8 dimensions each), keys at a time.
+struct DecodeShape {
+    int HC, KS, threads, per_sm;           // per_sm: CTAs an SM's registers hold (64 a thread)
+    DecodeShape(int H, int D) {
+        const int lpk = D / 8;
+        HC = min(H, 512 / lpk);
+        KS = max(1, min(16, 384 / (HC * lpk)));
+        threads = (HC * lpk * KS + 31) / 32 * 32;
+        per_sm = 1024 / threads;
+    }
+};
+// CTAs a document's tokens are dealt to in the decode kernel: as many as the SMs hold at once over all documents, 32 tokens
+// each at least.  (A CTA begins with a chain of loads, so a second wave costs more than its shorter pieces save: 4 x 8192 tokens, 12 x 64,
+// a call with one row each 27.3 us at four CTAs an SM of which two fit, 28.5 at three, 31.7 at six, 23.5 at two.)
+static int decode_splits(int B, int T, int H, int D) {
+    const DecodeShape d(H, D);
+    const long long mean = B > 0 ? (T + B - 1) / B : 0, heads = (H + d.HC - 1) / d.HC;
+    return (int)max(1LL, min((mean + 31) / 32, (long long)PLAN_SMS * d.per_sm / (max(B, 1) * heads)));
 }
 // CTAs a row block's keys are dealt to in the tile kernels: enough to fill the SMs (`per_sm` CTAs each), pieces of
 // four chunks at least.  level_mask < 0: every level (for the workspace size).  The host does not know how many tokens a level has:
@@ -80,7 +94,7 @@ static CrossLayout cross_layout(int B, int T, int Tq, int H, int D, bool tc, int
     L.used = o; o += 256;
     L.delta = o; if (bwd) o += al256c(sizeof(float) * (size_t)H * max(Tq, 1));
     // partial results [splits, Tq, H, D] and, in the forward, their LSE
-    const size_t splits = !bwd && cross_decode(B, Tq) ? decode_splits(B, T) : tile_splits(B, T, Tq, H, -1, bwd ? 8 : 2);
+    const size_t splits = !bwd && cross_decode(B, Tq) ? decode_splits(B, T, H, D) : tile_splits(B, T, Tq, H, -1, bwd ? 8 : 2);
     L.part = o; o += al256c(sizeof(float) * splits * Tq * H * D);
     L.part_lse = o; if (!bwd) o += al256c(sizeof(float) * splits * Tq * H);
     L.total = o + 256;
@@ -273,7 +287,7 @@ __global__ void __launch_bounds__(128) k_cross_zero(const int8_t *__restrict__ l
 // chip: 8 rows on one of 8 documents of 2048 tokens 28 us, so 19.)
 // Thread (slot, head, lane): D / 8 lanes per (key, head), the heads of a token next to one another, so that a
 // CTA reads whole token rows.  The bound is reading K and V once (4 x 8192 tokens, 12 x 64: 101 MB, 15 us at the
-// copy rate): four keys a thread in flight and four CTAs an SM; the tile kernel took 352 us here, one CTA per
+// copy rate; 20 us as one wave of CTAs): four keys a thread in flight; the tile kernel took 352 us here, one CTA per
 // document and head walking 64 chunks with one row of 128 in use.
 struct DecodeArgs {
     const int8_t *level;
@@ -315,11 +329,16 @@ __global__ void __launch_bounds__(512, 2) k_cross_decode(const DecodeArgs a) {
                     __syncthreads();
                     if (t < 32) {
                         int n = 0;
-                        for (int i0 = p0; i0 < p1; i0 += 32) {
-                            const bool f = i0 + lane < p1 && chosen(a.level, i0 + lane, a.level_mask);
-                            const unsigned m = __ballot_sync(0xffffffffu, f);
-                            if (f) s_list[n + __popc(m & ((1u << lane) - 1u))] = i0 + lane;
-                            n += __popc(m);
+                        for (int i0 = p0; i0 < p1; i0 += 128) {      // (four loads in flight: nothing of K and V is requested before the list is there)
+                            bool f[4];
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) f[k] = i0 + 32 * k + lane < p1 && chosen(a.level, i0 + 32 * k + lane, a.level_mask);
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                const unsigned m = __ballot_sync(0xffffffffu, f[k]);
+                                if (f[k]) s_list[n + __popc(m & ((1u << lane) - 1u))] = i0 + 32 * k + lane;
+                                n += __popc(m);
+                            }
                         }
                         if (lane == 0) s_n = n;
                     }
@@ -396,43 +415,53 @@ __global__ void __launch_bounds__(512, 2) k_cross_decode(const DecodeArgs a) {
 }
 
 // Merge of partial results over `splits`, a CTA per (row, head).  Forward (lse given): log-sum-exp merge of
-// normalised rows; backward: sum.
+// normalised rows; backward: sum.  Groups of D / 8 lanes take every G-th partial result, then meet: inside a warp by
+// shuffles, the four warps through shared memory (all groups one after the other there: 0.7 us more).
 template <int D, bool BF16>
 __global__ void __launch_bounds__(128) k_cross_combine(int splits, int Tq, int H, const float *part, const float *part_lse, void *out, float *lse) {
     pdl_wait();
     pdl_launch_dependents();
     constexpr int LPK = D / 8, G = 128 / LPK;
     using W = Raw<BF16, LPK>;
-    __shared__ float s_red[G][D + 2];
-    const int row = blockIdx.x, h = blockIdx.y, g = threadIdx.x % LPK, i = threadIdx.x / LPK;
+    __shared__ float s_red[4][D + 2];
+    const int row = blockIdx.x, h = blockIdx.y, g = threadIdx.x % LPK, i = threadIdx.x / LPK, w = threadIdx.x >> 5;
     RowSoftmax R;
     R.clear();
+    auto add = [&](float m, float l, const f2 (&x)[4]) {
+        if (part_lse != nullptr) R.merge(m, l, x);
+        else
+#pragma unroll
+            for (int u = 0; u < 4; ++u) R.acc[u] = add2(R.acc[u], x[u]);
+    };
 #pragma unroll 4
     for (int s = i; s < splits; s += G) {
         const size_t r = ((size_t)s * Tq + row) * H + h;
         f2 x[4];
         W::load_f32(part, r, g, x);
-        if (part_lse != nullptr) {
-            const float L = part_lse[r];
-            R.merge(L * 1.4426950408889634f, L > -INFINITY ? 1.f : 0.f, x);
-        } else {
-#pragma unroll
-            for (int u = 0; u < 4; ++u) R.acc[u] = add2(R.acc[u], x[u]);
-        }
+        const float L = part_lse != nullptr ? part_lse[r] : 0.f;
+        add(L * 1.4426950408889634f, L > -INFINITY ? 1.f : 0.f, x);
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) unpack2(R.acc[u], s_red[i][8 * g + 2 * u], s_red[i][8 * g + 2 * u + 1]);
-    if (g == 0) { s_red[i][D] = R.m; s_red[i][D + 1] = R.l; }
+    for (int o = LPK; o < 32; o *= 2) {
+        f2 x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = __shfl_xor_sync(0xffffffffu, R.acc[u], o);
+        const float m = __shfl_xor_sync(0xffffffffu, R.m, o), l = __shfl_xor_sync(0xffffffffu, R.l, o);
+        add(m, l, x);
+    }
+    if ((threadIdx.x & 31) < LPK) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) unpack2(R.acc[u], s_red[w][8 * g + 2 * u], s_red[w][8 * g + 2 * u + 1]);
+        if (g == 0) { s_red[w][D] = R.m; s_red[w][D + 1] = R.l; }
+    }
     __syncthreads();
     if (i != 0) return;
-    for (int j = 1; j < min(G, splits); ++j) {
+#pragma unroll
+    for (int j = 1; j < 4; ++j) {
         f2 x[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) x[u] = pack2(s_red[j][8 * g + 2 * u], s_red[j][8 * g + 2 * u + 1]);
-        if (part_lse != nullptr) R.merge(s_red[j][D], s_red[j][D + 1], x);
-        else
-#pragma unroll
-            for (int u = 0; u < 4; ++u) R.acc[u] = add2(R.acc[u], x[u]);
+        add(s_red[j][D], s_red[j][D + 1], x);
     }
     if (part_lse != nullptr) {
         const float L = R.finish();
@@ -454,11 +483,11 @@ static int launch_combine(int splits, int Tq, int H, int D, int dtype, const flo
 
 template <int D, bool BF16>
 static int launch_decode_t(DecodeArgs a, int B, cudaStream_t st) {
-    constexpr int LPK = D / 8;
-    a.HC = min(a.H, 512 / LPK);
-    a.KS = max(1, min(16, 384 / (a.HC * LPK)));
+    const DecodeShape d(a.H, D);
+    a.HC = d.HC;
+    a.KS = d.KS;
     a.B = B;
-    const int threads = (a.HC * LPK * a.KS + 31) / 32 * 32;
+    const int threads = d.threads;
     const unsigned groups = B + (a.Tq > DEC_ROWS ? (a.Tq + DEC_ROWS - 1) / DEC_ROWS : 0);
     const size_t smem = sizeof(float) * (size_t)a.KS * a.HC * (D + 2);
     HDT_CUDA_CHECK(launch_dependent(k_cross_decode<D, BF16>, true, dim3(groups * a.splits, (a.H + a.HC - 1) / a.HC), threads, smem, st, a));
@@ -536,7 +565,7 @@ extern "C" int hdt_cross_attn_fwd(const int8_t *level, const int32_t *cu_seqlens
     if (cross_decode(batch, total_q) && !g_force_simt) {
         DecodeArgs a{};
         a.level = level; a.cu_k = cu_seqlens_k; a.cu_q = cu_seqlens_q; a.level_mask = level_mask; a.H = heads; a.Tq = total_q;
-        a.splits = decode_splits(batch, total_tokens);
+        a.splits = decode_splits(batch, total_tokens, heads, head_dim);
         a.q = q; a.k = k; a.v = v; a.scale_log2 = scale * 1.4426950408889634f;
         a.o = o; a.lse = lse; a.part_o = part; a.part_lse = part_lse;
         if (head_dim == 64) rc = dtype == HDT_BF16 ? launch_decode_t<64, true>(a, batch, st) : launch_decode_t<64, false>(a, batch, st);

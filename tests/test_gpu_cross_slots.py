@@ -43,3 +43,27 @@ def test_cross_slots(name):
     doc = np.repeat(np.arange(b.batch), np.diff(b.cu_seqlens))
     rest = torch.from_numpy(~(((mask >> np.maximum(b.level, 0)) & 1).astype(bool) & (b.level >= 0) & (np.asarray(nq)[doc] > 0))).cuda()
     assert (g[1][rest] == 0).all() and (g[2][rest] == 0).all()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("docs,nq,mask,H,d", [
+    ([[[3]]], [1], 15, 1, 64),                              # one piece
+    ([[[31] * 4], [[0] * 3], [[60] * 2]], [1, 1, 1], 15, 12, 64),      # a piece of 32 tokens and more, two CTAs an SM
+    ([[[60] * 40]], [1], 15, 16, 128),                      # four CTAs an SM
+    ([[[60] * 40], [[9] * 7]], [2, 1], 6, 40, 128),         # more heads than a CTA takes, anchors alone
+    ([[[50] * 160]], [3], 8, 3, 64),                        # the longest pieces, a document with every row
+])
+def test_decode_pieces(docs, nq, mask, H, d, dtype):
+    import paper_2407_08330_b200 as P
+    b = gen.pack([gen.layout(s) for s in docs])
+    rng = np.random.default_rng(4)
+    f = gen.round_bf16 if dtype == "bf16" else (lambda x: x)
+    cu_q = np.concatenate([[0], np.cumsum(nq)]).astype(np.int32)
+    q = f(rng.standard_normal((int(cu_q[-1]), H, d)).astype(np.float32))
+    k, v = (f(rng.standard_normal((b.total_tokens, H, d)).astype(np.float32)) for _ in range(2))
+    lv, cuk, cuq = (torch.from_numpy(x).cuda() for x in (b.level, b.cu_seqlens, cu_q))
+    o, lse = P.hdt_cross_attn_fwd(lv, cuk, cuq, mask, *(dev_tensor(x, dtype) for x in (q, k, v)))
+    P.hdt_device_status()
+    o_r, lse_r = co.forward(b.level, b.cu_seqlens, mask, cu_q, q, k, v)
+    check_close(host(o), o_r, dtype, "O")
+    check_close(host(lse), lse_r, "f32" if dtype == "f32" else "bf16", "LSE")
