@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(ROW_THREADS, BF16 ? 4 : 3) k_bwd_rows(const Ro
 // A CTA takes 32 (head_dim 64) or 16 (128) rows of a block and the keys of their ranges, in pieces of KT; a
 // row is owned by D / 8 lanes as above.  The elements that live on leave their partial result in stage 1's
 // buffers.  What bounds it is the chain of a key chunk (loads, products, reduction, exponential, broadcast) at the
-// six warps a scheduler holds: 2 x 2048 tokens, 12 x 64, 53 us forward and 141 backward, against 100 and 191 for
+// six warps a scheduler holds: 2 x 2048 tokens, 12 x 64, 54 us forward and 143 backward (148 with loops that end row by row), against 100 and 191 for
 // the kernels that give 16 dimensions to a lane and walk a whole block's span in step.  Measured and not kept: a row
 // on 2 (forward) or 4 (backward) lanes (49 and 173 us: fewer warps, twice the registers), four and two rows to
 // eight lanes, so that a key read from shared memory serves several (58 and 213), going on to the
@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 3) k_fwd_tile(const TileFwdArgs 
     __shared__ int s_ab[2];
     float4 *sK = s_tile, *sV = sK + KT * U;
     const int h = blockIdx.y, lane = threadIdx.x & 31, g = lane % LPK, src = lane - g;
-    const unsigned mask = ((1u << LPK) - 1u) << src;
+    constexpr unsigned mask = 0xffffffffu;       // (the rows of a warp walk in step: with a mask per row their shuffles issue one after the other)
     TileRows T;
     T.find(a, ROWS, (a.block_rows + ROWS - 1) / ROWS, s_ab);
     if (T.n <= 0) return;
@@ -360,8 +360,10 @@ __global__ void __launch_bounds__(TILE_THREADS, 3) k_fwd_tile(const TileFwdArgs 
         tile_load<D>(sV, a.v, c0, n, a.H, h);
         cp_async_wait();
         __syncthreads();
-        const int jlo = max(r.x, c0), jhi = min(r.y, c0 + n);
-        for (int j0 = jlo; j0 < jhi; j0 += C) {
+        int jlo = max(r.x, c0), jhi = min(r.y, c0 + n);
+        if (jhi <= jlo) jlo = jhi = c0;
+        const int steps = __reduce_max_sync(mask, (jhi - jlo + C - 1) / C);
+        for (int it = 0, j0 = jlo; it < steps; ++it, j0 += C) {
             float sc[C];
             f2 qf[4];
             q.get(qf);
@@ -369,7 +371,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 3) k_fwd_tile(const TileFwdArgs 
             for (int i = 0; i < C; ++i) {
                 R x;
                 f2 k[4];
-                x.load_smem(sK + (min(j0 + i, jhi - 1) - c0) * U, g);      // (keys past the end: the last one, weight 0)
+                x.load_smem(sK + max(min(j0 + i, jhi - 1) - c0, 0) * U, g);      // (keys past the end: the last one, weight 0)
                 x.get(k);
                 sc[i] = dot8(qf, k);
             }
@@ -383,18 +385,18 @@ __global__ void __launch_bounds__(TILE_THREADS, 3) k_fwd_tile(const TileFwdArgs 
                 const f2 w2 = pack2(w, w);
                 R y;
                 f2 v[4];
-                y.load_smem(sV + (min(j0 + i, jhi - 1) - c0) * U, g);
+                y.load_smem(sV + max(min(j0 + i, jhi - 1) - c0, 0) * U, g);
                 y.get(v);
 #pragma unroll
                 for (int u = 0; u < 4; ++u) S.acc[u] = fma2(w2, v[u], S.acc[u]);
             }
         }
     }
-    if (!inb) return;
-    const int up = a.up ? __ldg(a.up + row) : -1;
     // (l over the C lanes that hold different keys)
 #pragma unroll
     for (int o = 1; o < C; o *= 2) S.l += __shfl_xor_sync(mask, S.l, o);
+    if (!inb) return;
+    const int up = a.up ? __ldg(a.up + row) : -1;
     const float lse = S.finish();
     if (up >= 0) {
         R::store(a.part_o, (unsigned)up * a.H + h, g, S.acc);
@@ -415,7 +417,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) k_bwd_tile(const TileBwdArgs 
     __shared__ float s_lse[KT], s_delta[KT];
     float4 *sK = s_tile, *sV = sK + KT * U, *sQ = sV + KT * U, *sG = sQ + KT * U;
     const int h = blockIdx.y, lane = threadIdx.x & 31, g = lane % LPK, src = lane - g;
-    const unsigned mask = ((1u << LPK) - 1u) << src;
+    constexpr unsigned mask = 0xffffffffu;       // (the rows of a warp walk in step: with a mask per row their shuffles issue one after the other)
     TileRows T;
     T.find(a, ROWS, (a.block_rows + ROWS - 1) / ROWS, s_ab);
     if (T.n <= 0) return;
@@ -433,7 +435,8 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) k_bwd_tile(const TileBwdArgs 
         tile_load<D>(sG, a.d_o, c0, n, a.H, h);
         cp_async_wait();
         __syncthreads();
-        for (int i = rl; i < n; i += ROWS) {           // rowsum(dO . O) of the tile's rows
+        for (int i0 = 0; i0 < n; i0 += ROWS) {         // rowsum(dO . O) of the tile's rows
+            const int i = min(i0 + rl, n - 1);
             R o, y;
             o.load(a.o, (unsigned)(c0 + i) * a.H + h, g);
             y.load_smem(sG + i * U, g);
@@ -446,23 +449,25 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) k_bwd_tile(const TileBwdArgs 
             }
         }
         __syncthreads();
-        const int jlo = max(r.x, c0), jhi = min(r.y, c0 + n);
-        for (int j0 = jlo; j0 < jhi; j0 += C) {
-            const int jm = j0 + (g & (C - 1)), jc = min(jm, jhi - 1);
+        int jlo = max(r.x, c0), jhi = min(r.y, c0 + n);
+        if (jhi <= jlo) jlo = jhi = c0;
+        const int steps = __reduce_max_sync(mask, (jhi - jlo + C - 1) / C);
+        for (int it = 0, j0 = jlo; it < steps; ++it, j0 += C) {
+            const int jm = j0 + (g & (C - 1)), jc = max(min(jm, jhi - 1), c0);
             const bool in = jm < jhi;
             const bool ok_q = in && (a.dirs == 7 || dir_ok(row, jm, r.x, a.dirs));
             const bool ok_k = in && (a.dirs == 7 || dir_ok_key(row, jm, r.x, a.dirs));
             R x[C], y[C];
 #pragma unroll
             for (int i = 0; i < C; ++i) {
-                const int o = (min(j0 + i, jhi - 1) - c0) * U;
+                const int o = max(min(j0 + i, jhi - 1) - c0, 0) * U;
                 x[i].load_smem(sK + o, g);
                 y[i].load_smem(sV + o, g);
             }
             S.template as_query<C>(x, y, ok_q, a.scale_log2, g, mask, src);
 #pragma unroll
             for (int i = 0; i < C; ++i) {
-                const int o = (min(j0 + i, jhi - 1) - c0) * U;
+                const int o = max(min(j0 + i, jhi - 1) - c0, 0) * U;
                 x[i].load_smem(sQ + o, g);
                 y[i].load_smem(sG + o, g);
             }
