@@ -27,7 +27,9 @@
 
 namespace hdt {
 
-static constexpr int ROW_THREADS = 128;
+// (small CTAs: one gives its place up when its longest row is done, and rows differ; 200 trees, forward and backward, 128 threads 244.8 us,
+// 64 240.0, 32 242.6)
+static constexpr int ROW_THREADS = 64;
 
 // The keys of a row over the stages it lives in, a chunk at a time.  What the next stage needs first (range,
 // next index) is loaded on entering a stage, and the tokens of a chunk while the one before it is worked
@@ -99,7 +101,7 @@ __device__ __forceinline__ void fwd_walk(const Args &a, const Raw<BF16, D / 8> &
 }
 
 template <int D, bool BF16, int KP, int C>
-__global__ void __launch_bounds__(ROW_THREADS, KP == 1 && C == 4 && BF16 ? 8 : 4) k_fwd_rows(const RowFwdArgs a) {
+__global__ void __launch_bounds__(ROW_THREADS, KP == 1 && C == 4 && BF16 ? 16 : 8) k_fwd_rows(const RowFwdArgs a) {
     constexpr int LPK = D / 8, G = LPK * KP;
     using R = Raw<BF16, LPK>;
     const int lane = threadIdx.x & 31, sub = lane % G, g = sub % LPK, kp = sub / LPK;
@@ -241,7 +243,7 @@ __device__ __forceinline__ void bwd_walk(const Args &a, RowGrad<BF16, D / 8> &S,
 }
 
 template <int D, bool BF16, int KP, bool DELTA>
-__global__ void __launch_bounds__(ROW_THREADS, BF16 ? 4 : 3) k_bwd_rows(const RowBwdArgs a) {
+__global__ void __launch_bounds__(ROW_THREADS, BF16 ? 8 : 6) k_bwd_rows(const RowBwdArgs a) {
     constexpr int LPK = D / 8, G = LPK * KP, C = 2;
     using R = Raw<BF16, LPK>;
     const int lane = threadIdx.x & 31, sub = lane % G, g = sub % LPK, kp = sub / LPK;
