@@ -271,6 +271,21 @@ static bool tile_f32(int dtype) { return dtype == HDT_F32 && !g_no_rows && !g_fo
 static bool tile_f32_rows(const hdt_index *ix, int heads, int head_dim) {
     return ix->n_stages == 1 || (rows_allowed() && ix->nnz_upper * heads * (head_dim / 64) <= 4000000);
 }
+// Documents (two or three stages, full rule) whose stages above 0 follow stage 0 on the caller's stream as programmatic
+// dependents, the merge behind them: no fork and no join, which cost the host 5 us a call, and no gap before the merge.  Every
+// kernel of the chain ends behind the one before it.  us forward and backward, in brackets with side streams: 3 x 3001
+// tokens, two layers, waiting builds 179.5 (184.4); 4 x 8192 219.8 (221.2), behind a deferred build, where the host is not waited for, 202.3 (202.7).
+static bool upper_chain(const hdt_index *ix) {
+    return rows_allowed() && ix->directions == 7 && ix->n_stages >= 2 && ix->n_stages <= 3;
+}
+
+// Stage 1 of a forward that completes its elements itself: see hdt_attn_fwd.
+static bool short_stage1(const hdt_index *ix, int heads) {
+    int n_sm = 0;
+    return sm_count(&n_sm) == HDT_OK && ix->n_stages > 1 && ix->desc[1].n_fused + ix->desc[1].n_empty == ix->desc[1].nb &&
+           (long long)ix->desc[1].nb * heads <= 2LL * n_sm;
+}
+
 static void row_stages(const hdt_index *ix, RowStage *st) {
     for (int s = 0; s < ix->n_stages; ++s) st[s] = RowStage{ix->st[s].tok, ix->st[s].rng, ix->st[s].up};
 }
@@ -395,6 +410,33 @@ extern "C" int hdt_attn_fwd(const hdt_index_t *ix, const void *q, const void *k,
         a.tok_rows = a.tok;
         return a;
     };
+    // (see hdt_attn_bwd; where stage 1 is not short enough to complete its elements itself, see below)
+    if (!up_rows && dtype == HDT_BF16 && !g_force_simt && ix->desc[0].n_fused == ix->desc[0].nb && upper_chain(ix) && !short_stage1(ix, heads)) {
+        if (!early) {
+            ProfScope ps(PROF_FWD_STAGE0, st);
+            rc = launch_fwd_tc(stage_args(0), head_dim, st);
+            if (rc) return rc;
+        }
+        ps_early.reset();
+        ProfScope ps(PROF_FWD_UPPER, st);
+        ChainArgs c{};
+        c.n1 = ix->desc[1].n; c.H = heads; c.T = ix->total_tokens; c.n_stages = ix->n_stages; c.nt = 1;
+        c.tok1 = ix->st[1].tok;
+        c.pdl = 1;
+        for (int s = 1; s < ix->n_stages; ++s) {
+            FwdStageArgs a = stage_args(s);
+            a.own_o = (float *)(ws + L.own[s][0]);
+            a.own_lse = (float *)(ws + L.own[s][1]);
+            c.up[s] = ix->st[s].up; c.own[s][0] = a.own_o; c.own_lse[s] = a.own_lse;
+            a.pdl = 2;
+            rc = launch_fwd_tc_upper(a, head_dim, st);
+            if (rc) return rc;
+        }
+        c.base[0] = (const float *)(ws + L.part[1][0]);
+        c.base_lse = (const float *)(ws + L.part[1][1]);
+        c.out[0] = o; c.lse = lse;
+        return launch_chain_merge(c, head_dim, dtype, st);
+    }
     // The stages above 0 do not depend on stage 0 until their results are merged: compute them on
     // the side stream while stage 0 runs, then finish each with an element-wise merge.
     const bool overlap = (ix->n_stages > 1 && !g_no_overlap) || early;
@@ -431,10 +473,7 @@ extern "C" int hdt_attn_fwd(const hdt_index_t *ix, const void *q, const void *k,
         // resident at once.  Otherwise (skewed documents with long sections: 47 us against 13; large
         // batches at head_dim 128: 59 against 23) stage 1 runs beside stage 0 like the others and the
         // merge kernel follows.
-        int n_sm1 = 0;
-        if (const int rc_ = sm_count(&n_sm1)) return rc_;
-        const bool short1 = ix->n_stages > 1 && ix->desc[1].n_fused + ix->desc[1].n_empty == ix->desc[1].nb &&
-                            (long long)ix->desc[1].nb * heads <= 2LL * n_sm1;
+        const bool short1 = short_stage1(ix, heads);
         const bool fold = tc_upper && !(g_no_fold & 1) && (short1 || (g_no_fold & 2)) && ix->n_stages > 1 && ix->n_stages <= 3;
         FwdStageArgs a1{};
         // (deep trees on the SIMT kernels: the stages above 0 are independent in own-partial mode and small, and a
@@ -649,6 +688,34 @@ extern "C" int hdt_attn_bwd(const hdt_index_t *ix, const void *q, const void *k,
         a.n_empty = ix->desc[s].n_empty;
         return a;
     };
+    // Stage 0 in one kernel: the stages above it and the merge follow as programmatic dependents on the caller's stream.  Their CTAs
+    // come when those of stage 0 leave, as they do from a side stream, without the events (see upper_chain).
+    if (!up_rows && tc_upper && dq_acc == nullptr && ix->desc[0].n_fused == ix->desc[0].nb && upper_chain(ix)) {
+        {
+            ProfScope ps(PROF_BWD_STAGE0, st);
+            rc = launch_bwd_tc(stage_args(0), head_dim, st);
+            if (rc) return rc;
+        }
+        ProfScope ps(PROF_BWD_UPPER, st);
+        ChainArgs c{};
+        c.n1 = ix->desc[1].n; c.H = heads; c.T = ix->total_tokens; c.n_stages = ix->n_stages; c.nt = 3;
+        c.tok1 = ix->st[1].tok;
+        c.pdl = 1;
+        for (int s = 1; s < ix->n_stages; ++s) {
+            BwdStageArgs a = stage_args(s);
+            a.own_dq = (float *)(ws + L.own[s][0]);
+            a.own_dk = (float *)(ws + L.own[s][1]);
+            a.own_dv = (float *)(ws + L.own[s][2]);
+            c.up[s] = ix->st[s].up;
+            c.own[s][0] = a.own_dq; c.own[s][1] = a.own_dk; c.own[s][2] = a.own_dv;
+            a.pdl = 2;
+            rc = launch_bwd_tc_upper(a, head_dim, st);
+            if (rc) return rc;
+        }
+        for (int k = 0; k < 3; ++k) c.base[k] = (const float *)(ws + L.part[1][k]);
+        c.out[0] = dq; c.out[1] = dk; c.out[2] = dv;
+        return launch_chain_merge(c, head_dim, dtype, st);
+    }
     if (overlap) {   // delta is ready: the upper stages' own gradients are computed beside stage 0
         Side *sd = nullptr;
         rc = get_side(&sd);

@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(128) k_fwd_tc(const __grid_constant__ CUtensor
     volatile int *abort_flag = (volatile int *)(slot + 1);
 
     const int tid = threadIdx.x, warp = tid >> 5;
-    if constexpr (GATHER) pdl_wait();
+    if constexpr (GATHER) { if (a.pdl != 2) pdl_wait(); }      // (2: what it reads is complete since the kernel of stage 0 has let this one start)
     // SINGLE: the first n_fused entries of queue_split; rest_only: the blocks after them
     const int blk = SINGLE ? a.queue_split[blockIdx.x]
                            : (a.rest_only ? a.queue_split[a.n_fused + blockIdx.x] : a.queue[blockIdx.x]);
@@ -121,6 +121,7 @@ __global__ void __launch_bounds__(128) k_fwd_tc(const __grid_constant__ CUtensor
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if constexpr (GATHER) { if (a.pdl == 2) pdl_launch_dependents(); }
     const uint32_t tmem = *slot;
     const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
 
@@ -465,6 +466,7 @@ __global__ void __launch_bounds__(128) k_fwd_tc(const __grid_constant__ CUtensor
         tc_fence_before();
         __syncthreads();
         if (warp == 0) tmem_dealloc(tmem, TM_COLS);
+        if (a.pdl == 2) pdl_wait();         // (what follows takes its end for the end of the kernels before it too)
         return;
     }
     float *po = nullptr;

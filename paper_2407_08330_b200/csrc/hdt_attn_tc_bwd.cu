@@ -176,7 +176,11 @@ __global__ void __maxnreg__(D == 64 ? 240 : 255) k_bwd_tc(const __grid_constant_
     const bool dead = (*abort_flag != 0);
     uint32_t ph_tma = 0, ph_mma = 0;
 
-    if constexpr (GATHER) { if (a.phase_split == 0) pdl_wait(); }
+    // (pdl = 2: what it reads is complete since the kernel of stage 0 has let this one start; it waits at its end)
+    if constexpr (GATHER) {
+        if (a.pdl == 2) pdl_launch_dependents();
+        else if (a.phase_split == 0) pdl_wait();
+    }
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
     // rest_only: take the blocks after the first n_fused entries of queue_split
     int qi = item, split = 0;
@@ -678,6 +682,7 @@ __global__ void __maxnreg__(D == 64 ? 240 : 255) k_bwd_tc(const __grid_constant_
     tc_fence_after();
     }
     if (warp == 0) tmem_dealloc(tmem, TM_COLS);
+    if constexpr (GATHER) { if (a.pdl == 2) pdl_wait(); }      // (what follows takes its end for the end of the kernels before it too)
 }
 
 

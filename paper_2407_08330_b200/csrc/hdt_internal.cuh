@@ -245,7 +245,8 @@ struct FwdStageArgs {
     // Gathering kernel in own-partial mode: splits > 1 gives the key span of a block to that many CTAs (grid.z), each with
     // a partial result of its own (own_o / own_lse hold splits x split_rows rows).
     int splits, split_rows;
-    int pdl;              // gathering kernel: launched as a programmatic dependent of the kernel before it on the stream
+    int pdl;              // gathering kernel: launched as a programmatic dependent of the kernel before it on the stream; 2: of a stage below,
+                          // of which it reads nothing, so that it only ends behind it
     const DevHeader *hdr; // set: the index build is still in flight; the looping kernel reads n_fused and stage 1's size here
     size_t ws_bytes;      // with hdr: bytes behind part_o (the caller's workspace)
     int n_empty;          // EMPTY blocks of the stage (0 where the caller does not know): when they are all that is left
@@ -382,6 +383,7 @@ int launch_bwd_rows(const RowBwdArgs &a, int head_dim, int dtype, cudaStream_t s
 // by following the `up` maps.  nt = 1 tensor (forward: O with LSE) or 3 (backward: dQ, dK, dV).
 struct ChainArgs {
     int n1, H, T, n_stages, nt;
+    int pdl;                                 // launched as a programmatic dependent of the last kernel whose results it merges
     const int *tok1;
     const int *up[HDT_MAX_STAGES];           // up[s]: stage s -> stage s+1
     const float *own[HDT_MAX_STAGES][3];     // own[s][t], s >= 1
