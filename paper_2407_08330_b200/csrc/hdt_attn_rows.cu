@@ -177,7 +177,7 @@ template <bool BF16, int N> struct RowGrad {
         dots<C>(go, y, v2);
         const float s = reduce_scatter<C, N>(v1, g, mask) * scale_log2, dp = reduce_scatter<C, N>(v2, g, mask);
         const float p = ok ? exp2f(s - lse) : 0.f;
-        axpys<C>(dq, p * (dp - delta), x, mask, src);
+        axpys<C>(dq, ok ? p * (dp - delta) : 0.f, x, mask, src);      // (a row that is none's query may hold anything in dO: see k_bwd_tile)
     }
     // The row as a key: Q rows x and dO rows y of queries that attend to it, with their LSE and delta.
     template <int C>
@@ -188,7 +188,7 @@ template <bool BF16, int N> struct RowGrad {
         dots<C>(v, y, v2);
         const float s = reduce_scatter<C, N>(v1, g, mask) * scale_log2, dp = reduce_scatter<C, N>(v2, g, mask);
         const float p = ok ? exp2f(s - lse_j) : 0.f;
-        axpys<C>(dk, p * (dp - delta_j), x, mask, src);
+        axpys<C>(dk, ok ? p * (dp - delta_j) : 0.f, x, mask, src);
         axpys<C>(dv, p, y, mask, src);
     }
     __device__ __forceinline__ void scale(float c) {
@@ -297,10 +297,21 @@ __global__ void __launch_bounds__(ROW_THREADS, BF16 ? 8 : 6) k_bwd_rows(const Ro
 // on 2 (forward) or 4 (backward) lanes (49 and 173 us: fewer warps, twice the registers), four and two rows to
 // eight lanes, so that a key read from shared memory serves several (58 and 213), going on to the
 // stages above 0 inside this kernel (70 and 185: one long row holds the CTA).
+// The rows of a warp walk in step: one with no keys left reads its last key again, one that has none in the piece a row of
+// zeros behind it (KT), at weight 0 both.  A key of another family there would carry an inf into a row that does not attend to it.
+// (KT: with the zero rows two backward CTAs take 196 KB of an SM, the step below the largest; at one row more, 228 KB, 28 instead of 60 are
+// left for L1, and 2 x 2048 tokens forward and backward take 219 us instead of 215, as much as without the zero rows.)
 static constexpr int TILE_THREADS = 256;
 template <int D> struct TileShape {
-    static constexpr int LPK = D / 8, ROWS = TILE_THREADS / LPK, KT = D == 64 ? 96 : 48;
+    static constexpr int LPK = D / 8, ROWS = TILE_THREADS / LPK, KT = D == 64 ? 95 : 47, PIECE = (KT + 1) * (D / 4);      // PIECE: float4s of a tensor's rows
 };
+// The keys [lo, hi) of a row in the piece of n from c0 on, counted from c0.
+template <int KT>
+__device__ __forceinline__ void piece_range(int2 r, int c0, int n, int &lo, int &hi) {
+    lo = max(r.x - c0, 0);
+    hi = min(r.y - c0, n);
+    if (hi <= lo) lo = hi = KT + 1;
+}
 __device__ __forceinline__ void cp_async16(float4 *dst, const float4 *src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
 }
@@ -339,7 +350,8 @@ __global__ void __launch_bounds__(TILE_THREADS, 3) k_fwd_tile(const TileFwdArgs 
     pdl_launch_dependents();
     extern __shared__ float4 s_tile[];
     __shared__ int s_ab[2];
-    float4 *sK = s_tile, *sV = sK + KT * U;
+    float4 *sK = s_tile, *sV = sK + TileShape<D>::PIECE;
+    for (int i = threadIdx.x; i < 2 * U; i += TILE_THREADS) s_tile[i / U * TileShape<D>::PIECE + KT * U + i % U] = make_float4(0.f, 0.f, 0.f, 0.f);
     const int h = blockIdx.y, lane = threadIdx.x & 31, g = lane % LPK, src = lane - g;
     constexpr unsigned mask = 0xffffffffu;       // (the rows of a warp walk in step: with a mask per row their shuffles issue one after the other)
     TileRows T;
@@ -362,10 +374,10 @@ __global__ void __launch_bounds__(TILE_THREADS, 3) k_fwd_tile(const TileFwdArgs 
         tile_load<D>(sV, a.v, c0, n, a.H, h);
         cp_async_wait();
         __syncthreads();
-        int jlo = max(r.x, c0), jhi = min(r.y, c0 + n);
-        if (jhi <= jlo) jlo = jhi = c0;
-        const int steps = __reduce_max_sync(mask, (jhi - jlo + C - 1) / C);
-        for (int it = 0, j0 = jlo; it < steps; ++it, j0 += C) {
+        int lo, hi;
+        piece_range<KT>(r, c0, n, lo, hi);
+        const int steps = __reduce_max_sync(mask, (hi - lo + C - 1) / C);
+        for (int it = 0, j0 = lo; it < steps; ++it, j0 += C) {
             float sc[C];
             f2 qf[4];
             q.get(qf);
@@ -373,12 +385,12 @@ __global__ void __launch_bounds__(TILE_THREADS, 3) k_fwd_tile(const TileFwdArgs 
             for (int i = 0; i < C; ++i) {
                 R x;
                 f2 k[4];
-                x.load_smem(sK + max(min(j0 + i, jhi - 1) - c0, 0) * U, g);      // (keys past the end: the last one, weight 0)
+                x.load_smem(sK + min(j0 + i, hi - 1) * U, g);      // (keys past the end: the last one or zeros, weight 0)
                 x.get(k);
                 sc[i] = dot8(qf, k);
             }
             const int jm = j0 + (g & (C - 1));
-            const bool ok = jm < jhi && (a.dirs == 7 || dir_ok(row, jm, r.x, a.dirs));
+            const bool ok = jm < hi && (a.dirs == 7 || dir_ok(row, c0 + jm, r.x, a.dirs));
             const float x = reduce_scatter<C, LPK>(sc, g, mask) * a.scale_log2;
             const float p = S.add<C>(ok ? x : -INFINITY, mask);
 #pragma unroll
@@ -387,7 +399,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 3) k_fwd_tile(const TileFwdArgs 
                 const f2 w2 = pack2(w, w);
                 R y;
                 f2 v[4];
-                y.load_smem(sV + max(min(j0 + i, jhi - 1) - c0, 0) * U, g);
+                y.load_smem(sV + min(j0 + i, hi - 1) * U, g);
                 y.get(v);
 #pragma unroll
                 for (int u = 0; u < 4; ++u) S.acc[u] = fma2(w2, v[u], S.acc[u]);
@@ -416,8 +428,11 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) k_bwd_tile(const TileBwdArgs 
     pdl_launch_dependents();
     extern __shared__ float4 s_tile[];
     __shared__ int s_ab[2];
-    __shared__ float s_lse[KT], s_delta[KT];
-    float4 *sK = s_tile, *sV = sK + KT * U, *sQ = sV + KT * U, *sG = sQ + KT * U;
+    __shared__ float s_lse[KT + 1], s_delta[KT + 1];
+    constexpr int PIECE = TileShape<D>::PIECE;
+    float4 *sK = s_tile, *sV = sK + PIECE, *sQ = sV + PIECE, *sG = sQ + PIECE;
+    for (int i = threadIdx.x; i < 4 * U; i += TILE_THREADS) s_tile[i / U * PIECE + KT * U + i % U] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (threadIdx.x == 0) s_lse[KT] = s_delta[KT] = 0.f;
     const int h = blockIdx.y, lane = threadIdx.x & 31, g = lane % LPK, src = lane - g;
     constexpr unsigned mask = 0xffffffffu;       // (the rows of a warp walk in step: with a mask per row their shuffles issue one after the other)
     TileRows T;
@@ -451,29 +466,29 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) k_bwd_tile(const TileBwdArgs 
             }
         }
         __syncthreads();
-        int jlo = max(r.x, c0), jhi = min(r.y, c0 + n);
-        if (jhi <= jlo) jlo = jhi = c0;
-        const int steps = __reduce_max_sync(mask, (jhi - jlo + C - 1) / C);
-        for (int it = 0, j0 = jlo; it < steps; ++it, j0 += C) {
-            const int jm = j0 + (g & (C - 1)), jc = max(min(jm, jhi - 1), c0);
-            const bool in = jm < jhi;
-            const bool ok_q = in && (a.dirs == 7 || dir_ok(row, jm, r.x, a.dirs));
-            const bool ok_k = in && (a.dirs == 7 || dir_ok_key(row, jm, r.x, a.dirs));
+        int lo, hi;
+        piece_range<KT>(r, c0, n, lo, hi);
+        const int steps = __reduce_max_sync(mask, (hi - lo + C - 1) / C);
+        for (int it = 0, j0 = lo; it < steps; ++it, j0 += C) {
+            const int jm = j0 + (g & (C - 1)), jc = min(jm, hi - 1);
+            const bool in = jm < hi;
+            const bool ok_q = in && (a.dirs == 7 || dir_ok(row, c0 + jm, r.x, a.dirs));
+            const bool ok_k = in && (a.dirs == 7 || dir_ok_key(row, c0 + jm, r.x, a.dirs));
             R x[C], y[C];
 #pragma unroll
             for (int i = 0; i < C; ++i) {
-                const int o = max(min(j0 + i, jhi - 1) - c0, 0) * U;
+                const int o = min(j0 + i, hi - 1) * U;
                 x[i].load_smem(sK + o, g);
                 y[i].load_smem(sV + o, g);
             }
             S.template as_query<C>(x, y, ok_q, a.scale_log2, g, mask, src);
 #pragma unroll
             for (int i = 0; i < C; ++i) {
-                const int o = max(min(j0 + i, jhi - 1) - c0, 0) * U;
+                const int o = min(j0 + i, hi - 1) * U;
                 x[i].load_smem(sQ + o, g);
                 y[i].load_smem(sG + o, g);
             }
-            S.template as_key<C>(x, y, ok_k, s_lse[jc - c0], s_delta[jc - c0], a.scale_log2, g, mask, src);
+            S.template as_key<C>(x, y, ok_k, s_lse[jc], s_delta[jc], a.scale_log2, g, mask, src);
         }
     }
     if (!inb) return;
@@ -490,7 +505,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) k_bwd_tile(const TileBwdArgs 
 template <int D>
 static int launch_fwd_tile_t(const TileFwdArgs &a, cudaStream_t st) {
     if (a.nb == 0) return HDT_OK;
-    constexpr int smem = 2 * TileShape<D>::KT * D * 4;
+    constexpr int smem = 2 * TileShape<D>::PIECE * 16;
     static DevOnce once;
     if (!once.done()) {
         HDT_CUDA_CHECK(cudaFuncSetAttribute(k_fwd_tile<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
@@ -503,7 +518,7 @@ static int launch_fwd_tile_t(const TileFwdArgs &a, cudaStream_t st) {
 template <int D>
 static int launch_bwd_tile_t(const TileBwdArgs &a, cudaStream_t st) {
     if (a.nb == 0) return HDT_OK;
-    constexpr int smem = 4 * TileShape<D>::KT * D * 4;
+    constexpr int smem = 4 * TileShape<D>::PIECE * 16;
     static DevOnce once;
     if (!once.done()) {
         HDT_CUDA_CHECK(cudaFuncSetAttribute(k_bwd_tile<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
