@@ -35,6 +35,9 @@
  *    must hold finite numbers: the tensor-core kernels load them with their tile and multiply them
  *    by exact zeros, and 0 x NaN or 0 x inf would reach real rows of the same tile (zero-fill them,
  *    as a padded batch normally is; nothing checks this).
+ *    A real row that is not finite reaches, in bf16 calls, the other rows of its tiles in the same way.  In
+ *    fp32 calls it reaches the rows of the families that it is in and no others (under mask_off also
+ *    those of them that do not attend to it), and PAD rows may hold anything.
  *  - `stream` is a cudaStream_t passed as void* (NULL = default stream).  hdt_attn_fwd/bwd are
  *    asynchronous on it.  hdt_build_index enqueues its kernels on it and then waits until they have
  *    read the structure arrays and sent the sizes the attention calls need.

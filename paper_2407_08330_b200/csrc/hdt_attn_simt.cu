@@ -147,7 +147,7 @@ __device__ __forceinline__ void fwd_simt_block(const FwdStageArgs &a, int bx) {
 #pragma unroll
                     for (int jj = 0; jj < 8; ++jj) {
                         const int j = j0 + jj;
-                        if (j < whi) {
+                        if (!(s[jj] == NEG)) {        // (another row's key: 0 x its V would be NaN where that is not finite)
                             const float p = exp2f(s[jj] - mn);
                             l += p;
                             const float4 *vr = sV + (j - c0) * U;

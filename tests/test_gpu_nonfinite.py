@@ -30,7 +30,7 @@ def _family(b, w):
 
 
 @pytest.mark.parametrize("d,H", [(64, 64), (128, 32)])
-@pytest.mark.parametrize("no_rows", [0])         # keys in shared memory
+@pytest.mark.parametrize("no_rows", [0, 1])      # the kernels with keys in shared memory; those that walk a whole block's span
 def test_infinite_row_stays_in_its_family(d, H, no_rows):
     import paper_2407_08330_b200 as P
     b = _batch()
