@@ -30,6 +30,7 @@
 namespace hdt {
 
 constexpr int XC = 32;      // CTAs (contiguous chunks) per document in the index kernel
+constexpr int DEC_LIST = 1024, DEC_ROWS = 8;     // decode kernel: tokens looked over at a time, rows of a document walked by one CTA
 
 struct CrossLayout {
     size_t sel, used, tokx, rngx, blocks, queue, delta, part, part_lse, total;
@@ -40,10 +41,10 @@ static size_t al256c(size_t v) { return (v + 255) & ~size_t(255); }
 
 // Decoding: few decoder rows a document on average (the host knows no more; k_cross_decode deals a document's rows beyond
 // its first DEC_ROWS to CTAs of their own).  Every row reads its document's K and V again, while the other path's 128-row tile costs the
-// same up to 128 rows.  us a forward call of 1, 4, 5 and 8 rows a document, bf16, there and (in brackets) on the tiles: 4 x 8192 tokens with
-// 12 x 64 heads 24, 52, 63, 95 (84); 8 x 2048 12, 31, 38, 56 (52); 1 x 4096 with 16 x 128 14, 32, 38, 56 (35); 64 x 2048 88, 293, 363,
-// 568 (261); 4 x 8192, anchors alone, 14, 20, 25, 34 (21).  All rows of a batch of 4 a document on one of 64 x 2048
-// 182 (98), of 256 x 512 166 (71).  (fp32 tiles cost far more: 4 x 2048 at 8 rows 53 (574); the line stays where bf16 has it.)
+// same up to 128 rows.  us a forward call of 1, 4, 5 and 8 rows a document, bf16, here and (in brackets) on the tiles: 4 x 8192 tokens with
+// 12 x 64 heads 23, 58, 68, 94 (85); 8 x 2048 15, 30, 35, 48 (54); 1 x 4096 with 16 x 128 19, 36, 45, 57 (36); 64 x 2048 72, 268, 335,
+// 528 (262); 4 x 8192, anchors alone, 9, 14, 16, 21 (21).  All rows of a batch of 4 a document on one of 64 x 2048
+// 202 (98), of 256 x 512 219 (72).  (fp32 tiles cost far more: 4 x 2048 at 8 rows 50 (722); the line stays where bf16 has it.)
 static bool cross_decode(int B, int Tq) { return (long long)Tq <= 4LL * B; }
 // Shape of a CTA of the decode kernel: heads side by side (lanes of 8 dimensions each), keys at a time.
 struct DecodeShape {
@@ -56,13 +57,53 @@ struct DecodeShape {
         per_sm = 1024 / threads;
     }
 };
-// CTAs a document's tokens are dealt to in the decode kernel: as many as the SMs hold at once over all documents, 32 tokens
-// each at least.  (A CTA begins with a chain of loads, so a second wave costs more than its shorter pieces save: 4 x 8192 tokens, 12 x 64,
-// a call with one row each 27.3 us at four CTAs an SM of which two fit, 28.5 at three, 31.7 at six, 23.5 at two.)
-static int decode_splits(int B, int T, int H, int D) {
-    const DecodeShape d(H, D);
-    const long long mean = B > 0 ? (T + B - 1) / B : 0, heads = (H + d.HC - 1) / d.HC;
-    return (int)max(1LL, min((mean + 31) / 32, (long long)PLAN_SMS * d.per_sm / (max(B, 1) * heads)));
+// How the decode kernel deals a batch's tokens: in pieces of at least P of them (32 or more).  A document of n tokens has
+// max(1, n / P), so a long one has its share whatever the others are.  P is the shortest of three of which there are no more
+// than CTAs fit on the SMs at once: the shortest of which documents of one length would have no more; the CTAs' mean share; and
+// that with a CTA kept for every document, which always fits.  A warp that sees all lengths at once (DEC_DOCS documents) chooses;
+// for more documents it is the mean share, of which every document leaves half a piece.  us a call of one row a document, bf16, 12 x 64 heads, and
+// in brackets with the same number of pieces for every document: documents of one length, 4 x 8192 23.1 (23.0), 8 x 2048 14.8
+// (14.4), 64 x 2048 72.0 (72.1); one long one, 8192 + 15 x 512 16 (46), 8192 + 63 x 256 22 (187), 4096 + 200 x 128 27 (366); 16 from
+// 200 to 16384, 47 (90).  (A CTA begins with a chain of loads, so a second wave costs more than its shorter pieces save: 4 x 8192 at four CTAs an
+// SM of which two fit 27.3, three 28.5, six 31.7, two 23.5.)
+constexpr int DEC_DOCS = 31;         // (a lane each, and the end of the last)
+struct DecodePieces {
+    int piece[3], ctas, most, rows;   // most: pieces of all documents of several, at most; rows: decoder rows of a document that leave partial results there
+    int splits;                       // pieces of a document for its rows beyond DEC_ROWS
+    DecodePieces() = default;
+    DecodePieces(int B, int T, int Tq, int H, int D) {
+        const DecodeShape d(H, D);
+        ctas = max(1, PLAN_SMS * d.per_sm / ((H + d.HC - 1) / d.HC));
+        B = max(B, 1);
+        const int mean = (int)(((long long)T + B - 1) / B);
+        auto share = [&](int n) { return max(32, (int)(((long long)T + n - 1) / n)); };
+        piece[0] = B > DEC_DOCS ? max(32, T / ctas) : max(32, mean / (max(1, ctas / B) + 1) + 1);
+        piece[1] = max(piece[0], share(ctas));
+        piece[2] = max(piece[1], share(max(1, ctas - B)));
+        most = T / piece[0];
+        rows = min(Tq, DEC_ROWS);
+        splits = max(1, (int)min((mean + 31LL) / 32, (4LL * PLAN_SMS + B - 1) / B));
+    }
+    size_t part(int Tq) const { return (size_t)most * rows + (Tq > DEC_ROWS ? (size_t)splits * Tq : 0); }      // rows of partial results in all
+};
+// x / d for 0 <= x, 0 < d, shorter than the integer division (a CTA of the decode kernel begins with three, each waiting for the one
+// before).  Both conversions and the quotient are off by 2^-21 of it at most, so below 2^20 the first guess is off by one at most.
+__device__ __forceinline__ int quotient(int x, int d) {
+    const int q = (int)__fdividef((float)x, (float)d);
+    if (q >= 1 << 20) return x / d;
+    const int r = x - q * d;
+    return q + (r >= d) - (r < 0);
+}
+__device__ __forceinline__ int doc_pieces(int tokens, int piece) { return max(1, quotient(tokens, piece)); }
+// P for at most DEC_DOCS documents, of `tokens` tokens this lane's; its document's pieces.  By a whole warp.
+__device__ __forceinline__ int choose_piece(const DecodePieces &p, int B, int tokens, int &n) {
+    const bool doc = (int)(threadIdx.x & 31) < B;
+    int n3[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) n3[i] = doc ? doc_pieces(tokens, p.piece[i]) : 0;
+    const bool fit0 = __reduce_add_sync(0xffffffffu, n3[0]) <= p.ctas, fit1 = __reduce_add_sync(0xffffffffu, n3[1]) <= p.ctas;
+    n = fit0 ? n3[0] : fit1 ? n3[1] : n3[2];
+    return fit0 ? p.piece[0] : fit1 ? p.piece[1] : p.piece[2];
 }
 // CTAs a row block's keys are dealt to in the tile kernels: enough to fill the SMs (`per_sm` CTAs each), pieces of
 // four chunks at least.  level_mask < 0: every level (for the workspace size).  The host does not know how many tokens a level has:
@@ -93,10 +134,10 @@ static CrossLayout cross_layout(int B, int T, int Tq, int H, int D, bool tc, int
     L.sel = o; o += al256c(sizeof(int) * (size_t)(B + 1));
     L.used = o; o += 256;
     L.delta = o; if (bwd) o += al256c(sizeof(float) * (size_t)H * max(Tq, 1));
-    // partial results [splits, Tq, H, D] and, in the forward, their LSE
-    const size_t splits = !bwd && cross_decode(B, Tq) ? decode_splits(B, T, H, D) : tile_splits(B, T, Tq, H, -1, bwd ? 8 : 2);
-    L.part = o; o += al256c(sizeof(float) * splits * Tq * H * D);
-    L.part_lse = o; if (!bwd) o += al256c(sizeof(float) * splits * Tq * H);
+    // partial results: rows of [H, D] and, in the forward, their LSE
+    const size_t rows = !bwd && cross_decode(B, Tq) ? DecodePieces(B, T, Tq, H, D).part(Tq) : (size_t)tile_splits(B, T, Tq, H, -1, bwd ? 8 : 2) * Tq;
+    L.part = o; o += al256c(sizeof(float) * rows * H * D);
+    L.part_lse = o; if (!bwd) o += al256c(sizeof(float) * rows * H);
     L.total = o + 256;
     return L;
 }
@@ -280,9 +321,9 @@ __global__ void __launch_bounds__(128) k_cross_zero(const int8_t *__restrict__ l
 }
 
 // ---- decoding ------------------------------------------------------------------------------------
-// CTA (group * splits + y, z): the y-th share of a document's tokens, heads z * HC ...  Group b < batch: the first DEC_ROWS decoder
-// rows of document b, in turn.  The groups behind take the rows beyond those, DEC_ROWS of all rows each, so that a
-// document that has most rows of the batch does not walk them on one CTA.  (All along x, where a grid has no limit that
+// CTA (x, y): a piece of a document's tokens (see DecodePieces) for its first DEC_ROWS decoder rows in turn, heads y * HC ...  The CTAs
+// behind those of the pieces take the rows beyond, DEC_ROWS of all rows and an even share of their document's
+// tokens each.  (All along x, where a grid has no limit that
 // matters; a document's CTAs follow one another, since some that lie a multiple of eight apart share a part of the
 // chip: 8 rows on one of 8 documents of 2048 tokens 28 us, so 19.)
 // Thread (slot, head, lane): D / 8 lanes per (key, head), the heads of a token next to one another, so that a
@@ -292,16 +333,37 @@ __global__ void __launch_bounds__(128) k_cross_zero(const int8_t *__restrict__ l
 struct DecodeArgs {
     const int8_t *level;
     const int32_t *cu_k, *cu_q;
-    int B, level_mask, H, HC, KS, Tq, splits;
+    int B, T, level_mask, H, HC, KS, Tq, pieces;      // pieces: CTAs of the documents' first DEC_ROWS rows
+    DecodePieces p;
     const void *q, *k, *v;
     float scale_log2;
     void *o;
-    float *lse, *part_o, *part_lse;       // splits > 1: [splits, Tq, H, D], [splits, Tq, H]
+    float *lse, *part_o, *part_lse;       // rows of partial results: [rows, most], then [splits, Tq]
 };
-static constexpr int DEC_LIST = 1024, DEC_ROWS = 8;
+// The last i of [0, n) with le(i); le holds for 0 and for no i behind one for which it does not.  By a whole warp.
+template <class F>
+__device__ __forceinline__ int warp_last(int n, F le) {
+    const int lane = threadIdx.x & 31;
+    int lo = 0;
+    while (n > 1) {
+        const int step = (n + 31) / 32, i = lane * step;
+        const int k = max(0, __popc(__ballot_sync(0xffffffffu, i < n && le(lo + i))) - 1) * step;
+        lo += k;
+        n = min(step, n - k);
+    }
+    return lo;
+}
 
 template <int D, bool BF16>
 __global__ void __launch_bounds__(512, 2) k_cross_decode(const DecodeArgs a) {
+    // What the CTA's first loads, one chain, will most likely need: into L2 while the kernel in front ends (a hint reads nothing;
+    // 4 x 8192 tokens 23.6 -> 23.2 us).
+    if (threadIdx.x < 4) {
+        const long long guess = min((long long)a.T - 1, (long long)blockIdx.x * a.T / a.pieces);       // (documents of one length)
+        const void *p = threadIdx.x == 0 ? (const void *)a.cu_k : threadIdx.x == 1 ? (const void *)a.cu_q
+                        : (const void *)(a.level + (threadIdx.x == 2 ? guess : min(a.T - 1LL, guess + 127)));
+        if (a.T > 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+    }
     pdl_wait();
     pdl_launch_dependents();
     constexpr int LPK = D / 8, C = 4;
@@ -309,174 +371,231 @@ __global__ void __launch_bounds__(512, 2) k_cross_decode(const DecodeArgs a) {
     extern __shared__ float s_red[];                 // [KS][HC][D + 2]
     __shared__ int s_list[DEC_LIST];
     __shared__ int s_n;
+    __shared__ int s_job[4];                         // tokens [0] .. [1], rows [2] .. [3]
+    __shared__ unsigned s_part[2];                   // row r leaves its partial result at [0] + r * [1]; [1] == 0: its result, since these are all the tokens
     const int t = threadIdx.x, lane = t & 31, g = t % LPK, src = lane - g;
     const unsigned mask = ((1u << LPK) - 1u) << src;
     const int pair = t / LPK, hl = pair % a.HC, ks = pair / a.HC, h = blockIdx.y * a.HC + hl;
     const bool on = ks < a.KS && h < a.H;
-    const int group = blockIdx.x / a.splits, split = blockIdx.x % a.splits;
-    // Rows [row0, row1) of document b.
-    auto walk = [&](int b, int row0, int row1) {
-        const int k0 = a.cu_k[b], k1 = a.cu_k[b + 1];
-        const int per = (k1 - k0 + a.splits - 1) / a.splits, c0 = min(k1, k0 + split * per), c1 = min(k1, c0 + per);
-        for (int row = row0; row < row1; ++row) {
-            RowSoftmax S;
-            S.clear();
-            W q;
-            if (on) q.load(a.q, (unsigned)row * a.H + h, g);
-            for (int p0 = c0; p0 < c1; p0 += DEC_LIST) {
-                const int p1 = min(c1, p0 + DEC_LIST);
-                if (row == row0 || c1 - c0 > DEC_LIST) {         // the chosen tokens of this piece, in order
-                    __syncthreads();
-                    if (t < 32) {
-                        int n = 0;
-                        for (int i0 = p0; i0 < p1; i0 += 128) {      // (four loads in flight: nothing of K and V is requested before the list is there)
-                            bool f[4];
+    auto list = [&](int p0, int p1) {                // by warp 0: the chosen tokens of [p0, p1), in order
+        int n = 0;
+        for (int i0 = p0; i0 < p1; i0 += 128) {      // (four loads in flight: nothing of K and V is requested before the list is there)
+            bool f[4];
 #pragma unroll
-                            for (int k = 0; k < 4; ++k) f[k] = i0 + 32 * k + lane < p1 && chosen(a.level, i0 + 32 * k + lane, a.level_mask);
+            for (int k = 0; k < 4; ++k) f[k] = i0 + 32 * k + lane < p1 && chosen(a.level, i0 + 32 * k + lane, a.level_mask);
 #pragma unroll
-                            for (int k = 0; k < 4; ++k) {
-                                const unsigned m = __ballot_sync(0xffffffffu, f[k]);
-                                if (f[k]) s_list[n + __popc(m & ((1u << lane) - 1u))] = i0 + 32 * k + lane;
-                                n += __popc(m);
-                            }
-                        }
-                        if (lane == 0) s_n = n;
-                    }
-                    __syncthreads();
-                }
-                const int n = s_n;
-                if (!on) continue;
-                for (int i0 = ks * C; i0 < n; i0 += a.KS * C) {
-                    W x[C], y[C];
-#pragma unroll
-                    for (int c = 0; c < C; ++c) {
-                        const unsigned r = (unsigned)s_list[min(i0 + c, n - 1)] * a.H + h;      // (past the end: the last key, weight 0)
-                        x[c].load(a.k, r, g);
-                        y[c].load(a.v, r, g);
-                    }
-                    float sc[C];
-                    dots<C>(q, x, sc);
-                    const float s = reduce_scatter<C, LPK>(sc, g, mask) * a.scale_log2;
-                    const float p = S.add<C>(i0 + (g & (C - 1)) < n ? s : -INFINITY, mask);
-                    axpys<C>(S.acc, p, y, mask, src);
-                }
+            for (int k = 0; k < 4; ++k) {
+                const unsigned m = __ballot_sync(0xffffffffu, f[k]);
+                if (f[k]) s_list[n + __popc(m & ((1u << lane) - 1u))] = i0 + 32 * k + lane;
+                n += __popc(m);
             }
-            // the slots of a head: one after the other through shared memory
-            if (on) {
-#pragma unroll
-                for (int o = 1; o < C; o *= 2) S.l += __shfl_xor_sync(mask, S.l, o);
-                float *d = s_red + (size_t)(ks * a.HC + hl) * (D + 2);
-                const float lse = S.finish();
-#pragma unroll
-                for (int u = 0; u < 4; ++u) unpack2(S.acc[u], d[8 * g + 2 * u], d[8 * g + 2 * u + 1]);
-                if (g == 0) d[D] = lse;
-            }
-            __syncthreads();
-            if (on && ks == 0) {
-                RowSoftmax R;
-                R.clear();
-                for (int i = 0; i < a.KS; ++i) {
-                    const float *d = s_red + (size_t)(i * a.HC + hl) * (D + 2);
-                    f2 x[4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) x[u] = pack2(d[8 * g + 2 * u], d[8 * g + 2 * u + 1]);
-                    R.merge(d[D] * 1.4426950408889634f, d[D] > -INFINITY ? 1.f : 0.f, x);
-                }
-                const float lse = R.finish();
-                if (a.splits == 1) {
-                    W::store(a.o, (unsigned)row * a.H + h, g, R.acc);
-                    if (g == 0) a.lse[(size_t)h * a.Tq + row] = lse;
-                } else {
-                    const size_t r = ((size_t)split * a.Tq + row) * a.H + h;
-                    W::store_f32(a.part_o, r, g, R.acc);
-                    if (g == 0) a.part_lse[r] = lse;
-                }
-            }
-            __syncthreads();
         }
+        if (lane == 0) s_n = n;
     };
-    if (group < a.B) {
-        const int q0 = a.cu_q[group], q1 = a.cu_q[group + 1];
-        walk(group, q0, min(q1, q0 + DEC_ROWS));
-        return;
-    }
-    auto document_of = [&](int row) {                // the last one that starts at or before the row
-        int lo = 0, hi = a.B;
-        while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (a.cu_q[mid] <= row) lo = mid; else hi = mid; }
-        return lo;
-    };
-    const int first = DEC_ROWS * (group - a.B), end = min(a.Tq, first + DEC_ROWS);
-    if (!__syncthreads_or(t < end - first && first + t >= a.cu_q[document_of(first + t)] + DEC_ROWS)) return;
-    for (int row = first; row < end;) {
-        const int b = document_of(row), q1 = a.cu_q[b + 1];
-        walk(b, max(row, a.cu_q[b] + DEC_ROWS), min(end, q1));
-        row = q1 > row ? q1 : end;
-    }
-}
-
-// Merge of partial results over `splits`, a CTA per (row, head).  Forward (lse given): log-sum-exp merge of
-// normalised rows; backward: sum.  Groups of D / 8 lanes take every G-th partial result, then meet: inside a warp by
-// shuffles, the four warps through shared memory (all groups one after the other there: 0.7 us more).
-template <int D, bool BF16>
-__global__ void __launch_bounds__(128) k_cross_combine(int splits, int Tq, int H, const float *part, const float *part_lse, void *out, float *lse) {
-    pdl_wait();
-    pdl_launch_dependents();
-    constexpr int LPK = D / 8, G = 128 / LPK;
-    using W = Raw<BF16, LPK>;
-    __shared__ float s_red[4][D + 2];
-    const int row = blockIdx.x, h = blockIdx.y, g = threadIdx.x % LPK, i = threadIdx.x / LPK, w = threadIdx.x >> 5;
-    RowSoftmax R;
-    R.clear();
-    auto add = [&](float m, float l, const f2 (&x)[4]) {
-        if (part_lse != nullptr) R.merge(m, l, x);
-        else
+    if (t < 32) {                                    // what to do, by one warp: the others' registers are the keys'
+        const int x = blockIdx.x;
+        int b = 0, j, n, k0, k1, row0 = 0, row1 = 0;
+        unsigned part = 0, step = 0;
+        if (x < a.pieces) {
+            int q0, q1, piece = a.p.piece[0];
+            if (a.B <= DEC_DOCS) {                          // one round of loads, the documents' pieces one behind the other
+                const int i = min(lane, a.B - 1);
+                k0 = a.cu_k[i]; k1 = a.cu_k[i + 1]; q0 = a.cu_q[i]; q1 = a.cu_q[i + 1];
+                piece = choose_piece(a.p, a.B, k1 - k0, n);
+                int end = n;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) R.acc[u] = add2(R.acc[u], x[u]);
-    };
-#pragma unroll 4
-    for (int s = i; s < splits; s += G) {
-        const size_t r = ((size_t)s * Tq + row) * H + h;
-        f2 x[4];
-        W::load_f32(part, r, g, x);
-        const float L = part_lse != nullptr ? part_lse[r] : 0.f;
-        add(L * 1.4426950408889634f, L > -INFINITY ? 1.f : 0.f, x);
-    }
-#pragma unroll
-    for (int o = LPK; o < 32; o *= 2) {
-        f2 x[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) x[u] = __shfl_xor_sync(0xffffffffu, R.acc[u], o);
-        const float m = __shfl_xor_sync(0xffffffffu, R.m, o), l = __shfl_xor_sync(0xffffffffu, R.l, o);
-        add(m, l, x);
-    }
-    if ((threadIdx.x & 31) < LPK) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) unpack2(R.acc[u], s_red[w][8 * g + 2 * u], s_red[w][8 * g + 2 * u + 1]);
-        if (g == 0) { s_red[w][D] = R.m; s_red[w][D + 1] = R.l; }
+                for (int o = 1; o < 32; o *= 2)
+                    if (o < a.B) { const int v = __shfl_up_sync(0xffffffffu, end, o); if (lane >= o) end += v; }
+                b = min(a.B - 1, __popc(__ballot_sync(0xffffffffu, lane < a.B && end <= x)));
+                j = x - __shfl_sync(0xffffffffu, end - n, b);
+                n = __shfl_sync(0xffffffffu, n, b);
+                k0 = __shfl_sync(0xffffffffu, k0, b); k1 = __shfl_sync(0xffffffffu, k1, b);
+                q0 = __shfl_sync(0xffffffffu, q0, b); q1 = __shfl_sync(0xffffffffu, q1, b);
+            } else {                                 // document b's from number cu[b] / piece + b on: some numbers are no piece's
+                b = warp_last(a.B, [&](int i) { return quotient(a.cu_k[i], piece) + i <= x; });
+                k0 = a.cu_k[b]; k1 = a.cu_k[b + 1]; q0 = a.cu_q[b]; q1 = a.cu_q[b + 1];
+                n = doc_pieces(k1 - k0, piece);
+                j = x - (quotient(k0, piece) + b);
+            }
+            row0 = q0;
+            row1 = j >= 0 && j < n ? min(q1, q0 + DEC_ROWS) : q0;
+            if (n > 1) { step = a.p.most; part = quotient(k0, piece) + j - q0 * step; }
+        } else {                                     // rows behind a document's first: DEC_ROWS of all rows hold those of one document at most
+            const int group = (x - a.pieces) / a.p.splits, row = DEC_ROWS * group + lane;
+            j = (x - a.pieces) % a.p.splits;
+            n = a.p.splits;
+            int hi = a.B;                            // its document: the last one that starts at or before the row
+            while (hi - b > 1) { const int mid = (b + hi) >> 1; if (a.cu_q[mid] <= row) b = mid; else hi = mid; }
+            const unsigned m = __ballot_sync(0xffffffffu, lane < DEC_ROWS && row >= a.cu_q[b] + DEC_ROWS && row < min(a.Tq, a.cu_q[b + 1]));
+            const int f = m ? __ffs(m) - 1 : 0;
+            b = __shfl_sync(0xffffffffu, b, f);
+            row0 = DEC_ROWS * group + f;
+            row1 = row0 + __popc(m);
+            k0 = a.cu_k[b]; k1 = a.cu_k[b + 1];
+            if (n > 1) { step = 1; part = a.p.most * a.p.rows + j * a.Tq; }
+        }
+        const int per = quotient(k1 - k0 + n - 1, n), c0 = min(k1, k0 + j * per), c1 = min(k1, c0 + per);
+        if (lane == 0) { s_job[0] = c0; s_job[1] = c1; s_job[2] = row0; s_job[3] = row1; s_part[0] = part; s_part[1] = step; }
+        if (row1 > row0) list(c0, min(c1, c0 + DEC_LIST));
     }
     __syncthreads();
-    if (i != 0) return;
+    const int c0 = s_job[0], c1 = s_job[1], row0 = s_job[2], row1 = s_job[3];
+    for (int row = row0; row < row1; ++row) {
+        RowSoftmax S;
+        S.clear();
+        W q;
+        if (on) q.load(a.q, (unsigned)row * a.H + h, g);
+        for (int p0 = c0; p0 < c1; p0 += DEC_LIST) {
+            if (c1 - c0 > DEC_LIST && (p0 != c0 || row != row0)) {
+                __syncthreads();
+                if (t < 32) list(p0, min(c1, p0 + DEC_LIST));
+                __syncthreads();
+            }
+            const int n = s_n;
+            if (!on) continue;
+            for (int i0 = ks * C; i0 < n; i0 += a.KS * C) {
+                W x[C], y[C];
 #pragma unroll
-    for (int j = 1; j < 4; ++j) {
-        f2 x[4];
+                for (int c = 0; c < C; ++c) {
+                    const unsigned r = (unsigned)s_list[min(i0 + c, n - 1)] * a.H + h;      // (past the end: the last key, weight 0)
+                    x[c].load(a.k, r, g);
+                    y[c].load(a.v, r, g);
+                }
+                float sc[C];
+                dots<C>(q, x, sc);
+                const float s = reduce_scatter<C, LPK>(sc, g, mask) * a.scale_log2;
+                const float p = S.add<C>(i0 + (g & (C - 1)) < n ? s : -INFINITY, mask);
+                axpys<C>(S.acc, p, y, mask, src);
+            }
+        }
+        // the slots of a head: one after the other through shared memory
+        if (on) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) x[u] = pack2(s_red[j][8 * g + 2 * u], s_red[j][8 * g + 2 * u + 1]);
-        add(s_red[j][D], s_red[j][D + 1], x);
+            for (int o = 1; o < C; o *= 2) S.l += __shfl_xor_sync(mask, S.l, o);
+            float *d = s_red + (size_t)(ks * a.HC + hl) * (D + 2);
+            const float lse = S.finish();
+#pragma unroll
+            for (int u = 0; u < 4; ++u) unpack2(S.acc[u], d[8 * g + 2 * u], d[8 * g + 2 * u + 1]);
+            if (g == 0) d[D] = lse;
+        }
+        __syncthreads();
+        if (on && ks == 0) {
+            RowSoftmax R;
+            R.clear();
+            for (int i = 0; i < a.KS; ++i) {
+                const float *d = s_red + (size_t)(i * a.HC + hl) * (D + 2);
+                f2 x[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) x[u] = pack2(d[8 * g + 2 * u], d[8 * g + 2 * u + 1]);
+                R.merge(d[D] * 1.4426950408889634f, d[D] > -INFINITY ? 1.f : 0.f, x);
+            }
+            const float lse = R.finish();
+            if (s_part[1] == 0) {
+                W::store(a.o, (unsigned)row * a.H + h, g, R.acc);
+                if (g == 0) a.lse[(size_t)h * a.Tq + row] = lse;
+            } else {
+                const size_t r = (size_t)(s_part[0] + row * s_part[1]) * a.H + h;
+                W::store_f32(a.part_o, r, g, R.acc);
+                if (g == 0) a.part_lse[r] = lse;
+            }
+        }
+        __syncthreads();
     }
-    if (part_lse != nullptr) {
-        const float L = R.finish();
-        if (g == 0) lse[(size_t)h * Tq + row] = L;
-    }
-    W::store(out, (unsigned)row * H + h, g, R.acc);
 }
 
-static int launch_combine(int splits, int Tq, int H, int D, int dtype, const float *part, const float *part_lse, void *out, float *lse, cudaStream_t st) {
-    const dim3 grid(Tq, H);
+// Where the partial results of decoder rows are, if not at [splits, Tq]: cu_k == nullptr says that they are.
+struct DecodeParts {
+    const int32_t *cu_k, *cu_q;
+    int B;
+    DecodePieces p;
+};
+// Merge of partial results over `splits`, a CTA per (row, head) or for some heads of a row.  Forward (lse given): log-sum-exp merge of
+// normalised rows; backward: sum.  Groups of D / 8 lanes take every G-th partial result, then meet: inside a warp by
+// shuffles, the warps through shared memory (all groups one after the other there: 0.7 us more).  Bound by the round trips to
+// L2: 256 threads where a row may have many partial results (decoding, 4 x 8192 tokens: 23.5 us a call with 128, 22.9 with 256).
+template <int D, bool BF16>
+__global__ void __launch_bounds__(256) k_cross_combine(int splits, int Tq, int H, const float *part, const float *part_lse, void *out, float *lse, const DecodeParts dp) {
+    constexpr int LPK = D / 8;
+    const int G = blockDim.x / LPK;
+    using W = Raw<BF16, LPK>;
+    __shared__ float s_red[8][D + 2];
+    const int row = blockIdx.x, g = threadIdx.x % LPK, i = threadIdx.x / LPK, w = threadIdx.x >> 5;
+    size_t first = row, step = Tq;
+    if (dp.cu_k != nullptr) {         // (before the wait: the kernel in front writes neither array, and began behind what did)
+        const int b = warp_last(dp.B, [&](int x) { return dp.cu_q[x] <= row; }), r = row - dp.cu_q[b], k0 = dp.cu_k[b];
+        if (r < 0) splits = 1;                       // (no document's row)
+        else if (r < DEC_ROWS) {
+            int piece = dp.p.piece[0];
+            if (dp.B <= DEC_DOCS) {
+                const int x = min((int)(threadIdx.x & 31), dp.B - 1);
+                piece = choose_piece(dp.p, dp.B, dp.cu_k[x + 1] - dp.cu_k[x], splits);
+            }
+            splits = doc_pieces(dp.cu_k[b + 1] - k0, piece);
+            first = (size_t)r * dp.p.most + quotient(k0, piece);
+            step = 1;
+        } else first += (size_t)dp.p.most * dp.p.rows;
+    }
+    pdl_wait();
+    pdl_launch_dependents();
+    if (dp.cu_k != nullptr && splits == 1) return;      // written by the one CTA that walked the row
+    for (int h = blockIdx.y; h < H; h += gridDim.y) {
+        if (h != (int)blockIdx.y) __syncthreads();
+        RowSoftmax R;
+        R.clear();
+        auto add = [&](float m, float l, const f2 (&x)[4]) {
+            if (part_lse != nullptr) R.merge(m, l, x);
+            else
+#pragma unroll
+                for (int u = 0; u < 4; ++u) R.acc[u] = add2(R.acc[u], x[u]);
+        };
+#pragma unroll 4
+        for (int s = i; s < splits; s += G) {
+            const size_t r = (first + s * step) * H + h;
+            f2 x[4];
+            W::load_f32(part, r, g, x);
+            const float L = part_lse != nullptr ? part_lse[r] : 0.f;
+            add(L * 1.4426950408889634f, L > -INFINITY ? 1.f : 0.f, x);
+        }
+#pragma unroll
+        for (int o = LPK; o < 32; o *= 2) {
+            f2 x[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) x[u] = __shfl_xor_sync(0xffffffffu, R.acc[u], o);
+            const float m = __shfl_xor_sync(0xffffffffu, R.m, o), l = __shfl_xor_sync(0xffffffffu, R.l, o);
+            add(m, l, x);
+        }
+        if ((threadIdx.x & 31) < LPK) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) unpack2(R.acc[u], s_red[w][8 * g + 2 * u], s_red[w][8 * g + 2 * u + 1]);
+            if (g == 0) { s_red[w][D] = R.m; s_red[w][D + 1] = R.l; }
+        }
+        __syncthreads();
+        if (i != 0) continue;
+        for (int j = 1; j < (int)blockDim.x / 32; ++j) {
+            f2 x[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) x[u] = pack2(s_red[j][8 * g + 2 * u], s_red[j][8 * g + 2 * u + 1]);
+            add(s_red[j][D], s_red[j][D + 1], x);
+        }
+        if (part_lse != nullptr) {
+            const float L = R.finish();
+            if (g == 0) lse[(size_t)h * Tq + row] = L;
+        }
+        W::store(out, (unsigned)row * H + h, g, R.acc);
+    }
+}
+
+static int launch_combine(int splits, int Tq, int H, int D, int dtype, const float *part, const float *part_lse, void *out, float *lse, cudaStream_t st,
+                          const DecodeParts &dp = DecodeParts{}) {
+    // (decoding: rows of documents of one piece have nothing to merge, so where there are many, few CTAs a row)
+    const bool decode = dp.cu_k != nullptr;
+    const dim3 grid(Tq, decode ? max(1, min(H, 8 * PLAN_SMS / Tq)) : H);
+    const int threads = decode ? 256 : 128;
     cudaError_t e;
-    if (D == 64) e = dtype == HDT_BF16 ? launch_dependent(k_cross_combine<64, true>, true, grid, 128, 0, st, splits, Tq, H, part, part_lse, out, lse)
-                                       : launch_dependent(k_cross_combine<64, false>, true, grid, 128, 0, st, splits, Tq, H, part, part_lse, out, lse);
-    else e = dtype == HDT_BF16 ? launch_dependent(k_cross_combine<128, true>, true, grid, 128, 0, st, splits, Tq, H, part, part_lse, out, lse)
-                               : launch_dependent(k_cross_combine<128, false>, true, grid, 128, 0, st, splits, Tq, H, part, part_lse, out, lse);
+    if (D == 64) e = dtype == HDT_BF16 ? launch_dependent(k_cross_combine<64, true>, true, grid, threads, 0, st, splits, Tq, H, part, part_lse, out, lse, dp)
+                                       : launch_dependent(k_cross_combine<64, false>, true, grid, threads, 0, st, splits, Tq, H, part, part_lse, out, lse, dp);
+    else e = dtype == HDT_BF16 ? launch_dependent(k_cross_combine<128, true>, true, grid, threads, 0, st, splits, Tq, H, part, part_lse, out, lse, dp)
+                               : launch_dependent(k_cross_combine<128, false>, true, grid, threads, 0, st, splits, Tq, H, part, part_lse, out, lse, dp);
     if (e != cudaSuccess) return set_error(HDT_ERR_CUDA, "launch of the combining kernel failed: %s", cudaGetErrorString(e));
     return HDT_OK;
 }
@@ -488,9 +607,11 @@ static int launch_decode_t(DecodeArgs a, int B, cudaStream_t st) {
     a.KS = d.KS;
     a.B = B;
     const int threads = d.threads;
-    const unsigned groups = B + (a.Tq > DEC_ROWS ? (a.Tq + DEC_ROWS - 1) / DEC_ROWS : 0);
+    // (At most DEC_DOCS documents have no more pieces than CTAs fit, or one each.)
+    a.pieces = B <= DEC_DOCS ? min(a.p.most + B, max(a.p.ctas, B)) : a.p.most + B;
+    const unsigned grid = a.pieces + (a.Tq > DEC_ROWS ? (unsigned)((a.Tq + DEC_ROWS - 1) / DEC_ROWS) * a.p.splits : 0u);
     const size_t smem = sizeof(float) * (size_t)a.KS * a.HC * (D + 2);
-    HDT_CUDA_CHECK(launch_dependent(k_cross_decode<D, BF16>, true, dim3(groups * a.splits, (a.H + a.HC - 1) / a.HC), threads, smem, st, a));
+    HDT_CUDA_CHECK(launch_dependent(k_cross_decode<D, BF16>, true, dim3(grid, (a.H + a.HC - 1) / a.HC), threads, smem, st, a));
     return HDT_OK;
 }
 
@@ -565,13 +686,16 @@ extern "C" int hdt_cross_attn_fwd(const int8_t *level, const int32_t *cu_seqlens
     if (cross_decode(batch, total_q) && !g_force_simt) {
         DecodeArgs a{};
         a.level = level; a.cu_k = cu_seqlens_k; a.cu_q = cu_seqlens_q; a.level_mask = level_mask; a.H = heads; a.Tq = total_q;
-        a.splits = decode_splits(batch, total_tokens, heads, head_dim);
+        const DecodePieces p(batch, total_tokens, total_q, heads, head_dim);
+        a.p = p;
+        a.T = total_tokens;
         a.q = q; a.k = k; a.v = v; a.scale_log2 = scale * 1.4426950408889634f;
         a.o = o; a.lse = lse; a.part_o = part; a.part_lse = part_lse;
         if (head_dim == 64) rc = dtype == HDT_BF16 ? launch_decode_t<64, true>(a, batch, st) : launch_decode_t<64, false>(a, batch, st);
         else rc = dtype == HDT_BF16 ? launch_decode_t<128, true>(a, batch, st) : launch_decode_t<128, false>(a, batch, st);
-        if (rc || a.splits == 1) return rc;
-        return launch_combine(a.splits, total_q, heads, head_dim, dtype, part, part_lse, o, lse, st);
+        if (rc || (p.most < 2 && (p.splits == 1 || total_q <= DEC_ROWS))) return rc;      // no document of several pieces
+        return launch_combine(p.splits, total_q, heads, head_dim, dtype, part, part_lse, o, lse, st,
+                              DecodeParts{cu_seqlens_k, cu_seqlens_q, batch, p});
     }
     rc = cross_build(L, ws, level, cu_seqlens_k, cu_seqlens_q, batch, total_tokens, total_q, level_mask, st);
     if (rc) return rc;
