@@ -23,9 +23,9 @@ extern "C" {
  *                    in a library built with HDT_WORKBENCH defined; otherwise as 0);
  *                    3: the forward kernel with one CTA per (block, head); 4: the self-contained
  *                    blocks of a head_dim 64 backward stay on the persistent 512-thread kernel
- *                    instead of the looping one; 5: the lock-step looping backward kernel
- *                    at head_dim 64; 6: one CTA per SM for the
- *                    transposed looping backward.
+ *                    instead of the looping one; 5: the general backward kernels, the
+ *                    forward's stage 0 on the default ones; 6: one CTA per SM for the transposed
+ *                    looping backward.
  *   "no_fwd_mc"      1: the blocks of a head_dim 64 forward that are not self-contained stay on the
  *                    128-thread general kernel instead of the 256-thread multi-chunk one (and with
  *                    it the EMPTY blocks of padded batches, which otherwise have a kernel of their
