@@ -42,9 +42,9 @@ static size_t al256c(size_t v) { return (v + 255) & ~size_t(255); }
 // Decoding: few decoder rows a document on average (the host knows no more; k_cross_decode deals a document's rows beyond
 // its first DEC_ROWS to CTAs of their own).  Every row reads its document's K and V again, while the other path's 128-row tile costs the
 // same up to 128 rows.  us a forward call of 1, 4, 5 and 8 rows a document, bf16, here and (in brackets) on the tiles: 4 x 8192 tokens with
-// 12 x 64 heads 23, 58, 68, 94 (85); 8 x 2048 15, 30, 35, 48 (54); 1 x 4096 with 16 x 128 19, 36, 45, 57 (36); 64 x 2048 72, 268, 335,
-// 528 (262); 4 x 8192, anchors alone, 9, 14, 16, 21 (21).  All rows of a batch of 4 a document on one of 64 x 2048
-// 202 (98), of 256 x 512 219 (72).  (fp32 tiles cost far more: 4 x 2048 at 8 rows 50 (722); the line stays where bf16 has it.)
+// 12 x 64 heads 19, 50, 58, 94 (85); 8 x 2048 14, 27, 31, 49 (53); 1 x 4096 with 16 x 128 14, 36, 43, 64 (35); 64 x 2048 75, 264, 326,
+// 512 (262); 4 x 8192, anchors alone, 10, 15, 17, 23 (36).  All rows of a batch of 4 a document on one of 64 x 2048
+// 186 (99), of 256 x 512 163 (72).  (fp32 tiles cost far more: 4 x 2048 at 8 rows 50 (722); the line stays where bf16 has it.)
 static bool cross_decode(int B, int Tq) { return (long long)Tq <= 4LL * B; }
 // Shape of a CTA of the decode kernel: heads side by side (lanes of 8 dimensions each), keys at a time.
 struct DecodeShape {
@@ -57,37 +57,43 @@ struct DecodeShape {
         per_sm = 1024 / threads;
     }
 };
-// How the decode kernel deals a batch's tokens: in pieces of at least P of them (32 or more).  A document of n tokens has
-// max(1, n / P), so a long one has its share whatever the others are.  P is the shortest of three of which there are no more
-// than CTAs fit on the SMs at once: the shortest of which documents of one length would have no more; the CTAs' mean share; and
-// that with a CTA kept for every document, which always fits.  A warp that sees all lengths at once (DEC_DOCS documents) chooses;
-// for more documents it is the mean share, of which every document leaves half a piece.  us a call of one row a document, bf16, 12 x 64 heads, and
-// in brackets with the same number of pieces for every document: documents of one length, 4 x 8192 23.1 (23.0), 8 x 2048 14.8
-// (14.4), 64 x 2048 72.0 (72.1); one long one, 8192 + 15 x 512 16 (46), 8192 + 63 x 256 22 (187), 4096 + 200 x 128 27 (366); 16 from
-// 200 to 16384, 47 (90).  (A CTA begins with a chain of loads, so a second wave costs more than its shorter pieces save: 4 x 8192 at four CTAs an
-// SM of which two fit 27.3, three 28.5, six 31.7, two 23.5.)
+// How the decode kernel deals a batch's tokens: in pieces of P of them, so that a long document has its share of the CTAs
+// whatever the others are.  Up to DEC_DOCS documents, whose lengths a warp sees at once: ceil(n / P) for a document of n tokens, P the
+// shortest of three (32 at least) of which there are no more than CTAs fit on the SMs at once: the shortest of which documents of one
+// length have no more; the CTAs' mean share, half a CTA a document kept back; and with one a document kept back, which always fits.
+// More documents: max(1, n / P) of even length, P the mean share, of which every document leaves half a piece.
+// us a call of one row a document, bf16, 12 x 64 heads, and in brackets with the same number of pieces for every document: documents of
+// one length, 4 x 8192 18.8 (18.4), 8 x 2048 13.5 (13.5), 64 x 2048 73.6 (72.2), 256 x 512 73.8 (71.0), with 16 x 128 8 x 1500 21.8 (21.3);
+// one long one, 8192 + 15 x 512 13.6 (25.3), 8192 + 63 x 256 18 (106), 4096 + 200 x 128 21 (282); 16 from 200 to 16384 72 (104).  (A CTA
+// begins with a chain of loads, so a second wave costs more than its shorter pieces save: 4 x 8192 at four CTAs an SM of which two fit 27.3, three
+// 28.5, six 31.7, two 23.5, timed one behind the other with the form before.)
 constexpr int DEC_DOCS = 31;         // (a lane each, and the end of the last)
 struct DecodePieces {
-    int piece[3], ctas, most, rows;   // most: pieces of all documents of several, at most; rows: decoder rows of a document that leave partial results there
-    int splits;                       // pieces of a document for its rows beyond DEC_ROWS
+    int piece[3], ctas, pieces, most, rows;   // pieces: CTAs for them; most: those of documents of several, at most; rows: decoder rows of a document that leave partial results there
+    float inv[3];                    // 1 / piece
+    int splits;                      // pieces of a document of more than DEC_ROWS decoder rows
+    bool several;                    // whether a document may have several
     DecodePieces() = default;
     DecodePieces(int B, int T, int Tq, int H, int D) {
         const DecodeShape d(H, D);
         ctas = max(1, PLAN_SMS * d.per_sm / ((H + d.HC - 1) / d.HC));
         B = max(B, 1);
-        const int mean = (int)(((long long)T + B - 1) / B);
-        auto share = [&](int n) { return max(32, (int)(((long long)T + n - 1) / n)); };
-        piece[0] = B > DEC_DOCS ? max(32, T / ctas) : max(32, mean / (max(1, ctas / B) + 1) + 1);
-        piece[1] = max(piece[0], share(ctas));
-        piece[2] = max(piece[1], share(max(1, ctas - B)));
-        most = T / piece[0];
+        const int mean = (int)(((long long)T + B - 1) / B), n = max(1, ctas / B);
+        auto share = [&](int c) { return (int)(((long long)T + max(1, c) - 1) / max(1, c)); };
+        piece[0] = max(32, B > DEC_DOCS ? T / ctas : (mean + n - 1) / n);
+        piece[1] = max(piece[0], share(ctas - B / 2));
+        piece[2] = max(piece[1], share(ctas - B));
+        for (int i = 0; i < 3; ++i) inv[i] = 1.0f / (float)piece[i];
+        most = B > DEC_DOCS ? T / piece[0] : min(T / piece[0] + B, max(ctas, B));      // (up to DEC_DOCS: no more than CTAs fit, or one each)
+        pieces = B > DEC_DOCS ? most + B : most;
+        several = B > DEC_DOCS ? most >= 2 : T > piece[0];
         rows = min(Tq, DEC_ROWS);
         splits = max(1, (int)min((mean + 31LL) / 32, (4LL * PLAN_SMS + B - 1) / B));
     }
     size_t part(int Tq) const { return (size_t)most * rows + (Tq > DEC_ROWS ? (size_t)splits * Tq : 0); }      // rows of partial results in all
 };
-// x / d for 0 <= x, 0 < d, shorter than the integer division (a CTA of the decode kernel begins with three, each waiting for the one
-// before).  Both conversions and the quotient are off by 2^-21 of it at most, so below 2^20 the first guess is off by one at most.
+// x / d for 0 <= x, 0 < d, shorter than the integer division.  Both conversions and the quotient are off by 2^-21 of it at most, so below 2^20
+// the first guess is off by one at most.
 __device__ __forceinline__ int quotient(int x, int d) {
     const int q = (int)__fdividef((float)x, (float)d);
     if (q >= 1 << 20) return x / d;
@@ -95,14 +101,23 @@ __device__ __forceinline__ int quotient(int x, int d) {
     return q + (r >= d) - (r < 0);
 }
 __device__ __forceinline__ int doc_pieces(int tokens, int piece) { return max(1, quotient(tokens, piece)); }
-// P for at most DEC_DOCS documents, of `tokens` tokens this lane's; its document's pieces.  By a whole warp.
-__device__ __forceinline__ int choose_piece(const DecodePieces &p, int B, int tokens, int &n) {
-    const bool doc = (int)(threadIdx.x & 31) < B;
+// Up to DEC_DOCS documents: P, and of lane b's document (k0, k1: its tokens) the pieces n and the number `base` of the first one.
+// By a whole warp.  (The division as above: there are fewer than 2^20 pieces.)
+__device__ __forceinline__ int choose_piece(const DecodePieces &p, int B, int tokens, int &n, int &base) {
+    const int lane = threadIdx.x & 31;
     int n3[3];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) n3[i] = doc ? doc_pieces(tokens, p.piece[i]) : 0;
+    for (int i = 0; i < 3; ++i) {
+        const int q = (int)((float)tokens * p.inv[i]), r = tokens - q * p.piece[i];
+        n3[i] = lane < B ? max(1, q + (r > 0) + (r > p.piece[i]) - (r <= -p.piece[i])) : 0;
+    }
     const bool fit0 = __reduce_add_sync(0xffffffffu, n3[0]) <= p.ctas, fit1 = __reduce_add_sync(0xffffffffu, n3[1]) <= p.ctas;
     n = fit0 ? n3[0] : fit1 ? n3[1] : n3[2];
+    int end = n;
+#pragma unroll
+    for (int o = 1; o < 32; o *= 2)
+        if (o < B) { const int v = __shfl_up_sync(0xffffffffu, end, o); if (lane >= o) end += v; }
+    base = end - n;
     return fit0 ? p.piece[0] : fit1 ? p.piece[1] : p.piece[2];
 }
 // CTAs a row block's keys are dealt to in the tile kernels: enough to fill the SMs (`per_sm` CTAs each), pieces of
@@ -321,8 +336,8 @@ __global__ void __launch_bounds__(128) k_cross_zero(const int8_t *__restrict__ l
 }
 
 // ---- decoding ------------------------------------------------------------------------------------
-// CTA (x, y): a piece of a document's tokens (see DecodePieces) for its first DEC_ROWS decoder rows in turn, heads y * HC ...  The CTAs
-// behind those of the pieces take the rows beyond, DEC_ROWS of all rows and an even share of their document's
+// CTA (x, y): a piece of a document's tokens (see DecodePieces) for its decoder rows in turn, heads y * HC ...  The CTAs behind those
+// of the pieces take the documents of more than DEC_ROWS rows, DEC_ROWS of all rows and an even share of their document's
 // tokens each.  (All along x, where a grid has no limit that
 // matters; a document's CTAs follow one another, since some that lie a multiple of eight apart share a part of the
 // chip: 8 rows on one of 8 documents of 2048 tokens 28 us, so 19.)
@@ -333,7 +348,7 @@ __global__ void __launch_bounds__(128) k_cross_zero(const int8_t *__restrict__ l
 struct DecodeArgs {
     const int8_t *level;
     const int32_t *cu_k, *cu_q;
-    int B, T, level_mask, H, HC, KS, Tq, pieces;      // pieces: CTAs of the documents' first DEC_ROWS rows
+    int B, level_mask, H, HC, KS, Tq;
     DecodePieces p;
     const void *q, *k, *v;
     float scale_log2;
@@ -354,16 +369,55 @@ __device__ __forceinline__ int warp_last(int n, F le) {
     return lo;
 }
 
+// What a CTA of the decode kernel does: tokens [c0, c1), rows [row0, row1); row r leaves its partial result at part + r * step (step
+// 0: its result, since these are all the tokens).
+struct DecodeJob {
+    int c0, c1, row0, row1;
+    unsigned part, step;
+};
+// The same for more than DEC_DOCS documents, and for documents of more than DEC_ROWS rows.  By a whole warp.
+__device__ __forceinline__ void decode_job(const DecodeArgs &a, int x, DecodeJob *out) {
+    const int lane = threadIdx.x & 31;
+    DecodeJob w{};
+    int b = 0, j, n;
+    if (x < a.p.pieces) {                            // document b's pieces from number cu[b] / piece + b on: some numbers are no piece's
+        const int piece = a.p.piece[0];
+        b = warp_last(a.B, [&](int i) { return quotient(a.cu_k[i], piece) + i <= x; });
+        const int k0 = a.cu_k[b], q0 = a.cu_q[b], q1 = a.cu_q[b + 1], base = quotient(k0, piece);
+        n = doc_pieces(a.cu_k[b + 1] - k0, piece);
+        j = x - (base + b);
+        w.row0 = q0;
+        w.row1 = j >= 0 && j < n && q1 - q0 <= DEC_ROWS ? q1 : q0;
+        if (n > 1) { w.step = a.p.most; w.part = base + j - q0 * w.step; }
+    } else {                                         // DEC_ROWS of all rows hold those of two documents of more at most
+        const int groups = (a.Tq + DEC_ROWS - 1) / DEC_ROWS, y = (x - a.p.pieces) / a.p.splits, second = y >= groups, group = y - second * groups, row = DEC_ROWS * group + lane;
+        j = (x - a.p.pieces) % a.p.splits;
+        n = a.p.splits;
+        int hi = a.B;                                // its document: the last one that starts at or before the row
+        while (hi - b > 1) { const int mid = (b + hi) >> 1; if (a.cu_q[mid] <= row) b = mid; else hi = mid; }
+        const int q0 = a.cu_q[b], q1 = a.cu_q[b + 1];
+        unsigned m = __ballot_sync(0xffffffffu, lane < DEC_ROWS && q1 - q0 > DEC_ROWS && row >= q0 && row < min(a.Tq, q1)), mine = 0;
+        int f = 0, d = 0;
+        for (int i = 0; i <= second; ++i) {
+            f = m ? __ffs(m) - 1 : 0;
+            d = __shfl_sync(0xffffffffu, b, f);
+            mine = m & __ballot_sync(0xffffffffu, b == d);
+            m &= ~mine;
+        }
+        b = d;
+        w.row0 = DEC_ROWS * group + f;
+        w.row1 = w.row0 + __popc(mine);
+        if (n > 1) { w.step = 1; w.part = a.p.most * a.p.rows + j * a.Tq; }
+    }
+    const int k0 = a.cu_k[b], k1 = a.cu_k[b + 1], per = quotient(k1 - k0 + n - 1, n);
+    w.c0 = min(k1, k0 + j * per);
+    w.c1 = min(k1, w.c0 + per);
+    if (lane == 0) *out = w;
+    __syncwarp();
+}
+
 template <int D, bool BF16>
 __global__ void __launch_bounds__(512, 2) k_cross_decode(const DecodeArgs a) {
-    // What the CTA's first loads, one chain, will most likely need: into L2 while the kernel in front ends (a hint reads nothing;
-    // 4 x 8192 tokens 23.6 -> 23.2 us).
-    if (threadIdx.x < 4) {
-        const long long guess = min((long long)a.T - 1, (long long)blockIdx.x * a.T / a.pieces);       // (documents of one length)
-        const void *p = threadIdx.x == 0 ? (const void *)a.cu_k : threadIdx.x == 1 ? (const void *)a.cu_q
-                        : (const void *)(a.level + (threadIdx.x == 2 ? guess : min(a.T - 1LL, guess + 127)));
-        if (a.T > 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-    }
     pdl_wait();
     pdl_launch_dependents();
     constexpr int LPK = D / 8, C = 4;
@@ -371,8 +425,7 @@ __global__ void __launch_bounds__(512, 2) k_cross_decode(const DecodeArgs a) {
     extern __shared__ float s_red[];                 // [KS][HC][D + 2]
     __shared__ int s_list[DEC_LIST];
     __shared__ int s_n;
-    __shared__ int s_job[4];                         // tokens [0] .. [1], rows [2] .. [3]
-    __shared__ unsigned s_part[2];                   // row r leaves its partial result at [0] + r * [1]; [1] == 0: its result, since these are all the tokens
+    __shared__ DecodeJob s_job;
     const int t = threadIdx.x, lane = t & 31, g = t % LPK, src = lane - g;
     const unsigned mask = ((1u << LPK) - 1u) << src;
     const int pair = t / LPK, hl = pair % a.HC, ks = pair / a.HC, h = blockIdx.y * a.HC + hl;
@@ -394,52 +447,22 @@ __global__ void __launch_bounds__(512, 2) k_cross_decode(const DecodeArgs a) {
     };
     if (t < 32) {                                    // what to do, by one warp: the others' registers are the keys'
         const int x = blockIdx.x;
-        int b = 0, j, n, k0, k1, row0 = 0, row1 = 0;
-        unsigned part = 0, step = 0;
-        if (x < a.pieces) {
-            int q0, q1, piece = a.p.piece[0];
-            if (a.B <= DEC_DOCS) {                          // one round of loads, the documents' pieces one behind the other
-                const int i = min(lane, a.B - 1);
-                k0 = a.cu_k[i]; k1 = a.cu_k[i + 1]; q0 = a.cu_q[i]; q1 = a.cu_q[i + 1];
-                piece = choose_piece(a.p, a.B, k1 - k0, n);
-                int end = n;
-#pragma unroll
-                for (int o = 1; o < 32; o *= 2)
-                    if (o < a.B) { const int v = __shfl_up_sync(0xffffffffu, end, o); if (lane >= o) end += v; }
-                b = min(a.B - 1, __popc(__ballot_sync(0xffffffffu, lane < a.B && end <= x)));
-                j = x - __shfl_sync(0xffffffffu, end - n, b);
-                n = __shfl_sync(0xffffffffu, n, b);
-                k0 = __shfl_sync(0xffffffffu, k0, b); k1 = __shfl_sync(0xffffffffu, k1, b);
-                q0 = __shfl_sync(0xffffffffu, q0, b); q1 = __shfl_sync(0xffffffffu, q1, b);
-            } else {                                 // document b's from number cu[b] / piece + b on: some numbers are no piece's
-                b = warp_last(a.B, [&](int i) { return quotient(a.cu_k[i], piece) + i <= x; });
-                k0 = a.cu_k[b]; k1 = a.cu_k[b + 1]; q0 = a.cu_q[b]; q1 = a.cu_q[b + 1];
-                n = doc_pieces(k1 - k0, piece);
-                j = x - (quotient(k0, piece) + b);
+        if (x < a.p.pieces && a.B <= DEC_DOCS) {     // one round of loads, the documents' pieces one behind the other
+            const int i = min(lane, a.B - 1), k0 = a.cu_k[i], k1 = a.cu_k[i + 1], q0 = a.cu_q[i], q1 = a.cu_q[i + 1];
+            int n, base;
+            const int piece = choose_piece(a.p, a.B, k1 - k0, n, base), j = x - base;
+            if (lane == 0) s_job.row0 = s_job.row1 = 0;      // (a number that is no piece's)
+            __syncwarp();
+            if (j >= 0 && j < n) {                   // (one lane)
+                const int c0 = min(k1, k0 + j * piece);
+                s_job = DecodeJob{c0, min(k1, c0 + piece), q0, q1 - q0 <= DEC_ROWS ? q1 : q0, n > 1 ? x - q0 * (unsigned)a.p.most : 0u, n > 1 ? (unsigned)a.p.most : 0u};
             }
-            row0 = q0;
-            row1 = j >= 0 && j < n ? min(q1, q0 + DEC_ROWS) : q0;
-            if (n > 1) { step = a.p.most; part = quotient(k0, piece) + j - q0 * step; }
-        } else {                                     // rows behind a document's first: DEC_ROWS of all rows hold those of one document at most
-            const int group = (x - a.pieces) / a.p.splits, row = DEC_ROWS * group + lane;
-            j = (x - a.pieces) % a.p.splits;
-            n = a.p.splits;
-            int hi = a.B;                            // its document: the last one that starts at or before the row
-            while (hi - b > 1) { const int mid = (b + hi) >> 1; if (a.cu_q[mid] <= row) b = mid; else hi = mid; }
-            const unsigned m = __ballot_sync(0xffffffffu, lane < DEC_ROWS && row >= a.cu_q[b] + DEC_ROWS && row < min(a.Tq, a.cu_q[b + 1]));
-            const int f = m ? __ffs(m) - 1 : 0;
-            b = __shfl_sync(0xffffffffu, b, f);
-            row0 = DEC_ROWS * group + f;
-            row1 = row0 + __popc(m);
-            k0 = a.cu_k[b]; k1 = a.cu_k[b + 1];
-            if (n > 1) { step = 1; part = a.p.most * a.p.rows + j * a.Tq; }
-        }
-        const int per = quotient(k1 - k0 + n - 1, n), c0 = min(k1, k0 + j * per), c1 = min(k1, c0 + per);
-        if (lane == 0) { s_job[0] = c0; s_job[1] = c1; s_job[2] = row0; s_job[3] = row1; s_part[0] = part; s_part[1] = step; }
-        if (row1 > row0) list(c0, min(c1, c0 + DEC_LIST));
+            __syncwarp();
+        } else decode_job(a, x, &s_job);
+        if (s_job.row1 > s_job.row0) list(s_job.c0, min(s_job.c1, s_job.c0 + DEC_LIST));
     }
     __syncthreads();
-    const int c0 = s_job[0], c1 = s_job[1], row0 = s_job[2], row1 = s_job[3];
+    const int c0 = s_job.c0, c1 = s_job.c1, row0 = s_job.row0, row1 = s_job.row1;
     for (int row = row0; row < row1; ++row) {
         RowSoftmax S;
         S.clear();
@@ -490,11 +513,11 @@ __global__ void __launch_bounds__(512, 2) k_cross_decode(const DecodeArgs a) {
                 R.merge(d[D] * 1.4426950408889634f, d[D] > -INFINITY ? 1.f : 0.f, x);
             }
             const float lse = R.finish();
-            if (s_part[1] == 0) {
+            if (s_job.step == 0) {
                 W::store(a.o, (unsigned)row * a.H + h, g, R.acc);
                 if (g == 0) a.lse[(size_t)h * a.Tq + row] = lse;
             } else {
-                const size_t r = (size_t)(s_part[0] + row * s_part[1]) * a.H + h;
+                const size_t r = (size_t)(s_job.part + row * s_job.step) * a.H + h;
                 W::store_f32(a.part_o, r, g, R.acc);
                 if (g == 0) a.part_lse[r] = lse;
             }
@@ -522,24 +545,37 @@ __global__ void __launch_bounds__(256) k_cross_combine(int splits, int Tq, int H
     const int row = blockIdx.x, g = threadIdx.x % LPK, i = threadIdx.x / LPK, w = threadIdx.x >> 5;
     size_t first = row, step = Tq;
     if (dp.cu_k != nullptr) {         // (before the wait: the kernel in front writes neither array, and began behind what did)
-        const int b = warp_last(dp.B, [&](int x) { return dp.cu_q[x] <= row; }), r = row - dp.cu_q[b], k0 = dp.cu_k[b];
+        int r, rows, n, base;
+        if (dp.B <= DEC_DOCS) {
+            const int lane = threadIdx.x & 31, x = min(lane, dp.B - 1), q0 = dp.cu_q[x];
+            choose_piece(dp.p, dp.B, dp.cu_k[x + 1] - dp.cu_k[x], n, base);
+            const int b = max(0, __popc(__ballot_sync(0xffffffffu, lane < dp.B && q0 <= row)) - 1);
+            r = row - __shfl_sync(0xffffffffu, q0, b);
+            rows = __shfl_sync(0xffffffffu, dp.cu_q[x + 1] - q0, b);
+            n = __shfl_sync(0xffffffffu, n, b);
+            base = __shfl_sync(0xffffffffu, base, b);
+        } else {
+            const int b = warp_last(dp.B, [&](int x) { return dp.cu_q[x] <= row; }), k0 = dp.cu_k[b];
+            r = row - dp.cu_q[b];
+            rows = dp.cu_q[b + 1] - dp.cu_q[b];
+            n = doc_pieces(dp.cu_k[b + 1] - k0, dp.p.piece[0]);
+            base = quotient(k0, dp.p.piece[0]);
+        }
         if (r < 0) splits = 1;                       // (no document's row)
-        else if (r < DEC_ROWS) {
-            int piece = dp.p.piece[0];
-            if (dp.B <= DEC_DOCS) {
-                const int x = min((int)(threadIdx.x & 31), dp.B - 1);
-                piece = choose_piece(dp.p, dp.B, dp.cu_k[x + 1] - dp.cu_k[x], splits);
-            }
-            splits = doc_pieces(dp.cu_k[b + 1] - k0, piece);
-            first = (size_t)r * dp.p.most + quotient(k0, piece);
+        else if (rows <= DEC_ROWS) {
+            splits = n;
+            first = (size_t)r * dp.p.most + base;
             step = 1;
         } else first += (size_t)dp.p.most * dp.p.rows;
     }
     pdl_wait();
     pdl_launch_dependents();
     if (dp.cu_k != nullptr && splits == 1) return;      // written by the one CTA that walked the row
-    for (int h = blockIdx.y; h < H; h += gridDim.y) {
-        if (h != (int)blockIdx.y) __syncthreads();
+    // (decoding: a warp for each head where there are few partial results)
+    const bool alone = dp.cu_k != nullptr && splits <= 4 * (32 / LPK);
+    const int s0 = alone ? (threadIdx.x & 31) / LPK : i, sG = alone ? 32 / LPK : G, hw = alone ? (int)blockDim.x / 32 : 1;
+    for (int h = blockIdx.y + (alone ? w * gridDim.y : 0); h < H; h += gridDim.y * hw) {
+        if (!alone && h != (int)blockIdx.y) __syncthreads();
         RowSoftmax R;
         R.clear();
         auto add = [&](float m, float l, const f2 (&x)[4]) {
@@ -549,7 +585,7 @@ __global__ void __launch_bounds__(256) k_cross_combine(int splits, int Tq, int H
                 for (int u = 0; u < 4; ++u) R.acc[u] = add2(R.acc[u], x[u]);
         };
 #pragma unroll 4
-        for (int s = i; s < splits; s += G) {
+        for (int s = s0; s < splits; s += sG) {
             const size_t r = (first + s * step) * H + h;
             f2 x[4];
             W::load_f32(part, r, g, x);
@@ -564,14 +600,14 @@ __global__ void __launch_bounds__(256) k_cross_combine(int splits, int Tq, int H
             const float m = __shfl_xor_sync(0xffffffffu, R.m, o), l = __shfl_xor_sync(0xffffffffu, R.l, o);
             add(m, l, x);
         }
-        if ((threadIdx.x & 31) < LPK) {
+        if (!alone && (threadIdx.x & 31) < LPK) {
 #pragma unroll
             for (int u = 0; u < 4; ++u) unpack2(R.acc[u], s_red[w][8 * g + 2 * u], s_red[w][8 * g + 2 * u + 1]);
             if (g == 0) { s_red[w][D] = R.m; s_red[w][D + 1] = R.l; }
         }
-        __syncthreads();
-        if (i != 0) continue;
-        for (int j = 1; j < (int)blockDim.x / 32; ++j) {
+        if (!alone) __syncthreads();
+        if (alone ? (threadIdx.x & 31) >= LPK : i != 0) continue;
+        for (int j = 1; !alone && j < (int)blockDim.x / 32; ++j) {
             f2 x[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) x[u] = pack2(s_red[j][8 * g + 2 * u], s_red[j][8 * g + 2 * u + 1]);
@@ -607,9 +643,7 @@ static int launch_decode_t(DecodeArgs a, int B, cudaStream_t st) {
     a.KS = d.KS;
     a.B = B;
     const int threads = d.threads;
-    // (At most DEC_DOCS documents have no more pieces than CTAs fit, or one each.)
-    a.pieces = B <= DEC_DOCS ? min(a.p.most + B, max(a.p.ctas, B)) : a.p.most + B;
-    const unsigned grid = a.pieces + (a.Tq > DEC_ROWS ? (unsigned)((a.Tq + DEC_ROWS - 1) / DEC_ROWS) * a.p.splits : 0u);
+    const unsigned grid = a.p.pieces + (a.Tq > DEC_ROWS ? 2u * ((a.Tq + DEC_ROWS - 1) / DEC_ROWS) * a.p.splits : 0u);
     const size_t smem = sizeof(float) * (size_t)a.KS * a.HC * (D + 2);
     HDT_CUDA_CHECK(launch_dependent(k_cross_decode<D, BF16>, true, dim3(grid, (a.H + a.HC - 1) / a.HC), threads, smem, st, a));
     return HDT_OK;
@@ -688,12 +722,11 @@ extern "C" int hdt_cross_attn_fwd(const int8_t *level, const int32_t *cu_seqlens
         a.level = level; a.cu_k = cu_seqlens_k; a.cu_q = cu_seqlens_q; a.level_mask = level_mask; a.H = heads; a.Tq = total_q;
         const DecodePieces p(batch, total_tokens, total_q, heads, head_dim);
         a.p = p;
-        a.T = total_tokens;
         a.q = q; a.k = k; a.v = v; a.scale_log2 = scale * 1.4426950408889634f;
         a.o = o; a.lse = lse; a.part_o = part; a.part_lse = part_lse;
         if (head_dim == 64) rc = dtype == HDT_BF16 ? launch_decode_t<64, true>(a, batch, st) : launch_decode_t<64, false>(a, batch, st);
         else rc = dtype == HDT_BF16 ? launch_decode_t<128, true>(a, batch, st) : launch_decode_t<128, false>(a, batch, st);
-        if (rc || (p.most < 2 && (p.splits == 1 || total_q <= DEC_ROWS))) return rc;      // no document of several pieces
+        if (rc || (!p.several && (p.splits == 1 || total_q <= DEC_ROWS))) return rc;      // no document of several pieces
         return launch_combine(p.splits, total_q, heads, head_dim, dtype, part, part_lse, o, lse, st,
                               DecodeParts{cu_seqlens_k, cu_seqlens_q, batch, p});
     }

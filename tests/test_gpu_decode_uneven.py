@@ -1,6 +1,6 @@
 """Decoding on documents of different lengths (forward of the cross-attention with few decoder rows a document): pieces dealt by
 length, at the lengths where a document gets one more, with documents without tokens or rows, fewer and more documents than
-a warp sees at once, rows beyond a document's first eight; against the oracle."""
+a warp sees at once, documents of more than eight rows; against the oracle."""
 import numpy as np
 import pytest
 import torch
@@ -17,7 +17,10 @@ CASES = {      # tokens and decoder rows of each document, level mask, heads, he
     "one_long": ([4000] + [40] * 30, [1] * 31, 15, 12, 64),
     "long_last": ([70] * 31 + [9000], [1] * 32, 15, 12, 64),            # pieces of more than 32 tokens
     "many": ([300, 0, 5] * 20 + [2000] + [33] * 40, [1, 2, 0] * 20 + [30] + [1] * 40, 15, 4, 64),
-    "rows_on_one": ([900] + [10] * 9, [20] + [1] * 9, 15, 2, 64),       # rows behind the first eight
+    "rows_on_one": ([900] + [10] * 9, [20] + [1] * 9, 15, 2, 64),       # a document of more than eight rows
+    "rows_on_some": ([100, 300, 50, 7, 900, 40] + [20] * 8, [3, 9, 11, 8, 9, 2] + [1] * 8, 15, 2, 128),      # two of them in eight rows of all
+    "rows_on_many": ([64, 200, 5, 31] * 10, [9, 0, 1, 5] * 10, 15, 12, 64),
+    "few_parts": ([120, 250, 500, 1000], [2, 1, 8, 1], 15, 20, 64),     # a warp and a CTA of the merge a head
     "many_rows": ([3] * 350 + [5000] + [40] * 350, [1] * 701, 15, 3, 64),      # several heads to a CTA of the merge
     "no_pieces": ([20], [1], 15, 2, 64),
     "long_pieces": ([700, 1, 40000], [1, 1, 1], 15, 33, 128),           # two groups of heads
