@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(256) k_cross_index(const CrossIndexArgs a) {
 
 // Zero dK, dV rows of the encoder tokens that no decoder row attends to.  n16: 16-byte pieces of a token's row.  A warp looks 32 tokens
 // over at a time, a lane each, then writes row after row.  CTAs of 128 threads have few enough registers to run beside those of
-// the tile kernel (which leaves 4096 an SM); see hdt_cross_attn_bwd.
+// the tile kernel at head_dim 64 (which leaves 4096 an SM; at 128 it leaves none); see hdt_cross_attn_bwd.
 __global__ void __launch_bounds__(128) k_cross_zero(const int8_t *__restrict__ level, const int32_t *__restrict__ cu_k, const int32_t *__restrict__ cu_q, int B,
                                                     int T, int level_mask, int n16, uint4 *dk, uint4 *dv) {
     const int lane = threadIdx.x & 31, warps = gridDim.x * 4;
@@ -775,6 +775,8 @@ extern "C" int hdt_cross_attn_bwd(const int8_t *level, const int32_t *cu_seqlens
     // their own, beside the other kernels, from one small CTA an SM on the stream of the highest priority.  On another it starts
     // only when the last CTA of the tile kernel has (so a backward of 4 x 8192 tokens and 256 rows ended 8 us behind that
     // kernel); half as many CTAs, so that the tile kernel has more of HBM, cost 1 us more, a quarter as many 5.
+    // At head_dim 128 an SM runs either kernel's CTA, and this grid is the better one too: 16 documents of 8192 tokens, 128 rows, 16 heads
+    // 375 us, 404 with sixteen CTAs an SM, 375 on a stream of no priority; 4 x 8192 with 256 rows 162, 161, 182.
     Side *sd = nullptr;
     if (total_tokens > 0 && batch == 0) {
         HDT_CUDA_CHECK(cudaMemsetAsync(dk, 0, (size_t)total_tokens * heads * head_dim * esz, st));
