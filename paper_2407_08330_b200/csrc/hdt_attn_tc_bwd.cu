@@ -152,10 +152,15 @@ __global__ void __maxnreg__(D == 64 ? 240 : 255) k_bwd_tc(const __grid_constant_
 
     // One block; with phase_split, where most block slots may be unused (the host does not know how many tokens a
     // level subset has, the index kernel leaves the number of slots in use), as many as the grid leaves to this CTA.  (Looking
-    // at every slot's record, 1.5 us each and seven a CTA, cost a backward of 4 x 8192 tokens and 256 rows 6 us.)
+    // at every slot's record, 1.5 us each and seven a CTA, cost a backward of 4 x 8192 tokens and 256 rows 6 us.)  A CTA that starts with
+    // the grid sets up while the index kernel ends and looks at its first slot's record beside the load of the number: 300 tokens, 256 rows,
+    // 12 x 64 16 us, 18 where all begin with the number.  Of a grid that does not fit at once those that start later and those behind the
+    // phase-1 blocks, which may have nothing to do, do begin with it: 8 x 8000 tokens, 16 rows, 3 heads 29.6 us, 31.5 where they do not.
     int n_items = (int)blockIdx.x + 1;
+    const bool later = GATHER && a.phase_split > 0 && gridDim.x * gridDim.y > (unsigned)PLAN_SMS &&
+                       ((int)blockIdx.x >= a.phase_split * a.splits || blockIdx.x + gridDim.x * blockIdx.y >= (unsigned)PLAN_SMS);
     if constexpr (GATHER) {
-        if (a.phase_split > 0) {
+        if (later) {
             pdl_wait();
             n_items = a.phase_split * a.splits + min(a.nb - a.phase_split, *a.used_slots);
             if ((int)blockIdx.x >= n_items) return;
@@ -179,9 +184,13 @@ __global__ void __maxnreg__(D == 64 ? 240 : 255) k_bwd_tc(const __grid_constant_
     // (pdl = 2: what it reads is complete since the kernel of stage 0 has let this one start; it waits at its end)
     if constexpr (GATHER) {
         if (a.pdl == 2) pdl_launch_dependents();
-        else if (a.phase_split == 0) pdl_wait();
+        else if (!later) {
+            pdl_wait();
+            if (a.phase_split > 0) n_items = a.phase_split * a.splits + min(a.nb - a.phase_split, *a.used_slots);
+        }
     }
-    for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+    int item = blockIdx.x;
+    do {
     // rest_only: take the blocks after the first n_fused entries of queue_split
     int qi = item, split = 0;
     if (GATHER && a.phase_split > 0) {      // (the phase-1 blocks come first, `splits` items each)
@@ -680,7 +689,7 @@ __global__ void __maxnreg__(D == 64 ? 240 : 255) k_bwd_tc(const __grid_constant_
         copy_out(sQ, a.dv);
     }
     tc_fence_after();
-    }
+    } while ((item += gridDim.x) < n_items);
     if (warp == 0) tmem_dealloc(tmem, TM_COLS);
     if constexpr (GATHER) { if (a.pdl == 2) pdl_wait(); }      // (what follows takes its end for the end of the kernels before it too)
 }
