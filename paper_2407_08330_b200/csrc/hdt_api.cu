@@ -610,7 +610,7 @@ extern "C" int hdt_attn_bwd(const hdt_index_t *ix, const void *q, const void *k,
     // Stages above 0 of bf16 calls: the gathering tensor-core kernels (see hdt_attn_fwd).
     const bool tc_upper = dtype == HDT_BF16 && !g_force_simt && !g_simt_upper;
     // No delta pass when every kernel of this call computes dO . O of its rows itself: stage 0
-    // entirely on the looping kernels (the transposed one at head_dim 64, the fused five-MMA one at
+    // entirely on the looping kernels (k_bwd_tc_t at head_dim 64, k_bwd_tc_x at
     // head_dim 128; every block self-contained), the stages above it on the gathering tensor-core kernels.
     const bool fused_delta = dtype == HDT_BF16 && !g_force_simt && (head_dim == 64 || head_dim == 128) && g_no_persistent == 0 &&
                              !g_no_fused_delta && ix->directions == 7 && ix->desc[0].n_fused == ix->desc[0].nb &&

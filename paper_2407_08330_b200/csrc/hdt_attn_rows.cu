@@ -8,8 +8,8 @@
 // All arithmetic is fp32 (P and dS are not rounded).
 //
 // What bounds them: the latency of a row's chain of loads at the occupancy their registers leave, then instruction
-// issue (200 trees: forward 56 us, 57 % of the issue slots and 39 % of the warps active; backward 130 us, 39 % and
-// 19 %).  Of whole calls (build, forward and, with b, backward) the kernels' first form made, with all else as it was
+// issue (200 trees: forward 56 us, 57 % of the issue slots and 40 % of the warps active; backward 125 us, 41 % and
+// 20 %).  Of whole calls (build, forward and, with b, backward) the kernels' first form made, with all else as it was
 // then: 200 trees 807 -> 260 us b, one tree 280 -> 82 b, 12 layers of 1 x 4096 tokens 389 -> 295,
 // 2 x 220 tokens fp32 133 -> 46 b, 8 x 2048 padded 56 -> 51.
 //
