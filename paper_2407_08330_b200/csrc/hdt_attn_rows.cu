@@ -292,13 +292,15 @@ __global__ void __launch_bounds__(ROW_THREADS, BF16 ? 8 : 6) k_bwd_rows(const Ro
 // A CTA takes 32 (head_dim 64) or 16 (128) rows of a block and the keys of their ranges, in pieces of KT; a
 // row is owned by D / 8 lanes as above.  The elements that live on leave their partial result in stage 1's
 // buffers.  What bounds it is the chain of a key chunk (loads, products, reduction, exponential, broadcast) at the
-// six warps a scheduler holds: 2 x 2048 tokens, 12 x 64, 54 us forward and 143 backward (148 with loops that end row by row), against 100 and 191 for
+// six warps a scheduler holds: 2 x 2048 tokens, 12 x 64, 54 us forward and 138 backward (148 with loops that end row by row), against 100 and 191 for
 // the kernels that give 16 dimensions to a lane and walk a whole block's span in step.  Measured and not kept: a row
 // on 2 (forward) or 4 (backward) lanes (49 and 173 us: fewer warps, twice the registers), four and two rows to
 // eight lanes, so that a key read from shared memory serves several (58 and 213), going on to the
 // stages above 0 inside this kernel (70 and 185: one long row holds the CTA).
 // The rows of a warp walk in step: one with no keys left reads its last key again, one that has none in the piece a row of
 // zeros behind it (KT), at weight 0 both.  A key of another family there would carry an inf into a row that does not attend to it.
+// Forward and backward in step and, in brackets, with loops that end row by row: 2 x 2048 tokens, 12 x 64, 213 us (220), 12 x 128 401 (409);
+// where all CTAs fit at once and the longest walk is what counts, 1 x 3119, 12 x 64, 207 (203), 4 x 741 196 (192).
 // (KT: with the zero rows two backward CTAs take 196 KB of an SM, the step below the largest; at one row more, 228 KB, 28 instead of 60 are
 // left for L1, and 2 x 2048 tokens forward and backward take 219 us instead of 215, as much as without the zero rows.)
 static constexpr int TILE_THREADS = 256;
