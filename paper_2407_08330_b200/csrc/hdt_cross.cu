@@ -536,7 +536,7 @@ struct DecodeParts {
 // normalised rows; backward: sum.  Groups of D / 8 lanes take every G-th partial result, then meet: inside a warp by
 // shuffles, the warps through shared memory (all groups one after the other there: 0.7 us more).  Bound by the round trips to
 // L2: 256 threads where a row may have many partial results (decoding, 4 x 8192 tokens: 23.5 us a call with 128, 22.9 with 256).
-template <int D, bool BF16>
+template <int D, bool BF16, bool PACK>
 __global__ void __launch_bounds__(256) k_cross_combine(int splits, int Tq, int H, const float *part, const float *part_lse, void *out, float *lse, const DecodeParts dp) {
     constexpr int LPK = D / 8;
     const int G = blockDim.x / LPK;
@@ -571,8 +571,8 @@ __global__ void __launch_bounds__(256) k_cross_combine(int splits, int Tq, int H
     pdl_wait();
     pdl_launch_dependents();
     if (dp.cu_k != nullptr && splits == 1) return;      // written by the one CTA that walked the row
-    // (decoding: a warp for each head where there are few partial results)
-    const bool alone = dp.cu_k != nullptr && splits <= 4 * (32 / LPK);
+    // (PACK, several heads to a CTA: a warp for each where there are few partial results)
+    const bool alone = PACK && splits <= 4 * (32 / LPK);
     const int s0 = alone ? (threadIdx.x & 31) / LPK : i, sG = alone ? 32 / LPK : G, hw = alone ? (int)blockDim.x / 32 : 1;
     for (int h = blockIdx.y + (alone ? w * gridDim.y : 0); h < H; h += gridDim.y * hw) {
         if (!alone && h != (int)blockIdx.y) __syncthreads();
@@ -627,11 +627,13 @@ static int launch_combine(int splits, int Tq, int H, int D, int dtype, const flo
     const bool decode = dp.cu_k != nullptr;
     const dim3 grid(Tq, decode ? max(1, min(H, 8 * PLAN_SMS / Tq)) : H);
     const int threads = decode ? 256 : 128;
+    const bool pack = (int)grid.y < H;
+    auto launch = [&](auto kernel) { return launch_dependent(kernel, true, grid, threads, 0, st, splits, Tq, H, part, part_lse, out, lse, dp); };
     cudaError_t e;
-    if (D == 64) e = dtype == HDT_BF16 ? launch_dependent(k_cross_combine<64, true>, true, grid, threads, 0, st, splits, Tq, H, part, part_lse, out, lse, dp)
-                                       : launch_dependent(k_cross_combine<64, false>, true, grid, threads, 0, st, splits, Tq, H, part, part_lse, out, lse, dp);
-    else e = dtype == HDT_BF16 ? launch_dependent(k_cross_combine<128, true>, true, grid, threads, 0, st, splits, Tq, H, part, part_lse, out, lse, dp)
-                               : launch_dependent(k_cross_combine<128, false>, true, grid, threads, 0, st, splits, Tq, H, part, part_lse, out, lse, dp);
+    if (D == 64) e = dtype == HDT_BF16 ? launch(pack ? k_cross_combine<64, true, true> : k_cross_combine<64, true, false>)
+                                       : launch(pack ? k_cross_combine<64, false, true> : k_cross_combine<64, false, false>);
+    else e = dtype == HDT_BF16 ? launch(pack ? k_cross_combine<128, true, true> : k_cross_combine<128, true, false>)
+                               : launch(pack ? k_cross_combine<128, false, true> : k_cross_combine<128, false, false>);
     if (e != cudaSuccess) return set_error(HDT_ERR_CUDA, "launch of the combining kernel failed: %s", cudaGetErrorString(e));
     return HDT_OK;
 }
